@@ -22,6 +22,7 @@
 #include <cub/device/device_select.cuh>
 
 #include "tg_host.hpp"
+#include "tg_local.cuh"
 
 namespace tg {
 
@@ -167,17 +168,30 @@ __global__ void k_rows(int64_t n, int L, const int64_t *__restrict__ rp, const u
 }
 
 // warp per node x: its higher-priority neighbours (the part of each type
-// segment past the pivot), packed (type << 29 | id), into one contiguous list
-__global__ void k_plus_fill(GraphView g, int32_t *plus_adj) {
+// segment past the pivot), packed (type << 29 | id), into one contiguous list,
+// with the edge ids; nodes with more than kTriWarpMax of them are listed by class
+__global__ void k_plus_fill(GraphView g, int32_t *plus_adj, int32_t *plus_eid, int32_t *mid, int32_t *big,
+                            int32_t *huge, unsigned long long *counts) {
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp;
     const int lane = threadIdx.x & (kWarp - 1);
     if (warp >= g.n) return;
     const int64_t x = warp, r = g.rp[x];
     int64_t out = g.plus_off[x];
+    if (lane == 0) {
+        const int64_t p = g.plus_off[x + 1] - out;
+        if (p > kTriWarpMax) {
+            const int c = p <= kTriMidMax ? 0 : p <= kTriBigMax ? 1 : 2;
+            const unsigned long long at = atomicAdd(&counts[c], 1ull);
+            (c == 0 ? mid : c == 1 ? big : huge)[at] = (int32_t)x;
+            atomicMax(&counts[3], (unsigned long long)p);
+        }
+    }
     for (int q = 0; q < g.L; ++q) {
         const int64_t b = r + g.pivot[x * g.L + q], e = r + g.toff[x * (g.L + 1) + q + 1];
-        for (int64_t k = b + lane; k < e; k += kWarp)
+        for (int64_t k = b + lane; k < e; k += kWarp) {
             plus_adj[out + (k - b)] = (int32_t)(((uint32_t)q << kTypeShift) | (uint32_t)g.adj[k]);
+            plus_eid[out + (k - b)] = g.slot_eid[k];
+        }
         out += e - b;
     }
 }
@@ -667,11 +681,25 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
     TG_CK(cudaStreamSynchronize(s));
     if (nplus_total != m) throw Error{TG_ERR_INTERNAL, "higher-priority neighbours"};
     G.plus_adj.alloc(sizeof(int32_t) * std::max<int64_t>(m, 1));
+    G.plus_eid.alloc(sizeof(int32_t) * std::max<int64_t>(m, 1));
+    // a class holds at most m / (its smallest |N+|) nodes
+    G.tri_list[0].alloc(sizeof(int32_t) * (size_t)(m / (kTriWarpMax + 1) + 1));
+    G.tri_list[1].alloc(sizeof(int32_t) * (size_t)(m / (kTriMidMax + 1) + 1));
+    G.tri_list[2].alloc(sizeof(int32_t) * (size_t)(m / (kTriBigMax + 1) + 1));
+    TBuf counts(sizeof(unsigned long long) * 4, s);
+    TG_CK(cudaMemsetAsync(counts.p, 0, sizeof(unsigned long long) * 4, s));
     if (n > 0) {
         ++G.last_launches;
-        k_plus_fill<<<blocks_for(n * kWarp, kThreads), kThreads, 0, s>>>(G.view(), G.plus_adj.as<int32_t>());
+        k_plus_fill<<<blocks_for(n * kWarp, kThreads), kThreads, 0, s>>>(
+            G.view(), G.plus_adj.as<int32_t>(), G.plus_eid.as<int32_t>(), G.tri_list[0].as<int32_t>(),
+            G.tri_list[1].as<int32_t>(), G.tri_list[2].as<int32_t>(), counts.as<unsigned long long>());
         TG_CK(cudaGetLastError());
     }
+    unsigned long long h_counts[4];
+    TG_CK(cudaMemcpyAsync(h_counts, counts.p, sizeof(h_counts), cudaMemcpyDeviceToHost, s));
+    TG_CK(cudaStreamSynchronize(s));
+    for (int c = 0; c < 3; ++c) G.tri_count[c] = (int64_t)h_counts[c];
+    G.max_nplus = (int64_t)h_counts[3];
 }
 
 }  // namespace tg

@@ -7,7 +7,7 @@
 // on hub-heavy graphs).  Instead it gathers these typed quantities
 // (t = type of the first node, t' = type of the second):
 //
-//   c[t]        |T_ij^t| (Cor. 1), by typed set intersection       (k_tri)
+//   c[t]        |T_ij^t| (Cor. 1), each triangle found once         (k_tri_*, tg_triangles.cu)
 //   TCi[t][t']  sum_{w in T^t} c_{iw}^{t'}                         (k_tsum)
 //   TCj[t][t']  sum_{w in T^t} c_{jw}^{t'}                         (k_tsum)
 //   DT[t][t']   sum_{w in T^t} d_w^{t'}                            (k_tsum)
@@ -55,15 +55,6 @@ constexpr int kAnchorThreads = 512;         // k_wedge_heavy: one anchor per CTA
 constexpr int kLightAnchorWarps = 4;        // k_wedge_light: one anchor per warp
 constexpr int kTile = 2048;                 // most edges per tile of k_epi4 and k_edge3 (tile_edges)
 
-__device__ __forceinline__ unsigned warp_sum_u32(unsigned v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // lexicographic rank of a sorted K-multiset over [0,L): the number of
 // non-decreasing K-tuples that precede it, counted position by position.
 __device__ __forceinline__ int multichoose(int n, int r) {   // C(n + r - 1, r), n >= 1
@@ -102,144 +93,6 @@ __device__ __forceinline__ int gblock_off(int L, int b) {
 
 __device__ __forceinline__ int pair_idx(int L, int t, int u) {   // t <= u
     return t * L - t * (t - 1) / 2 + (u - t);
-}
-
-// ------------------------------------------------------------------ k_tri
-// Warp per edge: c_e^t = |Gamma_i^t cap Gamma_j^t| (Cor. 1; Thm. 2's O(Delta)).
-// Binary search form: the shorter side of every typed pair, concatenated
-// over t, is one list of sum_t min(d_i^t, d_j^t) entries that the lanes
-// stride over (so the lanes are busy across type boundaries); each entry is
-// searched in the other side's segment of its type.  Lane q < L holds type
-// q's segments; per round every lane finds its entry's type from the
-// prefix ends (in registers) and the segments by shuffles.  Hits are
-// counted by type in the 8-bit fields of one register per lane (emptied
-// every 255 rounds).  Merge form (isect): one typed pair at a time.
-struct TypedPairs {
-    int64_t sa, sb;             // lane q < L: start of the shorter / longer type-q segment
-    int32_t nb;                 // length of the longer one
-    int32_t excl;               // entries of the shorter segments of types < q
-    int32_t incl[kMaxL];        // every lane: entries of types <= q, for each q
-    int32_t total;              // entries of all shorter segments
-};
-
-// the typed pairs of edge (i, j), each side's segment of type q on lane q
-__device__ __forceinline__ void typed_pairs(const GraphView &g, int32_t i, int32_t j, int lane, TypedPairs &tp) {
-    const int L = g.L;
-    int64_t si = 0, sj = 0;
-    int32_t di = 0, dj = 0;
-    if (lane < L) {
-        const int32_t *oi = g.toff + (int64_t)i * (L + 1), *oj = g.toff + (int64_t)j * (L + 1);
-        const int32_t a0 = oi[lane], b0 = oj[lane];
-        si = g.rp[i] + a0;
-        sj = g.rp[j] + b0;
-        di = oi[lane + 1] - a0;
-        dj = oj[lane + 1] - b0;
-    }
-    const bool sw = di > dj;
-    tp.sa = sw ? sj : si;
-    tp.sb = sw ? si : sj;
-    const int32_t na = sw ? dj : di;
-    tp.nb = sw ? di : dj;
-    int32_t inc = na;
-#pragma unroll
-    for (int s = 1; s < kMaxL; s <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, inc, s);
-        if (lane >= s) inc += y;
-    }
-    tp.excl = inc - na;
-#pragma unroll
-    for (int q = 0; q < kMaxL; ++q) tp.incl[q] = __shfl_sync(0xffffffffu, inc, q);   // = total for q >= L
-    tp.total = tp.incl[kMaxL - 1];
-}
-
-template <bool kMerge>
-__global__ void __launch_bounds__(256) k_tri(GraphView g, CountView cv) {
-    const int lane = threadIdx.x & 31;
-    const int L = g.L;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; e < g.m; e += nw) {
-        const int32_t i = g.e_lo[e], j = g.e_hi[e];
-        if (kMerge) {
-            for (int t = 0; t < L; ++t) {
-                int64_t bi = seg_begin(g, i, t), ei = seg_end(g, i, t);
-                int64_t bj = seg_begin(g, j, t), ej = seg_end(g, j, t);
-                if (ei == bi || ej == bj) {                 // an empty typed segment (warp-uniform)
-                    if (lane == 0) cv.C[e * L + t] = 0;
-                    continue;
-                }
-                if (ei - bi > ej - bj) {
-                    int64_t x = bi; bi = bj; bj = x;
-                    x = ei; ei = ej; ej = x;
-                }
-                unsigned cnt = 0;
-                isect<true>(g.adj, g.isect_modes, bi, ei, bj, ej, lane,
-                            [&](bool found, int64_t, int64_t, int32_t) { cnt += found ? 1u : 0u; });
-                cnt = warp_sum_u32(cnt);
-                if (lane == 0) cv.C[e * L + t] = cnt;
-            }
-            continue;
-        }
-        TypedPairs tp;
-        typed_pairs(g, i, j, lane, tp);
-        unsigned long long acc = 0, kreg = 0;
-        int since = 0;
-        for (int32_t p0 = 0; p0 < tp.total; p0 += 32) {
-            const int32_t p = p0 + lane;
-            int t = 0;
-#pragma unroll
-            for (int q = 0; q < kMaxL - 1; ++q) t += tp.incl[q] <= p ? 1 : 0;
-            const int64_t sa = __shfl_sync(0xffffffffu, tp.sa, t);
-            const int64_t sb = __shfl_sync(0xffffffffu, tp.sb, t);
-            const int32_t nb = __shfl_sync(0xffffffffu, tp.nb, t);
-            const int32_t ex = __shfl_sync(0xffffffffu, tp.excl, t);
-            if (p < tp.total) {
-                const int32_t w = g.adj[sa + (p - ex)];
-                const int64_t r = lower_bound_i32(g.adj, sb, sb + nb, w);
-                acc += (unsigned long long)(r < sb + nb && g.adj[r] == w) << (8 * t);
-            }
-            if (++since == 255) {
-                for (int q = 0; q < L; ++q) {
-                    const unsigned v = __reduce_add_sync(0xffffffffu, (unsigned)(acc >> (8 * q)) & 0xffu);
-                    kreg += lane == q ? v : 0u;
-                }
-                acc = 0;
-                since = 0;
-            }
-        }
-        for (int q = 0; q < L; ++q) {
-            const unsigned v = __reduce_add_sync(0xffffffffu, (unsigned)(acc >> (8 * q)) & 0xffu);
-            kreg += lane == q ? v : 0u;
-        }
-        if (lane < L) cv.C[e * L + lane] = (uint32_t)kreg;
-    }
-}
-
-// ------------------------------------------------------------------ k_tau
-// Warp per node x: tau_x[t][t'] = sum_{w in Gamma_x^t} c_{xw}^{t'}, the
-// ordered adjacent pairs inside Gamma_x by type.
-__global__ void __launch_bounds__(256) k_tau(GraphView g, CountView cv) {
-    const int lane = threadIdx.x & 31;
-    const int L = g.L;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t x = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; x < g.n; x += nw) {
-        for (int t = 0; t < L; ++t) {
-            unsigned long long acc[kMaxL];
-#pragma unroll
-            for (int q = 0; q < kMaxL; ++q) acc[q] = 0;
-            for (int64_t s = seg_begin(g, x, t) + lane; s < seg_end(g, x, t); s += 32) {
-                const uint32_t *c = cv.C + (int64_t)g.slot_eid[s] * L;
-#pragma unroll
-                for (int q = 0; q < kMaxL; ++q)
-                    if (q < L) acc[q] += c[q];
-            }
-#pragma unroll
-            for (int q = 0; q < kMaxL; ++q) {
-                if (q >= L) break;
-                unsigned long long v = warp_sum_u64(acc[q]);
-                if (lane == 0) cv.tau[(x * L + t) * L + q] = (int64_t)v;
-            }
-        }
-    }
 }
 
 // ------------------------------------------------------------ wedge kernels
@@ -1007,11 +860,6 @@ struct Tile {
     int32_t graph, pad;
 };
 
-__device__ __forceinline__ unsigned long long warp_allsum_u64(unsigned long long v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // |T_e| per edge of the chunk (input of the offset scan), and the device
 // list of edges whose T is too large for one warp's 4-clique pass.
 __global__ void k_tcount(GraphView g, CountView cv, int64_t e0, int64_t e1, int64_t big_t, int64_t *tcount,
@@ -1020,7 +868,7 @@ __global__ void k_tcount(GraphView g, CountView cv, int64_t e0, int64_t e1, int6
     if (e > e1) return;
     if (e == e1) { tcount[e1 - e0] = 0; return; }
     int64_t c = 0;
-    for (int t = 0; t < g.L; ++t) c += cv.C[e * g.L + t];
+    for (int t = 0; t < g.L; ++t) c += cv.C[e * kCRow + t];
     tcount[e - e0] = c;
     if (c > big_t) {
         const unsigned long long k = atomicAdd(big_count, 1ull);
@@ -1059,7 +907,7 @@ __global__ void __launch_bounds__(256, sizeof(Acc) == 4 ? 6 : 4) k_tsum(GraphVie
         int32_t pos = 0;
         for (int t = 0; t < L; ++t) {
             Acc s1 = 0, s2 = 0, s3 = 0;                     // lane q < L: the sums over T^t for type q
-            if (cv.C[e * L + t] != 0) {
+            if (cv.C[e * kCRow + t] != 0) {
                 int64_t bi = seg_begin(g, i, t), ei = seg_end(g, i, t);
                 int64_t bj = seg_begin(g, j, t), ej = seg_end(g, j, t);
                 bool swapped = false;
@@ -1076,8 +924,8 @@ __global__ void __launch_bounds__(256, sizeof(Acc) == 4 ? 6 : 4) k_tsum(GraphVie
                     const int32_t *o = g.toff;
                     if (found) {
                         tl[pos + __popc(bal & ((1u << lane) - 1u))] = w;
-                        ci = cv.C + (int64_t)g.slot_eid[swapped ? r : s] * L;
-                        cj = cv.C + (int64_t)g.slot_eid[swapped ? s : r] * L;
+                        ci = cv.C + (int64_t)g.slot_eid[swapped ? r : s] * kCRow;
+                        cj = cv.C + (int64_t)g.slot_eid[swapped ? s : r] * kCRow;
                         o = g.toff + (int64_t)w * (L + 1);
                     }
                     pos += __popc(bal);
@@ -1111,7 +959,7 @@ __device__ __forceinline__ void t_bounds(const CountView &cv, int L, int64_t e, 
 #pragma unroll
     for (int q = 0; q <= kMaxL; ++q) {
         ts[q] = acc;
-        if (q < L) acc += (int32_t)cv.C[e * L + q];
+        if (q < L) acc += (int32_t)cv.C[e * kCRow + q];
     }
 }
 
@@ -1656,7 +1504,7 @@ __global__ void __launch_bounds__(256, 3) k_epi4(GraphView g, CountView cv, cons
             // per-type scalars, lane t < L
             long long c = 0, di = 0, dj = 0;
             if (lane < L) {
-                c = cv.C[e * L + lane];
+                c = cv.C[e * kCRow + lane];
                 di = typed_degree(g, i, lane);
                 dj = typed_degree(g, j, lane);
             }
@@ -1830,7 +1678,7 @@ __global__ void __launch_bounds__(256) k_edge3(GraphView g, CountView cv, const 
             const int32_t i = g.e_lo[e], j = g.e_hi[e];
             const int p = g.ty[i], q = g.ty[j];
             for (int t = lane; t < L; t += 32) {
-                const int64_t c = cv.C[e * L + t];
+                const int64_t c = cv.C[e * kCRow + t];
                 const int64_t a = typed_degree(g, i, t) - c - (q == t ? 1 : 0);
                 const int64_t b = typed_degree(g, j, t) - c - (p == t ? 1 : 0);
                 if (per_edge_out) {
@@ -1907,7 +1755,7 @@ __global__ void __launch_bounds__(256) k_epi4_pa(GraphView g, CountView cv, PaVi
             const int p = g.ty[i], q = g.ty[j];
             long long c = 0, di = 0, dj = 0;
             if (lane < L) {
-                c = cv.C[e * L + lane];
+                c = cv.C[e * kCRow + lane];
                 di = typed_degree(g, i, lane);
                 dj = typed_degree(g, j, lane);
             }
@@ -2159,7 +2007,7 @@ static const Tile *tiles_for(Graph &G, int64_t e_begin, int64_t e_end, int64_t &
 __global__ void k_chunk_t(GraphView g, CountView cv, int64_t e0, int64_t e1, unsigned long long *out) {
     unsigned long long acc = 0;
     for (int64_t e = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < e1; e += (int64_t)gridDim.x * blockDim.x)
-        for (int t = 0; t < g.L; ++t) acc += cv.C[e * g.L + t];
+        for (int t = 0; t < g.L; ++t) acc += cv.C[e * kCRow + t];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, acc);
 }
@@ -2244,27 +2092,6 @@ void prepare_edges(Graph &G, int k, cudaStream_t s) {
         const size_t smem = (size_t)kLightAnchorWarps * cap * (1 + G.L) * sizeof(int32_t);
         raise_smem_limit((const void *)k_wedge_light, smem);
     }
-}
-
-// typed triangles per edge and per-node typed triangle sums: whole graph
-static int64_t launch_triangles(Graph &G, cudaStream_t s) {
-    const GraphView gv = G.view();
-    const CountView cv = G.cview();
-    const int sms = sm_count();
-    int64_t launches = 0;
-    if (G.m > 0) {
-        KernelTimer kt(G, s, "k_tri");
-        if (isect_any_merge(G.opt.isect_modes)) k_tri<true><<<grid_for(G.m, 8, sms * 16), 256, 0, s>>>(gv, cv);
-        else k_tri<false><<<grid_for(G.m, 8, sms * 16), 256, 0, s>>>(gv, cv);
-        ++launches;
-    }
-    if (G.n > 0) {
-        KernelTimer kt(G, s, "k_tau");
-        k_tau<<<grid_for(G.n, 8, sms * 16), 256, 0, s>>>(gv, cv);
-        ++launches;
-    }
-    TG_CK(cudaGetLastError());
-    return launches;
 }
 
 // Triangle-node entries of every chunk (a graph invariant, computed once
@@ -2616,8 +2443,9 @@ static int64_t launch_edges4(Graph &G, int64_t b, int64_t e, const Tile *tiles, 
 void prepare_counting(Graph &G, int k, cudaStream_t s) {
     const int L = G.L;
     const size_t m = (size_t)std::max<int64_t>(G.m, 1), n = (size_t)std::max<int64_t>(G.n, 1);
-    if (G.C.bytes < m * L * sizeof(uint32_t)) G.C.alloc(m * L * sizeof(uint32_t));
+    if (G.C.bytes < m * kCRow * sizeof(uint32_t)) G.C.alloc(m * kCRow * sizeof(uint32_t));
     if (G.tau.bytes < n * L * L * sizeof(int64_t)) G.tau.alloc(n * L * L * sizeof(int64_t));
+    prepare_triangles(G);
     const size_t gbytes = (size_t)G.ngraphs * global_slots(L, 4) * sizeof(unsigned long long);
     if (G.gacc.bytes < gbytes) G.gacc.alloc(gbytes);
     if (k == 4) {
@@ -2657,7 +2485,7 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
 // For a captured count: the T list size needs one k_tri before capture.
 void prepare_capture(Graph &G, int k, cudaStream_t s) {
     if (k == 4 && G.chunk_t.empty()) {
-        launch_triangles(G, s);
+        launch_triangles(G, true, s);
         ensure_t_sizes(G, s);
     }
 }
@@ -2665,9 +2493,11 @@ void prepare_capture(Graph &G, int k, cudaStream_t s) {
 int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per_edge_out, unsigned long long *gacc,
                   bool full, cudaStream_t s) {
     int64_t launches = 0;
-    if (full || G.prepared_k < 3) {
-        launches += launch_triangles(G, s);
+    // prepared_k 3: typed triangles only (all that k = 3 reads); 4: their per-node sums too
+    if (full || G.prepared_k < 3 || (k == 4 && !G.tau_ready)) {
+        launches += launch_triangles(G, k == 4, s);
         G.prepared_k = std::max(G.prepared_k, 3);
+        G.tau_ready = G.tau_ready || k == 4;
     }
     DBuf tmp;                                                // tiles of a range, stream-ordered
     tmp.owner = &G.stream;

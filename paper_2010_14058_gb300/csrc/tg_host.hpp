@@ -129,7 +129,10 @@ struct Graph {
 
     // graph (built once)
     DBuf node_off, edge_off, rp, adj, toff, pivot, nplus, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
-    DBuf plus_off, plus_adj;
+    DBuf plus_off, plus_adj, plus_eid;
+    // nodes by |N+| (tg_local.cuh): mid, big, and larger than shared memory holds
+    DBuf tri_list[3], local_scratch;
+    int64_t tri_count[3] = {0, 0, 0}, max_nplus = 0;
     // work lists
     DBuf anchors_light, anchors_heavy, edges_light, edges_heavy;
     int64_t n_anchors_light = 0, n_anchors_heavy = 0, n_edges_light = 0, n_edges_heavy = 0;
@@ -179,7 +182,8 @@ struct Graph {
     int64_t e_base = 0;
     int64_t table_stride = 0;
     int32_t n_tables = 0;
-    int32_t prepared_k = 0;             // 0: nothing, 3: C and tau, 4: C, tau and A
+    int32_t prepared_k = 0;             // 0: nothing, 3: C, 4: C and the chunk's per-slot and per-edge sums
+    bool tau_ready = false;             // tau of the current C
     int64_t last_launches = 0;
     // per-kernel event timing (tg_set_timing)
     bool timing = false;
@@ -217,6 +221,7 @@ struct Graph {
         v.delta = delta.as<int64_t>();
         v.plus_off = plus_off.as<int64_t>();
         v.plus_adj = plus_adj.as<int32_t>();
+        v.plus_eid = plus_eid.as<int32_t>();
         return v;
     }
     CountView cview() const {
@@ -251,7 +256,7 @@ struct Graph {
                              &e_slot_lo, &e_slot_hi, &delta, &anchors_light, &anchors_heavy, &edges_light,
                              &edges_heavy, &C, &tau, &A, &tables, &gacc, &status, &tiles_full, &stage_pe,
                              &stage_gl, &tcount, &toffs, &tlist, &tsum, &kmat, &big_list, &big_count, &scan_tmp,
-                             &set_scratch, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &hubs, &hub_base, &item_woff, &item_rec,
+                             &set_scratch, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
@@ -311,6 +316,20 @@ int sm_count();
 void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_t n, int64_t nnz,
                  const int64_t *row_ptr, const int32_t *col, const uint8_t *types, int32_t L,
                  const tg_options &opt, cudaStream_t s);
+
+// One class of nodes u by |N+(u)| and its launch shape (tg_local.cuh).
+struct LocalClass {
+    int64_t n;                  // nodes
+    const int32_t *list;
+    int threads, cap, lgf;      // CTA size, list capacity, log2 bits of the id filter
+};
+LocalClass local_class(const Graph &G, int cls);
+
+// shared-memory limits and scratch of launch_triangles (before any capture)
+void prepare_triangles(Graph &G);
+// typed triangles per edge and, with_tau, the per-node sums of the whole
+// graph (tg_triangles.cu); returns the kernel launches
+int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s);
 
 // count entries (tg_count.cu)
 void prepare_counting(Graph &G, int k, cudaStream_t s);

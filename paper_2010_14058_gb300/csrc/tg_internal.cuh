@@ -28,6 +28,7 @@ enum : uint32_t {
 
 constexpr int kMaxL = TG_MAX_TYPES;
 constexpr int kWarp = 32;
+constexpr int kCRow = 8;                           // words per row of typed triangle counts (one 32-byte sector)
 constexpr int kTypeShift = 29;                     // packed (type << 29 | id) sort keys
 constexpr int32_t kIdMask = (1 << kTypeShift) - 1;
 constexpr int kHeavyCap = 4096;                    // shared-memory hash rows of a heavy anchor
@@ -77,11 +78,12 @@ struct GraphView {
     const int64_t *plus_off;   // [n+1] start of x's higher-priority neighbours in plus_adj
     const int32_t *plus_adj;   // [m] higher-priority neighbours of each node, (type << 29 | id),
                                // grouped by type in (type, id) order
+    const int32_t *plus_eid;   // [m] edge id of each entry of plus_adj
 };
 
 // Per-count working arrays.
 struct CountView {
-    uint32_t *C;                // [m*L]   typed triangle counts c_e^t
+    uint32_t *C;                // [m][kCRow] typed triangle counts c_e^t (t < L)
     int64_t *tau;               // [n*L*L] ordered typed edges inside Gamma_x
     uint32_t *A;                // [L*L][a_stride] 4-cycle contributions per slot of the current chunk
     int64_t a_base;             // first adjacency slot of the current chunk
