@@ -8,12 +8,10 @@
 // (t = type of the first node, t' = type of the second):
 //
 //   c[t]        |T_ij^t| (Cor. 1), each triangle found once         (k_tri_*, tg_triangles.cu)
-//   TCi[t][t']  sum_{w in T^t} c_{iw}^{t'}                         (k_tsum)
-//   TCj[t][t']  sum_{w in T^t} c_{jw}^{t'}                         (k_tsum)
-//   DT[t][t']   sum_{w in T^t} d_w^{t'}                            (k_tsum)
-//   K[t][t']    ordered adjacent pairs (w,x) in T^t x T^t' (each pair is found
-//               once, from its smaller id, by k_clique / k_clique_big; the
-//               epilogue adds the transpose)
+//   TCi[t][t']  sum_{w in T^t} c_{iw}^{t'}                         (k_sum_*, tg_sums.cu)
+//   TCj[t][t']  sum_{w in T^t} c_{jw}^{t'}                         (k_sum_*)
+//   DT[t][t']   sum_{w in T^t} d_w^{t'}                            (k_sum_*)
+//   K[t][t']    ordered adjacent pairs (w,x) in T^t x T^t'          (k_sum_*)
 //   P[t][t']    3-paths j - w - r - i, w of type t, r of type t'   (k_wedge*)
 //   tau_x[t][t'] ordered adjacent pairs inside Gamma_x              (k_tau)
 //   delta_x[t][t'] sum_{w in Gamma_x^t} d_w^{t'}                    (build)
@@ -803,16 +801,10 @@ __global__ void __launch_bounds__(kHubThreads, 5) k_wedge_hub(GraphView g, Count
 }
 
 // ------------------------------------------------------------ per-edge 4-node
-// The per-edge stage runs as three lean warp-per-edge kernels with the
-// per-edge intermediates in HBM (all indexed relative to the chunk's first
-// edge e_base):
-//   k_tsum    T list of the edge (sorted by (type, id)) and the sums TCi, TCj,
-//             DT over its triangle nodes;
-//   k_clique  K: adjacent pairs inside T (warp per edge; CTA per edge for
-//             the edges with |T| above a threshold, collected on the device);
-//   k_epi4    every orbit of Table 3 from the gathered sums, one warp per
-//             edge with the L x L matrices held one entry per lane and
-//             transposed by shuffles; writes the row and the CTA histogram.
+// k_epi4: every orbit of Table 3 from the gathered sums (tg_sums.cu, the
+// wedge pass and the per-node sums), one warp per edge with the L x L
+// matrices held one entry per lane and transposed by shuffles; writes the
+// row and the CTA histogram.
 
 __device__ __forceinline__ uint32_t sat32(int64_t v, uint32_t *status) {
     if (v > 0xffffffffll) {
@@ -860,575 +852,6 @@ struct Tile {
     int32_t graph, pad;
 };
 
-// |T_e| per edge of the chunk (input of the offset scan), and the device
-// list of edges whose T is too large for one warp's 4-clique pass.
-__global__ void k_tcount(GraphView g, CountView cv, int64_t e0, int64_t e1, int64_t big_t, int64_t *tcount,
-                         int32_t *big_list, unsigned long long *big_count) {
-    const int64_t e = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e > e1) return;
-    if (e == e1) { tcount[e1 - e0] = 0; return; }
-    int64_t c = 0;
-    for (int t = 0; t < g.L; ++t) c += cv.C[e * kCRow + t];
-    tcount[e - e0] = c;
-    if (c > big_t) {
-        const unsigned long long k = atomicAdd(big_count, 1ull);
-        big_list[k] = (int32_t)e;
-    }
-}
-
-// Warp per edge: T list and the triangle-node sums (Cor. 1; gathers of the
-// typed triangle counts of the edges (i,w), (j,w) and of d_w^t').  The
-// sums of one type t are held by lane t' (three registers per lane); each
-// round of 32 candidates adds the found nodes' terms with one warp
-// reduction per (sum, t').  Acc = uint32_t when the maximum degree is below
-// 2^16 (every sum here is then below 2^32 and a warp reduction of 32 terms
-// below 2^21), else unsigned long long (terms split into 16-bit halves for
-// the 32-bit reductions).
-__device__ __forceinline__ unsigned long long warp_total(uint32_t v, uint32_t) {
-    return __reduce_add_sync(0xffffffffu, v);
-}
-__device__ __forceinline__ unsigned long long warp_total(uint32_t v, unsigned long long) {
-    const unsigned long long lo = __reduce_add_sync(0xffffffffu, v & 0xffffu);
-    const unsigned long long hi = __reduce_add_sync(0xffffffffu, v >> 16);
-    return lo + (hi << 16);
-}
-
-template <class Acc, bool kMerge>
-__global__ void __launch_bounds__(256, sizeof(Acc) == 4 ? 6 : 4) k_tsum(GraphView g, CountView cv, int64_t e0,
-                                                                        int64_t e1) {
-    const int L = g.L, LL = L * L;
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = e0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); e < e1; e += nw) {
-        const int64_t er = e - e0;
-        const int32_t i = g.e_lo[e], j = g.e_hi[e];
-        int32_t *tl = cv.tlist + cv.toffs[er];
-        unsigned long long *sum = cv.tsum + er * 3 * LL;
-        int32_t pos = 0;
-        for (int t = 0; t < L; ++t) {
-            Acc s1 = 0, s2 = 0, s3 = 0;                     // lane q < L: the sums over T^t for type q
-            if (cv.C[e * kCRow + t] != 0) {
-                int64_t bi = seg_begin(g, i, t), ei = seg_end(g, i, t);
-                int64_t bj = seg_begin(g, j, t), ej = seg_end(g, j, t);
-                bool swapped = false;
-                if (ei - bi > ej - bj) {
-                    int64_t x = bi; bi = bj; bj = x;
-                    x = ei; ei = ej; ej = x;
-                    swapped = true;
-                }
-                isect<kMerge>(g.adj, g.isect_modes, bi, ei, bj, ej, lane, [&](bool found, int64_t s, int64_t r,
-                                                                                 int32_t w) {
-                    const unsigned bal = __ballot_sync(0xffffffffu, found);
-                    if (bal == 0) return;                   // warp-uniform
-                    const uint32_t *ci = cv.C, *cj = cv.C;
-                    const int32_t *o = g.toff;
-                    if (found) {
-                        tl[pos + __popc(bal & ((1u << lane) - 1u))] = w;
-                        ci = cv.C + (int64_t)g.slot_eid[swapped ? r : s] * kCRow;
-                        cj = cv.C + (int64_t)g.slot_eid[swapped ? s : r] * kCRow;
-                        o = g.toff + (int64_t)w * (L + 1);
-                    }
-                    pos += __popc(bal);
-                    for (int q = 0; q < L; ++q) {
-                        const uint32_t v1 = found ? ci[q] : 0u;
-                        const uint32_t v2 = found ? cj[q] : 0u;
-                        const uint32_t v3 = found ? (uint32_t)(o[q + 1] - o[q]) : 0u;
-                        const unsigned long long t1 = warp_total(v1, Acc()), t2 = warp_total(v2, Acc());
-                        const unsigned long long t3 = warp_total(v3, Acc());
-                        if (lane == q) {
-                            s1 += (Acc)t1;
-                            s2 += (Acc)t2;
-                            s3 += (Acc)t3;
-                        }
-                    }
-                });
-            }
-            if (lane < L) {
-                sum[t * L + lane] = (unsigned long long)s1;
-                sum[LL + t * L + lane] = (unsigned long long)s2;
-                sum[2 * LL + t * L + lane] = (unsigned long long)s3;
-            }
-        }
-    }
-}
-
-// type boundaries of an edge's T list, from its typed triangle counts
-// (indices unrolled, so ts[] stays in registers)
-__device__ __forceinline__ void t_bounds(const CountView &cv, int L, int64_t e, int32_t *ts) {
-    int32_t acc = 0;
-#pragma unroll
-    for (int q = 0; q <= kMaxL; ++q) {
-        ts[q] = acc;
-        if (q < L) acc += (int32_t)cv.C[e * kCRow + q];
-    }
-}
-
-// type of T's member k (0 <= k < |T|): ts[q] = |T| > k for q >= L
-__device__ __forceinline__ int type_of_index(const int32_t *ts, int32_t k) {
-    int t = 0;
-#pragma unroll
-    for (int q = 1; q < kMaxL; ++q) t += ts[q] <= k ? 1 : 0;
-    return t;
-}
-
-// ------------------------------------------------------------- 4-cliques
-// K[t][t'] of an edge counts the adjacent pairs (w, x) inside T, w of type
-// t and x of type t', each pair once, from its lower-priority node w: x is
-// then one of w's higher-priority neighbours N+(w) (a contiguous list of
-// (type << 29 | id) entries grouped by type, built once per graph).  So
-// every member w of T scans N+(w) and looks each entry up in a set of T:
-// sum_{w in T} |N+(w)| lookups.
-//
-// The set.  Ids are degree ranks, and on power-law graphs the members of T
-// and the entries of their N+ lists crowd at the top of the id range: the
-// members within B below the largest member tmax (B = 2^13 for a warp's
-// edge, 2^15 for a CTA's) take over 98% of the lookups on the graphs
-// measured.  When at least 3/4 of the members lie in that window, they are
-// a bitmap indexed by tmax - x (one 32-bit shared-memory load per lookup)
-// and the members below it a hash set, looked up only by entries between
-// the smallest member and the window.  Otherwise all members are in the
-// hash set.  The hash set: buckets of 4 slots (one 16-byte load per
-// lookup), slots taken in order by atomicCAS, -1 when empty, so a bucket
-// whose last slot is empty is not full and a lookup stops there; with at
-// least 4 slots per member almost every lookup reads one bucket.  The
-// bitmap is all zero between edges: the words of an edge's members are
-// cleared after its scan.
-// The scan: one whole warp per member, lanes striding over N+(w) (coalesced
-// loads, 4 in flight per lane) -- the lists behind almost all lookups are
-// tens to thousands of entries long.  A window lookup has no branch; the
-// hash lookups (entries between the smallest member and the window, and
-// every entry within T's range in the hash form) are taken by the lanes
-// that need them, once per round of four, when any lane of the warp
-// does.  Only members below the window check for them: N+(w) holds ids
-// above w, so a member in the window meets no member below it.  Each lane
-// counts its hits by
-// type of x in the fields of one register (no warp-wide step inside the
-// scan, so a lane's four lookups overlap); the warp sums the fields with
-// __reduce_add_sync before any can overflow and when the member type t
-// changes (T is sorted by type), and lane q adds the count for x of type q
-// to K[t][q].
-
-__device__ __forceinline__ uint32_t t_hash(int32_t x, int lgnb) {      // lgnb >= 1
-    return ((uint32_t)x * 2654435761u) >> (32 - lgnb);
-}
-
-__device__ __forceinline__ void group_sync(int gsize) {
-    if (gsize > 32) __syncthreads(); else __syncwarp();
-}
-
-// the members x <= xmax of T (nT distinct ids) in 2^lgnb buckets, built by the group
-__device__ void tset_build(const int32_t *T, int32_t nT, int4 *set, int lgnb, int gsize, int gr, int32_t xmax) {
-    const int nb = 1 << lgnb;
-    int32_t *slot = reinterpret_cast<int32_t *>(set);
-    for (int k = gr; k < 4 * nb; k += gsize) slot[k] = -1;
-    group_sync(gsize);
-    for (int32_t k = gr; k < nT; k += gsize) {
-        const int32_t x = T[k];
-        if (x > xmax) continue;
-        uint32_t b = t_hash(x, lgnb);
-        bool done = false;
-        for (int probe = 0; probe < nb && !done; ++probe) {   // 4 nb >= 2 nT: a free slot exists
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (!done) done = atomicCAS(&slot[4 * b + q], -1, x) == -1;
-            b = (b + 1) & (nb - 1);
-        }
-    }
-    group_sync(gsize);
-}
-
-__device__ __forceinline__ bool bucket_has(const int4 &k, int32_t x) {
-    return (k.x == x) | (k.y == x) | (k.z == x) | (k.w == x);
-}
-
-__device__ __forceinline__ bool tset_has(const int4 *set, int lgnb, int32_t x) {
-    uint32_t b = t_hash(x, lgnb);
-    int4 k = set[b];
-    if (bucket_has(k, x)) return true;
-    if (k.w == -1) return false;                            // the bucket is not full
-    const int nb = 1 << lgnb;                               // rare: continue in the next buckets
-    for (int probe = 1; probe < nb; ++probe) {
-        b = (b + 1) & (nb - 1);
-        k = set[b];
-        if (bucket_has(k, x)) return true;
-        if (k.w == -1) return false;
-    }
-    return false;
-}
-
-// buckets for nT members: 4 slots per member when they fit max_slots, else
-// 2 (2^lgnb buckets of 4 slots); -1 when even that exceeds max_slots
-__device__ __forceinline__ int tset_lgnb(int32_t nT, int max_slots) {
-    int lg = 1;
-    while ((4 << lg) < 4 * nT) ++lg;
-    if ((4 << lg) <= max_slots) return lg;
-    lg = 1;
-    while ((4 << lg) < 2 * nT) ++lg;
-    return (4 << lg) <= max_slots ? lg : -1;
-}
-
-// T of one edge: the window bitmap and the hash set
-struct TWin {
-    const uint32_t *bm;         // bit d: member tmax - d, for d < wbits; word wbits / 32 is zero
-    const int4 *set;            // the members below the window (all of them in the hash form)
-    int32_t tmax, tmin, lowmax; // lowmax: the largest id the hash set may hold, else -1
-    uint32_t wbits;             // the window's width: B, or 0 in the hash form
-    uint32_t lowspan;           // ids tmin .. tmin + lowspan - 1 are looked up in the hash set
-    int lgnb;
-};
-
-// smallest and largest member of T (each type's run is in increasing id order)
-__device__ __forceinline__ void t_range(const int32_t *T, const int32_t *ts, int L, int32_t &tmin, int32_t &tmax) {
-    tmin = INT32_MAX;
-    tmax = -1;
-#pragma unroll
-    for (int q = 0; q < kMaxL; ++q) {
-        if (q < L && ts[q + 1] > ts[q]) {
-            tmin = min(tmin, T[ts[q]]);
-            tmax = max(tmax, T[ts[q + 1] - 1]);
-        }
-    }
-}
-
-// members of the group (strided by gsize from gr) below the window of B
-template <int B>
-__device__ __forceinline__ int32_t twin_below(const int32_t *T, int32_t nT, int32_t tmax, int gsize, int gr) {
-    int32_t low = 0;
-    for (int32_t k = gr; k < nT; k += gsize) low += (uint32_t)(tmax - T[k]) >= (uint32_t)B ? 1 : 0;
-    return low;
-}
-
-// sets (or, set = false, clears the words of) the window bits of the group's members
-template <int B>
-__device__ __forceinline__ void twin_bits(const int32_t *T, int32_t nT, int32_t tmax, uint32_t *bm, int gsize, int gr,
-                                          bool set) {
-    for (int32_t k = gr; k < nT; k += gsize) {
-        const uint32_t d = (uint32_t)(tmax - T[k]);
-        if (d < (uint32_t)B) {
-            if (set) atomicOr(&bm[d >> 5], 1u << (d & 31u));
-            else bm[d >> 5] = 0u;
-        }
-    }
-}
-
-// Per-lane hit counters of one warp: field q (F bits of `acc`) counts the
-// lane's hits on entries of type q; `since` counts scan rounds (at most 4
-// hits per field each) since the fields were last emptied into `kreg`,
-// where lane q holds the warp's count for type q.  Two layouts: 6-bit
-// fields in 32 bits for L <= 5 (emptied every 15 rounds), 8-bit fields in
-// 64 bits otherwise (every 63).  Warp-uniform control flow.
-template <class A>
-struct CliqueAcc {
-    static constexpr int F = sizeof(A) == 4 ? 6 : 8;
-    static constexpr int R = ((1 << F) - 1) / 4;
-    A acc = 0;
-    unsigned long long kreg = 0;
-    int since = 0;
-    __device__ __forceinline__ void add(bool hit, uint32_t ent) {
-        acc += (A)hit << (F * (ent >> kTypeShift));
-    }
-    __device__ __forceinline__ void add_bit(uint32_t bit, uint32_t ent) {   // bit: 0 or 1
-        acc += (A)bit << (F * (ent >> kTypeShift));
-    }
-    __device__ __forceinline__ void drain(int L) {
-        for (int q = 0; q < L; ++q) {
-            const unsigned v = __reduce_add_sync(0xffffffffu, (unsigned)(acc >> (F * q)) & ((1u << F) - 1u));
-            kreg += (threadIdx.x & 31) == (unsigned)q ? (unsigned long long)v : 0ull;
-        }
-        acc = 0;
-        since = 0;
-    }
-};
-
-// lanes q < L add the warp's counts to K[tw][q]
-template <class A>
-__device__ __forceinline__ void flush_k(CliqueAcc<A> &a, int tw, unsigned long long *K, int L, int lane, bool shared_k) {
-    a.drain(L);
-    if (tw >= 0 && lane < L && a.kreg) {
-        if (shared_k) atomicAdd(&K[tw * kMaxL + lane], a.kreg);
-        else K[tw * kMaxL + lane] += a.kreg;
-    }
-    a.kreg = 0;
-}
-
-// one lookup of entry `ent` (slot u of a round): the window bit (d is
-// clamped to wbits, whose word and bit are always zero) counted at once,
-// and bit u of `slow` set when the entry falls in the hash set's range
-template <bool kSlow, class A>
-__device__ __forceinline__ void look(const TWin &tw, uint32_t ent, CliqueAcc<A> &a, unsigned &slow, int u) {
-    const int32_t x = (int32_t)(ent & (uint32_t)kIdMask);
-    const uint32_t d = min((uint32_t)(tw.tmax - x), tw.wbits);
-    const uint32_t word = tw.bm[d >> 5];
-    a.add_bit(__funnelshift_r(word, 0u, d) & 1u, ent);       // bit d % 32 of the word
-    if (kSlow) slow |= ((uint32_t)(x - tw.tmin) < tw.lowspan ? 1u : 0u) << u;
-}
-
-// the hash lookups of the round's slow entries, when any lane has one
-template <bool kSlow, class A>
-__device__ __forceinline__ void look_slow(const TWin &tw, const uint32_t *ent, CliqueAcc<A> &a, unsigned slow) {
-    if (kSlow && __any_sync(0xffffffffu, slow != 0u)) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if ((slow >> u) & 1u) a.add(tset_has(tw.set, tw.lgnb, (int32_t)(ent[u] & (uint32_t)kIdMask)), ent[u]);
-    }
-}
-
-// member w of T: the whole warp scans N+(w), 128 entries a round (full
-// rounds without bounds checks, then the partial one); returns |N+(w)|.
-// kSlow: w may have hash-set members in N+(w), i.e. w <= lowmax (N+(w)
-// holds ids above w only, so a member in the window meets window members
-// only).
-template <bool kSlow, class A>
-__device__ __forceinline__ int32_t scan_list(const GraphView &g, int32_t w, const TWin &tw, CliqueAcc<A> &a,
-                                             int lane) {
-    const int64_t pb = g.plus_off[w];
-    const int32_t np = (int32_t)(g.plus_off[w + 1] - pb);
-    const int32_t *p = g.plus_adj + pb + lane;
-    int32_t r0 = 0;
-    for (; r0 + 128 <= np; r0 += 128, p += 128) {
-        uint32_t ent[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ent[u] = (uint32_t)__ldg(p + 32 * u);
-        unsigned slow = 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) look<kSlow>(tw, ent[u], a, slow, u);
-        look_slow<kSlow>(tw, ent, a, slow);
-        if (++a.since == CliqueAcc<A>::R) a.drain(g.L);
-    }
-    if (r0 < np) {
-        // entries past the list are looked up as id kIdMask of type 0, above
-        // every member: no hit, and not in the hash set's range
-        uint32_t ent[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ent[u] = r0 + 32 * u + lane < np ? (uint32_t)__ldg(p + 32 * u) : 0u;
-        unsigned slow = 0, valid = 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool v = r0 + 32 * u + lane < np;
-            valid |= (v ? 1u : 0u) << u;
-            uint32_t e = v ? ent[u] : (uint32_t)kIdMask;    // an id above every member: no hit, not slow
-            look<kSlow>(tw, e, a, slow, u);
-        }
-        look_slow<kSlow>(tw, ent, a, slow & valid);
-        if (++a.since == CliqueAcc<A>::R) a.drain(g.L);
-    }
-    return np;
-}
-
-template <class A>
-__device__ __forceinline__ int32_t scan_member(const GraphView &g, int32_t w, const TWin &tw, CliqueAcc<A> &a,
-                                               int lane) {
-    return w <= tw.lowmax ? scan_list<true>(g, w, tw, a, lane) : scan_list<false>(g, w, tw, a, lane);
-}
-
-// the members of T, warp-serially, into K (sK) by member type
-template <class A>
-__device__ __forceinline__ unsigned long long scan_members_warp(const GraphView &g, const int32_t *T, int32_t nT,
-                                                                const int32_t *ts, const TWin &tw,
-                                                                unsigned long long *sK, int lane) {
-    CliqueAcc<A> acc;
-    unsigned long long probes = 0;
-    int t = -1;
-    for (int32_t k = 0; k < nT; ++k) {
-        const int tk = type_of_index(ts, k);
-        if (tk != t) {
-            flush_k(acc, t, sK, g.L, lane, false);
-            t = tk;
-        }
-        probes += (unsigned long long)scan_member(g, T[k], tw, acc, lane);
-    }
-    flush_k(acc, t, sK, g.L, lane, false);
-    return probes;
-}
-
-// few pairs: every pair (a, b) of T checked by a binary search in the
-// smaller id's typed row; K by (type of smaller, type of larger)
-__device__ void clique_pairs_search(const GraphView &g, const int32_t *T, int32_t nT, const int32_t *ts,
-                                    unsigned long long *sK, int gsize, int gr) {
-    const long long npair = (long long)nT * (nT - 1) / 2;
-    for (long long pk = gr; pk < npair; pk += gsize) {
-        int32_t a = 0;
-        long long rem = pk;
-        while (rem >= nT - 1 - a) { rem -= nT - 1 - a; ++a; }
-        const int32_t b = a + 1 + (int32_t)rem;
-        int32_t w = T[a], x = T[b];
-        int tw = type_of_index(ts, a), tx = type_of_index(ts, b);
-        if (x < w) { int32_t y = w; w = x; x = y; int ty = tw; tw = tx; tx = ty; }
-        const int64_t sb = seg_begin(g, w, tx), se = seg_end(g, w, tx);
-        const int64_t r = lower_bound_i32(g.adj, sb, se, x);
-        if (r < se && g.adj[r] == x) atomicAdd(&sK[tw * kMaxL + tx], 1ull);
-    }
-}
-
-// optional diagnostic work counters (bench): lookups of the scans, pair searches
-__device__ __forceinline__ void add_work(unsigned long long *work, int slot, unsigned long long v, int lane) {
-    if (work && lane == 0 && v) atomicAdd(&work[slot], v);
-}
-
-// the window form when at least 3/4 of the members lie in the window
-__device__ __forceinline__ bool use_window(int32_t nlow, int32_t nT) { return 4 * nlow <= nT; }
-
-// Warp per edge (edges with |T| <= big_t): K into kmat.  A = the counter
-// register type (uint32_t for L <= 5).
-constexpr int kCliqueWarpSlots = 1024;       // per-warp set: 4 slots per member up to |T| = 256
-constexpr int kCliqueWarpWin = 1 << 13;      // per-warp window bits (1 KB)
-template <class A>
-__global__ void __launch_bounds__(256, 5) k_clique(GraphView g, CountView cv, int64_t e0, int64_t e1, int64_t big_t) {
-    __shared__ unsigned long long sKw[8][kMaxL * kMaxL];
-    __shared__ int4 setw[8][kCliqueWarpSlots / 4];
-    __shared__ uint32_t bmw[8][kCliqueWarpWin / 32 + 1];   // + the zero word of clamped lookups
-    const int L = g.L, LL = L * L;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long *sK = sKw[wid];
-    uint32_t *bm = bmw[wid];
-    for (int k = lane; k <= kCliqueWarpWin / 32; k += 32) bm[k] = 0u;
-    __syncwarp();
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = e0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); e < e1; e += nw) {
-        const int64_t er = e - e0;
-        const int32_t nT = (int32_t)(cv.toffs[er + 1] - cv.toffs[er]);
-        if (nT > big_t) continue;                           // done by k_clique_big
-        unsigned long long *km = cv.kmat + er * LL;
-        if (nT < 2) {
-            for (int k = lane; k < LL; k += 32) km[k] = 0;
-            continue;
-        }
-        for (int k = lane; k < kMaxL * kMaxL; k += 32) sK[k] = 0;
-        __syncwarp();
-        int32_t ts[kMaxL + 1];
-        t_bounds(cv, L, e, ts);
-        const int32_t *T = cv.tlist + cv.toffs[er];
-        const long long npair = (long long)nT * (nT - 1) / 2;
-        if (npair <= 64) {
-            clique_pairs_search(g, T, nT, ts, sK, 32, lane);
-            add_work(cv.work, kWorkCliqueSearches, (unsigned long long)npair, lane);
-        } else {
-            TWin tw;
-            t_range(T, ts, L, tw.tmin, tw.tmax);
-            const int32_t nlow = (int32_t)__reduce_add_sync(
-                0xffffffffu, (unsigned)twin_below<kCliqueWarpWin>(T, nT, tw.tmax, 32, lane));
-            const bool win = use_window(nlow, nT);
-            const int32_t nset = win ? nlow : nT;           // members in the hash set
-            tw.bm = bm;
-            tw.set = setw[wid];
-            tw.wbits = win ? kCliqueWarpWin : 0u;
-            tw.lowmax = !win ? tw.tmax : nlow > 0 ? tw.tmax - kCliqueWarpWin : -1;
-            tw.lowspan = tw.lowmax >= tw.tmin ? (uint32_t)(tw.lowmax - tw.tmin) + 1u : 0u;
-            tw.lgnb = nset > 0 ? tset_lgnb(nset, kCliqueWarpSlots) : 1;   // nset <= 256: 4 slots per member
-            if (tw.lgnb < 0) {                              // the options clamp big_t to 256
-                if (lane == 0) set_status(cv.status, ST_INTERNAL);
-                continue;
-            }
-            if (win) twin_bits<kCliqueWarpWin>(T, nT, tw.tmax, bm, 32, lane, true);
-            if (nset > 0) tset_build(T, nT, setw[wid], tw.lgnb, 32, lane, tw.lowmax);
-            else __syncwarp();                              // (tset_build ends with __syncwarp)
-            const unsigned long long probes = scan_members_warp<A>(g, T, nT, ts, tw, sK, lane);
-            add_work(cv.work, kWorkCliqueProbes, probes, lane);
-            __syncwarp();
-            if (win) twin_bits<kCliqueWarpWin>(T, nT, tw.tmax, bm, 32, lane, false);
-        }
-        __syncwarp();
-        for (int k = lane; k < LL; k += 32) km[k] = sK[(k / L) * kMaxL + (k % L)];
-        __syncwarp();
-    }
-}
-
-// the members of T taken by the CTA's warps from a shared counter (in
-// order, so each warp's member types only rise)
-template <class A>
-__device__ __forceinline__ unsigned long long big_members(const GraphView &g, const int32_t *T, int32_t nT,
-                                                          const int32_t *ts, const TWin &tw, unsigned long long *sK,
-                                                          int *next, int lane) {
-    CliqueAcc<A> acc;
-    unsigned long long probes = 0;
-    int t = -1;
-    for (;;) {
-        int32_t m = 0;
-        if (lane == 0) m = atomicAdd(next, 1);
-        m = __shfl_sync(0xffffffffu, m, 0);
-        if (m >= nT) break;
-        const int tm = type_of_index(ts, m);
-        if (tm != t) {
-            flush_k(acc, t, sK, g.L, lane, true);
-            t = tm;
-        }
-        probes += (unsigned long long)scan_member(g, T[m], tw, acc, lane);
-    }
-    flush_k(acc, t, sK, g.L, lane, true);
-    return probes;
-}
-
-// CTA per edge for the listed edges with a large T; the hash set lives in
-// shared memory up to kBigSetSmem slots, else in this CTA's global slice
-// (2 slots per member).
-constexpr int kBigSetSmem = 1 << 13;
-constexpr int kBigThreads = 256;
-constexpr int kBigWin = 1 << 15;             // window bits (4 KB)
-template <class A>
-__global__ void __launch_bounds__(kBigThreads, 5) k_clique_big(GraphView g, CountView cv, int64_t e0,
-                                                          const int32_t *__restrict__ big_list,
-                                                          const unsigned long long *__restrict__ big_count,
-                                                          int32_t *set_scratch, int64_t set_stride) {
-    __shared__ unsigned long long sK[kMaxL * kMaxL];
-    __shared__ uint32_t bm[kBigWin / 32 + 1];            // + the zero word of clamped lookups
-    __shared__ int s_next, s_low;
-    extern __shared__ int4 set_smem[];
-    const int L = g.L, LL = L * L;
-    const int lane = threadIdx.x & 31;
-    const int64_t nb = (int64_t)*big_count;
-    unsigned long long probes = 0;
-    for (int x = threadIdx.x; x <= kBigWin / 32; x += blockDim.x) bm[x] = 0u;
-    for (int64_t k = blockIdx.x; k < nb; k += gridDim.x) {
-        const int64_t e = big_list[k];
-        const int64_t er = e - e0;
-        const int32_t nT = (int32_t)(cv.toffs[er + 1] - cv.toffs[er]);
-        for (int x = threadIdx.x; x < kMaxL * kMaxL; x += blockDim.x) sK[x] = 0;
-        if (threadIdx.x == 0) {
-            s_next = 0;
-            s_low = 0;
-        }
-        int32_t ts[kMaxL + 1];
-        t_bounds(cv, L, e, ts);
-        const int32_t *T = cv.tlist + cv.toffs[er];
-        TWin tw;
-        t_range(T, ts, L, tw.tmin, tw.tmax);
-        __syncthreads();                                    // s_low zero, the previous edge done
-        const unsigned low = __reduce_add_sync(0xffffffffu,
-                                               (unsigned)twin_below<kBigWin>(T, nT, tw.tmax, blockDim.x, threadIdx.x));
-        if (lane == 0 && low) atomicAdd(&s_low, (int)low);
-        __syncthreads();
-        const int32_t nlow = s_low;
-        const bool win = use_window(nlow, nT);              // CTA-uniform
-        const int32_t nset = win ? nlow : nT;
-        tw.bm = bm;
-        tw.wbits = win ? kBigWin : 0u;
-        tw.lowmax = !win ? tw.tmax : nlow > 0 ? tw.tmax - kBigWin : -1;
-        tw.lowspan = tw.lowmax >= tw.tmin ? (uint32_t)(tw.lowmax - tw.tmin) + 1u : 0u;
-        const int32_t xmax = tw.lowmax;
-        if (win) twin_bits<kBigWin>(T, nT, tw.tmax, bm, blockDim.x, threadIdx.x, true);
-        const int lgs = nset > 0 ? tset_lgnb(nset, kBigSetSmem) : 1;
-        if (lgs >= 0) {
-            tw.set = set_smem;
-            tw.lgnb = lgs;
-            if (nset > 0) tset_build(T, nT, set_smem, lgs, blockDim.x, threadIdx.x, xmax);   // ends with a barrier
-            else __syncthreads();
-        } else {                                            // global slice: 2^lg >= 2 nset slots
-            int lg = 1;
-            while ((4 << lg) < 2 * nset) ++lg;
-            int4 *set = reinterpret_cast<int4 *>(set_scratch + (int64_t)blockIdx.x * set_stride);
-            tw.set = set;
-            tw.lgnb = lg;
-            tset_build(T, nT, set, lg, blockDim.x, threadIdx.x, xmax);
-        }
-        probes += big_members<A>(g, T, nT, ts, tw, sK, &s_next, lane);
-        __syncthreads();
-        for (int x = threadIdx.x; x < LL; x += blockDim.x) cv.kmat[er * LL + x] = sK[(x / L) * kMaxL + (x % L)];
-        if (win) twin_bits<kBigWin>(T, nT, tw.tmax, bm, blockDim.x, threadIdx.x, false);
-        __syncthreads();
-    }
-    add_work(cv.work, kWorkCliqueBigProbes, probes, lane);
-}
-
 // value of matrix entry k (0 <= k < L*L) held as (r0 on lane k, or r1 on lane k-32)
 __device__ __forceinline__ long long mat_get(long long r0, long long r1, int k) {
     const long long v0 = __shfl_sync(0xffffffffu, r0, k & 31);
@@ -1451,6 +874,7 @@ __host__ __device__ __forceinline__ size_t epi4_smem_bytes(int L, int copies) {
            (size_t)(L * L + L * L * L + L * L * P + 1) * sizeof(uint16_t);
 }
 
+template <class Acc>
 __global__ void __launch_bounds__(256, 3) k_epi4(GraphView g, CountView cv, const Tile *__restrict__ tiles,
                                              int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
                                              unsigned long long *gacc, int copies) {
@@ -1511,8 +935,8 @@ __global__ void __launch_bounds__(256, 3) k_epi4(GraphView g, CountView cv, cons
             const long long a = di - c - (q == lane ? 1 : 0);  // |S_i^t|
             const long long b = dj - c - (p == lane ? 1 : 0);  // |S_j^t|
             // gathered matrices
-            const unsigned long long *sum = cv.tsum + er * 3 * LL;
-            const unsigned long long *km = cv.kmat + er * LL;
+            const Acc *sum = reinterpret_cast<const Acc *>(cv.xsum) + er * 4 * LL;
+            const long long cA = lane_get(c, xA < L ? xA : 0), cB = lane_get(c, xB < L ? xB : 0);
             const int64_t *tau_i = cv.tau + (int64_t)i * LL, *tau_j = cv.tau + (int64_t)j * LL;
             const int64_t *del_i = g.delta + (int64_t)i * LL, *del_j = g.delta + (int64_t)j * LL;
             const uint32_t *A = cv.A - cv.a_base;
@@ -1524,10 +948,13 @@ __global__ void __launch_bounds__(256, 3) k_epi4(GraphView g, CountView cv, cons
                 const bool has = h ? hasB : hasA;
                 const int k = h ? kB : kA, x = h ? xB : xA, y = h ? yB : yA;
                 if (has) {
-                    TCi[h] = (long long)sum[k];
-                    TCj[h] = (long long)sum[LL + k];
-                    DT[h] = (long long)sum[2 * LL + k];
-                    Kd[h] = (long long)km[k];
+                    if (h ? cB : cA) {                       // rows of types without a triangle node are not kept
+                        const Acc *r = sum + x * 4 * L + y;
+                        TCi[h] = (long long)r[0];
+                        TCj[h] = (long long)r[L];
+                        DT[h] = (long long)r[2 * L];
+                        Kd[h] = (long long)r[3 * L];
+                    }
                     // P[x][y]: slot i->j holds [type next to i][type next to j], slot j->i the reverse
                     Pm[h] = (long long)A[(int64_t)(y * L + x) * cv.a_stride + sij] +
                             (long long)A[(int64_t)(x * L + y) * cv.a_stride + sji];
@@ -1537,10 +964,10 @@ __global__ void __launch_bounds__(256, 3) k_epi4(GraphView g, CountView cv, cons
                     dJ[h] = del_j[k];
                 }
             }
-            // Ks = K + K^T
+            // Ks: ordered adjacent pairs of T (K' + K'^T counts each twice)
             long long Ks[2];
-            Ks[0] = Kd[0] + mat_get(Kd[0], Kd[1], hasA ? tA : 0);
-            Ks[1] = Kd[1] + mat_get(Kd[0], Kd[1], hasB ? tB : 0);
+            Ks[0] = (Kd[0] + mat_get(Kd[0], Kd[1], hasA ? tA : 0)) >> 1;
+            Ks[1] = (Kd[1] + mat_get(Kd[0], Kd[1], hasB ? tB : 0)) >> 1;
             // CTi, CTj
             long long CTi[2], CTj[2];
 #pragma unroll
@@ -1725,6 +1152,7 @@ struct PaView {
 
 __host__ __device__ __forceinline__ size_t epi4_pa_hist_words(int G) { return (size_t)((G + 1) & ~1); }
 
+template <class Acc>
 __global__ void __launch_bounds__(256) k_epi4_pa(GraphView g, CountView cv, PaView pv, const Tile *__restrict__ tiles,
                                                  int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
                                                  unsigned long long *gacc, int copies) {
@@ -1761,8 +1189,8 @@ __global__ void __launch_bounds__(256) k_epi4_pa(GraphView g, CountView cv, PaVi
             }
             const long long a = di - c - (q == lane ? 1 : 0);  // |S_i^t|
             const long long b = dj - c - (p == lane ? 1 : 0);  // |S_j^t|
-            const unsigned long long *sum = cv.tsum + er * 3 * LL;
-            const unsigned long long *km = cv.kmat + er * LL;
+            const Acc *sum = reinterpret_cast<const Acc *>(cv.xsum) + er * 4 * LL;
+            const long long cA = lane_get(c, xA < L ? xA : 0), cB = lane_get(c, xB < L ? xB : 0);
             const int64_t *tau_i = cv.tau + (int64_t)i * LL, *tau_j = cv.tau + (int64_t)j * LL;
             const int64_t *del_i = g.delta + (int64_t)i * LL, *del_j = g.delta + (int64_t)j * LL;
             const uint32_t *A = cv.A - cv.a_base;
@@ -1774,10 +1202,13 @@ __global__ void __launch_bounds__(256) k_epi4_pa(GraphView g, CountView cv, PaVi
                 const bool has = h ? hasB : hasA;
                 const int k = h ? kB : kA, x = h ? xB : xA, y = h ? yB : yA;
                 if (has) {
-                    TCi[h] = (long long)sum[k];
-                    TCj[h] = (long long)sum[LL + k];
-                    DT[h] = (long long)sum[2 * LL + k];
-                    Kd[h] = (long long)km[k];
+                    if (h ? cB : cA) {                       // rows of types without a triangle node are not kept
+                        const Acc *r = sum + x * 4 * L + y;
+                        TCi[h] = (long long)r[0];
+                        TCj[h] = (long long)r[L];
+                        DT[h] = (long long)r[2 * L];
+                        Kd[h] = (long long)r[3 * L];
+                    }
                     Pm[h] = (long long)A[(int64_t)(y * L + x) * cv.a_stride + sij] +
                             (long long)A[(int64_t)(x * L + y) * cv.a_stride + sji];
                     ti_[h] = tau_i[k];
@@ -1787,8 +1218,8 @@ __global__ void __launch_bounds__(256) k_epi4_pa(GraphView g, CountView cv, PaVi
                 }
             }
             long long Ks[2];
-            Ks[0] = Kd[0] + mat_get(Kd[0], Kd[1], hasA ? tA : 0);
-            Ks[1] = Kd[1] + mat_get(Kd[0], Kd[1], hasB ? tB : 0);
+            Ks[0] = (Kd[0] + mat_get(Kd[0], Kd[1], hasA ? tA : 0)) >> 1;
+            Ks[1] = (Kd[1] + mat_get(Kd[0], Kd[1], hasB ? tB : 0)) >> 1;
             long long CTi[2], CTj[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -1951,11 +1382,11 @@ static std::vector<Tile> make_tiles(const Graph &G, int64_t e_begin, int64_t e_e
 static void plan_chunks(Graph &G) {
     G.chunks.clear();
     // working bytes of a chunk: the 4-cycle array (4 L^2 per slot) and the
-    // per-edge sums, K and offsets (32 L^2 + 28 per edge)
+    // per-edge sums (4 L^2 words per edge)
     const int64_t LL = (int64_t)G.L * G.L;
     const int64_t budget = std::max<int64_t>((int64_t)G.opt.cycle_budget_mb << 20, 1);
     auto bytes_of = [&](int a, int b) {
-        return (G.h_slot_off[b] - G.h_slot_off[a]) * 4 * LL + (G.h_edge_off[b] - G.h_edge_off[a]) * (32 * LL + 28);
+        return (G.h_slot_off[b] - G.h_slot_off[a]) * 4 * LL + (G.h_edge_off[b] - G.h_edge_off[a]) * LL * (G.wide_sums() ? 32 : 16);
     };
     // tile index ranges follow graph boundaries (make_tiles emits graph after graph)
     std::vector<int64_t> tile_off(G.ngraphs + 1, 0);
@@ -2003,15 +1434,6 @@ static const Tile *tiles_for(Graph &G, int64_t e_begin, int64_t e_end, int64_t &
     return dst.as<Tile>();
 }
 
-// |T_e| summed over the edges of each chunk (from c_e^t)
-__global__ void k_chunk_t(GraphView g, CountView cv, int64_t e0, int64_t e1, unsigned long long *out) {
-    unsigned long long acc = 0;
-    for (int64_t e = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < e1; e += (int64_t)gridDim.x * blockDim.x)
-        for (int t = 0; t < g.L; ++t) acc += cv.C[e * kCRow + t];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0 && acc) atomicAdd(out, acc);
-}
-
 int light_anchor_limit(int L) {
     int dev = 0, optin = 0;
     TG_CK(cudaGetDevice(&dev));
@@ -2054,8 +1476,9 @@ static int epi4_pa_copies(int G) {
 }
 
 void prepare_epi4_pa(Graph &G) {
-    raise_smem_limit((const void *)k_epi4_pa,
-                     epi4_pa_hist_words((int)G.pa.G) * epi4_pa_copies((int)G.pa.G) * sizeof(unsigned long long));
+    const size_t bytes = epi4_pa_hist_words((int)G.pa.G) * epi4_pa_copies((int)G.pa.G) * sizeof(unsigned long long);
+    raise_smem_limit((const void *)k_epi4_pa<uint32_t>, bytes);
+    raise_smem_limit((const void *)k_epi4_pa<unsigned long long>, bytes);
 }
 
 static PaView pa_view(const Graph &G) {
@@ -2070,18 +1493,9 @@ static PaView pa_view(const Graph &G) {
 
 void prepare_edges(Graph &G, int k, cudaStream_t s) {
     raise_smem_limit((const void *)k_edge3, hist_bytes(G.L, 3));
-    raise_smem_limit((const void *)k_epi4, epi4_smem_bytes(G.L, epi4_copies(G.L)));
-    raise_smem_limit((const void *)k_clique_big<uint32_t>, kBigSetSmem * sizeof(int32_t));
-    raise_smem_limit((const void *)k_clique_big<unsigned long long>, kBigSetSmem * sizeof(int32_t));
+    raise_smem_limit((const void *)k_epi4<uint32_t>, epi4_smem_bytes(G.L, epi4_copies(G.L)));
+    raise_smem_limit((const void *)k_epi4<unsigned long long>, epi4_smem_bytes(G.L, epi4_copies(G.L)));
     raise_smem_limit((const void *)k_wedge_heavy, (size_t)kHeavyCap * (1 + G.L) * sizeof(int32_t));
-    if (k == 4 && !G.set_scratch.p) {
-        // a set of capacity >= 2 max degree per CTA, for edges whose T exceeds shared memory
-        int64_t cap = 1;
-        while (cap < 2 * std::max<int64_t>(G.max_degree, 1)) cap <<= 1;
-        G.big_blocks = sm_count() * 5;
-        G.set_stride = cap > kBigSetSmem ? cap : 1;
-        G.set_scratch.alloc(sizeof(int32_t) * (size_t)(G.set_stride * G.big_blocks));
-    }
     DBuf unused;
     unused.owner = &G.stream;
     int64_t nt = 0;
@@ -2091,33 +1505,6 @@ void prepare_edges(Graph &G, int k, cudaStream_t s) {
         while (cap < 2 * G.opt.light_anchor_max_wedges) cap <<= 1;
         const size_t smem = (size_t)kLightAnchorWarps * cap * (1 + G.L) * sizeof(int32_t);
         raise_smem_limit((const void *)k_wedge_light, smem);
-    }
-}
-
-// Triangle-node entries of every chunk (a graph invariant, computed once
-// after the first k_tri; synchronises) and the T list buffer sized for the
-// largest chunk.
-static void ensure_t_sizes(Graph &G, cudaStream_t s) {
-    if (!G.chunk_t.empty()) return;
-    TBuf cnt(sizeof(unsigned long long) * G.chunks.size(), s);
-    TG_CK(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long) * G.chunks.size(), s));
-    const GraphView gv = G.view();
-    const CountView cv = G.cview();
-    for (size_t x = 0; x < G.chunks.size(); ++x) {
-        const Graph::Chunk &c = G.chunks[x];
-        if (c.e1 > c.e0)
-            k_chunk_t<<<grid_for(c.e1 - c.e0, 256, sm_count() * 8), 256, 0, s>>>(gv, cv, c.e0, c.e1,
-                                                                               cnt.as<unsigned long long>() + x);
-    }
-    TG_CK(cudaGetLastError());
-    std::vector<unsigned long long> h(G.chunks.size());
-    TG_CK(cudaMemcpyAsync(h.data(), cnt.p, sizeof(unsigned long long) * h.size(), cudaMemcpyDeviceToHost, s));
-    TG_CK(cudaStreamSynchronize(s));
-    G.chunk_t.assign(h.begin(), h.end());
-    const int64_t cap = std::max<int64_t>(*std::max_element(G.chunk_t.begin(), G.chunk_t.end()), 1);
-    if (G.tlist_cap < cap) {
-        G.tlist.alloc(sizeof(int32_t) * (size_t)cap);
-        G.tlist_cap = cap;
     }
 }
 
@@ -2366,72 +1753,36 @@ static int64_t launch_wedges(Graph &G, const Graph::Chunk &c, cudaStream_t s) {
     return launches;
 }
 
-// per-edge 4-node stage of edges [b, e) (inside one chunk, whose wedge pass
-// is in A): T offsets, T lists and sums, K, orbits
-static int64_t launch_edges4(Graph &G, int64_t b, int64_t e, const Tile *tiles, int64_t n_tiles, int64_t row_base,
-                             uint32_t *per_edge_out, unsigned long long *gacc, cudaStream_t s) {
+// orbits of edges [b, e) (inside one chunk, whose wedge pass and sums are done)
+static int64_t launch_edges4(Graph &G, const Graph::Chunk &c, int64_t b, int64_t e, const Tile *tiles, int64_t n_tiles,
+                             int64_t row_base, uint32_t *per_edge_out, unsigned long long *gacc, cudaStream_t s) {
     if (e <= b) return 0;
-    G.e_base = b;
+    G.a_base = c.s0;
+    G.e_base = c.e0;
     const GraphView gv = G.view();
     const CountView cv = G.cview();
     const int sms = sm_count();
-    const int64_t ne = e - b;
-    const int64_t big_t = std::max<int64_t>(G.opt.light_edge_max_degree, 32);
     int64_t launches = 0;
-    TG_CK(cudaMemsetAsync(G.big_count.p, 0, sizeof(unsigned long long), s));
-    {
-        KernelTimer kt(G, s, "k_tcount");
-        k_tcount<<<grid_for(ne + 1, 256, 1 << 30), 256, 0, s>>>(gv, cv, b, e, big_t, G.tcount.as<int64_t>(),
-                                                                G.big_list.as<int32_t>(),
-                                                                G.big_count.as<unsigned long long>());
-        ++launches;
-    }
-    size_t tmp_bytes = G.scan_tmp_bytes;
-    TG_CK(cub::DeviceScan::ExclusiveSum(G.scan_tmp.p, tmp_bytes, G.tcount.as<int64_t>(), G.toffs.as<int64_t>(),
-                                        ne + 1, s));
-    {
-        KernelTimer kt(G, s, "k_tsum");
-        const unsigned grid = (unsigned)grid_for(ne, 8, sms * 32);
-        const bool merge = isect_any_merge(G.opt.isect_modes);
-        if (G.max_degree < (1 << 16)) {
-            if (merge) k_tsum<uint32_t, true><<<grid, 256, 0, s>>>(gv, cv, b, e);
-            else k_tsum<uint32_t, false><<<grid, 256, 0, s>>>(gv, cv, b, e);
-        } else {
-            if (merge) k_tsum<unsigned long long, true><<<grid, 256, 0, s>>>(gv, cv, b, e);
-            else k_tsum<unsigned long long, false><<<grid, 256, 0, s>>>(gv, cv, b, e);
-        }
-        ++launches;
-    }
-    {
-        KernelTimer kt(G, s, "k_clique");
-        if (G.L <= 5) k_clique<uint32_t><<<grid_for(ne, 8, sms * 32), 256, 0, s>>>(gv, cv, b, e, big_t);
-        else k_clique<unsigned long long><<<grid_for(ne, 8, sms * 32), 256, 0, s>>>(gv, cv, b, e, big_t);
-        ++launches;
-    }
-    {
-        KernelTimer kt(G, s, "k_clique_big");
-        if (G.L <= 5)
-            k_clique_big<uint32_t><<<G.big_blocks, 256, kBigSetSmem * sizeof(int32_t), s>>>(
-                gv, cv, b, G.big_list.as<int32_t>(), G.big_count.as<unsigned long long>(), G.set_scratch.as<int32_t>(),
-                G.set_stride);
-        else
-            k_clique_big<unsigned long long><<<G.big_blocks, 256, kBigSetSmem * sizeof(int32_t), s>>>(
-                gv, cv, b, G.big_list.as<int32_t>(), G.big_count.as<unsigned long long>(), G.set_scratch.as<int32_t>(),
-                G.set_stride);
-        ++launches;
-    }
     if (n_tiles > 0 && G.pa_active) {
         KernelTimer kt(G, s, "k_epi4_pa");
         const int copies = epi4_pa_copies((int)G.pa.G);
-        k_epi4_pa<<<grid_for(n_tiles, 1, sms * G.opt.ctas_per_sm), 256,
-                    epi4_pa_hist_words((int)G.pa.G) * copies * sizeof(unsigned long long), s>>>(
-            gv, cv, pa_view(G), tiles, n_tiles, row_base, per_edge_out, gacc, copies);
+        auto launch = [&](auto kern) {
+            kern<<<grid_for(n_tiles, 1, sms * G.opt.ctas_per_sm), 256,
+                   epi4_pa_hist_words((int)G.pa.G) * copies * sizeof(unsigned long long), s>>>(
+                gv, cv, pa_view(G), tiles, n_tiles, row_base, per_edge_out, gacc, copies);
+        };
+        if (G.wide_sums()) launch(k_epi4_pa<unsigned long long>);
+        else launch(k_epi4_pa<uint32_t>);
         ++launches;
     } else if (n_tiles > 0) {
         KernelTimer kt(G, s, "k_epi4");
         const int copies = epi4_copies(G.L);
-        k_epi4<<<grid_for(n_tiles, 1, sms * G.opt.ctas_per_sm), 256, epi4_smem_bytes(G.L, copies), s>>>(
-            gv, cv, tiles, n_tiles, row_base, per_edge_out, gacc, copies);
+        auto launch = [&](auto kern) {
+            kern<<<grid_for(n_tiles, 1, sms * G.opt.ctas_per_sm), 256, epi4_smem_bytes(G.L, copies), s>>>(
+                gv, cv, tiles, n_tiles, row_base, per_edge_out, gacc, copies);
+        };
+        if (G.wide_sums()) launch(k_epi4<unsigned long long>);
+        else launch(k_epi4<uint32_t>);
         ++launches;
     }
     TG_CK(cudaGetLastError());
@@ -2444,6 +1795,7 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
     const int L = G.L;
     const size_t m = (size_t)std::max<int64_t>(G.m, 1), n = (size_t)std::max<int64_t>(G.n, 1);
     if (G.C.bytes < m * kCRow * sizeof(uint32_t)) G.C.alloc(m * kCRow * sizeof(uint32_t));
+    if (G.tri_any.bytes < n) G.tri_any.alloc(n);
     if (G.tau.bytes < n * L * L * sizeof(int64_t)) G.tau.alloc(n * L * L * sizeof(int64_t));
     prepare_triangles(G);
     const size_t gbytes = (size_t)G.ngraphs * global_slots(L, 4) * sizeof(unsigned long long);
@@ -2453,19 +1805,9 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
         const size_t ab = (size_t)G.a_stride * L * L * sizeof(uint32_t);
         if (G.A.bytes < ab) G.A.alloc(ab);
         const size_t me = (size_t)std::max<int64_t>(G.max_chunk_edges, 1);
-        if (G.tcount.bytes < (me + 1) * sizeof(int64_t)) {
-            G.tcount.alloc((me + 1) * sizeof(int64_t));
-            G.toffs.alloc((me + 1) * sizeof(int64_t));
-            G.tsum.alloc(me * 3 * L * L * sizeof(unsigned long long));
-            G.kmat.alloc(me * L * L * sizeof(unsigned long long));
-            G.big_list.alloc(me * sizeof(int32_t));
-            G.big_count.alloc(sizeof(unsigned long long));
-            size_t tb = 0;
-            TG_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, G.tcount.as<int64_t>(), G.toffs.as<int64_t>(),
-                                                (int64_t)me + 1, s));
-            G.scan_tmp.alloc(tb);
-            G.scan_tmp_bytes = tb;
-        }
+        const size_t xb = me * 4 * L * L * (G.wide_sums() ? sizeof(unsigned long long) : sizeof(uint32_t));
+        if (G.xsum.bytes < xb) G.xsum.alloc(xb);
+        prepare_sums(G);
         if (G.n_hubs > 0 && !G.hubs_ready) prepare_hubs(G, s);
         if (G.n_hubs > 0 && G.hub_plans.empty()) plan_hubs(G, s);
         if (G.n_anchors_heavy > 0 && G.n_tables == 0) {
@@ -2479,14 +1821,6 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
             G.table_stride = stride;
             G.n_tables = (int32_t)nt;
         }
-    }
-}
-
-// For a captured count: the T list size needs one k_tri before capture.
-void prepare_capture(Graph &G, int k, cudaStream_t s) {
-    if (k == 4 && G.chunk_t.empty()) {
-        launch_triangles(G, true, s);
-        ensure_t_sizes(G, s);
     }
 }
 
@@ -2514,19 +1848,18 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
             TG_CK(cudaGetLastError());
         }
     } else {
-        ensure_t_sizes(G, s);
         const bool whole = e_begin == 0 && e_end == G.m;
         std::vector<Tile> host;
         if (!whole) host = make_tiles(G, e_begin, e_end);
         for (const Graph::Chunk &c : G.chunks) {
             const int64_t b = std::max(e_begin, c.e0), e = std::min(e_end, c.e1);
             if (b >= e) continue;
-            // the wedge pass of a single-chunk handle is reused by later range calls
+            // the wedge pass and sums of a single-chunk handle are reused by later range calls
             if (full || G.chunks.size() > 1 || G.prepared_k != 4) {
+                launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
                 launches += launch_wedges(G, c, s);
                 if (G.chunks.size() == 1) G.prepared_k = 4;
             }
-            G.a_base = c.s0;
             const Tile *ct = tiles;
             int64_t nct = n_tiles;
             if (whole) {
@@ -2540,7 +1873,7 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
                 ct = tiles + a;
                 nct = y - a;
             }
-            launches += launch_edges4(G, b, e, ct, nct, e_begin, per_edge_out, gacc, s);
+            launches += launch_edges4(G, c, b, e, ct, nct, e_begin, per_edge_out, gacc, s);
         }
     }
     if (tmp.p) TG_CK(cudaStreamSynchronize(s));

@@ -171,14 +171,10 @@ struct Graph {
     bool hub_packed = false;                    // two 16-bit counters per word
     // counting state
     DBuf C, tau, A, tables, gacc, status, tiles_full, stage_pe, stage_gl;
-    DBuf tcount, toffs, tlist, tsum, kmat, big_list, big_count, scan_tmp, set_scratch;
+    DBuf xsum, tri_any;
     DBuf work;                          // [kWorkSlots] work counters (tg_set_work_counting)
     bool work_on = false;
-    int64_t set_stride = 1;
-    int32_t big_blocks = 1;
-    int64_t n_tiles_full = 0, max_chunk_edges = 0, tlist_cap = 0;
-    size_t scan_tmp_bytes = 0;
-    std::vector<int64_t> chunk_t;       // triangle-node entries per chunk (graph invariant)
+    int64_t n_tiles_full = 0, max_chunk_edges = 0;
     int64_t e_base = 0;
     int64_t table_stride = 0;
     int32_t n_tables = 0;
@@ -201,6 +197,8 @@ struct Graph {
     const void *batch_pe = nullptr, *batch_gl = nullptr;
     cudaStream_t batch_stream = nullptr;
 
+    // sums over triangle nodes may reach 2^32 only when a degree reaches 2^16
+    bool wide_sums() const { return max_degree >= (1 << 16); }
     GraphView view() const {
         GraphView v;
         v.ngraphs = ngraphs; v.L = L; v.n = n; v.nnz = nnz; v.m = m;
@@ -232,10 +230,8 @@ struct Graph {
         c.a_base = a_base;
         c.a_stride = a_stride;
         c.e_base = e_base;
-        c.toffs = toffs.as<int64_t>();
-        c.tlist = tlist.as<int32_t>();
-        c.tsum = tsum.as<unsigned long long>();
-        c.kmat = kmat.as<unsigned long long>();
+        c.xsum = xsum.p;
+        c.tri_any = tri_any.as<uint8_t>();
         c.tables = tables.as<uint32_t>();
         c.table_stride = table_stride;
         c.gacc = gacc.as<unsigned long long>();
@@ -255,8 +251,7 @@ struct Graph {
         return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &anchors_light, &anchors_heavy, &edges_light,
                              &edges_heavy, &C, &tau, &A, &tables, &gacc, &status, &tiles_full, &stage_pe,
-                             &stage_gl, &tcount, &toffs, &tlist, &tsum, &kmat, &big_list, &big_count, &scan_tmp,
-                             &set_scratch, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
+                             &stage_gl, &xsum, &tri_any, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
@@ -331,10 +326,14 @@ void prepare_triangles(Graph &G);
 // graph (tg_triangles.cu); returns the kernel launches
 int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s);
 
+// sums over the triangle nodes and 4-cliques of the edges [e0, e1) of whole
+// graphs with nodes [n0, n1) (tg_sums.cu); prepare_sums before any capture
+void prepare_sums(Graph &G);
+int64_t launch_sums(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s);
+
 // count entries (tg_count.cu)
 void prepare_counting(Graph &G, int k, cudaStream_t s);
 void prepare_edges(Graph &G, int k, cudaStream_t s);
-void prepare_capture(Graph &G, int k, cudaStream_t s);
 // Runs the counting stages for edges [e_begin, e_end) into per_edge_out
 // (row 0 = e_begin) and the raw sums gacc.  full: the whole graph, every
 // stage recomputed (no cached state).  Returns the kernel launches.

@@ -88,11 +88,9 @@ struct CountView {
     uint32_t *A;                // [L*L][a_stride] 4-cycle contributions per slot of the current chunk
     int64_t a_base;             // first adjacency slot of the current chunk
     int64_t a_stride;           // slots per type-pair row of A
-    int64_t e_base;             // first edge of the current range (per-edge arrays are relative to it)
-    int64_t *toffs;             // [edges + 1] T list offsets of the range
-    int32_t *tlist;             // T lists of the range, each sorted by (type, id)
-    unsigned long long *tsum;   // [edges][3][L*L] TCi, TCj, DT
-    unsigned long long *kmat;   // [edges][L*L] adjacent pairs inside T, (smaller id type, larger id type)
+    int64_t e_base;             // first edge of the current chunk (xsum is relative to it)
+    void *xsum;                 // [edges][L][4][L] TCi, TCj, DT, K' (tg_sums.cu): uint32, or uint64 when wide
+    uint8_t *tri_any;           // [n] 1 if a triangle has the node as its lowest
     uint32_t *tables;           // dense per-CTA wedge tables
     int64_t table_stride;       // entries (uint32) per CTA table
     unsigned long long *gacc;   // [ngraphs*G] raw per-graphlet edge sums

@@ -19,13 +19,18 @@ namespace {
 
 // Warp per node u with 2 <= |N+(u)| <= kTriWarpMax: one pair of N+(u) per
 // lane, looked up in the lower node's N+ list.
-__global__ void __launch_bounds__(256) k_tri_warp(GraphView g, uint32_t *C) {
+__global__ void __launch_bounds__(256) k_tri_warp(GraphView g, uint32_t *C, uint8_t *any) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; u < g.n; u += nw) {
         const int64_t pb = g.plus_off[u];
         const int p = (int)(g.plus_off[u + 1] - pb);
-        if (p < 2 || p > kTriWarpMax) continue;
+        if (p > kTriWarpMax) continue;
+        if (p < 2) {
+            if (lane == 0) any[u] = 0;
+            continue;
+        }
+        bool found = false;
         const uint32_t tu = g.ty[u];
         const uint32_t ent = lane < p ? (uint32_t)g.plus_adj[pb + lane] : 0u;
         const uint32_t eid = lane < p ? (uint32_t)g.plus_eid[pb + lane] : 0u;
@@ -40,17 +45,20 @@ __global__ void __launch_bounds__(256) k_tri_warp(GraphView g, uint32_t *C) {
             const bool kl = (ek & (uint32_t)kIdMask) < (el & (uint32_t)kIdMask);
             const int64_t pos = plus_find(g, (int32_t)((kl ? ek : el) & (uint32_t)kIdMask), kl ? el : ek);
             if (pos < 0) continue;
+            found = true;
             atomicAdd(&C[(int64_t)dk * kCRow + (el >> kTypeShift)], 1u);
             atomicAdd(&C[(int64_t)dl * kCRow + (ek >> kTypeShift)], 1u);
             atomicAdd(&C[(int64_t)g.plus_eid[pos] * kCRow + tu], 1u);
         }
+        found = __any_sync(0xffffffffu, found);
+        if (lane == 0) any[u] = found ? 1 : 0;
     }
 }
 
 // CTA per listed node u: the counts of u's own edges in shared memory (or,
 // kSmem = false, in the CTA's global slice), those of {a, b} added in place.
 template <int kThreadsT, bool kSmem>
-__global__ void __launch_bounds__(kThreadsT) k_tri_cta(GraphView g, uint32_t *C, const int32_t *__restrict__ list,
+__global__ void __launch_bounds__(kThreadsT) k_tri_cta(GraphView g, uint32_t *C, uint8_t *any, const int32_t *__restrict__ list,
                                                        int64_t n_list, int cap, int lgf, unsigned char *scratch,
                                                        int64_t stride) {
     extern __shared__ unsigned char tri_smem[];
@@ -81,11 +89,14 @@ __global__ void __launch_bounds__(kThreadsT) k_tri_cta(GraphView g, uint32_t *C,
             atomicAdd(&C[(int64_t)g.plus_eid[pos] * kCRow + tu], 1u);
         });
         __syncthreads();
+        bool found = false;
         for (int k = threadIdx.x; k < p * L; k += kThreadsT) {
             const uint32_t v = cnt[k];
             if (v) atomicAdd(&C[(int64_t)q.eid[k / L] * kCRow + k % L], v);
+            found = found || v;
         }
-        __syncthreads();
+        found = __syncthreads_or(found);
+        if (threadIdx.x == 0) any[u] = found ? 1 : 0;
     }
 }
 
@@ -158,7 +169,7 @@ int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s) {
     if (G.m > 0) {
         KernelTimer kt(G, s, "k_tri");
         TG_CK(cudaMemsetAsync(G.C.p, 0, (size_t)G.m * kCRow * sizeof(uint32_t), s));
-        k_tri_warp<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sms * 64), 256, 0, s>>>(gv, cv.C);
+        k_tri_warp<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sms * 64), 256, 0, s>>>(gv, cv.C, cv.tri_any);
         ++launches;
         for (int cls = 0; cls < 3; ++cls) {
             const LocalClass c = local_class(G, cls);
@@ -168,13 +179,13 @@ int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s) {
             if (cls == 2) {
                 const int64_t grid = std::min<int64_t>(c.n, sms);
                 k_tri_cta<kTriBigThreads, false><<<(unsigned)grid, kTriBigThreads, 0, s>>>(
-                    gv, cv.C, c.list, c.n, c.cap, c.lgf, G.local_scratch.as<unsigned char>(), (int64_t)bytes);
+                    gv, cv.C, cv.tri_any, c.list, c.n, c.cap, c.lgf, G.local_scratch.as<unsigned char>(), (int64_t)bytes);
                 continue;
             }
             auto launch = [&](auto kern) {
                 const int per_sm = std::max(1, std::min<int>(2048 / c.threads, (int)((220u << 10) / (bytes + 1024))));
                 kern<<<(unsigned)std::min<int64_t>(c.n, (int64_t)sms * per_sm), c.threads, bytes, s>>>(
-                    gv, cv.C, c.list, c.n, c.cap, c.lgf, nullptr, 0);
+                    gv, cv.C, cv.tri_any, c.list, c.n, c.cap, c.lgf, nullptr, 0);
             };
             if (cls == 0) launch(k_tri_cta<kTriMidThreads, true>);
             else launch(k_tri_cta<kTriBigThreads, true>);

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import graphgen
+import oracle
 from gpu_helpers import gpu_count
 
 pytestmark = pytest.mark.gpu
@@ -55,3 +56,22 @@ def test_typed_triangles_match_dense_products(n, density, L):
     for t in range(L):
         c = ((A * (g["types"] == t)) @ A)[i, j]               # below 2^53: exact
         np.testing.assert_array_equal(pe[:, L + t], c)
+
+
+@pytest.mark.parametrize("n,density,L", CASES)
+def test_four_node_rows_match_oracle(n, density, L):
+    """Sums over triangle nodes and 4-cliques: sampled rows against Alg. 1-3; the 4-clique slots add up to six times
+    the total, which is C(n, 4) on a complete graph."""
+    g = dense_graph(n, density, L, seed=12)
+    pe, gl, st = gpu_count(g)
+    assert st == 0, tg.STATUS[st]
+    rng = np.random.default_rng(5)
+    ids = np.unique(rng.integers(0, g["m"], 40))
+    rows, _ = oracle.paper_edges(g, ids)
+    np.testing.assert_array_equal(pe[ids], rows)
+    lay = tg.tg_layout(L, 4)
+    off, size = lay["global_block_offset"][8], lay["global_block_size"][8]
+    k4 = pe[:, lay["orbit_offset"][12]:lay["orbit_offset"][12] + lay["pairs"]]
+    assert int(k4.sum()) == 6 * int(gl[off:off + size].sum())
+    if density == 1.0:
+        assert int(gl[off:off + size].sum()) == n * (n - 1) * (n - 2) * (n - 3) // 24
