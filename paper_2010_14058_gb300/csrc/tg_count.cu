@@ -51,47 +51,6 @@ namespace {
 
 constexpr int kAnchorThreads = 512;         // k_wedge_heavy: one anchor per CTA
 constexpr int kLightAnchorWarps = 4;        // k_wedge_light: one anchor per warp
-constexpr int kTile = 2048;                 // most edges per tile of k_epi4 and k_edge3 (tile_edges)
-
-// lexicographic rank of a sorted K-multiset over [0,L): the number of
-// non-decreasing K-tuples that precede it, counted position by position.
-__device__ __forceinline__ int multichoose(int n, int r) {   // C(n + r - 1, r), n >= 1
-    int64_t v = 1;
-    for (int k = 1; k <= r; ++k) v = v * (n + k - 1) / k;
-    return (int)v;
-}
-__device__ int multiset_rank_dev(int L, int K, const int *s) {
-    int r = 0, prev = 0;
-    for (int k = 0; k < K; ++k) {
-        for (int v = prev; v < s[k]; ++v) r += multichoose(L - v, K - k - 1);
-        prev = s[k];
-    }
-    return r;
-}
-__device__ __forceinline__ void sort4(int *s) {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 3 - a; ++b)
-            if (s[b] > s[b + 1]) { int x = s[b]; s[b] = s[b + 1]; s[b + 1] = x; }
-}
-__device__ __forceinline__ void sort3(int *s) {
-    if (s[0] > s[1]) { int x = s[0]; s[0] = s[1]; s[1] = x; }
-    if (s[1] > s[2]) { int x = s[1]; s[1] = s[2]; s[2] = x; }
-    if (s[0] > s[1]) { int x = s[0]; s[0] = s[1]; s[1] = x; }
-}
-
-// global block offsets (block 0 edges, 1 3-path, 2 triangle, 3..8 four-node)
-__device__ __forceinline__ int gblock_off(int L, int b) {
-    int c2 = multichoose(L, 2), c3 = multichoose(L, 3), c4 = multichoose(L, 4);
-    if (b == 0) return 0;
-    if (b <= 2) return c2 + (b - 1) * c3;
-    return c2 + 2 * c3 + (b - 3) * c4;
-}
-
-__device__ __forceinline__ int pair_idx(int L, int t, int u) {   // t <= u
-    return t * L - t * (t - 1) / 2 + (u - t);
-}
 
 // ------------------------------------------------------------ wedge kernels
 // For an anchor u, V_u = {v in Gamma_u : v < u} and, for v in V_u, the
@@ -800,554 +759,6 @@ __global__ void __launch_bounds__(kHubThreads, 5) k_wedge_hub(GraphView g, Count
     }
 }
 
-// ------------------------------------------------------------ per-edge 4-node
-// k_epi4: every orbit of Table 3 from the gathered sums (tg_sums.cu, the
-// wedge pass and the per-node sums), one warp per edge with the L x L
-// matrices held one entry per lane and transposed by shuffles; writes the
-// row and the CTA histogram.
-
-__device__ __forceinline__ uint32_t sat32(int64_t v, uint32_t *status) {
-    if (v > 0xffffffffll) {
-        set_status(status, ST_OVERFLOW);
-        return 0xffffffffu;
-    }
-    return (uint32_t)v;
-}
-
-// orbit o (3..12) -> global block of its graphlet (Sec. 4.4)
-__device__ __forceinline__ int graphlet_block(int o) {
-    switch (o) {
-        case 3: case 4: return 3;
-        case 5: return 4;
-        case 6: return 5;
-        case 7: case 8: case 9: return 6;
-        case 10: case 11: return 7;
-        default: return 8;
-    }
-}
-
-__device__ void flush_hist(unsigned long long *hist, int G, unsigned long long *gacc, int graph, int gsize, int gr) {
-    for (int s = gr; s < G; s += gsize) {
-        unsigned long long v = hist[s];
-        if (v) atomicAdd(&gacc[(int64_t)graph * G + s], v);
-        hist[s] = 0;
-    }
-}
-
-// the sum of `copies` histograms of one graph into gacc; clears them
-__device__ void flush_hist_copies(unsigned long long *hist, int hw, int copies, int G, unsigned long long *gacc,
-                                  int graph, int gsize, int gr) {
-    for (int s = gr; s < G; s += gsize) {
-        unsigned long long v = 0;
-        for (int c = 0; c < copies; ++c) {
-            v += hist[c * hw + s];
-            hist[c * hw + s] = 0;
-        }
-        if (v) atomicAdd(&gacc[(int64_t)graph * G + s], v);
-    }
-}
-
-struct Tile {
-    int64_t begin, end;
-    int32_t graph, pad;
-};
-
-// value of matrix entry k (0 <= k < L*L) held as (r0 on lane k, or r1 on lane k-32)
-__device__ __forceinline__ long long mat_get(long long r0, long long r1, int k) {
-    const long long v0 = __shfl_sync(0xffffffffu, r0, k & 31);
-    const long long v1 = __shfl_sync(0xffffffffu, r1, k & 31);
-    return k < 32 ? v0 : v1;
-}
-__device__ __forceinline__ long long lane_get(long long v, int t) { return __shfl_sync(0xffffffffu, v, t); }
-
-// Warp per edge: all orbits of Table 3 from the gathered sums (the
-// inclusion-exclusion of Thm. 1 over S_i, S_j, T, I; then Lemmas 1-4).
-// Lane l holds entry k = l (and k = l + 32 when L*L > 32) of each L x L
-// matrix, (x, y) = (k / L, k % L); transposed entries come by shuffle.
-// Shared memory of k_epi4: `copies` histograms of G(L) u64 (warp w adds into
-// copy w % copies, so fewer warps contend per entry), then the multiset
-// rank tables: rank2[p][q], rank3[p][q][t], rank4[p][q][pair] (uint16).
-__host__ __device__ __forceinline__ size_t epi4_hist_words(int L) { return (size_t)((global_slots(L, 4) + 1) & ~1); }
-__host__ __device__ __forceinline__ size_t epi4_smem_bytes(int L, int copies) {
-    const int P = L * (L + 1) / 2;
-    return epi4_hist_words(L) * copies * sizeof(unsigned long long) +
-           (size_t)(L * L + L * L * L + L * L * P + 1) * sizeof(uint16_t);
-}
-
-template <class Acc>
-__global__ void __launch_bounds__(256, 3) k_epi4(GraphView g, CountView cv, const Tile *__restrict__ tiles,
-                                             int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
-                                             unsigned long long *gacc, int copies) {
-    extern __shared__ unsigned long long hist_all[];
-    const int L = g.L, LL = L * L, P = L * (L + 1) / 2;
-    const int G = (int)global_slots(L, 4);
-    const int S = (int)per_edge_slots(L, 4);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const int HW = (int)epi4_hist_words(L);
-    unsigned long long *hist = hist_all + (wid % copies) * HW;
-    uint16_t *rank2 = reinterpret_cast<uint16_t *>(hist_all + (size_t)copies * HW);
-    uint16_t *rank3 = rank2 + LL;
-    uint16_t *rank4 = rank3 + LL * L;
-    for (int s = threadIdx.x; s < copies * HW; s += blockDim.x) hist_all[s] = 0;
-    for (int k = threadIdx.x; k < LL * P; k += blockDim.x) {
-        const int pq = k / P, pi = k % P;
-        int t = 0;
-        while (pair_idx(L, t, L - 1) < pi) ++t;
-        int ms[4] = {pq / L, pq % L, t, t + (pi - pair_idx(L, t, t))};
-        sort4(ms);
-        rank4[k] = (uint16_t)multiset_rank_dev(L, 4, ms);
-    }
-    for (int k = threadIdx.x; k < LL * L; k += blockDim.x) {
-        int ms[3] = {k / LL, (k / L) % L, k % L};
-        sort3(ms);
-        rank3[k] = (uint16_t)multiset_rank_dev(L, 3, ms);
-    }
-    for (int k = threadIdx.x; k < LL; k += blockDim.x) {
-        int ms[2] = {k / L < k % L ? k / L : k % L, k / L < k % L ? k % L : k / L};
-        rank2[k] = (uint16_t)multiset_rank_dev(L, 2, ms);
-    }
-    const int off1 = gblock_off(L, 1), off2 = gblock_off(L, 2), off4 = gblock_off(L, 3), c4 = multichoose(L, 4);
-    __syncthreads();
-    int cur_graph = -1;
-    const int kA = lane, kB = lane + 32;                     // this lane's matrix entries
-    const int xA = kA / L, yA = kA % L, xB = kB / L, yB = kB % L;
-    const bool hasA = kA < LL, hasB = kB < LL;
-    const int tA = yA * L + xA, tB = yB * L + xB;            // transposed entries
-    for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
-        const Tile tile = tiles[ti];
-        if (tile.graph != cur_graph) {
-            __syncthreads();
-            if (cur_graph >= 0) flush_hist_copies(hist_all, HW, copies, G, gacc, cur_graph, blockDim.x, threadIdx.x);
-            __syncthreads();
-            cur_graph = tile.graph;
-        }
-        for (int64_t e = tile.begin + wid; e < tile.end; e += nwarp) {
-            const int64_t er = e - cv.e_base;
-            const int32_t i = g.e_lo[e], j = g.e_hi[e];
-            const int p = g.ty[i], q = g.ty[j];
-            // per-type scalars, lane t < L
-            long long c = 0, di = 0, dj = 0;
-            if (lane < L) {
-                c = cv.C[e * kCRow + lane];
-                di = typed_degree(g, i, lane);
-                dj = typed_degree(g, j, lane);
-            }
-            const long long a = di - c - (q == lane ? 1 : 0);  // |S_i^t|
-            const long long b = dj - c - (p == lane ? 1 : 0);  // |S_j^t|
-            // gathered matrices
-            const Acc *sum = reinterpret_cast<const Acc *>(cv.xsum) + er * 4 * LL;
-            const long long cA = lane_get(c, xA < L ? xA : 0), cB = lane_get(c, xB < L ? xB : 0);
-            const int64_t *tau_i = cv.tau + (int64_t)i * LL, *tau_j = cv.tau + (int64_t)j * LL;
-            const int64_t *del_i = g.delta + (int64_t)i * LL, *del_j = g.delta + (int64_t)j * LL;
-            const uint32_t *A = cv.A - cv.a_base;
-            const int64_t sij = g.e_slot_lo[e], sji = g.e_slot_hi[e];
-            long long TCi[2] = {0, 0}, TCj[2] = {0, 0}, DT[2] = {0, 0}, Kd[2] = {0, 0}, Pm[2] = {0, 0};
-            long long ti_[2] = {0, 0}, tj_[2] = {0, 0}, dI[2] = {0, 0}, dJ[2] = {0, 0};
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const bool has = h ? hasB : hasA;
-                const int k = h ? kB : kA, x = h ? xB : xA, y = h ? yB : yA;
-                if (has) {
-                    if (h ? cB : cA) {                       // rows of types without a triangle node are not kept
-                        const Acc *r = sum + x * 4 * L + y;
-                        TCi[h] = (long long)r[0];
-                        TCj[h] = (long long)r[L];
-                        DT[h] = (long long)r[2 * L];
-                        Kd[h] = (long long)r[3 * L];
-                    }
-                    // P[x][y]: slot i->j holds [type next to i][type next to j], slot j->i the reverse
-                    Pm[h] = (long long)A[(int64_t)(y * L + x) * cv.a_stride + sij] +
-                            (long long)A[(int64_t)(x * L + y) * cv.a_stride + sji];
-                    ti_[h] = tau_i[k];
-                    tj_[h] = tau_j[k];
-                    dI[h] = del_i[k];
-                    dJ[h] = del_j[k];
-                }
-            }
-            // Ks: ordered adjacent pairs of T (K' + K'^T counts each twice)
-            long long Ks[2];
-            Ks[0] = (Kd[0] + mat_get(Kd[0], Kd[1], hasA ? tA : 0)) >> 1;
-            Ks[1] = (Kd[1] + mat_get(Kd[0], Kd[1], hasB ? tB : 0)) >> 1;
-            // CTi, CTj
-            long long CTi[2], CTj[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int x = h ? xB : xA, y = h ? yB : yA;
-                const long long cx = lane_get(c, x < L ? x : 0);
-                CTi[h] = TCi[h] - Ks[h] - (y == q ? cx : 0);
-                CTj[h] = TCj[h] - Ks[h] - (y == p ? cx : 0);
-            }
-            long long CTiT[2], CTjT[2];
-            CTiT[0] = mat_get(CTi[0], CTi[1], hasA ? tA : 0);
-            CTiT[1] = mat_get(CTi[0], CTi[1], hasB ? tB : 0);
-            CTjT[0] = mat_get(CTj[0], CTj[1], hasA ? tA : 0);
-            CTjT[1] = mat_get(CTj[0], CTj[1], hasB ? tB : 0);
-            // W, Q
-            long long Wi[2], Wj[2], Q[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int x = h ? xB : xA, y = h ? yB : yA;
-                const long long cx = lane_get(c, x < L ? x : 0), cy = lane_get(c, y < L ? y : 0);
-                Wi[h] = ti_[h] - CTi[h] - CTiT[h] - Ks[h] - (x == q ? cy : 0) - (y == q ? cx : 0);
-                Wj[h] = tj_[h] - CTj[h] - CTjT[h] - Ks[h] - (x == p ? cy : 0) - (y == p ? cx : 0);
-                Q[h] = Pm[h] - CTjT[h] - CTi[h] - Ks[h];
-            }
-            long long QT[2];
-            QT[0] = mat_get(Q[0], Q[1], hasA ? tA : 0);
-            QT[1] = mat_get(Q[0], Q[1], hasB ? tB : 0);
-            // R = Ri + Rj, G8, W = Wi + Wj, CT = CTi + CTj
-            long long R[2], G8[2], W[2], CT[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int x = h ? xB : xA, y = h ? yB : yA;
-                const long long cx = lane_get(c, x < L ? x : 0);
-                const long long ax = lane_get(a, x < L ? x : 0), bx = lane_get(b, x < L ? x : 0);
-                const long long djy = lane_get(dj, y < L ? y : 0), diy = lane_get(di, y < L ? y : 0);
-                const long long Ri = dI[h] - DT[h] - (x == q ? djy : 0) - (y == p ? ax : 0) - Wi[h] - CTiT[h] - QT[h];
-                const long long Rj = dJ[h] - DT[h] - (x == p ? diy : 0) - (y == q ? bx : 0) - Wj[h] - CTjT[h] - Q[h];
-                R[h] = Ri + Rj;
-                G8[h] = DT[h] - ((y == p ? 1 : 0) + (y == q ? 1 : 0)) * cx - Ks[h] - CTi[h] - CTj[h];
-                W[h] = Wi[h] + Wj[h];
-                CT[h] = CTi[h] + CTj[h];
-            }
-            uint32_t *row = per_edge_out ? per_edge_out + (e - row_base) * S : nullptr;
-            // 3-node slots, typed edge and 3-node global blocks
-            if (lane < L) {
-                const long long s3 = a + b;
-                if (a < 0 || b < 0) set_status(cv.status, ST_INTERNAL);
-                if (row) {
-                    row[lane] = sat32(s3, cv.status);
-                    row[L + lane] = sat32(c, cv.status);
-                }
-                const int r = rank3[(p * L + q) * L + lane];
-                if (s3) atomicAdd(&hist[off1 + r], (unsigned long long)s3);
-                if (c) atomicAdd(&hist[off2 + r], (unsigned long long)c);
-            }
-            if (lane == 0) atomicAdd(&hist[rank2[p * L + q]], 1ull);
-            // orbits, one type pair (t <= u) per lane (two rounds when P > 32)
-            for (int base = 0; base < P; base += 32) {
-                const int pi = base + lane;
-                int t = 0;
-                if (pi < P)
-                    while (pair_idx(L, t, L - 1) < pi) ++t;
-                const int u = pi < P ? t + (pi - pair_idx(L, t, t)) : 0;
-                const int ktu = t * L + u, kut = u * L + t;
-                const long long Rtu = mat_get(R[0], R[1], ktu), Rut = mat_get(R[0], R[1], kut);
-                const long long Qtu = mat_get(Q[0], Q[1], ktu), Qut = mat_get(Q[0], Q[1], kut);
-                const long long Wtu = mat_get(W[0], W[1], ktu);
-                const long long Gtu = mat_get(G8[0], G8[1], ktu), Gut = mat_get(G8[0], G8[1], kut);
-                const long long CTtu = mat_get(CT[0], CT[1], ktu), CTut = mat_get(CT[0], CT[1], kut);
-                const long long Ktu = mat_get(Ks[0], Ks[1], ktu);
-                const long long at = lane_get(a, t), au = lane_get(a, u), bt = lane_get(b, t), bu = lane_get(b, u);
-                const long long ct = lane_get(c, t), cu = lane_get(c, u);
-                if (pi >= P) continue;
-                long long gv[10];
-                bool ok = true;
-                if (t != u) {
-                    gv[0] = Rtu + Rut;                                 // g3
-                    gv[3] = Qtu + Qut;                                 // g6
-                    gv[4] = Wtu;                                       // g7
-                    gv[5] = Gtu + Gut;                                 // g8
-                    gv[7] = CTtu + CTut;                               // g10
-                    gv[9] = Ktu;                                       // g12
-                    gv[1] = at * bu + au * bt - gv[3];                 // Lemma 1
-                    gv[2] = at * au + bt * bu - gv[4];                 // Lemma 2
-                    gv[6] = ct * (au + bu) + cu * (at + bt) - gv[7];   // Lemma 3
-                    gv[8] = ct * cu - gv[9];                           // Lemma 4
-                } else {
-                    ok = !(Wtu & 1) && !(Ktu & 1);
-                    gv[0] = Rtu;
-                    gv[3] = Qtu;
-                    gv[4] = Wtu / 2;
-                    gv[5] = Gtu;
-                    gv[7] = CTtu;
-                    gv[9] = Ktu / 2;
-                    gv[1] = at * bt - gv[3];
-                    gv[2] = at * (at - 1) / 2 + bt * (bt - 1) / 2 - gv[4];
-                    gv[6] = ct * (at + bt) - gv[7];
-                    gv[8] = ct * (ct - 1) / 2 - gv[9];
-                }
-                const int r = rank4[(p * L + q) * P + pi];
-#pragma unroll
-                for (int o = 3; o <= 12; ++o) {
-                    const long long v = gv[o - 3];
-                    ok = ok && v >= 0;
-                    if (row) row[2 * L + (o - 3) * P + pi] = sat32(v, cv.status);
-                    if (v > 0) atomicAdd(&hist[off4 + (graphlet_block(o) - 3) * c4 + r], (unsigned long long)v);
-                }
-                if (!ok) set_status(cv.status, ST_INTERNAL);
-            }
-        }
-    }
-    __syncthreads();
-    if (cur_graph >= 0) flush_hist_copies(hist_all, HW, copies, G, gacc, cur_graph, blockDim.x, threadIdx.x);
-}
-
-// k = 3: 3-node slots and global blocks 0..2 only (warp per edge)
-__global__ void __launch_bounds__(256) k_edge3(GraphView g, CountView cv, const Tile *__restrict__ tiles, int64_t n_tiles,
-                                               int64_t e_begin, uint32_t *per_edge_out, unsigned long long *gacc) {
-    extern __shared__ unsigned long long hist[];
-    const int L = g.L;
-    const int G = (int)global_slots(L, 3);
-    const int S = 2 * L;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    for (int s = threadIdx.x; s < G; s += blockDim.x) hist[s] = 0;
-    __syncthreads();
-    int cur_graph = -1;
-    for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
-        const Tile tile = tiles[ti];
-        if (tile.graph != cur_graph) {
-            if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph, blockDim.x, threadIdx.x);
-            __syncthreads();
-            cur_graph = tile.graph;
-        }
-        for (int64_t e = tile.begin + wid; e < tile.end; e += nwarp) {
-            const int32_t i = g.e_lo[e], j = g.e_hi[e];
-            const int p = g.ty[i], q = g.ty[j];
-            for (int t = lane; t < L; t += 32) {
-                const int64_t c = cv.C[e * kCRow + t];
-                const int64_t a = typed_degree(g, i, t) - c - (q == t ? 1 : 0);
-                const int64_t b = typed_degree(g, j, t) - c - (p == t ? 1 : 0);
-                if (per_edge_out) {
-                    uint32_t *row = per_edge_out + (e - e_begin) * S;
-                    row[t] = sat32(a + b, cv.status);
-                    row[L + t] = sat32(c, cv.status);
-                }
-                int ms[3] = {p, q, t};
-                sort3(ms);
-                const int r = multiset_rank_dev(L, 3, ms);
-                if (a + b) atomicAdd(&hist[gblock_off(L, 1) + r], (unsigned long long)(a + b));
-                if (c) atomicAdd(&hist[gblock_off(L, 2) + r], (unsigned long long)c);
-            }
-            if (lane == 0) {
-                int ms[2] = {p < q ? p : q, p < q ? q : p};
-                atomicAdd(&hist[multiset_rank_dev(L, 2, ms)], 1ull);
-            }
-        }
-        __syncthreads();
-    }
-    if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph, blockDim.x, threadIdx.x);
-}
-
-// ------------------------------------------------- position-aware epilogue
-// Sec. 5 (Def. 8): before k_epi4 folds them into unordered type pairs, its
-// matrices already keep the positions of an instance apart: Ri / Rj (4-path
-// end edges with inner endpoint i / j: w the inner endpoint's other
-// neighbour, r the far end), Q (4-cycles; first index the type of j's
-// neighbour), Wi / Wj (adjacent pairs inside S_i / S_j), CTi / CTj (a
-// triangle node and an adjacent node of S_i / S_j), G8 (a triangle node and
-// its tail in I) and K (adjacent pairs inside T).  k_epi4_pa writes them by
-// position -- the row layout of tg_pa.cu, sides named by caller ids (lo =
-// the smaller) -- and adds every count to the class that the slot and the
-// endpoint types fix (host table).  One warp per edge, as k_epi4; the gather
-// and the matrices Ks, CTi, CTj, Wi, Wj, Q below repeat k_epi4's line for
-// line, and the two kernels must change together.
-struct PaView {
-    const int32_t *cls;       // [L*L][S+1] class of (phi_lo, phi_hi, slot); slot S: the edge itself
-    const int32_t *old_of;    // [n] caller id of each internal node
-    int32_t S;                // per-edge slots
-    int32_t G;                // classes (global slots) per graph
-    int32_t off[13];          // first slot of blocks O1..O12
-};
-
-__host__ __device__ __forceinline__ size_t epi4_pa_hist_words(int G) { return (size_t)((G + 1) & ~1); }
-
-template <class Acc>
-__global__ void __launch_bounds__(256) k_epi4_pa(GraphView g, CountView cv, PaView pv, const Tile *__restrict__ tiles,
-                                                 int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
-                                                 unsigned long long *gacc, int copies) {
-    extern __shared__ unsigned long long hist_all[];
-    const int L = g.L, LL = L * L, P = L * (L + 1) / 2;
-    const int S = pv.S, G = pv.G;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const int HW = (int)epi4_pa_hist_words(G);
-    unsigned long long *hist = hist_all + (wid % copies) * HW;
-    for (int s = threadIdx.x; s < copies * HW; s += blockDim.x) hist_all[s] = 0;
-    __syncthreads();
-    int cur_graph = -1;
-    const int kA = lane, kB = lane + 32;                     // this lane's matrix entries
-    const int xA = kA / L, yA = kA % L, xB = kB / L, yB = kB % L;
-    const bool hasA = kA < LL, hasB = kB < LL;
-    const int tA = yA * L + xA, tB = yB * L + xB;            // transposed entries
-    for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
-        const Tile tile = tiles[ti];
-        if (tile.graph != cur_graph) {
-            __syncthreads();
-            if (cur_graph >= 0) flush_hist_copies(hist_all, HW, copies, G, gacc, cur_graph, blockDim.x, threadIdx.x);
-            __syncthreads();
-            cur_graph = tile.graph;
-        }
-        for (int64_t e = tile.begin + wid; e < tile.end; e += nwarp) {
-            const int64_t er = e - cv.e_base;
-            const int32_t i = g.e_lo[e], j = g.e_hi[e];
-            const int p = g.ty[i], q = g.ty[j];
-            long long c = 0, di = 0, dj = 0;
-            if (lane < L) {
-                c = cv.C[e * kCRow + lane];
-                di = typed_degree(g, i, lane);
-                dj = typed_degree(g, j, lane);
-            }
-            const long long a = di - c - (q == lane ? 1 : 0);  // |S_i^t|
-            const long long b = dj - c - (p == lane ? 1 : 0);  // |S_j^t|
-            const Acc *sum = reinterpret_cast<const Acc *>(cv.xsum) + er * 4 * LL;
-            const long long cA = lane_get(c, xA < L ? xA : 0), cB = lane_get(c, xB < L ? xB : 0);
-            const int64_t *tau_i = cv.tau + (int64_t)i * LL, *tau_j = cv.tau + (int64_t)j * LL;
-            const int64_t *del_i = g.delta + (int64_t)i * LL, *del_j = g.delta + (int64_t)j * LL;
-            const uint32_t *A = cv.A - cv.a_base;
-            const int64_t sij = g.e_slot_lo[e], sji = g.e_slot_hi[e];
-            long long TCi[2] = {0, 0}, TCj[2] = {0, 0}, DT[2] = {0, 0}, Kd[2] = {0, 0}, Pm[2] = {0, 0};
-            long long ti_[2] = {0, 0}, tj_[2] = {0, 0}, dI[2] = {0, 0}, dJ[2] = {0, 0};
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const bool has = h ? hasB : hasA;
-                const int k = h ? kB : kA, x = h ? xB : xA, y = h ? yB : yA;
-                if (has) {
-                    if (h ? cB : cA) {                       // rows of types without a triangle node are not kept
-                        const Acc *r = sum + x * 4 * L + y;
-                        TCi[h] = (long long)r[0];
-                        TCj[h] = (long long)r[L];
-                        DT[h] = (long long)r[2 * L];
-                        Kd[h] = (long long)r[3 * L];
-                    }
-                    Pm[h] = (long long)A[(int64_t)(y * L + x) * cv.a_stride + sij] +
-                            (long long)A[(int64_t)(x * L + y) * cv.a_stride + sji];
-                    ti_[h] = tau_i[k];
-                    tj_[h] = tau_j[k];
-                    dI[h] = del_i[k];
-                    dJ[h] = del_j[k];
-                }
-            }
-            long long Ks[2];
-            Ks[0] = (Kd[0] + mat_get(Kd[0], Kd[1], hasA ? tA : 0)) >> 1;
-            Ks[1] = (Kd[1] + mat_get(Kd[0], Kd[1], hasB ? tB : 0)) >> 1;
-            long long CTi[2], CTj[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int x = h ? xB : xA, y = h ? yB : yA;
-                const long long cx = lane_get(c, x < L ? x : 0);
-                CTi[h] = TCi[h] - Ks[h] - (y == q ? cx : 0);
-                CTj[h] = TCj[h] - Ks[h] - (y == p ? cx : 0);
-            }
-            long long CTiT[2], CTjT[2];
-            CTiT[0] = mat_get(CTi[0], CTi[1], hasA ? tA : 0);
-            CTiT[1] = mat_get(CTi[0], CTi[1], hasB ? tB : 0);
-            CTjT[0] = mat_get(CTj[0], CTj[1], hasA ? tA : 0);
-            CTjT[1] = mat_get(CTj[0], CTj[1], hasB ? tB : 0);
-            long long Wi[2], Wj[2], Q[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int x = h ? xB : xA, y = h ? yB : yA;
-                const long long cx = lane_get(c, x < L ? x : 0), cy = lane_get(c, y < L ? y : 0);
-                Wi[h] = ti_[h] - CTi[h] - CTiT[h] - Ks[h] - (x == q ? cy : 0) - (y == q ? cx : 0);
-                Wj[h] = tj_[h] - CTj[h] - CTjT[h] - Ks[h] - (x == p ? cy : 0) - (y == p ? cx : 0);
-                Q[h] = Pm[h] - CTjT[h] - CTi[h] - Ks[h];
-            }
-            long long QT[2];
-            QT[0] = mat_get(Q[0], Q[1], hasA ? tA : 0);
-            QT[1] = mat_get(Q[0], Q[1], hasB ? tB : 0);
-            // orientation: side 0 is the endpoint with the smaller caller id
-            const bool lo_is_i = pv.old_of[i] < pv.old_of[j];
-            const int sI = lo_is_i ? 0 : 1, sJ = 1 - sI;
-            const int pl = lo_is_i ? p : q, ph = lo_is_i ? q : p;
-            const int32_t *cls = pv.cls + (int64_t)(pl * L + ph) * (S + 1);
-            uint32_t *row = per_edge_out ? per_edge_out + (e - row_base) * S : nullptr;
-            bool ok = true;
-            auto emit = [&](int slot, long long v) {
-                ok = ok && v >= 0;
-                if (row) row[slot] = sat32(v, cv.status);
-                if (v > 0) atomicAdd(&hist[cls[slot]], (unsigned long long)v);
-            };
-            if (lane == 0) atomicAdd(&hist[cls[S]], 1ull);            // the edge itself
-            if (lane < L) {
-                if (a < 0 || b < 0) set_status(cv.status, ST_INTERNAL);
-                emit(pv.off[1] + sI * L + lane, a);                  // 3-path centred at i
-                emit(pv.off[1] + sJ * L + lane, b);                  // centred at j
-                emit(pv.off[2] + lane, c);
-            }
-            // ordered blocks: entry (x, y) of each matrix on this lane
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const bool has = h ? hasB : hasA;
-                const int k = h ? kB : kA, x = h ? xB : xA, y = h ? yB : yA;
-                const int kt = h ? tB : tA;                          // (y, x)
-                const long long cx = lane_get(c, x < L ? x : 0);
-                const long long ax = lane_get(a, x < L ? x : 0), ay = lane_get(a, y < L ? y : 0);
-                const long long bx = lane_get(b, x < L ? x : 0), by = lane_get(b, y < L ? y : 0);
-                const long long djy = lane_get(dj, y < L ? y : 0), diy = lane_get(di, y < L ? y : 0);
-                if (!has) continue;
-                const long long Ri = dI[h] - DT[h] - (x == q ? djy : 0) - (y == p ? ax : 0) - Wi[h] - CTiT[h] - QT[h];
-                const long long Rj = dJ[h] - DT[h] - (x == p ? diy : 0) - (y == q ? bx : 0) - Wj[h] - CTjT[h] - Q[h];
-                const long long G8 = DT[h] - ((y == p ? 1 : 0) + (y == q ? 1 : 0)) * cx - Ks[h] - CTi[h] - CTj[h];
-                emit(pv.off[3] + sI * LL + k, Ri);                   // inner endpoint i: near x, far y
-                emit(pv.off[3] + sJ * LL + k, Rj);
-                emit(pv.off[4] + (lo_is_i ? k : kt), ax * by - QT[h]);   // i's neighbour x, j's y (Lemma 1)
-                emit(pv.off[6] + (lo_is_i ? k : kt), QT[h]);         // 4-cycle: i's neighbour x, j's y
-                emit(pv.off[8] + k, G8);                             // triangle node x, tail y
-                emit(pv.off[9] + sI * LL + k, cx * ay - CTi[h]);     // Lemma 3, degree-3 node i
-                emit(pv.off[9] + sJ * LL + k, cx * by - CTj[h]);
-                emit(pv.off[10] + sI * LL + k, CTi[h]);              // chordal outer edge, degree-3 node i
-                emit(pv.off[10] + sJ * LL + k, CTj[h]);
-            }
-            // unordered pairs (t <= u), one per lane
-            for (int base = 0; base < P; base += 32) {
-                const int pi = base + lane;
-                int t = 0;
-                if (pi < P)
-                    while (pair_idx(L, t, L - 1) < pi) ++t;
-                const int u = pi < P ? t + (pi - pair_idx(L, t, t)) : 0;
-                const int ktu = t * L + u;
-                const long long Witu = mat_get(Wi[0], Wi[1], ktu), Wjtu = mat_get(Wj[0], Wj[1], ktu);
-                const long long Ktu = mat_get(Ks[0], Ks[1], ktu);
-                const long long at = lane_get(a, t), au = lane_get(a, u), bt = lane_get(b, t), bu = lane_get(b, u);
-                const long long ct = lane_get(c, t), cu = lane_get(c, u);
-                if (pi >= P) continue;
-                long long star_i, star_j, tail_i, tail_j, chord, clique;
-                if (t != u) {
-                    star_i = at * au - Witu;                         // Lemma 2, centre i
-                    star_j = bt * bu - Wjtu;
-                    tail_i = Witu;
-                    tail_j = Wjtu;
-                    chord = ct * cu - Ktu;                           // Lemma 4
-                    clique = Ktu;
-                } else {
-                    ok = ok && !(Witu & 1) && !(Wjtu & 1) && !(Ktu & 1);
-                    star_i = at * (at - 1) / 2 - Witu / 2;
-                    star_j = bt * (bt - 1) / 2 - Wjtu / 2;
-                    tail_i = Witu / 2;
-                    tail_j = Wjtu / 2;
-                    chord = ct * (ct - 1) / 2 - Ktu / 2;
-                    clique = Ktu / 2;
-                }
-                emit(pv.off[5] + sI * P + pi, star_i);
-                emit(pv.off[5] + sJ * P + pi, star_j);
-                emit(pv.off[7] + sI * P + pi, tail_i);
-                emit(pv.off[7] + sJ * P + pi, tail_j);
-                emit(pv.off[11] + pi, chord);
-                emit(pv.off[12] + pi, clique);
-            }
-            if (!ok) set_status(cv.status, ST_INTERNAL);
-        }
-    }
-    __syncthreads();
-    if (cur_graph >= 0) flush_hist_copies(hist_all, HW, copies, G, gacc, cur_graph, blockDim.x, threadIdx.x);
-}
-
-// global totals: C_H = (1/|E(H)|) * sum_e x_e (Sec. 6), exact division
-__global__ void k_finalize(int ngraphs, int L, int k, const unsigned long long *__restrict__ gacc, int64_t *out,
-                           uint32_t *status) {
-    const int G = (int)global_slots(L, k);
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)ngraphs * G) return;
-    const int s = (int)(idx % G);
-    const int nb = k == 4 ? 9 : 3;
-    int b = 0;
-    while (b + 1 < nb && gblock_off(L, b + 1) <= s) ++b;
-    const int edges_of[9] = {1, 2, 3, 3, 3, 4, 4, 5, 6};
-    const unsigned long long v = gacc[idx];
-    if (v % edges_of[b]) set_status(status, ST_INTERNAL);
-    out[idx] = (int64_t)(v / edges_of[b]);
-}
-
 int grid_for(int64_t items, int per_block, int cap) {
     int64_t b = (items + per_block - 1) / per_block;
     if (b < 1) b = 1;
@@ -1381,12 +792,12 @@ static std::vector<Tile> make_tiles(const Graph &G, int64_t e_begin, int64_t e_e
 // its own), and sizes the array for the largest chunk.
 static void plan_chunks(Graph &G) {
     G.chunks.clear();
-    // working bytes of a chunk: the 4-cycle array (4 L^2 per slot) and the
+    // working bytes of a chunk: the 4-cycle array by plane and by slot (8 L^2 per slot) and the
     // per-edge sums (4 L^2 words per edge)
     const int64_t LL = (int64_t)G.L * G.L;
     const int64_t budget = std::max<int64_t>((int64_t)G.opt.cycle_budget_mb << 20, 1);
     auto bytes_of = [&](int a, int b) {
-        return (G.h_slot_off[b] - G.h_slot_off[a]) * 4 * LL + (G.h_edge_off[b] - G.h_edge_off[a]) * LL * (G.wide_sums() ? 32 : 16);
+        return (G.h_slot_off[b] - G.h_slot_off[a]) * 8 * LL + (G.h_edge_off[b] - G.h_edge_off[a]) * LL * (G.wide_sums() ? 32 : 16);
     };
     // tile index ranges follow graph boundaries (make_tiles emits graph after graph)
     std::vector<int64_t> tile_off(G.ngraphs + 1, 0);
@@ -1411,8 +822,6 @@ static void plan_chunks(Graph &G) {
     }
     G.a_stride = std::max<int64_t>(widest, 1);
 }
-
-static size_t hist_bytes(int L, int k) { return (size_t)((global_slots(L, k) + 1) & ~1) * sizeof(unsigned long long); }
 
 // Device tile list of [e_begin, e_end); the full range is cached by the
 // handle (so that a captured CUDA graph never copies from host memory).
@@ -1459,42 +868,9 @@ void raise_smem_limit(const void *func, size_t bytes) {
     else set.push_back({func, dev, bytes});
 }
 
-// Allocations and kernel attributes of the per-edge stage (done before any
-// capture).
-// histogram copies of k_epi4: one per warp while they fit in 64 KB
-static int epi4_copies(int L) {
-    int c = 8;
-    while (c > 1 && epi4_hist_words(L) * c * sizeof(unsigned long long) > (64u << 10)) c >>= 1;
-    return c;
-}
-
-// histogram copies of k_epi4_pa: as many as fit 64 KB (at least one)
-static int epi4_pa_copies(int G) {
-    int c = 8;
-    while (c > 1 && epi4_pa_hist_words(G) * c * sizeof(unsigned long long) > (64u << 10)) c >>= 1;
-    return c;
-}
-
-void prepare_epi4_pa(Graph &G) {
-    const size_t bytes = epi4_pa_hist_words((int)G.pa.G) * epi4_pa_copies((int)G.pa.G) * sizeof(unsigned long long);
-    raise_smem_limit((const void *)k_epi4_pa<uint32_t>, bytes);
-    raise_smem_limit((const void *)k_epi4_pa<unsigned long long>, bytes);
-}
-
-static PaView pa_view(const Graph &G) {
-    PaView v;
-    v.cls = G.pa_cls.as<int32_t>();
-    v.old_of = G.old_of.as<int32_t>();
-    v.S = G.pa.S;
-    v.G = (int32_t)G.pa.G;
-    for (int o = 0; o < 13; ++o) v.off[o] = G.pa.off[o];
-    return v;
-}
-
+// Tiles and kernel attributes of the count (done before any capture).
 void prepare_edges(Graph &G, int k, cudaStream_t s) {
-    raise_smem_limit((const void *)k_edge3, hist_bytes(G.L, 3));
-    raise_smem_limit((const void *)k_epi4<uint32_t>, epi4_smem_bytes(G.L, epi4_copies(G.L)));
-    raise_smem_limit((const void *)k_epi4<unsigned long long>, epi4_smem_bytes(G.L, epi4_copies(G.L)));
+    if (k == 4) prepare_epi(G);
     raise_smem_limit((const void *)k_wedge_heavy, (size_t)kHeavyCap * (1 + G.L) * sizeof(int32_t));
     DBuf unused;
     unused.owner = &G.stream;
@@ -1753,43 +1129,6 @@ static int64_t launch_wedges(Graph &G, const Graph::Chunk &c, cudaStream_t s) {
     return launches;
 }
 
-// orbits of edges [b, e) (inside one chunk, whose wedge pass and sums are done)
-static int64_t launch_edges4(Graph &G, const Graph::Chunk &c, int64_t b, int64_t e, const Tile *tiles, int64_t n_tiles,
-                             int64_t row_base, uint32_t *per_edge_out, unsigned long long *gacc, cudaStream_t s) {
-    if (e <= b) return 0;
-    G.a_base = c.s0;
-    G.e_base = c.e0;
-    const GraphView gv = G.view();
-    const CountView cv = G.cview();
-    const int sms = sm_count();
-    int64_t launches = 0;
-    if (n_tiles > 0 && G.pa_active) {
-        KernelTimer kt(G, s, "k_epi4_pa");
-        const int copies = epi4_pa_copies((int)G.pa.G);
-        auto launch = [&](auto kern) {
-            kern<<<grid_for(n_tiles, 1, sms * G.opt.ctas_per_sm), 256,
-                   epi4_pa_hist_words((int)G.pa.G) * copies * sizeof(unsigned long long), s>>>(
-                gv, cv, pa_view(G), tiles, n_tiles, row_base, per_edge_out, gacc, copies);
-        };
-        if (G.wide_sums()) launch(k_epi4_pa<unsigned long long>);
-        else launch(k_epi4_pa<uint32_t>);
-        ++launches;
-    } else if (n_tiles > 0) {
-        KernelTimer kt(G, s, "k_epi4");
-        const int copies = epi4_copies(G.L);
-        auto launch = [&](auto kern) {
-            kern<<<grid_for(n_tiles, 1, sms * G.opt.ctas_per_sm), 256, epi4_smem_bytes(G.L, copies), s>>>(
-                gv, cv, tiles, n_tiles, row_base, per_edge_out, gacc, copies);
-        };
-        if (G.wide_sums()) launch(k_epi4<unsigned long long>);
-        else launch(k_epi4<uint32_t>);
-        ++launches;
-    }
-    TG_CK(cudaGetLastError());
-    return launches;
-}
-
-
 // Allocates the working arrays of a count with this k (kept by the handle).
 void prepare_counting(Graph &G, int k, cudaStream_t s) {
     const int L = G.L;
@@ -1804,6 +1143,7 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
         if (G.chunks.empty()) plan_chunks(G);
         const size_t ab = (size_t)G.a_stride * L * L * sizeof(uint32_t);
         if (G.A.bytes < ab) G.A.alloc(ab);
+        if (G.slot_rows.bytes < ab) G.slot_rows.alloc(ab);
         const size_t me = (size_t)std::max<int64_t>(G.max_chunk_edges, 1);
         const size_t xb = me * 4 * L * L * (G.wide_sums() ? sizeof(unsigned long long) : sizeof(uint32_t));
         if (G.xsum.bytes < xb) G.xsum.alloc(xb);
@@ -1838,15 +1178,7 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
     int64_t n_tiles = 0;
     const Tile *tiles = tiles_for(G, e_begin, e_end, n_tiles, tmp, s);
     if (k == 3) {
-        if (n_tiles > 0) {
-            const GraphView gv = G.view();
-            const CountView cv = G.cview();
-            KernelTimer kt(G, s, "k_edge3");
-            k_edge3<<<grid_for(n_tiles, 1, sm_count() * 8), 256, hist_bytes(G.L, 3), s>>>(gv, cv, tiles, n_tiles, e_begin,
-                                                                                       per_edge_out, gacc);
-            ++launches;
-            TG_CK(cudaGetLastError());
-        }
+        launches += launch_edges3(G, tiles, n_tiles, e_begin, per_edge_out, gacc, s);
     } else {
         const bool whole = e_begin == 0 && e_end == G.m;
         std::vector<Tile> host;
@@ -1858,6 +1190,7 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
             if (full || G.chunks.size() > 1 || G.prepared_k != 4) {
                 launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
                 launches += launch_wedges(G, c, s);
+                launches += launch_slot_rows(G, c.s1 - c.s0, s);
                 if (G.chunks.size() == 1) G.prepared_k = 4;
             }
             const Tile *ct = tiles;
@@ -1873,20 +1206,13 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
                 ct = tiles + a;
                 nct = y - a;
             }
-            launches += launch_edges4(G, c, b, e, ct, nct, e_begin, per_edge_out, gacc, s);
+            G.a_base = c.s0;
+            G.e_base = c.e0;
+            launches += launch_edges4(G, ct, nct, e_begin, per_edge_out, gacc, s);
         }
     }
     if (tmp.p) TG_CK(cudaStreamSynchronize(s));
     return launches;
-}
-
-int64_t launch_finalize(Graph &G, int k, int64_t *global_out, cudaStream_t s) {
-    const int64_t total = (int64_t)G.ngraphs * global_slots(G.L, k);
-    KernelTimer kt(G, s, "k_finalize");
-    k_finalize<<<grid_for(total, 256, 1 << 20), 256, 0, s>>>(G.ngraphs, G.L, k, G.gacc.as<unsigned long long>(), global_out,
-                                                              G.status.as<uint32_t>());
-    TG_CK(cudaGetLastError());
-    return 1;
 }
 
 }  // namespace tg

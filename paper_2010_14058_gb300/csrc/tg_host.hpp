@@ -6,6 +6,7 @@
 #include <cstring>
 #include <memory>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 #include <cuda_runtime.h>
@@ -171,7 +172,7 @@ struct Graph {
     bool hub_packed = false;                    // two 16-bit counters per word
     // counting state
     DBuf C, tau, A, tables, gacc, status, tiles_full, stage_pe, stage_gl;
-    DBuf xsum, tri_any;
+    DBuf xsum, tri_any, slot_rows;
     DBuf work;                          // [kWorkSlots] work counters (tg_set_work_counting)
     bool work_on = false;
     int64_t n_tiles_full = 0, max_chunk_edges = 0;
@@ -227,10 +228,12 @@ struct Graph {
         c.C = C.as<uint32_t>();
         c.tau = tau.as<int64_t>();
         c.A = A.as<uint32_t>();
+        c.slot_rows = slot_rows.as<uint32_t>();
         c.a_base = a_base;
         c.a_stride = a_stride;
         c.e_base = e_base;
         c.xsum = xsum.p;
+        c.wide = wide_sums();
         c.tri_any = tri_any.as<uint8_t>();
         c.tables = tables.as<uint32_t>();
         c.table_stride = table_stride;
@@ -251,7 +254,7 @@ struct Graph {
         return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &anchors_light, &anchors_heavy, &edges_light,
                              &edges_heavy, &C, &tau, &A, &tables, &gacc, &status, &tiles_full, &stage_pe,
-                             &stage_gl, &xsum, &tri_any, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
+                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
@@ -339,8 +342,16 @@ void prepare_edges(Graph &G, int k, cudaStream_t s);
 // stage recomputed (no cached state).  Returns the kernel launches.
 int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per_edge_out,
                   unsigned long long *gacc, bool full, cudaStream_t s);
+// rows and raw sums of the edges of the tiles (tg_epi.cu)
+void prepare_epi(Graph &G);
+int64_t launch_edges3(Graph &G, const Tile *tiles, int64_t n_tiles, int64_t e_begin, uint32_t *per_edge_out,
+                      unsigned long long *gacc, cudaStream_t s);
+// the per-slot 4-cycle planes of a chunk as rows, one per slot
+int64_t launch_slot_rows(Graph &G, int64_t n_slots, cudaStream_t s);
+int64_t launch_edges4(Graph &G, const Tile *tiles, int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
+                      unsigned long long *gacc, cudaStream_t s);
 int64_t launch_finalize(Graph &G, int k, int64_t *global_out, cudaStream_t s);
-// Position-aware typed graphlets (tg_pa.cu; epilogue in tg_count.cu).
+// Position-aware typed graphlets (tg_pa.cu; epilogue in tg_epi.cu).
 PaLayout pa_layout(int L);
 bool pa_labelling(int L, int block, int64_t rank, int32_t *labelling);
 std::vector<int32_t> pa_class_table(const PaLayout &Y);

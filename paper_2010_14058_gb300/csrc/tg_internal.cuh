@@ -55,6 +55,13 @@ struct HubSegment {
 };
 constexpr int64_t kHubTicketWords = 1 << 16;
 
+// Edges of one graph that a CTA of the per-edge kernels takes at a time.
+struct Tile {
+    int64_t begin, end;
+    int32_t graph, pad;
+};
+constexpr int kTile = 2048;                 // most edges per tile
+
 // Read-only view of a built graph, passed to kernels by value.
 struct GraphView {
     int32_t ngraphs;
@@ -86,10 +93,12 @@ struct CountView {
     uint32_t *C;                // [m][kCRow] typed triangle counts c_e^t (t < L)
     int64_t *tau;               // [n*L*L] ordered typed edges inside Gamma_x
     uint32_t *A;                // [L*L][a_stride] 4-cycle contributions per slot of the current chunk
+    const uint32_t *slot_rows;  // [slots][L*L] the same by slot (k_slot_rows), read by the epilogue
     int64_t a_base;             // first adjacency slot of the current chunk
     int64_t a_stride;           // slots per type-pair row of A
     int64_t e_base;             // first edge of the current chunk (xsum is relative to it)
     void *xsum;                 // [edges][L][4][L] TCi, TCj, DT, K' (tg_sums.cu): uint32, or uint64 when wide
+    bool wide;                  // xsum holds uint64
     uint8_t *tri_any;           // [n] 1 if a triangle has the node as its lowest
     uint32_t *tables;           // dense per-CTA wedge tables
     int64_t table_stride;       // entries (uint32) per CTA table
