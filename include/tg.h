@@ -114,18 +114,17 @@ typedef struct {
 
 /* Tuning knobs (0 = library default).  Results never depend on them. */
 typedef struct {
-    int32_t light_edge_max_degree;    /* edges whose triangle set T has at most max(this, 32) nodes:
-                                         warp per edge in the 4-clique pass (CTA per edge above) */
+    int32_t light_edge_max_degree;    /* accepted and ignored (the 4-cliques have one form) */
     int32_t light_anchor_max_wedges;  /* wedge anchors with at most this many wedges: warp per anchor
                                          (at most 2048, and what one CTA's shared memory holds for L) */
-    int32_t anchor_table_budget_mb;   /* device memory for the dense node tables of heavy anchors with
-                                         too many wedges for shared memory, one per CTA that takes them
-                                         (default 12,288; at most two CTAs per SM get one) */
+    int32_t anchor_table_budget_mb;   /* accepted and ignored (every anchor's table is in shared memory
+                                         or a hub table) */
     int32_t ctas_per_sm;              /* resident CTAs per SM for the per-edge kernels */
     int32_t cycle_budget_mb;          /* device memory for the per-slot 4-cycle array; a batch whose
                                          array would exceed it is counted in chunks of whole graphs */
-    int32_t hub_min_wedges;           /* anchors with more wedges than this are hubs: each is counted
-                                         by the whole GPU against one node table shared by all CTAs */
+    int32_t hub_min_wedges;           /* anchors with more wedges than this, or than a CTA's shared memory
+                                         holds, are hubs: each is counted by the whole GPU against one
+                                         node table shared by all CTAs */
     int32_t hub_l2_mb;                /* MB of hub node tables of the persistent hub pass: one group
                                          of hubs fills at most half of it (about the L2 size) */
     int32_t isect_modes;              /* typed set intersection per bucket of the shorter segment's

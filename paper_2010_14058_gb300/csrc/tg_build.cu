@@ -10,7 +10,7 @@
 //   * edge ids in the caller's lexicographic (u < v) order, the two slots of
 //     each edge and the edge id of every slot;
 //   * per-node typed degree sums delta_x[t][t'] = sum_{w in Gamma_x^t} d_w^t';
-//   * work lists: wedge anchors by wedge count, edges by min endpoint degree.
+//   * work lists: wedge anchors by class.
 // Sorting and compaction use CUB device primitives.
 #include <algorithm>
 #include <cstdint>
@@ -19,7 +19,6 @@
 
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
-#include <cub/device/device_select.cuh>
 
 #include "tg_host.hpp"
 #include "tg_local.cuh"
@@ -274,16 +273,19 @@ __global__ void k_delta(GraphView g, int64_t *delta) {
     }
 }
 
-// warp per anchor x: number of wedges x - v - w with v < x and w < x
-__global__ void k_anchor_work(GraphView g, int64_t *work) {
+// warp per anchor x: number of wedges x - v - w with v < x and w < x, and
+// the most lower-priority neighbours of one type
+__global__ void k_anchor_work(GraphView g, int64_t *work, int32_t *most) {
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp;
     int lane = threadIdx.x & (kWarp - 1);
     if (warp >= g.n) return;
     int32_t x = (int32_t)warp;
     int64_t total = 0;
+    int32_t mx = 0;
     for (int t = 0; t < g.L; ++t) {
         int64_t b = seg_begin(g, x, t), e = seg_end(g, x, t);
         int64_t cut = lower_bound_i32(g.adj, b, e, x);
+        mx = max(mx, (int32_t)(cut - b));
         for (int64_t s = b + lane; s < cut; s += kWarp) {
             int32_t v = g.adj[s];
             for (int q = 0; q < g.L; ++q) {
@@ -293,33 +295,10 @@ __global__ void k_anchor_work(GraphView g, int64_t *work) {
         }
     }
     for (int off = 16; off > 0; off >>= 1) total += __shfl_down_sync(0xffffffffu, total, off);
-    if (lane == 0) work[x] = total;
-}
-
-__global__ void k_classify_anchors(int64_t n, const int64_t *__restrict__ work, int64_t light_max, int64_t hub_min,
-                                   uint8_t *is_light, uint8_t *is_heavy, uint8_t *is_hub, int32_t *ids,
-                                   unsigned long long *heavy_key) {
-    int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    int64_t w = work[x];
-    is_light[x] = (w > 0 && w <= light_max) ? 1 : 0;
-    is_heavy[x] = (w > light_max && w <= hub_min) ? 1 : 0;
-    is_hub[x] = (w > hub_min) ? 1 : 0;
-    ids[x] = (int32_t)x;
-    heavy_key[x] = (unsigned long long)w;
-}
-
-__global__ void k_classify_edges(int64_t m, GraphView g, int64_t light_max_deg, uint8_t *is_light,
-                                 uint8_t *is_heavy, int32_t *ids, unsigned long long *cost) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= m) return;
-    int32_t a = g.e_lo[e], b = g.e_hi[e];
-    int64_t da = g.rp[a + 1] - g.rp[a], db = g.rp[b + 1] - g.rp[b];
-    int64_t mn = da < db ? da : db;
-    is_light[e] = mn <= light_max_deg ? 1 : 0;
-    is_heavy[e] = mn > light_max_deg ? 1 : 0;
-    ids[e] = (int32_t)e;
-    cost[e] = (unsigned long long)(da + db);
+    if (lane == 0) {
+        work[x] = total;
+        most[x] = mx;
+    }
 }
 
 template <class F>
@@ -336,52 +315,16 @@ int bits_for(int64_t v) {
     return b;
 }
 
-// Selects the flagged ids into a new device buffer; returns the count.
-int64_t select_flagged(const int32_t *ids, const uint8_t *flags, int64_t n, DBuf &out, cudaStream_t s) {
-    TBuf sel(sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1), s);
-    TBuf cnt(sizeof(int64_t), s);
-    cub_call([&](void *t, size_t &b) {
-        return cub::DeviceSelect::Flagged(t, b, ids, flags, sel.as<int32_t>(), cnt.as<int64_t>(), n, s);
-    }, s);
-    int64_t c = 0;
-    TG_CK(cudaMemcpyAsync(&c, cnt.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TG_CK(cudaStreamSynchronize(s));
-    out.alloc(sizeof(int32_t) * (size_t)std::max<int64_t>(c, 1));
-    TG_CK(cudaMemcpyAsync(out.p, sel.p, sizeof(int32_t) * (size_t)c, cudaMemcpyDeviceToDevice, s));
-    return c;
-}
-
 __global__ void k_widen(int64_t n, const int32_t *__restrict__ in, int64_t *out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) out[i] = in[i];
 }
 
-__global__ void k_count_above(int64_t c, const int32_t *__restrict__ ids, const unsigned long long *__restrict__ key,
-                              unsigned long long limit, unsigned long long *count) {
+// work of the listed nodes
+__global__ void k_gather_work(int64_t c, const int32_t *__restrict__ ids, const int64_t *__restrict__ work,
+                              int64_t *out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < c && key[ids[i]] > limit) atomicAdd(count, 1ull);
-}
-
-// Sorts `ids` (count c) by descending key (keys indexed by id).
-__global__ void k_gather_keys(int64_t c, const int32_t *__restrict__ ids, const unsigned long long *__restrict__ key,
-                              unsigned long long *out) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < c) out[i] = key[ids[i]];
-}
-
-void sort_desc_by_key(DBuf &ids, int64_t c, const unsigned long long *key, cudaStream_t s, int64_t &launches) {
-    if (c <= 1) return;
-    ++launches;
-    TBuf k_in(sizeof(unsigned long long) * c, s), k_out(sizeof(unsigned long long) * c, s);
-    TBuf v_out(sizeof(int32_t) * c, s);
-    k_gather_keys<<<blocks_for(c, kThreads), kThreads, 0, s>>>(c, ids.as<int32_t>(), key, k_in.as<unsigned long long>());
-    TG_CK(cudaGetLastError());
-    cub_call([&](void *t, size_t &b) {
-        return cub::DeviceRadixSort::SortPairsDescending(t, b, k_in.as<unsigned long long>(),
-                                                         k_out.as<unsigned long long>(), ids.as<int32_t>(),
-                                                         v_out.as<int32_t>(), c, 0, 64, s);
-    }, s);
-    TG_CK(cudaMemcpyAsync(ids.p, v_out.p, sizeof(int32_t) * c, cudaMemcpyDeviceToDevice, s));
+    if (i < c) out[i] = work[ids[i]];
 }
 
 uint32_t read_status(const DBuf &st, cudaStream_t s) {
@@ -599,66 +542,31 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
         TG_CK(cudaGetLastError());
     }
 
-    // 6. work lists
+    // 6. wedge anchors by class; hubs in ascending id order
     {
-        TBuf work(sizeof(int64_t) * std::max<int64_t>(n, 1), s);
-        TBuf fl(std::max<int64_t>(n, 1), s), fh(std::max<int64_t>(n, 1), s), ids(sizeof(int32_t) * std::max<int64_t>(n, 1), s);
-        TBuf key(sizeof(unsigned long long) * std::max<int64_t>(n, 1), s);
-        TBuf fhub(std::max<int64_t>(n, 1), s);
+        TBuf work(sizeof(int64_t) * std::max<int64_t>(n, 1), s), most(sizeof(int32_t) * std::max<int64_t>(n, 1), s);
         if (n > 0) {
             ++G.last_launches;
-            k_anchor_work<<<blocks_for(n * kWarp, kThreads), kThreads, 0, s>>>(G.view(), work.as<int64_t>());
-            ++G.last_launches;
-            k_classify_anchors<<<blocks_for(n, kThreads), kThreads, 0, s>>>(
-                n, work.as<int64_t>(), opt.light_anchor_max_wedges, opt.hub_min_wedges, fl.as<uint8_t>(),
-                fh.as<uint8_t>(), fhub.as<uint8_t>(), ids.as<int32_t>(), key.as<unsigned long long>());
+            k_anchor_work<<<blocks_for(n * kWarp, kThreads), kThreads, 0, s>>>(G.view(), work.as<int64_t>(),
+                                                                              most.as<int32_t>());
             TG_CK(cudaGetLastError());
         }
-        G.n_anchors_light = select_flagged(ids.as<int32_t>(), fl.as<uint8_t>(), n, G.anchors_light, s);
-        G.n_anchors_heavy = select_flagged(ids.as<int32_t>(), fh.as<uint8_t>(), n, G.anchors_heavy, s);
-        sort_desc_by_key(G.anchors_heavy, G.n_anchors_heavy, key.as<unsigned long long>(), s, G.last_launches);
-        {   // heavy anchors above the shared-memory hash's limit (they lead the sorted list)
-            TBuf cnt(sizeof(unsigned long long), s);
-            TG_CK(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long), s));
-            if (G.n_anchors_heavy > 0) {
-                ++G.last_launches;
-                k_count_above<<<blocks_for(G.n_anchors_heavy, kThreads), kThreads, 0, s>>>(
-                    G.n_anchors_heavy, G.anchors_heavy.as<int32_t>(), key.as<unsigned long long>(), kHeavyFit,
-                    cnt.as<unsigned long long>());
-                TG_CK(cudaGetLastError());
-            }
-            unsigned long long c = 0;
-            TG_CK(cudaMemcpyAsync(&c, cnt.p, sizeof(c), cudaMemcpyDeviceToHost, s));
-            TG_CK(cudaStreamSynchronize(s));
-            G.n_heavy_dense = (int64_t)c;
-        }
-        G.n_hubs = select_flagged(ids.as<int32_t>(), fhub.as<uint8_t>(), n, G.hubs, s);
+        list_anchors(G, work.as<int64_t>(), most.as<int32_t>(), s);
         G.h_hub_id.assign((size_t)G.n_hubs, 0);
         G.h_hub_wedges.assign((size_t)G.n_hubs, 0);
         if (G.n_hubs > 0) {
-            TBuf wk(sizeof(unsigned long long) * (size_t)G.n_hubs, s);
-            ++G.last_launches;
-            k_gather_keys<<<blocks_for(G.n_hubs, kThreads), kThreads, 0, s>>>(
-                G.n_hubs, G.hubs.as<int32_t>(), key.as<unsigned long long>(), wk.as<unsigned long long>());
-            TG_CK(cudaGetLastError());
+            TBuf wk(sizeof(int64_t) * (size_t)G.n_hubs, s);
             TG_CK(cudaMemcpyAsync(G.h_hub_id.data(), G.hubs.p, sizeof(int32_t) * G.n_hubs, cudaMemcpyDeviceToHost, s));
+            TG_CK(cudaStreamSynchronize(s));
+            std::sort(G.h_hub_id.begin(), G.h_hub_id.end());
+            TG_CK(cudaMemcpyAsync(G.hubs.p, G.h_hub_id.data(), sizeof(int32_t) * G.n_hubs, cudaMemcpyHostToDevice, s));
+            ++G.last_launches;
+            k_gather_work<<<blocks_for(G.n_hubs, kThreads), kThreads, 0, s>>>(G.n_hubs, G.hubs.as<int32_t>(),
+                                                                             work.as<int64_t>(), wk.as<int64_t>());
+            TG_CK(cudaGetLastError());
             TG_CK(cudaMemcpyAsync(G.h_hub_wedges.data(), wk.p, sizeof(int64_t) * G.n_hubs, cudaMemcpyDeviceToHost, s));
             TG_CK(cudaStreamSynchronize(s));
         }
-    }
-    {
-        TBuf fl(std::max<int64_t>(m, 1), s), fh(std::max<int64_t>(m, 1), s), ids(sizeof(int32_t) * std::max<int64_t>(m, 1), s);
-        TBuf cost(sizeof(unsigned long long) * std::max<int64_t>(m, 1), s);
-        if (m > 0) {
-            ++G.last_launches;
-            k_classify_edges<<<blocks_for(m, kThreads), kThreads, 0, s>>>(
-                m, G.view(), opt.light_edge_max_degree, fl.as<uint8_t>(), fh.as<uint8_t>(), ids.as<int32_t>(),
-                cost.as<unsigned long long>());
-            TG_CK(cudaGetLastError());
-        }
-        G.n_edges_light = select_flagged(ids.as<int32_t>(), fl.as<uint8_t>(), m, G.edges_light, s);
-        G.n_edges_heavy = select_flagged(ids.as<int32_t>(), fh.as<uint8_t>(), m, G.edges_heavy, s);
-        sort_desc_by_key(G.edges_heavy, G.n_edges_heavy, cost.as<unsigned long long>(), s, G.last_launches);
     }
     if (read_status(G.status, s) & ST_INVALID_GRAPH) throw Error{TG_ERR_INVALID_GRAPH, "asymmetric rows"};
 

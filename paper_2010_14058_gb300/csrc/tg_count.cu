@@ -49,346 +49,6 @@ namespace tg {
 
 namespace {
 
-constexpr int kAnchorThreads = 512;         // k_wedge_heavy: one anchor per CTA
-constexpr int kLightAnchorWarps = 4;        // k_wedge_light: one anchor per warp
-
-// ------------------------------------------------------------ wedge kernels
-// For an anchor u, V_u = {v in Gamma_u : v < u} and, for v in V_u, the
-// wedge ends {w in Gamma_v : w < u}.  Phase 1 counts, per wedge end w and
-// per type t of the middle node, the wedges u - v - w (table H_u[w][t]).
-// Phase 2 revisits every wedge u - v - w: the other middles x of (u,w) of
-// type t number cnt_t = H_u[w][t] - [phi_v = t]; each closes the 4-cycle
-// u - v - w - x - u, which is recorded on
-//   slot (v -> w): A[phi_u][t]   (v's other cycle neighbour u, w's is x)
-//   slot (u -> v): A[t][phi_w]   (u's other cycle neighbour x, v's is w).
-// A[s][t] of a slot (a -> b) counts 4-cycles a - b - y - z - a with
-// phi_z = s (a's other neighbour) and phi_y = t (b's other neighbour).
-
-// cut of typed segment (x, t) at id < bound
-__device__ __forceinline__ void seg_prefix(const GraphView &g, int64_t x, int t, int32_t bound, int64_t &b,
-                                           int64_t &cut) {
-    b = seg_begin(g, x, t);
-    cut = lower_bound_i32(g.adj, b, seg_end(g, x, t), bound);
-}
-
-__device__ __forceinline__ int hash_slot(int32_t w, int cap) {
-    return (int)(((uint32_t)w * 2654435761u) & (uint32_t)(cap - 1));
-}
-
-// open addressing in shared memory; returns the slot or -1 when full
-__device__ int hash_insert(int32_t *keys, int cap, int32_t w) {
-    int h = hash_slot(w, cap);
-    for (int probe = 0; probe < cap; ++probe) {
-        int32_t k = keys[h];
-        if (k == w) return h;
-        if (k == -1) {
-            int32_t old = atomicCAS(&keys[h], -1, w);
-            if (old == -1 || old == w) return h;
-        }
-        h = (h + 1) & (cap - 1);
-    }
-    return -1;
-}
-__device__ int hash_find(const int32_t *keys, int cap, int32_t w) {
-    int h = hash_slot(w, cap);
-    for (int probe = 0; probe < cap; ++probe) {
-        int32_t k = keys[h];
-        if (k == w) return h;
-        if (k == -1) return -1;
-        h = (h + 1) & (cap - 1);
-    }
-    return -1;
-}
-
-// ------------------------------------------------------------ wedges of one v
-// The wedges u - v - w (v, w below the anchor u) of one neighbour v, all
-// types of w flattened: lane t < L finds the part of v's type-t segment
-// below u (one binary search per lane, in parallel) and its exclusive
-// offset; wedge p of v then has type tw = the last lane t whose offset is
-// <= p, and lanes take 32 wedges at a time whatever their types.
-struct VRuns {
-    int64_t b;          // lane t < L: first slot of type t in v's row
-    int32_t off;        // lane t < L: wedges of types < t (total on lanes >= L)
-    int32_t total;      // wedges of v
-};
-
-__device__ __forceinline__ VRuns v_runs(const GraphView &g, int32_t v, int32_t u, int lane) {
-    VRuns r;
-    r.b = 0;
-    int32_t n = 0;
-    if (lane < g.L) {
-        int64_t cut;
-        seg_prefix(g, v, lane, u, r.b, cut);
-        n = (int32_t)(cut - r.b);
-    }
-    int32_t inc = n;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    r.off = inc - n;
-    r.total = __shfl_sync(0xffffffffu, inc, kMaxL - 1);
-    return r;
-}
-
-// per-(v, type of w) sums of phase 1 over the lanes (runs of equal tw are
-// contiguous): tail lanes add them to the 4-cycle slot of (u, v)
-__device__ __forceinline__ void flush_runs(uint32_t *A, int64_t nnz, int L, const uint32_t *c, int key, int tw,
-                                           int64_t sv, int lane) {
-    unsigned same = 0;
-#pragma unroll
-    for (int s = 0; s < 5; ++s) {
-        const int kk = __shfl_up_sync(0xffffffffu, key, 1 << s);
-        if (lane >= (1 << s) && kk == key) same |= 1u << s;
-    }
-    const int knext = __shfl_down_sync(0xffffffffu, key, 1);
-    const bool tail = key >= 0 && (lane == 31 || knext != key);
-#pragma unroll
-    for (int t = 0; t < kMaxL; ++t) {
-        if (t >= L) break;
-        uint32_t v = c[t];
-#pragma unroll
-        for (int s = 0; s < 5; ++s) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, v, 1 << s);
-            if (same & (1u << s)) v += y;
-        }
-        if (tail && v) atomicAdd(&A[(int64_t)(t * L + tw) * nnz + sv], v);
-    }
-}
-
-// One phase of the wedges of v for one warp.  rows(w, insert) gives w's
-// counter row (L entries): phase 0 inserts and adds 1 at t_v; phase 1 adds
-// h[w][t] - [t = t_v] to the slot of (v, w) and the per-type sums to the
-// slot of (u, v); phase 2 clears the row (dense tables only).
-template <class Rows>
-__device__ __forceinline__ void wedge_v(const GraphView &g, uint32_t *A, int64_t nnz, int32_t u, int tu, int32_t v,
-                                        int tv, int64_t sv, int phase, int lane, Rows rows) {
-    const int L = g.L;
-    const VRuns r = v_runs(g, v, u, lane);
-    for (int32_t p0 = 0; p0 < r.total; p0 += 32) {
-        const int32_t p = p0 + lane;
-        int tw = 0;
-#pragma unroll
-        for (int st = kMaxL / 2; st > 0; st >>= 1) {
-            const int32_t c = __shfl_sync(0xffffffffu, r.off, tw + st);
-            if (c <= p) tw += st;
-        }
-        const int64_t k = __shfl_sync(0xffffffffu, r.b, tw) + (p - __shfl_sync(0xffffffffu, r.off, tw));
-        const bool act = p < r.total;
-        uint32_t c[kMaxL];
-#pragma unroll
-        for (int t = 0; t < kMaxL; ++t) c[t] = 0;
-        if (act) {
-            const int32_t w = g.adj[k];
-            uint32_t *row = rows(w, phase == 0);
-            if (row) {
-                if (phase == 0) {
-                    atomicAdd(row + tv, 1u);
-                } else if (phase == 1) {
-#pragma unroll
-                    for (int t = 0; t < kMaxL; ++t) {
-                        if (t >= L) break;
-                        const uint32_t x = row[t] - (t == tv ? 1u : 0u);
-                        c[t] = x;
-                        if (x) atomicAdd(&A[(int64_t)(tu * L + t) * nnz + k], x);
-                    }
-                } else {
-                    for (int t = 0; t < L; ++t) row[t] = 0;
-                }
-            }
-        }
-        if (phase == 1) flush_runs(A, nnz, L, c, act ? tw : -1, tw, sv, lane);
-    }
-}
-
-// lower-priority neighbours of u by type: lane t < L gets the first slot
-// of type t and the exclusive offset of its part; returns their number
-__device__ __forceinline__ int32_t u_runs(const GraphView &g, int32_t u, int lane, int64_t &ub, int32_t &uoff) {
-    int32_t n = 0;
-    ub = 0;
-    if (lane < g.L) {
-        int64_t cut;
-        seg_prefix(g, u, lane, u, ub, cut);
-        n = (int32_t)(cut - ub);
-    }
-    int32_t inc = n;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    uoff = inc - n;
-    return __shfl_sync(0xffffffffu, inc, kMaxL - 1);
-}
-
-// neighbour number kv of u's lower-priority neighbours -> (slot, type)
-__device__ __forceinline__ int64_t u_slot(int64_t ub, int32_t uoff, int32_t kv, int &tv) {
-    tv = 0;
-#pragma unroll
-    for (int st = kMaxL / 2; st > 0; st >>= 1) {
-        const int32_t c = __shfl_sync(0xffffffffu, uoff, tv + st);
-        if (c <= kv) tv += st;
-    }
-    return __shfl_sync(0xffffffffu, ub, tv) + (kv - __shfl_sync(0xffffffffu, uoff, tv));
-}
-
-// Light anchors (few wedges): one warp per anchor, table in shared memory
-// (a hash of capacity `cap` >= 2 x the anchor's wedges).
-__global__ void __launch_bounds__(kLightAnchorWarps * 32) k_wedge_light(GraphView g, CountView cv,
-                                                                        const int32_t *__restrict__ anchors,
-                                                                        int64_t n_anchors, int cap, int64_t n0,
-                                                                        int64_t n1) {
-    extern __shared__ int32_t smem[];
-    const int L = g.L;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int32_t *keys = smem + wid * cap * (1 + L);
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(keys + cap);
-    for (int k = lane; k < cap; k += 32) keys[k] = -1;
-    for (int k = lane; k < cap * L; k += 32) cnt[k] = 0;
-    __syncwarp();
-    const int64_t nw = (int64_t)gridDim.x * kLightAnchorWarps;
-    const int64_t nnz = cv.a_stride;
-    uint32_t *A = cv.A - cv.a_base;                          // indexed by absolute slot
-    auto rows = [&](int32_t w, bool insert) -> uint32_t * {
-        const int h = insert ? hash_insert(keys, cap, w) : hash_find(keys, cap, w);
-        if (h < 0) {
-            if (insert) set_status(cv.status, ST_INTERNAL);
-            return nullptr;
-        }
-        return cnt + h * L;
-    };
-    for (int64_t a = (int64_t)blockIdx.x * kLightAnchorWarps + wid; a < n_anchors; a += nw) {
-        const int32_t u = anchors[a];
-        if (u < n0 || u >= n1) continue;                    // anchor outside this chunk
-        const int tu = g.ty[u];
-        int64_t ub;
-        int32_t uoff;
-        const int32_t nV = u_runs(g, u, lane, ub, uoff);
-        for (int phase = 0; phase < 2; ++phase) {
-            for (int32_t kv = 0; kv < nV; ++kv) {
-                int tv;
-                const int64_t sv = u_slot(ub, uoff, kv, tv);
-                wedge_v(g, A, nnz, u, tu, g.adj[sv], tv, sv, phase, lane, rows);
-            }
-            __syncwarp();
-        }
-        for (int k = lane; k < cap; k += 32) keys[k] = -1;
-        for (int k = lane; k < cap * L; k += 32) cnt[k] = 0;
-        __syncwarp();
-    }
-}
-
-// Heavy anchors: one CTA per anchor, warps over the anchor's lower-priority
-// neighbours v.  The rows h[w][.] live in a shared-memory hash of kHeavyCap
-// entries.  Anchors with more wedges than 3/4 of it go to a dense node table
-// in global memory (cleared again by phase 2): on power-law graphs their
-// wedge ends are almost all distinct.  Only the first n_tables CTAs own a
-// table (the budget of anchor_table_budget_mb); the grid may be larger, and
-// the CTAs without a table take hash anchors only.
-
-__device__ int hash_insert_bounded(int32_t *keys, int cap, int32_t w, int *fill, int limit) {
-    int h = hash_slot(w, cap);
-    for (int probe = 0; probe < cap; ++probe) {
-        int32_t k = keys[h];
-        if (k == w) return h;
-        if (k == -1) {
-            if (atomicAdd(fill, 1) >= limit) return -1;     // over the load limit
-            const int32_t old = atomicCAS(&keys[h], -1, w);
-            if (old == -1) return h;
-            atomicSub(fill, 1);
-            if (old == w) return h;
-        }
-        h = (h + 1) & (cap - 1);
-    }
-    return -1;
-}
-
-__global__ void __launch_bounds__(kAnchorThreads, 2) k_wedge_heavy(GraphView g, CountView cv,
-                                                               const int32_t *__restrict__ anchors,
-                                                               int64_t n_anchors, int64_t n_dense, int64_t n_tables,
-                                                               int64_t n0, int64_t n1) {
-    extern __shared__ int32_t hsm[];
-    __shared__ int s_fill, s_over;
-    const int L = g.L;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    int32_t *keys = hsm;
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(hsm + kHeavyCap);
-    const bool has_table = blockIdx.x < n_tables;
-    uint32_t *tbl = cv.tables + (int64_t)(has_table ? blockIdx.x : 0) * cv.table_stride;
-    // a CTA without a dense table never falls back to one: its hash anchors
-    // have at most kHeavyFit distinct wedge ends, and with the limit at the
-    // capacity the fill count (distinct ends plus at most one in-flight
-    // insert per thread) cannot reach it
-    const int limit = has_table ? kHeavyFit : kHeavyCap - 1;
-    const int64_t nnz = cv.a_stride;
-    uint32_t *A = cv.A - cv.a_base;                          // indexed by absolute slot
-    // pass 0: the first n_dense anchors (more wedges than the hash's load
-    // limit, sorted first) against the dense tables, by the CTAs that own
-    // one; pass 1: the other anchors against the shared-memory hash, by all
-    for (int pass = 0; pass < 2; ++pass) {
-        const int64_t a_end = pass == 0 ? (has_table ? n_dense : 0) : n_anchors;
-        const int64_t a_step = pass == 0 ? n_tables : gridDim.x;
-        for (int64_t a = (pass == 0 ? 0 : n_dense) + blockIdx.x; a < a_end; a += a_step) {
-            const int32_t u = anchors[a];
-            if (u < n0 || u >= n1) continue;                // anchor outside this chunk (uniform per CTA)
-            const int tu = g.ty[u];
-            const int64_t base = g.node_off[graph_of_node(g, u)];
-            const bool pre_dense = pass == 0;
-            if (!pre_dense) {
-                for (int k = threadIdx.x; k < kHeavyCap; k += blockDim.x) keys[k] = -1;
-                for (int k = threadIdx.x; k < kHeavyCap * L; k += blockDim.x) cnt[k] = 0;
-            }
-            if (threadIdx.x == 0) { s_fill = 0; s_over = pre_dense ? 1 : 0; }
-            __syncthreads();
-            int64_t ub;
-            int32_t uoff;
-            const int32_t nV = u_runs(g, u, lane, ub, uoff);
-            auto hash_rows = [&](int32_t w, bool insert) -> uint32_t * {
-                int h;
-                if (insert) {
-                    h = hash_insert_bounded(keys, kHeavyCap, w, &s_fill, limit);
-                    if (h < 0) { s_over = 1; return nullptr; }
-                } else {
-                    h = hash_find(keys, kHeavyCap, w);
-                    if (h < 0) return nullptr;
-                }
-                return cnt + h * L;
-            };
-            auto dense_rows = [&](int32_t w, bool) -> uint32_t * { return tbl + (int64_t)(w - base) * L; };
-            if (!pre_dense) {
-                for (int32_t kv = wid; kv < nV; kv += nwarp) {
-                    int tv;
-                    const int64_t sv = u_slot(ub, uoff, kv, tv);
-                    wedge_v(g, A, nnz, u, tu, g.adj[sv], tv, sv, 0, lane, hash_rows);
-                }
-                __syncthreads();
-            }
-            const bool dense = s_over != 0;                 // uniform after the barrier
-            if (dense && !has_table) {                      // excluded above; reported, never miscounted
-                if (threadIdx.x == 0) set_status(cv.status, ST_INTERNAL);
-                __syncthreads();
-                continue;
-            }
-            if (dense)
-                for (int32_t kv = wid; kv < nV; kv += nwarp) {
-                    int tv;
-                    const int64_t sv = u_slot(ub, uoff, kv, tv);
-                    wedge_v(g, A, nnz, u, tu, g.adj[sv], tv, sv, 0, lane, dense_rows);
-                }
-            __syncthreads();
-            for (int phase = 1; phase < (dense ? 3 : 2); ++phase) {
-                for (int32_t kv = wid; kv < nV; kv += nwarp) {
-                    int tv;
-                    const int64_t sv = u_slot(ub, uoff, kv, tv);
-                    if (dense) wedge_v(g, A, nnz, u, tu, g.adj[sv], tv, sv, phase, lane, dense_rows);
-                    else wedge_v(g, A, nnz, u, tu, g.adj[sv], tv, sv, phase, lane, hash_rows);
-                }
-                __syncthreads();
-            }
-        }
-    }
-}
 
 // ------------------------------------------------------------ hub anchors
 // An anchor u with very many wedges (a hub) is counted by the whole GPU at
@@ -399,7 +59,7 @@ __global__ void __launch_bounds__(kAnchorThreads, 2) k_wedge_heavy(GraphView g, 
 // (hub, v, type of w) with at least one wedge; item_woff is the exclusive
 // prefix of the items' wedge counts, so wedge x of the flattened order is
 // w = adj[item_vb[it] + x - item_woff[it]] for the item it containing x.
-// The counts are the same as k_wedge_heavy's: phase 0 fills h_u[w][t] (the
+// The counts are those of tg_wedge.cu: phase 0 fills h_u[w][t] (the
 // number of type-t neighbours v of u below u that are adjacent to w),
 // phase 1 adds h_u[w][t] - [t = t_v] to the 4-cycle slot of (v, w) and the
 // per-(v, type of w) sums to the slot of (u, v), phase 2 clears the rows.
@@ -843,15 +503,6 @@ static const Tile *tiles_for(Graph &G, int64_t e_begin, int64_t e_end, int64_t &
     return dst.as<Tile>();
 }
 
-int light_anchor_limit(int L) {
-    int dev = 0, optin = 0;
-    TG_CK(cudaGetDevice(&dev));
-    TG_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    int cap = 1;                                              // per-warp hash of k_wedge_light
-    while ((size_t)kLightAnchorWarps * (cap * 2) * (1 + L) * sizeof(int32_t) <= (size_t)optin) cap *= 2;
-    return cap / 2;                                           // capacity >= 2 x wedges
-}
-
 void raise_smem_limit(const void *func, size_t bytes) {
     struct Limit { const void *func; int dev; size_t bytes; };
     static std::mutex mu;
@@ -871,17 +522,11 @@ void raise_smem_limit(const void *func, size_t bytes) {
 // Tiles and kernel attributes of the count (done before any capture).
 void prepare_edges(Graph &G, int k, cudaStream_t s) {
     if (k == 4) prepare_epi(G);
-    raise_smem_limit((const void *)k_wedge_heavy, (size_t)kHeavyCap * (1 + G.L) * sizeof(int32_t));
+    if (k == 4) prepare_wedges(G);
     DBuf unused;
     unused.owner = &G.stream;
     int64_t nt = 0;
     tiles_for(G, 0, G.m, nt, unused, s);
-    if (k == 4 && G.n_anchors_light > 0) {
-        int cap = 1;
-        while (cap < 2 * G.opt.light_anchor_max_wedges) cap <<= 1;
-        const size_t smem = (size_t)kLightAnchorWarps * cap * (1 + G.L) * sizeof(int32_t);
-        raise_smem_limit((const void *)k_wedge_light, smem);
-    }
 }
 
 // words of one hub's counter table (one row of L counters per node of its graph)
@@ -1108,23 +753,8 @@ static int64_t launch_wedges(Graph &G, const Graph::Chunk &c, cudaStream_t s) {
     if (c.s1 > c.s0)
         TG_CK(cudaMemset2DAsync(G.A.p, (size_t)G.a_stride * sizeof(uint32_t), 0, (size_t)(c.s1 - c.s0) * sizeof(uint32_t),
                                 (size_t)L * L, s));
-    if (G.n_anchors_light > 0) {
-        int cap = 1;
-        while (cap < 2 * G.opt.light_anchor_max_wedges) cap <<= 1;
-        const size_t smem = (size_t)kLightAnchorWarps * cap * (1 + L) * sizeof(int32_t);
-        KernelTimer kt(G, s, "k_wedge_light");
-        k_wedge_light<<<grid_for(G.n_anchors_light, kLightAnchorWarps, sms * 8), kLightAnchorWarps * 32, smem, s>>>(
-            gv, cv, G.anchors_light.as<int32_t>(), G.n_anchors_light, cap, c.n0, c.n1);
-        ++launches;
-    }
     if (G.n_hubs > 0) launches += launch_hubs(G, (size_t)(&c - G.chunks.data()), s);
-    if (G.n_anchors_heavy > 0) {
-        KernelTimer kt(G, s, "k_wedge_heavy");
-        const int grid = (int)std::min<int64_t>(std::max<int64_t>(G.n_tables, 2 * sms), G.n_anchors_heavy);
-        k_wedge_heavy<<<std::max(grid, G.n_tables), kAnchorThreads, (size_t)kHeavyCap * (1 + L) * sizeof(int32_t), s>>>(
-            gv, cv, G.anchors_heavy.as<int32_t>(), G.n_anchors_heavy, G.n_heavy_dense, G.n_tables, c.n0, c.n1);
-        ++launches;
-    }
+    launches += launch_anchor_wedges(G, c.n0, c.n1, s);
     TG_CK(cudaGetLastError());
     return launches;
 }
@@ -1150,17 +780,6 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
         prepare_sums(G);
         if (G.n_hubs > 0 && !G.hubs_ready) prepare_hubs(G, s);
         if (G.n_hubs > 0 && G.hub_plans.empty()) plan_hubs(G, s);
-        if (G.n_anchors_heavy > 0 && G.n_tables == 0) {
-            const int64_t stride = std::max<int64_t>(G.max_graph_nodes, 1) * L;
-            const int64_t per = stride * (int64_t)sizeof(uint32_t);
-            int64_t budget = (int64_t)G.opt.anchor_table_budget_mb << 20;
-            const int64_t need = G.n_anchors_heavy;
-            int64_t nt = std::min<int64_t>({(int64_t)2 * sm_count(), need, std::max<int64_t>(budget / per, 1)});
-            G.tables.alloc((size_t)(nt * per));
-            TG_CK(cudaMemsetAsync(G.tables.p, 0, (size_t)(nt * per), s));
-            G.table_stride = stride;
-            G.n_tables = (int32_t)nt;
-        }
     }
 }
 

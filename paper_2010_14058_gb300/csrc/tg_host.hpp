@@ -40,7 +40,7 @@ inline void throw_cuda(cudaError_t e, const char *what) {
 void raise_smem_limit(const void *func, size_t bytes);
 
 // Largest light_anchor_max_wedges whose per-warp hashes of k_wedge_light fit
-// one CTA's shared memory for L types.  Defined in tg_count.cu.
+// one CTA's shared memory for L types.  Defined in tg_wedge.cu.
 int light_anchor_limit(int L);
 
 #define TG_CK(call) ::tg::throw_cuda((call), #call)
@@ -135,9 +135,8 @@ struct Graph {
     DBuf tri_list[3], local_scratch;
     int64_t tri_count[3] = {0, 0, 0}, max_nplus = 0;
     // work lists
-    DBuf anchors_light, anchors_heavy, edges_light, edges_heavy;
-    int64_t n_anchors_light = 0, n_anchors_heavy = 0, n_edges_light = 0, n_edges_heavy = 0;
-    int64_t n_heavy_dense = 0;          // leading heavy anchors with more than kHeavyFit wedges
+    DBuf anchors[kHubClass], anchor_wedges;     // wedge anchors by class (tg_wedge.cu); wedges of every node
+    int64_t n_anchors[kHubClass] = {};
     // hub anchors (ascending id) and their wedge items: one item per
     // (hub, lower-priority neighbour v, type of w) with at least one wedge
     DBuf hubs, hub_base, item_woff, item_rec;
@@ -171,14 +170,12 @@ struct Graph {
     int64_t hub_stride = 0, hub_buf_words = 0;  // words per hub table, per buffer
     bool hub_packed = false;                    // two 16-bit counters per word
     // counting state
-    DBuf C, tau, A, tables, gacc, status, tiles_full, stage_pe, stage_gl;
+    DBuf C, tau, A, gacc, status, tiles_full, stage_pe, stage_gl;
     DBuf xsum, tri_any, slot_rows;
     DBuf work;                          // [kWorkSlots] work counters (tg_set_work_counting)
     bool work_on = false;
     int64_t n_tiles_full = 0, max_chunk_edges = 0;
     int64_t e_base = 0;
-    int64_t table_stride = 0;
-    int32_t n_tables = 0;
     int32_t prepared_k = 0;             // 0: nothing, 3: C, 4: C and the chunk's per-slot and per-edge sums
     bool tau_ready = false;             // tau of the current C
     int64_t last_launches = 0;
@@ -235,8 +232,6 @@ struct Graph {
         c.xsum = xsum.p;
         c.wide = wide_sums();
         c.tri_any = tri_any.as<uint8_t>();
-        c.tables = tables.as<uint32_t>();
-        c.table_stride = table_stride;
         c.gacc = gacc.as<unsigned long long>();
         c.status = status.as<uint32_t>();
         c.work = work_on ? work.as<unsigned long long>() : nullptr;
@@ -252,8 +247,8 @@ struct Graph {
     }
     std::vector<const DBuf *> cbuffers() const {
         return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
-                             &e_slot_lo, &e_slot_hi, &delta, &anchors_light, &anchors_heavy, &edges_light,
-                             &edges_heavy, &C, &tau, &A, &tables, &gacc, &status, &tiles_full, &stage_pe,
+                             &e_slot_lo, &e_slot_hi, &delta, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
+                             &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
                              &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
                 &pa_cls, &pa_gacc};
     }
@@ -333,6 +328,13 @@ int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s);
 // graphs with nodes [n0, n1) (tg_sums.cu); prepare_sums before any capture
 void prepare_sums(Graph &G);
 int64_t launch_sums(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s);
+
+// wedge anchors (tg_wedge.cu): class lists from the wedges and the most
+// lower-priority neighbours of one type of every node (the hubs unsorted);
+// the wedge pass of the anchors of [n0, n1) that are not hubs
+void list_anchors(Graph &G, const int64_t *work, const int32_t *most, cudaStream_t s);
+void prepare_wedges(Graph &G);
+int64_t launch_anchor_wedges(Graph &G, int64_t n0, int64_t n1, cudaStream_t s);
 
 // count entries (tg_count.cu)
 void prepare_counting(Graph &G, int k, cudaStream_t s);

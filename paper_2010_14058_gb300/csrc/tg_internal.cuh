@@ -31,12 +31,17 @@ constexpr int kWarp = 32;
 constexpr int kCRow = 8;                           // words per row of typed triangle counts (one 32-byte sector)
 constexpr int kTypeShift = 29;                     // packed (type << 29 | id) sort keys
 constexpr int32_t kIdMask = (1 << kTypeShift) - 1;
-constexpr int kHeavyCap = 4096;                    // shared-memory hash rows of a heavy anchor
 // slots of the optional work counters (tg_set_work_counting; TG_WORK_*)
 enum : int { kWorkCliqueProbes = 0, kWorkCliqueSearches = 1, kWorkCliqueBigProbes = 2, kWorkHubWait = 3,
              kWorkHubKind = 4 /* + ticket kind 0..3 */, kWorkHubWedges = 8, kWorkHubSlotUpdates = 9,
              kWorkSlots = 16 };
-constexpr int kHeavyFit = kHeavyCap / 4 * 3;       // its load limit (distinct wedge ends)
+
+// Wedge anchors by class (tg_wedge.cu): 0 a warp, 1-4 a CTA by table size, kHubClass hubs.
+constexpr int kHubClass = 5;
+struct WedgeLimits {
+    int64_t light, hub;         // most wedges of class 0, and of the shared-memory classes
+    int64_t bytes[4];           // table bytes of classes 1 to 4
+};
 
 // Persistent hub pass (tg_count.cu): a group of hubs whose counter tables
 // share one table buffer, and the ticket queue as runs of tickets of one
@@ -100,8 +105,6 @@ struct CountView {
     void *xsum;                 // [edges][L][4][L] TCi, TCj, DT, K' (tg_sums.cu): uint32, or uint64 when wide
     bool wide;                  // xsum holds uint64
     uint8_t *tri_any;           // [n] 1 if a triangle has the node as its lowest
-    uint32_t *tables;           // dense per-CTA wedge tables
-    int64_t table_stride;       // entries (uint32) per CTA table
     unsigned long long *gacc;   // [ngraphs*G] raw per-graphlet edge sums
     uint32_t *status;           // device status word
     unsigned long long *work;   // [kWorkSlots] work counters, or nullptr (counting off)
@@ -231,6 +234,13 @@ __device__ __forceinline__ int64_t seg_end(const GraphView &g, int64_t x, int t)
 __device__ __forceinline__ int32_t typed_degree(const GraphView &g, int64_t x, int t) {
     const int32_t *o = g.toff + x * (g.L + 1);
     return o[t + 1] - o[t];
+}
+
+// cut of typed segment (x, t) at id < bound
+__device__ __forceinline__ void seg_prefix(const GraphView &g, int64_t x, int t, int32_t bound, int64_t &b,
+                                           int64_t &cut) {
+    b = seg_begin(g, x, t);
+    cut = lower_bound_i32(g.adj, b, seg_end(g, x, t), bound);
 }
 
 __device__ __forceinline__ void set_status(uint32_t *status, uint32_t bits) {
