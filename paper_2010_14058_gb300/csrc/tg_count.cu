@@ -70,6 +70,8 @@ namespace {
 struct HubView {
     const int32_t *hubs;        // hub node ids
     const int64_t *hub_base;    // first node of each hub's graph (read when batched)
+    const int32_t *hub_nlow;    // nodes of each hub's graph with one-word rows (read when batched)
+    int32_t nlow;               // the same when there is one graph
     const int64_t *woff;        // [n_items + 1] first wedge of each item
     const int4 *item;           // per item: adj position of its first w, adj position of v in the
                                 // hub's row, hub index, type of u << 8 | type of v << 4 | type of w
@@ -78,8 +80,15 @@ struct HubView {
 
 constexpr int kHubThreads = 256;
 
+// Table rows.  A counter h_u[w][t] is at most d_w^t, so a node w of degree
+// below 2^(32 / L) has all its types in one word; the nodes of a graph are
+// in degree order, so these are a prefix of its ids (L = 5: degree 63 and
+// less, 96% of a Chung-Lu graph of average degree 20), and its table is a
+// third of one with 16-bit counters throughout.
+__host__ __device__ __forceinline__ int low_bits(int L) { return 32 / L; }
+
 __global__ void k_hub_nv(GraphView g, const int32_t *__restrict__ hubs, int64_t n_hubs, int64_t *nv,
-                         int64_t *hub_base) {
+                         int64_t *hub_base, int32_t *hub_nlow) {
     const int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (h > n_hubs) return;
     if (h == n_hubs) { nv[h] = 0; return; }
@@ -91,7 +100,15 @@ __global__ void k_hub_nv(GraphView g, const int32_t *__restrict__ hubs, int64_t 
         acc += cut - b;
     }
     nv[h] = acc;
-    hub_base[h] = g.node_off[graph_of_node(g, u)];
+    const int gr = graph_of_node(g, u);
+    const int64_t base = g.node_off[gr];
+    hub_base[h] = base;
+    int64_t lo = base, hi = g.node_off[gr + 1];             // first node whose degree has no room in a field
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if ((g.rp[mid + 1] - g.rp[mid]) >> low_bits(g.L)) hi = mid; else lo = mid + 1;
+    }
+    hub_nlow[h] = (int32_t)(lo - base);
 }
 
 // CTA per hub: wedge count of every (v, type of w) of the hub
@@ -179,18 +196,19 @@ __device__ __forceinline__ int64_t hub_find_item(const int64_t *__restrict__ wof
 // hubs (items [i0, i1), first hub h0; hub h's table at tbl + (h - h0) *
 // stride).  Warp wi of nwi takes one contiguous run of the range, 32 wedges
 // at a time, one wedge per lane; the item window of the next 32 wedges is
-// loaded while the current ones are worked on.  Counters: kPacked = two
-// 16-bit counters per 32-bit word (types 2k and 2k+1; every count is at
-// most the hub's degree, below 2^16 when this layout is chosen), else one
-// 32-bit counter per type.  The tables are read and cleared at L2
-// (ld/st.cg): other CTAs of the same launch update them, so no L1 copy may
-// be trusted.
+// loaded while the current ones are worked on.  Counters: one word per node
+// for the graph's low nodes (above); for the others kPacked = two 16-bit
+// counters per 32-bit word (types 2k and 2k+1; every count is at most the
+// hub's degree, below 2^16 when this layout is chosen), else one 32-bit
+// counter per type.  The tables are read and cleared at L2 (ld/st.cg): other
+// CTAs of the same launch update them, so no L1 copy may be trusted.
 template <bool kPacked, bool kCount>
 __device__ void hub_wedges(const GraphView &g, const CountView &cv, const HubView &hv, int64_t i0, int64_t i1,
                            int64_t x0r, int64_t x1r, int32_t h0, uint32_t *tbl, int64_t stride, int phase, int wi,
                            int nwi, int lane) {
     const int L = g.L;
-    const int RW = kPacked ? (L + 1) / 2 : L;               // words per table row
+    const int RW = kPacked ? (L + 1) / 2 : L;               // words per row of a node that is not low
+    const int lb = low_bits(L);                             // bits per type in a low node's word
     const int64_t per = (((x1r - x0r) + nwi - 1) / nwi + 31) & ~(int64_t)31;
     int64_t x0 = x0r + wi * per;
     const int64_t xe = min(x1r, x0 + per);
@@ -233,25 +251,34 @@ __device__ void hub_wedges(const GraphView &g, const CountView &cv, const HubVie
             const int64_t pos = (int64_t)rec.x + (x - wstart);
             const int32_t w = g.adj[pos];
             const int64_t base = hv.batched ? hv.hub_base[hh] : 0;
-            uint32_t *row = tbl + (int64_t)(hh - h0) * stride + (w - base) * RW;
+            const int32_t nlow = hv.batched ? hv.hub_nlow[hh] : hv.nlow;
+            const int32_t rel = (int32_t)(w - base);
+            const bool low = rel < nlow;
+            uint32_t *row = tbl + (int64_t)(hh - h0) * stride + (low ? rel : nlow + (int64_t)(rel - nlow) * RW);
             if (phase == 0) {
-                if (kPacked) atomicAdd(row + (tv >> 1), 1u << (16 * (tv & 1)));
+                if (low) atomicAdd(row, 1u << (lb * tv));
+                else if (kPacked) atomicAdd(row + (tv >> 1), 1u << (16 * (tv & 1)));
                 else atomicAdd(row + tv, 1u);
             } else if (phase == 1) {
                 const int tu = rec.w >> 8;
                 uint32_t words[kMaxL];
+                words[0] = __ldcg(row);
 #pragma unroll
-                for (int q = 0; q < kMaxL; ++q) words[q] = q < RW ? __ldcg(row + q) : 0u;
+                for (int q = 1; q < kMaxL; ++q) words[q] = !low && q < RW ? __ldcg(row + q) : 0u;
+                if (!low || words[0] != 1u << (lb * tv)) {  // (else this wedge alone: it closes nothing)
+                    const uint32_t lm = lb == 32 ? 0xffffffffu : (1u << lb) - 1u;
 #pragma unroll
-                for (int t = 0; t < kMaxL; ++t) {
-                    if (t >= L) break;
-                    const uint32_t h = kPacked ? (words[t >> 1] >> (16 * (t & 1))) & 0xffffu : words[t];
-                    const uint32_t v = h - (t == tv ? 1u : 0u);
-                    c[t] = v;
-                    if (v) atomicAdd(&A[(int64_t)(tu * L + t) * nnz + pos], v);
+                    for (int t = 0; t < kMaxL; ++t) {
+                        if (t >= L) break;
+                        const uint32_t hi = kPacked ? (words[t >> 1] >> (16 * (t & 1))) & 0xffffu : words[t];
+                        const uint32_t h = low ? (words[0] >> (lb * t)) & lm : hi;
+                        const uint32_t v = h - (t == tv ? 1u : 0u);
+                        c[t] = v;
+                        if (v) atomicAdd(&A[(int64_t)(tu * L + t) * nnz + pos], v);
+                    }
                 }
             } else {
-                for (int q = 0; q < RW; ++q) __stcg(row + q, 0u);
+                for (int q = 0; q < (low ? 1 : RW); ++q) __stcg(row + q, 0u);
             }
         }
         if (phase == 1) {
@@ -529,16 +556,23 @@ void prepare_edges(Graph &G, int k, cudaStream_t s) {
     tiles_for(G, 0, G.m, nt, unused, s);
 }
 
-// words of one hub's counter table (one row of L counters per node of its graph)
+// words of the largest hub's counter table
 static int64_t hub_words_per_table(const Graph &G) {
     const int64_t rw = G.hub_packed ? (G.L + 1) / 2 : G.L;
-    return std::max<int64_t>(G.max_graph_nodes, 1) * rw;
+    int64_t most = 1;
+    for (size_t h = 0; h < G.h_hub_nlow.size(); ++h) {
+        const size_t gr = std::upper_bound(G.h_node_off.begin(), G.h_node_off.end(), (int64_t)G.h_hub_id[h]) -
+                          G.h_node_off.begin() - 1;
+        const int64_t nodes = G.h_node_off[gr + 1] - G.h_node_off[gr];
+        most = std::max(most, G.h_hub_nlow[h] + (nodes - G.h_hub_nlow[h]) * rw);
+    }
+    return most;
 }
 
 // hubs of one group: their tables fill at most half of hub_l2_mb (the
 // persistent pass fills one group's tables while it reads the previous one's)
 static int64_t hub_group_max(const Graph &G) {
-    const int64_t per = hub_words_per_table(G) * (int64_t)sizeof(uint32_t);
+    const int64_t per = G.hub_stride * (int64_t)sizeof(uint32_t);
     return std::max<int64_t>(((int64_t)G.opt.hub_l2_mb << 20) / 2 / per, 1);
 }
 
@@ -556,6 +590,8 @@ static HubView hub_view(const Graph &G) {
     HubView h;
     h.hubs = G.hubs.as<int32_t>();
     h.hub_base = G.hub_base.as<int64_t>();
+    h.hub_nlow = G.hub_nlow.as<int32_t>();
+    h.nlow = G.h_hub_nlow.empty() ? 0 : G.h_hub_nlow[0];
     h.woff = G.item_woff.as<int64_t>();
     h.item = G.item_rec.as<int4>();
     h.batched = G.ngraphs > 1;
@@ -569,8 +605,9 @@ static void prepare_hubs(Graph &G, cudaStream_t s) {
     const GraphView gv = G.view();
     TBuf nv(sizeof(int64_t) * (nh + 1), s), vbase(sizeof(int64_t) * (nh + 1), s);
     G.hub_base.alloc(sizeof(int64_t) * nh);
+    G.hub_nlow.alloc(sizeof(int32_t) * nh);
     k_hub_nv<<<grid_for(nh + 1, 256, 1 << 20), 256, 0, s>>>(gv, G.hubs.as<int32_t>(), nh, nv.as<int64_t>(),
-                                                            G.hub_base.as<int64_t>());
+                                                            G.hub_base.as<int64_t>(), G.hub_nlow.as<int32_t>());
     TG_CK(cudaGetLastError());
     exclusive_sum(nv.as<int64_t>(), vbase.as<int64_t>(), nh + 1, s);
     int64_t NV = 0;
@@ -606,6 +643,8 @@ static void prepare_hubs(Graph &G, cudaStream_t s) {
                                                                 G.item_woff.as<int64_t>(), fi.as<int64_t>(),
                                                                 fw.as<int64_t>());
     TG_CK(cudaGetLastError());
+    G.h_hub_nlow.assign(nh, 0);
+    TG_CK(cudaMemcpyAsync(G.h_hub_nlow.data(), G.hub_nlow.p, sizeof(int32_t) * nh, cudaMemcpyDeviceToHost, s));
     G.h_hub_item.assign(nh + 1, 0);
     G.h_hub_woff.assign(nh + 1, 0);
     TG_CK(cudaMemcpyAsync(G.h_hub_item.data(), fi.p, sizeof(int64_t) * (nh + 1), cudaMemcpyDeviceToHost, s));

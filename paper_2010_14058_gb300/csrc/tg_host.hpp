@@ -139,9 +139,10 @@ struct Graph {
     int64_t n_anchors[kHubClass] = {};
     // hub anchors (ascending id) and their wedge items: one item per
     // (hub, lower-priority neighbour v, type of w) with at least one wedge
-    DBuf hubs, hub_base, item_woff, item_rec;
+    DBuf hubs, hub_base, hub_nlow, item_woff, item_rec;
     int64_t n_hubs = 0, n_items = 0;
     std::vector<int32_t> h_hub_id;      // hub node ids
+    std::vector<int32_t> h_hub_nlow;    // nodes of the hub's graph with one-word table rows
     std::vector<int64_t> h_hub_wedges;  // wedges of each hub
     std::vector<int64_t> h_hub_item;    // first item of each hub (n_hubs + 1)
     std::vector<int64_t> h_hub_woff;    // first wedge of each hub (n_hubs + 1)
@@ -249,7 +250,7 @@ struct Graph {
         return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
-                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &item_woff, &item_rec,
+                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &item_woff, &item_rec,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
