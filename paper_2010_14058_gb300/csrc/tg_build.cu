@@ -320,11 +320,11 @@ __global__ void k_widen(int64_t n, const int32_t *__restrict__ in, int64_t *out)
     if (i < n) out[i] = in[i];
 }
 
-// work of the listed nodes
+// work << 4 | type of the listed nodes
 __global__ void k_gather_work(int64_t c, const int32_t *__restrict__ ids, const int64_t *__restrict__ work,
-                              int64_t *out) {
+                              const uint8_t *__restrict__ ty, int64_t *out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < c) out[i] = work[ids[i]];
+    if (i < c) out[i] = work[ids[i]] << 4 | ty[ids[i]];
 }
 
 uint32_t read_status(const DBuf &st, cudaStream_t s) {
@@ -542,7 +542,7 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
         TG_CK(cudaGetLastError());
     }
 
-    // 6. wedge anchors by class; hubs in ascending id order
+    // 6. wedge anchors by class
     {
         TBuf work(sizeof(int64_t) * std::max<int64_t>(n, 1), s), most(sizeof(int32_t) * std::max<int64_t>(n, 1), s);
         if (n > 0) {
@@ -555,17 +555,29 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
         G.h_hub_id.assign((size_t)G.n_hubs, 0);
         G.h_hub_wedges.assign((size_t)G.n_hubs, 0);
         if (G.n_hubs > 0) {
+            // hub order: by graph, type and id, as the entries of the N+ lists
             TBuf wk(sizeof(int64_t) * (size_t)G.n_hubs, s);
-            TG_CK(cudaMemcpyAsync(G.h_hub_id.data(), G.hubs.p, sizeof(int32_t) * G.n_hubs, cudaMemcpyDeviceToHost, s));
-            TG_CK(cudaStreamSynchronize(s));
-            std::sort(G.h_hub_id.begin(), G.h_hub_id.end());
-            TG_CK(cudaMemcpyAsync(G.hubs.p, G.h_hub_id.data(), sizeof(int32_t) * G.n_hubs, cudaMemcpyHostToDevice, s));
+            std::vector<int32_t> id((size_t)G.n_hubs);
+            std::vector<int64_t> wt((size_t)G.n_hubs);
             ++G.last_launches;
-            k_gather_work<<<blocks_for(G.n_hubs, kThreads), kThreads, 0, s>>>(G.n_hubs, G.hubs.as<int32_t>(),
-                                                                             work.as<int64_t>(), wk.as<int64_t>());
+            k_gather_work<<<blocks_for(G.n_hubs, kThreads), kThreads, 0, s>>>(
+                G.n_hubs, G.hubs.as<int32_t>(), work.as<int64_t>(), G.ty.as<uint8_t>(), wk.as<int64_t>());
             TG_CK(cudaGetLastError());
-            TG_CK(cudaMemcpyAsync(G.h_hub_wedges.data(), wk.p, sizeof(int64_t) * G.n_hubs, cudaMemcpyDeviceToHost, s));
+            TG_CK(cudaMemcpyAsync(id.data(), G.hubs.p, sizeof(int32_t) * G.n_hubs, cudaMemcpyDeviceToHost, s));
+            TG_CK(cudaMemcpyAsync(wt.data(), wk.p, sizeof(int64_t) * G.n_hubs, cudaMemcpyDeviceToHost, s));
             TG_CK(cudaStreamSynchronize(s));
+            std::vector<std::pair<std::pair<int64_t, int64_t>, int64_t>> order((size_t)G.n_hubs);   // ((graph, type), id), wedges
+            for (size_t h = 0; h < order.size(); ++h) {
+                const int64_t gr = std::upper_bound(G.h_node_off.begin(), G.h_node_off.end(), (int64_t)id[h]) -
+                                   G.h_node_off.begin();
+                order[h] = {{gr, (wt[h] & 15) << kTypeShift | id[h]}, wt[h] >> 4};
+            }
+            std::sort(order.begin(), order.end());
+            for (size_t h = 0; h < order.size(); ++h) {
+                G.h_hub_id[h] = (int32_t)(order[h].first.second & kIdMask);
+                G.h_hub_wedges[h] = order[h].second;
+            }
+            TG_CK(cudaMemcpyAsync(G.hubs.p, G.h_hub_id.data(), sizeof(int32_t) * G.n_hubs, cudaMemcpyHostToDevice, s));
         }
     }
     if (read_status(G.status, s) & ST_INVALID_GRAPH) throw Error{TG_ERR_INVALID_GRAPH, "asymmetric rows"};

@@ -597,21 +597,6 @@ __global__ void k_finalize(int ngraphs, int L, int k, const unsigned long long *
     out[idx] = (int64_t)(v / edges_of[b]);
 }
 
-// f(std::integral_constant<int, L>) for the handle's L
-template <class F>
-void with_types(int L, F f) {
-    switch (L) {
-        case 1: f(std::integral_constant<int, 1>()); break;
-        case 2: f(std::integral_constant<int, 2>()); break;
-        case 3: f(std::integral_constant<int, 3>()); break;
-        case 4: f(std::integral_constant<int, 4>()); break;
-        case 5: f(std::integral_constant<int, 5>()); break;
-        case 6: f(std::integral_constant<int, 6>()); break;
-        case 7: f(std::integral_constant<int, 7>()); break;
-        default: f(std::integral_constant<int, 8>()); break;
-    }
-}
-
 PaView pa_view(const Graph &G) {
     PaView v;
     v.cls = G.pa_cls.as<int32_t>();

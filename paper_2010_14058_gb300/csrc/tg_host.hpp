@@ -137,17 +137,12 @@ struct Graph {
     // work lists
     DBuf anchors[kHubClass], anchor_wedges;     // wedge anchors by class (tg_wedge.cu); wedges of every node
     int64_t n_anchors[kHubClass] = {};
-    // hub anchors (ascending id) and their wedge items: one item per
-    // (hub, lower-priority neighbour v, type of w) with at least one wedge
-    DBuf hubs, hub_base, hub_nlow, item_woff, item_rec;
-    int64_t n_hubs = 0, n_items = 0;
+    // hub anchors in (graph, type, id) order and the pieces of their wedges (tg_hub.cu)
+    DBuf hubs, hub_base, hub_nlow, hub_piece;
+    int64_t n_hubs = 0;
     std::vector<int32_t> h_hub_id;      // hub node ids
-    std::vector<int32_t> h_hub_nlow;    // nodes of the hub's graph with one-word table rows
     std::vector<int64_t> h_hub_wedges;  // wedges of each hub
-    std::vector<int64_t> h_hub_item;    // first item of each hub (n_hubs + 1)
-    std::vector<int64_t> h_hub_woff;    // first wedge of each hub (n_hubs + 1)
-    bool hubs_ready = false;
-    // persistent hub pass (tg_count.cu): per chunk, its ticket queue; the
+    // persistent hub pass (tg_hub.cu): per chunk, its ticket queue; the
     // table buffers shared by all chunks
     struct HubPlan {
         DBuf segs, groups, ntick, ctr;
@@ -250,7 +245,7 @@ struct Graph {
         return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
-                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &item_woff, &item_rec,
+                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
@@ -329,6 +324,26 @@ int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s);
 // graphs with nodes [n0, n1) (tg_sums.cu); prepare_sums before any capture
 void prepare_sums(Graph &G);
 int64_t launch_sums(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s);
+
+// the hub anchors (tg_hub.cu): groups, items and ticket queues (before any
+// capture), and the pass over the hubs of chunk ci
+void prepare_hubs(Graph &G, cudaStream_t s);
+int64_t launch_hubs(Graph &G, size_t ci, cudaStream_t s);
+
+// f(std::integral_constant<int, L>) for the handle's L
+template <class F>
+void with_types(int L, F f) {
+    switch (L) {
+        case 1: f(std::integral_constant<int, 1>()); break;
+        case 2: f(std::integral_constant<int, 2>()); break;
+        case 3: f(std::integral_constant<int, 3>()); break;
+        case 4: f(std::integral_constant<int, 4>()); break;
+        case 5: f(std::integral_constant<int, 5>()); break;
+        case 6: f(std::integral_constant<int, 6>()); break;
+        case 7: f(std::integral_constant<int, 7>()); break;
+        default: f(std::integral_constant<int, 8>()); break;
+    }
+}
 
 // wedge anchors (tg_wedge.cu): class lists from the wedges and the most
 // lower-priority neighbours of one type of every node (the hubs unsorted);

@@ -43,14 +43,13 @@ struct WedgeLimits {
     int64_t bytes[4];           // table bytes of classes 1 to 4
 };
 
-// Persistent hub pass (tg_count.cu): a group of hubs whose counter tables
+// Persistent hub pass (tg_hub.cu): a group of hubs whose counter tables
 // share one table buffer, and the ticket queue as runs of tickets of one
 // (group, kind) in queue order; kinds 0 fill, 1 read, 2 clear by walking the
 // wedges, 3 clear by zeroing the group's table words.
 struct HubGroup {
-    int64_t i0, i1;             // items
-    int64_t w0, w1;             // wedges
-    int64_t tw;                 // wedges per fill / read / walk-clear ticket
+    int64_t x0, x1;             // pieces
+    int64_t tx;                 // pieces per fill / read / walk-clear ticket
     int64_t zwords;             // table words of the group (zeroing tickets: kHubTicketWords each)
     int32_t h0, buf;            // first hub, table buffer
 };
