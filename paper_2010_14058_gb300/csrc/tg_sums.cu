@@ -20,8 +20,13 @@
 // Measured against one pass over every edge's typed intersection for the sums
 // and one over every T list for the cliques: 61.4 + 62.9 + 32.7 -> 25.9 + 1.1
 // (zeroing) ms on that graph, 18.2 + 12.0 -> 5.6 + 0.6 ms on 256 dense graphs
-// of 14 M edges.  What bounds it now: the atomics' instructions (one triangle
-// of 4 L lanes per warp step) and their sectors in L2.
+// of 14 M edges.  With each node's triangles kept in a list, so that its lists
+// are scanned once and every warp step has 32 triangles, 25.3 -> 21.2 ms; with
+// the number of types compiled in 18.5 ms (5.6 -> 4.3 ms).  What bounds it now:
+// the atomics' instructions (one triangle of 4 L lanes per warp step) and
+// their sectors in L2 (three rows of 80 bytes per triangle at L = 5).  Visiting
+// the nodes u grouped by type, so that 1 / L of the rows of {a, b} is live,
+// changed nothing (21.3 against 21.2 ms).
 #include <algorithm>
 
 #include "tg_host.hpp"
@@ -33,22 +38,21 @@ namespace {
 
 constexpr int kSumWarps = 8;                 // warps per CTA of the warp form
 
-// Per-warp staging of up to 32 triangles.
+// Per-warp staging of up to 32 triangles: what the lanes of add_terms read
+// of each, worked out by one lane per triangle.
 struct Stage {
-    uint32_t *ab;               // [32] edge id of {a, b}
+    int64_t *at;                // [32][3] words of X: row ty_b of {u, a}, ty_a of {u, b}, ty_u of {a, b}
     uint32_t *kk;               // [32] list position of a << 16 | of b
-    uint32_t *cab;              // [32][L] triangle counts of {a, b}
-    uint32_t *nq;               // [32][L] nodes adjacent to u, a and b by type
+    uint32_t *val;              // [32][2 L] triangle counts of {a, b}, then the nodes adjacent to u, a and b by type
 };
 
-__host__ __device__ inline size_t stage_words(int L) { return 32 * (2 + 2 * (size_t)L); }
+__host__ __device__ inline size_t stage_words(int L) { return 32 * (7 + 2 * (size_t)L); }
 
-__device__ __forceinline__ Stage stage_carve(uint32_t *mem, int L) {
+__device__ __forceinline__ Stage stage_carve(uint32_t *mem, int L) {   // mem: 8-byte aligned
     Stage s;
-    s.ab = mem;
-    s.kk = s.ab + 32;
-    s.cab = s.kk + 32;
-    s.nq = s.cab + 32 * L;
+    s.at = reinterpret_cast<int64_t *>(mem);
+    s.kk = mem + 32 * 6;
+    s.val = s.kk + 32;
     return s;
 }
 
@@ -79,36 +83,41 @@ __device__ __forceinline__ void load_vec(const GraphView &g, const uint32_t *C, 
     }
 }
 
+// stages triangle number i of the warp (nq is filled in by the caller)
+__device__ __forceinline__ void stage_put(const CountView &cv, int L, const Stage &s, int i, uint32_t ab, int ka, int kb,
+                                          const uint32_t *ent, const uint32_t *eid, uint32_t tu) {
+    const int row = 4 * L;
+    s.at[3 * i] = ((int64_t)eid[ka] - cv.e_base) * (L * row) + (ent[kb] >> kTypeShift) * row;
+    s.at[3 * i + 1] = ((int64_t)eid[kb] - cv.e_base) * (L * row) + (ent[ka] >> kTypeShift) * row;
+    s.at[3 * i + 2] = ((int64_t)ab - cv.e_base) * (L * row) + tu * row;
+    s.kk[i] = (uint32_t)ka << 16 | (uint32_t)kb;
+    load_c(cv.C, ab, L, s.val + i * 2 * L);
+}
+
 // Adds the terms of the warp's `cnt` staged triangles.  vec: the local
-// nodes' rows, vu: lane's word of u's own typed degrees (component 2), ent /
-// eid: the local list.  Lanes take 4 L words of one triangle, 32 / (4 L)
-// triangles at a time.
-template <class Acc>
-__device__ __forceinline__ void add_terms(Acc *X, int64_t e_base, int L, const Stage &s, int cnt, const uint32_t *vec,
-                                          uint32_t du, const uint32_t *ent, const uint32_t *eid, uint32_t tu,
+// nodes' rows, du: the lane's word of u's own typed degrees (component 2).
+// Lanes take 4 L words of one triangle, 32 / (4 L) triangles at a time.
+template <class Acc, int kL>
+__device__ __forceinline__ void add_terms(Acc *X, int rt_L, const Stage &s, int cnt, const uint32_t *vec, uint32_t du,
                                           int lane) {
+    const int L = kL ? kL : rt_L;
     const int row = 4 * L, per = 32 / row;
     const int grp = lane / row, comp = lane - grp * row;
     const int k = comp / L, q = comp - k * L;
     const int off = k == 2 ? L + q : q;                     // word of vec (components 0 and 2)
-    for (int i0 = 0; i0 < cnt; i0 += per) {
-        const int i = i0 + grp;
-        if (grp >= per || i >= cnt) continue;
+    const int val = k == 3 ? L + q : q;                     // word of the staged values (components 1 and 3)
+    Acc *Xc = X + comp;
+#pragma unroll 2
+    for (int i = grp < per ? grp : cnt; i < cnt; i += per) {
         const uint32_t kk = s.kk[i];
-        const int ka = (int)(kk >> 16), kb = (int)(kk & 0xffffu);
-        const uint32_t va = vec[ka * 2 * L + off], vb = vec[kb * 2 * L + off];
-        uint32_t xa, xb, xab;
-        if (k & 1) {                                        // 1: {a, b}'s counts; 3: the 4-cliques
-            xa = xb = k == 1 ? s.cab[i * L + q] : s.nq[i * L + q];
-            xab = k == 1 ? vb : 2 * xa;
-        } else {                                            // 0: u's counts of the other node; 2: its degrees
-            xa = vb;
-            xb = va;
-            xab = k == 0 ? va : du;
-        }
-        if (xa) atomicAdd(&X[((int64_t)eid[ka] - e_base) * (L * row) + (ent[kb] >> kTypeShift) * row + comp], (Acc)xa);
-        if (xb) atomicAdd(&X[((int64_t)eid[kb] - e_base) * (L * row) + (ent[ka] >> kTypeShift) * row + comp], (Acc)xb);
-        if (xab) atomicAdd(&X[((int64_t)s.ab[i] - e_base) * (L * row) + tu * row + comp], (Acc)xab);
+        const uint32_t va = vec[(kk >> 16) * 2 * L + off], vb = vec[(kk & 0xffffu) * 2 * L + off];
+        const uint32_t sv = s.val[i * 2 * L + val];
+        // 0: u's counts of the other node; 1: {a, b}'s counts; 2: degrees; 3: the 4-cliques
+        const uint32_t xa = k & 1 ? sv : vb, xb = k & 1 ? sv : va;
+        const uint32_t xab = k == 0 ? va : k == 1 ? vb : k == 2 ? du : 2 * sv;
+        if (xa) atomicAdd(Xc + s.at[3 * i], (Acc)xa);
+        if (xb) atomicAdd(Xc + s.at[3 * i + 1], (Acc)xb);
+        if (xab) atomicAdd(Xc + s.at[3 * i + 2], (Acc)xab);
     }
 }
 
@@ -132,12 +141,12 @@ __global__ void __launch_bounds__(256) k_sum_zero(int64_t e0, int64_t e1, int L,
 
 // Warp per node u of [n0, n1) with 2 <= |N+(u)| <= kTriWarpMax: the bit
 // matrix is one word per local node, type q's columns a mask of that word.
-template <class Acc>
+template <class Acc, int kL>
 __global__ void __launch_bounds__(kSumWarps * 32) k_sum_warp(GraphView g, CountView cv, int64_t n0, int64_t n1) {
     extern __shared__ uint32_t sw_smem[];
-    const int L = g.L;
+    const int L = kL ? kL : g.L;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int per_warp = (int)stage_words(L) + 32 * 2 * L + 32 * 3;
+    const int per_warp = (int)stage_words(L) + 32 * 2 * L + 32 * 3;   // even: the staging is 8-byte aligned
     uint32_t *mem = sw_smem + wid * per_warp;
     const Stage s = stage_carve(mem, L);
     uint32_t *vec = mem + stage_words(L), *ents = vec + 32 * 2 * L, *eids = ents + 32, *B = eids + 32;
@@ -191,17 +200,15 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_warp(GraphView g, CountV
                 const int64_t pos = find(r * 32 + lane, k, l);
                 const uint32_t e = (uint32_t)g.plus_eid[pos];
                 const int at = __popc(bal & ((1u << lane) - 1u));
-                s.ab[at] = e;
-                s.kk[at] = (uint32_t)k << 16 | (uint32_t)l;
-                load_c(cv.C, e, L, s.cab + at * L);
+                stage_put(cv, L, s, at, e, k, l, ents, eids, tu);
                 const uint32_t both = B[k] & B[l];
 #pragma unroll
                 for (int q = 0; q < kMaxL; ++q)
-                    if (q < L) s.nq[at * L + q] = __popc(both & mask[q]);
+                    if (q < L) s.val[at * 2 * L + L + q] = __popc(both & mask[q]);
                 words += 1;
             }
             __syncwarp();
-            add_terms<Acc>(X, cv.e_base, L, s, __popc(bal), vec, du, ents, eids, tu, lane);
+            add_terms<Acc, kL>(X, L, s, __popc(bal), vec, du, lane);
             __syncwarp();
         }
     }
@@ -213,23 +220,34 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_warp(GraphView g, CountV
 __host__ __device__ inline int bit_words(int cap, int L) { return ((cap + 31) / 32 + L) | 1; }
 
 __host__ __device__ inline size_t sum_bytes(int cap, int lgf, int warps, int L) {
-    return 4 * ((size_t)cap * bit_words(cap, L) + (size_t)cap * 2 * L + (size_t)warps * stage_words(L) + 2 * kMaxL + 2) +
+    return 4 * ((((size_t)cap * bit_words(cap, L) + 1) & ~(size_t)1) + (size_t)cap * 2 * L +
+                (size_t)warps * stage_words(L) + 2 * kMaxL + 2) +
            local_bytes(cap, lgf, warps);
 }
 
+// Triangles of one node: its list positions and the edge of the other two.
+struct Found {
+    uint32_t ab, kk;
+};
+
+__host__ __device__ inline int64_t most_found(int64_t cap) { return cap * (cap - 1) / 2; }
+
 // CTA per listed node u of [n0, n1)
-template <class Acc, int kThreadsT, bool kSmem>
+template <class Acc, int kL, int kThreadsT, bool kSmem>
 __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv, const int32_t *__restrict__ list,
                                                        int64_t n_list, int64_t n0, int64_t n1, int cap, int lgf,
                                                        unsigned char *scratch, int64_t stride) {
+    // kSmem: the arrays in shared memory, and in the CTA's global slice the
+    // triangles of one node, so that its lists are scanned once; else the
+    // arrays in the slice and a second scan
     extern __shared__ uint32_t sc_smem[];
-    const int L = g.L;
+    const int L = kL ? kL : g.L;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int kWarps = kThreadsT / 32;
     uint32_t *mem = kSmem ? sc_smem : reinterpret_cast<uint32_t *>(scratch + (int64_t)blockIdx.x * stride);
     const int W = bit_words(cap, L);
     uint32_t *B = mem;
-    uint32_t *vec = B + (size_t)cap * W;
+    uint32_t *vec = B + (((size_t)cap * W + 1) & ~(size_t)1);
     const Stage s = stage_carve(vec + (size_t)cap * 2 * L + wid * stage_words(L), L);
     int *ws = reinterpret_cast<int *>(vec + (size_t)cap * 2 * L + kWarps * stage_words(L));   // [L + 1] first word of a type
     int *shift = ws + kMaxL + 1;                            // [L] column of list position k of type t: k + shift[t]
@@ -237,6 +255,8 @@ __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv
     local_carve(q, reinterpret_cast<unsigned char *>(ws + 2 * kMaxL + 2), cap, lgf, kWarps, wid);
     Acc *X = reinterpret_cast<Acc *>(cv.xsum);
     unsigned long long words = 0;
+    __shared__ int s_found, s_next;
+    Found *found = reinterpret_cast<Found *>(scratch + (int64_t)blockIdx.x * stride);
     for (int64_t x = blockIdx.x; x < n_list; x += gridDim.x) {
         const int32_t u = list[x];
         if (u < n0 || u >= n1 || !cv.tri_any[u]) continue;  // uniform over the CTA
@@ -273,35 +293,60 @@ __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv
                 if (lane == L - 1) ws[L] = inc;
             }
         }
+        if (threadIdx.x == 0) s_found = s_next = 0;
         __syncthreads();
-        local_pairs(g, p, q, lane, wid, kWarps, [&](bool hit, int ka, int kb, uint32_t) {
-            if (!hit) return;
+        auto set_bits = [&](int ka, int kb) {
             const int ca = ka + shift[q.ent[ka] >> kTypeShift], cb = kb + shift[q.ent[kb] >> kTypeShift];
             atomicOr(&B[ka * W + (cb >> 5)], 1u << (cb & 31));
             atomicOr(&B[kb * W + (ca >> 5)], 1u << (ca & 31));
-        });
-        __syncthreads();
-        local_pairs(g, p, q, lane, wid, kWarps, [&](bool hit, int ka, int kb, uint32_t pos) {
+        };
+        // stages one triangle per lane that has one and adds the warp's terms
+        auto terms = [&](bool hit, uint32_t ab, int ka, int kb) {
             const unsigned bal = __ballot_sync(0xffffffffu, hit);
             if (bal == 0) return;
             if (hit) {
-                const uint32_t e = (uint32_t)g.plus_eid[pos];
                 const int at = __popc(bal & ((1u << lane) - 1u));
-                s.ab[at] = e;
-                s.kk[at] = (uint32_t)ka << 16 | (uint32_t)kb;
-                load_c(cv.C, e, L, s.cab + at * L);
+                stage_put(cv, L, s, at, ab, ka, kb, q.ent, q.eid, tu);
                 const uint32_t *ra = B + ka * W, *rb = B + kb * W;
                 int w = 0;
                 for (int t = 0; t < L; ++t) {
                     uint32_t n = 0;
                     for (const int we = ws[t + 1]; w < we; ++w) n += __popc(ra[w] & rb[w]);
-                    s.nq[at * L + t] = n;
+                    s.val[at * 2 * L + L + t] = n;
                 }
                 words += (unsigned)w;
             }
             __syncwarp();
-            add_terms<Acc>(X, cv.e_base, L, s, __popc(bal), vec, du, q.ent, q.eid, tu, lane);
+            add_terms<Acc, kL>(X, L, s, __popc(bal), vec, du, lane);
+            __syncwarp();
+        };
+        local_pairs(g, p, q, lane, wid, kWarps, [&](bool hit, int ka, int kb, uint32_t pos) {
+            if (hit) set_bits(ka, kb);
+            if (!kSmem) return;
+            const unsigned bal = __ballot_sync(0xffffffffu, hit);
+            if (bal == 0) return;
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_found, __popc(bal));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+            if (hit) found[at] = Found{(uint32_t)g.plus_eid[pos], (uint32_t)ka << 16 | (uint32_t)kb};
         });
+        __syncthreads();
+        if (kSmem) {
+            const int nf = s_found;
+            for (;;) {
+                int i = 0;
+                if (lane == 0) i = atomicAdd(&s_next, 32);
+                i = __shfl_sync(0xffffffffu, i, 0);
+                if (i >= nf) break;
+                Found f{0, 0};
+                if (i + lane < nf) f = found[i + lane];
+                terms(i + lane < nf, f.ab, (int)(f.kk >> 16), (int)(f.kk & 0xffffu));
+            }
+        } else {
+            local_pairs(g, p, q, lane, wid, kWarps, [&](bool hit, int ka, int kb, uint32_t pos) {
+                terms(hit, hit ? (uint32_t)g.plus_eid[pos] : 0u, ka, kb);
+            });
+        }
         __syncthreads();
     }
     if (cv.work && words) atomicAdd(&cv.work[kWorkCliqueProbes], words);
@@ -319,23 +364,42 @@ size_t class_bytes(const Graph &G, const LocalClass &c) {
 
 size_t warp_bytes(int L) { return sizeof(uint32_t) * kSumWarps * (stage_words(L) + 32 * 2 * (size_t)L + 32 * 3); }
 
-template <class Acc>
+// CTAs of a class and bytes of a CTA's global slice
+struct SumShape {
+    size_t smem, slice;
+    int64_t ctas;
+};
+
+SumShape shape_of(const Graph &G, const LocalClass &c, int cls) {
+    SumShape r;
+    const size_t bytes = class_bytes(G, c);
+    if (cls == 2) {
+        r.smem = 0;
+        r.slice = bytes;
+        r.ctas = huge_ctas(bytes, c.n);
+    } else {
+        r.smem = bytes;
+        r.slice = sizeof(Found) * (size_t)most_found(c.cap);
+        const int per_sm = std::max(1, std::min<int>(2048 / c.threads, (int)((226u << 10) / (bytes + 1024))));
+        r.ctas = std::min<int64_t>(c.n, (int64_t)sm_count() * per_sm);
+    }
+    return r;
+}
+
+template <class Acc, int kL>
 void prepare(Graph &G) {
-    raise_smem_limit((const void *)k_sum_warp<Acc>, warp_bytes(G.L));
+    raise_smem_limit((const void *)k_sum_warp<Acc, kL>, warp_bytes(G.L));
     for (int cls = 0; cls < 3; ++cls) {
         const LocalClass c = local_class(G, cls);
         if (c.n == 0) continue;
-        const size_t bytes = class_bytes(G, c);
-        if (cls == 0) raise_smem_limit((const void *)k_sum_cta<Acc, kTriMidThreads, true>, bytes);
-        else if (cls == 1) raise_smem_limit((const void *)k_sum_cta<Acc, kTriBigThreads, true>, bytes);
-        else {
-            const size_t want = bytes * (size_t)huge_ctas(bytes, c.n);
-            if (G.local_scratch.bytes < want) G.local_scratch.alloc(want);
-        }
+        const SumShape r = shape_of(G, c, cls);
+        if (cls == 0) raise_smem_limit((const void *)k_sum_cta<Acc, kL, kTriMidThreads, true>, r.smem);
+        else if (cls == 1) raise_smem_limit((const void *)k_sum_cta<Acc, kL, kTriBigThreads, true>, r.smem);
+        if (G.local_scratch.bytes < r.slice * (size_t)r.ctas) G.local_scratch.alloc(r.slice * (size_t)r.ctas);
     }
 }
 
-template <class Acc>
+template <class Acc, int kL>
 int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s) {
     G.e_base = e0;
     const GraphView gv = G.view();
@@ -353,28 +417,22 @@ int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStr
     {
         const size_t bytes = warp_bytes(G.L);
         const int per_sm = std::max(1, std::min<int>(2048 / (kSumWarps * 32), (int)((220u << 10) / (bytes + 1024))));
-        k_sum_warp<Acc><<<(unsigned)std::min<int64_t>((n1 - n0 + kSumWarps - 1) / kSumWarps, (int64_t)sms * per_sm * 8),
+        k_sum_warp<Acc, kL><<<(unsigned)std::min<int64_t>((n1 - n0 + kSumWarps - 1) / kSumWarps, (int64_t)sms * per_sm * 8),
                           kSumWarps * 32, bytes, s>>>(gv, cv, n0, n1);
         ++launches;
     }
     for (int cls = 0; cls < 3; ++cls) {
         const LocalClass c = local_class(G, cls);
         if (c.n == 0) continue;
-        const size_t bytes = class_bytes(G, c);
+        const SumShape r = shape_of(G, c, cls);
         ++launches;
-        if (cls == 2) {
-            k_sum_cta<Acc, kTriBigThreads, false><<<(unsigned)huge_ctas(bytes, c.n), kTriBigThreads, 0, s>>>(
-                gv, cv, c.list, c.n, n0, n1, c.cap, c.lgf, G.local_scratch.as<unsigned char>(), (int64_t)bytes);
-            continue;
-        }
-        const int per_sm = std::max(1, std::min<int>(2048 / c.threads, (int)((220u << 10) / (bytes + 1024))));
-        const unsigned grid = (unsigned)std::min<int64_t>(c.n, (int64_t)sms * per_sm);
-        if (cls == 0)
-            k_sum_cta<Acc, kTriMidThreads, true><<<grid, c.threads, bytes, s>>>(gv, cv, c.list, c.n, n0, n1, c.cap,
-                                                                               c.lgf, nullptr, 0);
-        else
-            k_sum_cta<Acc, kTriBigThreads, true><<<grid, c.threads, bytes, s>>>(gv, cv, c.list, c.n, n0, n1, c.cap,
-                                                                               c.lgf, nullptr, 0);
+        auto run = [&](auto kern) {
+            kern<<<(unsigned)r.ctas, c.threads, r.smem, s>>>(gv, cv, c.list, c.n, n0, n1, c.cap, c.lgf,
+                                                             G.local_scratch.as<unsigned char>(), (int64_t)r.slice);
+        };
+        if (cls == 0) run(k_sum_cta<Acc, kL, kTriMidThreads, true>);
+        else if (cls == 1) run(k_sum_cta<Acc, kL, kTriBigThreads, true>);
+        else run(k_sum_cta<Acc, kL, kTriBigThreads, false>);
     }
     TG_CK(cudaGetLastError());
     return launches;
@@ -382,13 +440,18 @@ int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStr
 
 }  // namespace
 
+// kernels of 32-bit sums are compiled per number of types (the terms' index
+// arithmetic is most of their instructions), those of 64-bit sums once
 void prepare_sums(Graph &G) {
-    if (G.wide_sums()) prepare<unsigned long long>(G);
-    else prepare<uint32_t>(G);
+    if (G.wide_sums()) prepare<unsigned long long, 0>(G);
+    else with_types(G.L, [&](auto l) { prepare<uint32_t, decltype(l)::value>(G); });
 }
 
 int64_t launch_sums(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s) {
-    return G.wide_sums() ? launch<unsigned long long>(G, n0, n1, e0, e1, s) : launch<uint32_t>(G, n0, n1, e0, e1, s);
+    if (G.wide_sums()) return launch<unsigned long long, 0>(G, n0, n1, e0, e1, s);
+    int64_t launches = 0;
+    with_types(G.L, [&](auto l) { launches = launch<uint32_t, decltype(l)::value>(G, n0, n1, e0, e1, s); });
+    return launches;
 }
 
 }  // namespace tg
