@@ -127,11 +127,8 @@ typedef struct {
                                          node table shared by all CTAs */
     int32_t hub_l2_mb;                /* MB of hub node tables of the persistent hub pass: one group
                                          of hubs fills at most half of it (about the L2 size) */
-    int32_t isect_modes;              /* typed set intersection per bucket of the shorter segment's
-                                         length (buckets [1,32) [32,128) [128,512) [512,inf), two bits
-                                         each from bit 0): 0 default = 1, 1 binary search of each
-                                         shorter entry in the longer segment, 2 warp-wide merge of
-                                         both segments, 3 whichever a dependent-load count favours */
+    int32_t isect_modes;              /* accepted and ignored (typed triangles are found from the lists of
+                                         higher-priority neighbours, not by intersecting rows) */
 } tg_options;
 
 /* ---- layout ---------------------------------------------------------- */

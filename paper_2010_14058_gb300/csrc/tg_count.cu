@@ -49,7 +49,7 @@ namespace tg {
 
 // Edges per tile: kTile, or fewer for a small handle so that its tiles
 // still fill the GPU (at least about 12 tiles per SM, 64 edges or more each).
-static int64_t tile_edges(const Graph &G) {
+int64_t tile_edges(const Graph &G) {
     const int64_t want = (G.m + (int64_t)sm_count() * 12 - 1) / ((int64_t)sm_count() * 12);
     int64_t t = 64;
     while (t < want && t < kTile) t <<= 1;

@@ -4,13 +4,16 @@
 // out-neighbours Gamma_i^{t,+} and in-neighbours Gamma_i^{t,-}, and the sets
 // T_ij^t, S_i^t, S_j^t of Alg. 1 with it.  On the GPU an oriented graph is
 // held as its underlying undirected graph (the ordinary tg_build layout:
-// rows by (type, id), per-type segments) plus one sign per adjacency slot
-// (+1 when the row's node is the arc's tail) and the typed out-degrees of
-// every node.  Per edge {i, j}, one warp intersects the typed segments of i
-// and j (binary search or merge, isect); each triangle node w falls into
-// T^t(sign at i, sign at j), counted with ballots; the S sets follow from the typed out- and in-degrees by
-// Cor. 1-2: |S_i^{t,+}| = d_i^{t,+} - |T^t(+,.)| - [phi_j = t, i -> j] and
-// so on.  Per-edge layout and class ranks: include/tg.h.
+// rows by (type, id), per-type segments) plus one label per edge (bit 0: the
+// internal endpoint of lower priority is the arc's tail; bit 1: it has the
+// larger caller id) and the typed out-degrees of every node.  Every triangle
+// is found once (tg_visit.cuh); its three labels give the signs of each node
+// at the ends of the opposite edge, and one atomic per edge counts it in the
+// cell T^t(sign at lower, sign at higher endpoint).  A second kernel, one
+// thread per (edge, type), forms the rows: the S sets follow from the typed
+// out- and in-degrees by Cor. 1-2: |S_i^{t,+}| = d_i^{t,+} - |T^t(+,.)| -
+// [phi_j = t, i -> j] and so on.  Per-edge layout and class ranks:
+// include/tg.h.
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -18,6 +21,8 @@
 #include <cub/device/device_scan.cuh>
 
 #include "tg_host.hpp"
+#include "tg_tiles.cuh"
+#include "tg_visit.cuh"
 
 namespace tg {
 
@@ -169,70 +174,105 @@ __global__ void __launch_bounds__(256) k_out_degree(GraphView g, const int8_t *_
     }
 }
 
+// edge labels from the slots' signs
+__global__ void k_arc_labels(GraphView g, const int8_t *__restrict__ sign, const int32_t *__restrict__ old_of,
+                             uint8_t *lab) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= g.m) return;
+    lab[e] = (uint8_t)((sign[g.e_slot_lo[e]] > 0 ? 1 : 0) | (old_of[g.e_lo[e]] > old_of[g.e_hi[e]] ? 2 : 0));
+}
+
 // ---------------------------------------------------------------- count
-// Warp per edge {i, j} (i the smaller caller id): T^t by signs at i and j
-// with ballots (lane t keeps type t's four counts), then S^t from the
-// typed out- and in-degrees, the row, and the per-CTA class histogram.
-template <bool kMerge>
-__global__ void __launch_bounds__(256) k_directed3(GraphView g, const int8_t *__restrict__ sign,
-                                                   const int32_t *__restrict__ outdeg,
-                                                   const int32_t *__restrict__ old_of,
-                                                   const int32_t *__restrict__ slot_class, int G,
-                                                   uint32_t *per_edge_out, unsigned long long *gacc,
-                                                   uint32_t *status) {
+// cells [edge][type of the third node][sign at lower endpoint - ? 2 : 0 |
+// sign at higher endpoint - ? 1 : 0]
+struct DirectedCells {
+    uint32_t *cell;
+    const uint8_t *lab;
+    int L;
+    __device__ __forceinline__ void add(int64_t e, int t, bool minus_lo, bool minus_hi) const {
+        atomicAdd(&cell[(e * L + t) * 4 + (minus_lo ? 2 : 0) + (minus_hi ? 1 : 0)], 1u);
+    }
+    __device__ __forceinline__ void operator()(int64_t ua, int64_t ub, int64_t ab, int tu, int ta, int tb) const {
+        const bool u_a = lab[ua] & 1, u_b = lab[ub] & 1, a_b = lab[ab] & 1;   // the lower node is the tail
+        add(ua, tb, !u_b, !a_b);                            // b seen from u and a
+        add(ub, ta, !u_a, a_b);                             // a seen from u and b
+        add(ab, tu, u_a, u_b);                              // u seen from a and b
+    }
+};
+
+constexpr int kRowThreads = 256;
+
+// Thread per (edge, type): T^t by signs at i and j (i the smaller caller id)
+// from the cells, then S^t from the typed out- and in-degrees, the row, and
+// the class sums, kept in registers while the endpoints' types and the arc's
+// direction stay the same.
+template <int L>
+__global__ void __launch_bounds__(kRowThreads) k_directed_rows(GraphView g, const uint32_t *__restrict__ cell,
+                                                               const uint8_t *__restrict__ lab,
+                                                               const int32_t *__restrict__ outdeg,
+                                                               const int32_t *__restrict__ slot_class, int G,
+                                                               int64_t tile, uint32_t *per_edge_out,
+                                                               unsigned long long *gacc, uint32_t *status) {
+    constexpr int LL = L * L, E = kRowThreads / L;
     extern __shared__ unsigned long long dhist[];
-    const int L = g.L, LL = L * L;
-    const int lane = threadIdx.x & 31;
+    __shared__ TileOrder<2 * LL> o;
     for (int s = threadIdx.x; s < G; s += blockDim.x) dhist[s] = 0;
-    __syncthreads();
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; e < g.m; e += nw) {
-        const int32_t a = g.e_lo[e], b = g.e_hi[e];
-        const bool swap = old_of[a] > old_of[b];
-        const int32_t i = swap ? b : a, j = swap ? a : b;
-        const int64_t sij = swap ? g.e_slot_hi[e] : g.e_slot_lo[e];     // slot of j in row i
-        const int o = sign[sij] > 0 ? 0 : 1;                             // 0: i -> j
-        const int pi = g.ty[i], pj = g.ty[j];
-        unsigned c0 = 0, c1 = 0, c2 = 0, c3 = 0;                         // lane t: T^t(++ +- -+ --)
-        for (int t = 0; t < L; ++t) {
-            int64_t bi = seg_begin(g, i, t), ei = seg_end(g, i, t);
-            int64_t bj = seg_begin(g, j, t), ej = seg_end(g, j, t);
-            if (ei == bi || ej == bj) continue;                          // warp-uniform
-            const bool i_short = ei - bi <= ej - bj;
-            const int64_t sb = i_short ? bi : bj, se = i_short ? ei : ej;
-            const int64_t lb = i_short ? bj : bi, le = i_short ? ej : ei;
-            isect<kMerge>(g.adj, g.isect_modes, sb, se, lb, le, lane, [&](bool found, int64_t s, int64_t r, int32_t) {
-                int q = -1;
-                if (found) {
-                    const int8_t at_i = sign[i_short ? s : r], at_j = sign[i_short ? r : s];
-                    q = (at_i > 0 ? 0 : 2) + (at_j > 0 ? 0 : 1);
-                }
-                const unsigned n0 = __popc(__ballot_sync(0xffffffffu, q == 0));
-                const unsigned n1 = __popc(__ballot_sync(0xffffffffu, q == 1));
-                const unsigned n2 = __popc(__ballot_sync(0xffffffffu, q == 2));
-                const unsigned n3 = __popc(__ballot_sync(0xffffffffu, q == 3));
-                if (lane == t) { c0 += n0; c1 += n1; c2 += n2; c3 += n3; }
-            });
+    const int slice = threadIdx.x / L, t = threadIdx.x % L;
+    for (int64_t b = blockIdx.x * tile; b < g.m; b += gridDim.x * tile) {
+        const int n = (int)min(tile, g.m - b);
+        // key ((phi_i * L + phi_j) * 2 + o), o = 0: i -> j
+        tile_order(b, n, o, [&](int64_t e) {
+            const int l = lab[e];
+            const bool swap = l & 2;
+            const int i = swap ? g.e_hi[e] : g.e_lo[e], j = swap ? g.e_lo[e] : g.e_hi[e];
+            return (g.ty[i] * L + g.ty[j]) * 2 + (((l & 1) != 0) != swap ? 0 : 1);
+        });
+        for (int k = threadIdx.x; k < 2 * LL; k += blockDim.x) {        // the edges: (tail type, head type)
+            const int pi = k / 2 / L, pj = k / 2 % L;
+            if (o.count[k]) atomicAdd(&dhist[k & 1 ? pj * L + pi : pi * L + pj], (unsigned long long)o.count[k]);
         }
-        if (lane < L) {
-            const int t = lane;
+        if (slice >= E) continue;
+        int xb, xe;
+        slice_of(n, slice, E, xb, xe);
+        unsigned long long acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        int key = -1;
+        auto flush = [&]() {
+            const int32_t *cls = slot_class + (int64_t)key * 8 * L;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (acc[k]) atomicAdd(&dhist[LL + cls[k * L + t]], acc[k]);
+                acc[k] = 0;
+            }
+        };
+        for (int x = xb; x < xe; ++x) {
+            const int64_t e = b + o.order[x];
+            const int k = o.key[o.order[x]];
+            if (k != key) {
+                if (key >= 0) flush();
+                key = k;
+            }
+            const int pi = k / 2 / L, pj = k / 2 % L, dir = k & 1;
+            const bool swap = lab[e] & 2;
+            const int32_t i = swap ? g.e_hi[e] : g.e_lo[e], j = swap ? g.e_lo[e] : g.e_hi[e];
+            const uint4 c = *reinterpret_cast<const uint4 *>(cell + (e * L + t) * 4);
+            const int64_t c0 = c.x, c1 = swap ? c.z : c.y, c2 = swap ? c.y : c.z, c3 = c.w;   // (++ +- -+ --)
             const int64_t di = typed_degree(g, i, t), dj = typed_degree(g, j, t);
             const int64_t oi = outdeg[(int64_t)i * L + t], oj = outdeg[(int64_t)j * L + t];
             const int64_t v[8] = {
-                oi - c0 - c1 - ((pj == t && o == 0) ? 1 : 0),                   // S_i^{t,+}
-                (di - oi) - c2 - c3 - ((pj == t && o == 1) ? 1 : 0),            // S_i^{t,-}
-                oj - c0 - c2 - ((pi == t && o == 1) ? 1 : 0),                   // S_j^{t,+}
-                (dj - oj) - c1 - c3 - ((pi == t && o == 0) ? 1 : 0),            // S_j^{t,-}
+                oi - c0 - c1 - ((pj == t && dir == 0) ? 1 : 0),                 // S_i^{t,+}
+                (di - oi) - c2 - c3 - ((pj == t && dir == 1) ? 1 : 0),          // S_i^{t,-}
+                oj - c0 - c2 - ((pi == t && dir == 1) ? 1 : 0),                 // S_j^{t,+}
+                (dj - oj) - c1 - c3 - ((pi == t && dir == 0) ? 1 : 0),          // S_j^{t,-}
                 c0, c1, c2, c3};
-            const int32_t *cls = slot_class + (((int64_t)pi * L + pj) * 2 + o) * 8 * L;
             uint32_t *row = per_edge_out ? per_edge_out + e * 8 * L : nullptr;
-            for (int k = 0; k < 8; ++k) {
-                if (v[k] < 0) set_status(status, ST_INTERNAL);
-                if (row) row[k * L + t] = (uint32_t)(v[k] < 0 ? 0 : v[k]);
-                if (v[k] > 0) atomicAdd(&dhist[LL + cls[k * L + t]], (unsigned long long)v[k]);
+#pragma unroll
+            for (int y = 0; y < 8; ++y) {
+                if (v[y] < 0) set_status(status, ST_INTERNAL);
+                if (row) row[y * L + t] = (uint32_t)(v[y] < 0 ? 0 : v[y]);
+                acc[y] += (unsigned long long)(v[y] < 0 ? 0 : v[y]);
             }
         }
-        if (lane == 0) atomicAdd(&dhist[o == 0 ? pi * L + pj : pj * L + pi], 1ull);   // (tail type, head type)
+        if (key >= 0) flush();
     }
     __syncthreads();
     for (int s = threadIdx.x; s < G; s += blockDim.x)
@@ -297,18 +337,22 @@ void symmetrize_arcs(int64_t n, int64_t na, const int64_t *orp, const int32_t *o
 // symmetric CSR of these arcs; the class tables of L on the device.
 void prepare_directed(Graph &G, int64_t na, const int32_t *src, const int32_t *ocol, cudaStream_t s) {
     const GraphView gv = G.view();
-    G.dsign.alloc(std::max<int64_t>(G.nnz, 1));
+    TBuf sign(std::max<int64_t>(G.nnz, 1), s);
+    G.dlab.alloc(std::max<int64_t>(G.m, 1));
     G.doutdeg.alloc(sizeof(int32_t) * (size_t)std::max<int64_t>(G.n * G.L, 1));
-    TG_CK(cudaMemsetAsync(G.dsign.p, 0, std::max<int64_t>(G.nnz, 1), s));
+    TG_CK(cudaMemsetAsync(sign.p, 0, std::max<int64_t>(G.nnz, 1), s));
     TBuf new_of(sizeof(int32_t) * std::max<int64_t>(G.n, 1), s);
     if (G.n > 0)
         k_new_of<<<(unsigned)((G.n + 255) / 256), 256, 0, s>>>(G.n, G.old_of.as<int32_t>(), new_of.as<int32_t>());
     if (na > 0)
         k_arc_sign<<<(unsigned)((na + 255) / 256), 256, 0, s>>>(gv, na, src, ocol, new_of.as<int32_t>(),
-                                                                 G.dsign.as<int8_t>(), G.status.as<uint32_t>());
+                                                                 sign.as<int8_t>(), G.status.as<uint32_t>());
     if (G.n > 0)
         k_out_degree<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sm_count() * 16), 256, 0, s>>>(
-            gv, G.dsign.as<int8_t>(), G.doutdeg.as<int32_t>(), G.status.as<uint32_t>());
+            gv, sign.as<int8_t>(), G.doutdeg.as<int32_t>(), G.status.as<uint32_t>());
+    if (G.m > 0)
+        k_arc_labels<<<(unsigned)((G.m + 255) / 256), 256, 0, s>>>(gv, sign.as<int8_t>(), G.old_of.as<int32_t>(),
+                                                                   G.dlab.as<uint8_t>());
     TG_CK(cudaGetLastError());
     const DirectedTables &D = directed_tables(G.L);
     G.dcls.alloc(sizeof(int32_t) * D.slot_class.size());
@@ -326,21 +370,25 @@ int64_t run_directed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, cud
     const int Gs = (int)G.d_global;
     TG_CK(cudaMemsetAsync(G.dgacc.p, 0, sizeof(unsigned long long) * (size_t)Gs, s));
     const size_t smem = sizeof(unsigned long long) * (size_t)Gs;
-    const bool merge = isect_any_merge(G.opt.isect_modes);
-    const void *fn = merge ? (const void *)k_directed3<true> : (const void *)k_directed3<false>;
-    raise_smem_limit(fn, smem);
     int64_t launches = 0;
     if (G.m > 0) {
-        KernelTimer kt(G, s, "k_directed3");
-        const unsigned grid = (unsigned)std::min<int64_t>((G.m + 7) / 8, (int64_t)sm_count() * 16);
-        if (merge)
-            k_directed3<true><<<grid, 256, smem, s>>>(G.view(), G.dsign.as<int8_t>(), G.doutdeg.as<int32_t>(),
-                                                       G.old_of.as<int32_t>(), G.dcls.as<int32_t>(), Gs, per_edge_out,
-                                                       G.dgacc.as<unsigned long long>(), G.status.as<uint32_t>());
-        else
-            k_directed3<false><<<grid, 256, smem, s>>>(G.view(), G.dsign.as<int8_t>(), G.doutdeg.as<int32_t>(),
-                                                        G.old_of.as<int32_t>(), G.dcls.as<int32_t>(), Gs, per_edge_out,
-                                                        G.dgacc.as<unsigned long long>(), G.status.as<uint32_t>());
+        const size_t bytes = sizeof(uint32_t) * 4 * (size_t)G.L * (size_t)G.m;
+        if (G.dcell.bytes < bytes) G.dcell.alloc(bytes);
+        {
+            KernelTimer kt(G, s, "k_directed_cells");
+            TG_CK(cudaMemsetAsync(G.dcell.p, 0, bytes, s));
+            launches += visit_triangles(G, DirectedCells{G.dcell.as<uint32_t>(), G.dlab.as<uint8_t>(), G.L}, s);
+        }
+        KernelTimer kt(G, s, "k_directed_rows");
+        const int64_t tile = tile_edges(G);
+        const unsigned grid = (unsigned)std::min<int64_t>((G.m + tile - 1) / tile, (int64_t)sm_count() * 6);
+        with_types(G.L, [&](auto l) {
+            constexpr int L = decltype(l)::value;
+            raise_smem_limit((const void *)k_directed_rows<L>, smem);
+            k_directed_rows<L><<<grid, kRowThreads, smem, s>>>(
+                G.view(), G.dcell.as<uint32_t>(), G.dlab.as<uint8_t>(), G.doutdeg.as<int32_t>(), G.dcls.as<int32_t>(), Gs,
+                tile, per_edge_out, G.dgacc.as<unsigned long long>(), G.status.as<uint32_t>());
+        });
         ++launches;
     }
     if (global_out) {

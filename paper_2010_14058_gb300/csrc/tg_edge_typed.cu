@@ -4,20 +4,23 @@
 // edge types).
 //
 // The handle is the ordinary tg_build layout (rows by (type, id), per-type
-// segments) plus one edge type per adjacency slot and, per node x, node type
-// t and edge type q, the number d_x^{t,q} of x's type-t neighbours joined to
-// x by an edge of type q.  Per edge {i, j}, one warp intersects the typed
-// segments of i and j (binary search or merge, isect); each triangle node w
-// of type t adds 1 to the warp's cell (t, type of {i,w}, type of {j,w}).
-// The sets S_i, S_j follow by Cor. 1-2, split by edge type:
+// segments) plus one edge type per edge and, per node x, node type t and edge
+// type q, the number d_x^{t,q} of x's type-t neighbours joined to x by an
+// edge of type q.  Every triangle is found once (tg_visit.cuh) and counted at
+// each of its edges in the slot (t, {types of the other two edges}); these
+// cells are the row's triangle slots.  A second kernel forms the 3-path slots
+// and the class sums.  The sets S_i, S_j follow by Cor. 1-2, split by edge
+// type:
 //   |S_i^{t,x}| = d_i^{t,x} - |{w in T^t : xi_iw = x}| - [phi_j = t, xi_ij = x]
 // and likewise for S_j.  A 3-path's slot is (t, x) whichever endpoint is its
-// centre (its class ({phi_i, phi_j, t}, {xi_ij, x}) is the same), a
-// triangle's slot (t, {xi_iw, xi_jw}).  Per-edge layout and class ranks:
-// include/tg.h.
+// centre (its class ({phi_i, phi_j, t}, {xi_ij, x}) is the same), so it needs
+// |{w : xi_iw = x}| + |{w : xi_jw = x}|, which the unordered cells give.
+// Per-edge layout and class ranks: include/tg.h.
 #include <algorithm>
 
 #include "tg_host.hpp"
+#include "tg_tiles.cuh"
+#include "tg_visit.cuh"
 
 namespace tg {
 
@@ -92,12 +95,13 @@ __global__ void k_et_fill(GraphView g, int64_t nnz, const int64_t *__restrict__ 
     etype[s] = t;
 }
 
-// both slots of every edge hold the same type
-__global__ void k_et_check(GraphView g, const uint8_t *__restrict__ etype, uint32_t *status) {
+// both slots of every edge hold the same type, which is the edge's
+__global__ void k_et_check(GraphView g, const uint8_t *__restrict__ etype, uint8_t *by_edge, uint32_t *status) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= g.m) return;
     const uint8_t a = etype[g.e_slot_lo[e]], b = etype[g.e_slot_hi[e]];
     if (a == 0xff || a != b) set_status(status, ST_INVALID_GRAPH);
+    by_edge[e] = a;
 }
 
 // d_x^{t,q}: warp per node, one warp sum per (type, edge type)
@@ -126,88 +130,128 @@ __global__ void __launch_bounds__(256) k_et_degree(GraphView g, const uint8_t *_
 }
 
 // ---------------------------------------------------------------- count
-// Warp per edge {i, j}: the triangle cells in the warp's shared-memory
-// histogram, then per lane the path and triangle slots, the row, and the
-// per-CTA class histogram (block 0 edges, block 1 3-paths, block 2
-// triangles).
-template <bool kMerge>
-__global__ void __launch_bounds__(256) k_edge_typed3(GraphView g, const uint8_t *__restrict__ etype,
-                                                     const int32_t *__restrict__ etdeg, int X, int G,
-                                                     uint32_t *per_edge_out, unsigned long long *gacc,
-                                                     uint32_t *status) {
+// position of the unordered pair {x, y} among the pairs of X edge types
+__device__ __forceinline__ int x_pair(int X, int x, int y) {
+    const int a = x < y ? x : y, b = x < y ? y : x;
+    return a * X - a * (a - 1) / 2 + (b - a);
+}
+
+// cells [edge][type of the third node][pair of its edges' types]
+struct EdgeTypedCells {
+    uint32_t *cell;
+    int64_t stride;             // words from edge to edge
+    const uint8_t *xi;
+    int X, P;
+    __device__ __forceinline__ void operator()(int64_t ua, int64_t ub, int64_t ab, int tu, int ta, int tb) const {
+        const int xa = xi[ua], xb = xi[ub], xab = xi[ab];
+        atomicAdd(&cell[ua * stride + tb * P + x_pair(X, xb, xab)], 1u);
+        atomicAdd(&cell[ub * stride + ta * P + x_pair(X, xa, xab)], 1u);
+        atomicAdd(&cell[ab * stride + tu * P + x_pair(X, xa, xb)], 1u);
+    }
+};
+
+constexpr int kRowThreads = 256;
+
+// zeroes the cells of every edge
+__global__ void k_et_zero(int64_t m, int64_t stride, int words, uint32_t *cell) {
+    const int64_t n = m * words;
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
+        cell[x / words * stride + x % words] = 0u;
+}
+
+// Thread per (edge, slot): the 3-path slot from the typed degrees and the
+// cells, or the triangle slot's cell; class sums (block 0 edges, block 1
+// 3-paths, block 2 triangles) are kept in registers while the endpoints'
+// types and the edge's type stay the same.
+template <int L, int X>
+__global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, const uint32_t *__restrict__ cell,
+                                                                 int64_t stride, const uint8_t *__restrict__ xi,
+                                                                 const int32_t *__restrict__ etdeg, int G, int64_t tile,
+                                                                 uint32_t *per_edge_out,
+                                                                 unsigned long long *gacc, uint32_t *status) {
     extern __shared__ unsigned long long ehist[];
-    __shared__ uint32_t wh_all[8][kMaxL * kMaxX * kMaxX];
-    const int L = g.L;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t *wh = wh_all[wid];
-    const int XX = X * X, P = X * (X + 1) / 2;
-    const int64_t S = (int64_t)L * X + (int64_t)L * P;
+    __shared__ TileOrder<L * L * X> o;
+    constexpr int P = X * (X + 1) / 2, S = L * X + L * P, E = kRowThreads / S;
     const int64_t off1 = mchoose(L, 2) * X, off2 = off1 + mchoose(L, 3) * mchoose(X, 2);
     const int64_t w2 = mchoose(X, 2), w3 = mchoose(X, 3);
     for (int s = threadIdx.x; s < G; s += blockDim.x) ehist[s] = 0;
-    __syncthreads();
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; e < g.m; e += nw) {
-        const int32_t i = g.e_lo[e], j = g.e_hi[e];
-        const int pi = g.ty[i], pj = g.ty[j];
-        const int xij = etype[g.e_slot_lo[e]];
-        for (int k = lane; k < L * XX; k += 32) wh[k] = 0;
-        __syncwarp();
-        for (int t = 0; t < L; ++t) {
-            const int64_t bi = seg_begin(g, i, t), ei = seg_end(g, i, t);
-            const int64_t bj = seg_begin(g, j, t), ej = seg_end(g, j, t);
-            if (ei == bi || ej == bj) continue;                          // warp-uniform
-            const bool i_short = ei - bi <= ej - bj;
-            const int64_t sb = i_short ? bi : bj, se = i_short ? ei : ej;
-            const int64_t lb = i_short ? bj : bi, le = i_short ? ej : ei;
-            isect<kMerge>(g.adj, g.isect_modes, sb, se, lb, le, lane, [&](bool found, int64_t s, int64_t r, int32_t) {
-                if (found) {
-                    const int xa = etype[i_short ? s : r], xb = etype[i_short ? r : s];   // edges {i,w}, {j,w}
-                    atomicAdd(&wh[(t * X + xa) * X + xb], 1u);
+    // ranks of the multisets {phi_i, phi_j, t}, {xi_ij, x}, {xi_ij, x, y}
+    __shared__ uint16_t rank_n[L * L * L], rank_2[X * X], rank_3[X * X * X];
+    for (int k = threadIdx.x; k < L * L * L; k += blockDim.x) {
+        int n3[3] = {k / (L * L), k / L % L, k % L};
+        sort3v(n3);
+        rank_n[k] = (uint16_t)ms_rank(L, 3, n3);
+    }
+    for (int k = threadIdx.x; k < X * X * X; k += blockDim.x) {
+        int e3[3] = {k / (X * X), k / X % X, k % X}, e2[2] = {k / X, k % X};
+        sort3v(e3);
+        rank_3[k] = (uint16_t)ms_rank(X, 3, e3);
+        if (k >= X * X) continue;
+        sort2(e2);
+        rank_2[k] = (uint16_t)ms_rank(X, 2, e2);
+    }
+    const int slice = threadIdx.x / S, slot = threadIdx.x % S;
+    const bool path = slot < L * X;
+    const int t = path ? slot / X : (slot - L * X) / P;
+    const int pair = path ? 0 : (slot - L * X) % P;
+    int x_at[X];                                            // pairs {x0, z} of a path slot
+    int x0 = 0, y0 = 0;                                     // the slot's edge types: {x} or {x, y}
+    if (path) {
+        x0 = slot % X;
+    } else {
+        int r = pair;
+        while (r >= X - x0) { r -= X - x0; ++x0; }
+        y0 = x0 + r;
+    }
+#pragma unroll
+    for (int z = 0; z < X; ++z) x_at[z] = x_pair(X, x0, z);
+    for (int64_t b = blockIdx.x * tile; b < g.m; b += gridDim.x * tile) {
+        const int n = (int)min(tile, g.m - b);
+        tile_order(b, n, o, [&](int64_t e) { return (g.ty[g.e_lo[e]] * L + g.ty[g.e_hi[e]]) * X + xi[e]; });
+        for (int k = threadIdx.x; k < L * L * X; k += blockDim.x)
+            if (o.count[k]) {
+                int n2[2] = {k / X / L, k / X % L};
+                sort2(n2);
+                atomicAdd(&ehist[ms_rank(L, 2, n2) * X + k % X], (unsigned long long)o.count[k]);
+            }
+        if (slice >= E) continue;
+        int xb, xe;
+        slice_of(n, slice, E, xb, xe);
+        unsigned long long acc = 0;
+        int key = -1;
+        auto flush = [&]() {
+            const int n3 = rank_n[(key / X) * L + t];
+            if (acc)
+                atomicAdd(&ehist[path ? off1 + n3 * w2 + rank_2[key % X * X + x0]
+                                      : off2 + n3 * w3 + rank_3[(key % X * X + x0) * X + y0]], acc);
+            acc = 0;
+        };
+        for (int x = xb; x < xe; ++x) {
+            const int rel = o.order[x], k = o.key[rel];
+            const int64_t e = b + rel;
+            if (k != key) {
+                if (key >= 0) flush();
+                key = k;
+            }
+            const uint32_t *c = cell + e * stride + t * P;
+            int64_t v;
+            if (path) {
+                const int pi = k / X / L, pj = k / X % L, xij = k % X;
+                v = (int64_t)etdeg[((int64_t)g.e_lo[e] * L + t) * X + x0] + etdeg[((int64_t)g.e_hi[e] * L + t) * X + x0] -
+                    ((pj == t && xij == x0) ? 1 : 0) - ((pi == t && xij == x0) ? 1 : 0);
+#pragma unroll
+                for (int z = 0; z < X; ++z) v -= (int64_t)c[x_at[z]] * (z == x0 ? 2 : 1);
+                if (v < 0) {
+                    set_status(status, ST_INTERNAL);
+                    v = 0;
                 }
-            });
-        }
-        __syncwarp();
-        uint32_t *row = per_edge_out ? per_edge_out + e * S : nullptr;
-        for (int p = lane; p < L * X; p += 32) {                        // 3-paths (t, x)
-            const int t = p / X, x = p - t * X;
-            int64_t ti = 0, tj = 0;
-            for (int y = 0; y < X; ++y) {
-                ti += wh[(t * X + x) * X + y];
-                tj += wh[(t * X + y) * X + x];
+                if (per_edge_out) per_edge_out[e * S + slot] = (uint32_t)v;   // (the cells are in place)
+            } else {
+                v = c[pair];
             }
-            const int64_t a = etdeg[((int64_t)i * L + t) * X + x] - ti - ((pj == t && xij == x) ? 1 : 0);
-            const int64_t b = etdeg[((int64_t)j * L + t) * X + x] - tj - ((pi == t && xij == x) ? 1 : 0);
-            if (a < 0 || b < 0) set_status(status, ST_INTERNAL);
-            const int64_t v = (a < 0 ? 0 : a) + (b < 0 ? 0 : b);
-            if (row) row[p] = (uint32_t)v;
-            if (v) {
-                int n3[3] = {pi, pj, t}, e2[2] = {xij, x};
-                sort3v(n3);
-                sort2(e2);
-                atomicAdd(&ehist[off1 + ms_rank(L, 3, n3) * w2 + ms_rank(X, 2, e2)], (unsigned long long)v);
-            }
+            acc += (unsigned long long)v;
         }
-        for (int q = lane; q < L * P; q += 32) {                        // triangles (t, {x, y})
-            const int t = q / P;
-            int r = q - t * P, x = 0;
-            while (r >= X - x) { r -= X - x; ++x; }
-            const int y = x + r;
-            const uint32_t v = wh[(t * X + x) * X + y] + (x != y ? wh[(t * X + y) * X + x] : 0u);
-            if (row) row[(int64_t)L * X + q] = v;
-            if (v) {
-                int n3[3] = {pi, pj, t}, e3[3] = {xij, x, y};
-                sort3v(n3);
-                sort3v(e3);
-                atomicAdd(&ehist[off2 + ms_rank(L, 3, n3) * w3 + ms_rank(X, 3, e3)], (unsigned long long)v);
-            }
-        }
-        if (lane == 0) {
-            int n2[2] = {pi, pj};
-            sort2(n2);
-            atomicAdd(&ehist[ms_rank(L, 2, n2) * X + xij], 1ull);
-        }
-        __syncwarp();                                                   // the cells are cleared next
+        if (key >= 0) flush();
     }
     __syncthreads();
     for (int s = threadIdx.x; s < G; s += blockDim.x)
@@ -238,19 +282,21 @@ int64_t edge_typed_global_slots(int L, int X) {
 void prepare_edge_typed(Graph &G, int X, const int64_t *row_ptr, const int32_t *col, const uint8_t *edge_types,
                         cudaStream_t s) {
     const GraphView gv = G.view();
-    G.etype.alloc(std::max<int64_t>(G.nnz, 1));
+    TBuf by_slot(std::max<int64_t>(G.nnz, 1), s);
+    G.etype.alloc(std::max<int64_t>(G.m, 1));
     G.etdeg.alloc(sizeof(int32_t) * (size_t)std::max<int64_t>(G.n * G.L * X, 1));
-    TG_CK(cudaMemsetAsync(G.etype.p, 0xff, std::max<int64_t>(G.nnz, 1), s));
+    TG_CK(cudaMemsetAsync(by_slot.p, 0xff, std::max<int64_t>(G.nnz, 1), s));
     TG_CK(cudaMemsetAsync(G.status.p, 0, sizeof(uint32_t), s));
     TBuf new_of(sizeof(int32_t) * std::max<int64_t>(G.n, 1), s);
     if (G.n > 0)
         k_et_new_of<<<(unsigned)((G.n + 255) / 256), 256, 0, s>>>(G.n, G.old_of.as<int32_t>(), new_of.as<int32_t>());
     if (G.nnz > 0)
         k_et_fill<<<(unsigned)((G.nnz + 255) / 256), 256, 0, s>>>(gv, G.nnz, row_ptr, col, edge_types, X,
-                                                                   new_of.as<int32_t>(), G.etype.as<uint8_t>(),
+                                                                   new_of.as<int32_t>(), by_slot.as<uint8_t>(),
                                                                    G.status.as<uint32_t>());
     if (G.m > 0)
-        k_et_check<<<(unsigned)((G.m + 255) / 256), 256, 0, s>>>(gv, G.etype.as<uint8_t>(), G.status.as<uint32_t>());
+        k_et_check<<<(unsigned)((G.m + 255) / 256), 256, 0, s>>>(gv, by_slot.as<uint8_t>(), G.etype.as<uint8_t>(),
+                                                                 G.status.as<uint32_t>());
     TG_CK(cudaGetLastError());
     uint32_t st = 0;
     TG_CK(cudaMemcpyAsync(&st, G.status.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
@@ -259,7 +305,7 @@ void prepare_edge_typed(Graph &G, int X, const int64_t *row_ptr, const int32_t *
     if (st) throw Error{TG_ERR_INTERNAL, "edge type slots"};
     if (G.n > 0)
         k_et_degree<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sm_count() * 16), 256, 0, s>>>(
-            gv, G.etype.as<uint8_t>(), X, G.etdeg.as<int32_t>());
+            gv, by_slot.as<uint8_t>(), X, G.etdeg.as<int32_t>());
     TG_CK(cudaGetLastError());
     G.et_X = X;
     G.et_global = edge_typed_global_slots(G.L, X);
@@ -271,21 +317,39 @@ int64_t run_edge_typed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, c
     const int Gs = (int)G.et_global, X = G.et_X, L = G.L;
     TG_CK(cudaMemsetAsync(G.etgacc.p, 0, sizeof(unsigned long long) * (size_t)Gs, s));
     const size_t smem = sizeof(unsigned long long) * (size_t)Gs;
-    const bool merge = isect_any_merge(G.opt.isect_modes);
-    const void *fn = merge ? (const void *)k_edge_typed3<true> : (const void *)k_edge_typed3<false>;
-    raise_smem_limit(fn, smem);
     int64_t launches = 0;
     if (G.m > 0) {
-        KernelTimer kt(G, s, "k_edge_typed3");
-        const unsigned grid = (unsigned)std::min<int64_t>((G.m + 7) / 8, (int64_t)sm_count() * 16);
-        if (merge)
-            k_edge_typed3<true><<<grid, 256, smem, s>>>(G.view(), G.etype.as<uint8_t>(), G.etdeg.as<int32_t>(), X, Gs,
-                                                         per_edge_out, G.etgacc.as<unsigned long long>(),
-                                                         G.status.as<uint32_t>());
-        else
-            k_edge_typed3<false><<<grid, 256, smem, s>>>(G.view(), G.etype.as<uint8_t>(), G.etdeg.as<int32_t>(), X, Gs,
-                                                          per_edge_out, G.etgacc.as<unsigned long long>(),
-                                                          G.status.as<uint32_t>());
+        const int P = X * (X + 1) / 2, S = L * X + L * P;
+        // the rows hold the cells; without rows, a buffer of the handle
+        uint32_t *cell = per_edge_out ? per_edge_out + L * X : nullptr;
+        const int64_t stride = per_edge_out ? S : L * P;
+        if (!cell) {
+            const size_t bytes = sizeof(uint32_t) * (size_t)(stride * G.m);
+            if (G.etcell.bytes < bytes) G.etcell.alloc(bytes);
+            cell = G.etcell.as<uint32_t>();
+        }
+        {
+            KernelTimer kt(G, s, "k_edge_typed_cells");
+            k_et_zero<<<(unsigned)std::min<int64_t>((G.m * L * P + 255) / 256, (int64_t)sm_count() * 32), 256, 0, s>>>(
+                G.m, stride, L * P, cell);
+            launches += 1 + visit_triangles(G, EdgeTypedCells{cell, stride, G.etype.as<uint8_t>(), X, P}, s);
+        }
+        KernelTimer kt(G, s, "k_edge_typed_rows");
+        const int64_t tile = tile_edges(G);
+        const unsigned grid = (unsigned)std::min<int64_t>((G.m + tile - 1) / tile, (int64_t)sm_count() * 6);
+        with_types(L, [&](auto l) {
+            constexpr int kL = decltype(l)::value;
+            auto run = [&](auto kern) {
+                raise_smem_limit((const void *)kern, smem);
+                kern<<<grid, kRowThreads, smem, s>>>(G.view(), cell, stride, G.etype.as<uint8_t>(), G.etdeg.as<int32_t>(),
+                                                     Gs, tile, per_edge_out, G.etgacc.as<unsigned long long>(),
+                                                     G.status.as<uint32_t>());
+            };
+            if (X == 1) run(k_edge_typed_rows<kL, 1>);
+            else if (X == 2) run(k_edge_typed_rows<kL, 2>);
+            else if (X == 3) run(k_edge_typed_rows<kL, 3>);
+            else run(k_edge_typed_rows<kL, 4>);
+        });
         ++launches;
     }
     if (global_out) {

@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "tg_host.hpp"
+#include "tg_tiles.cuh"
 
 namespace tg {
 
@@ -90,56 +91,16 @@ __device__ void flush_hist(unsigned long long *hist, int G, unsigned long long *
     }
 }
 
-// ------------------------------------------------------------ tile order
-struct TileOrder {
-    uint16_t order[kTile];      // the tile's edges (relative to its first) grouped by key
-    uint8_t key[kTile];         // types of the endpoints, p * L + q, by edge
-    int count[kMaxL * kMaxL];   // edges of each key
-    int next[kMaxL * kMaxL];
-};
-
-// groups the tile's edges by the types of their endpoints; by_caller: p is
-// the type of the endpoint with the smaller caller id, else of e_lo.  Begins
-// and ends with a barrier.
+// the types of the endpoints, p * L + q; by_caller: p is the type of the
+// endpoint with the smaller caller id, else of e_lo
 template <int L>
-__device__ __forceinline__ void tile_order(const GraphView &g, const Tile &tile, TileOrder &o, bool by_caller,
-                                           const int32_t *__restrict__ old_of) {
-    constexpr int LL = L * L;
-    __syncthreads();
-    for (int k = threadIdx.x; k < LL; k += blockDim.x) o.count[k] = 0;
-    __syncthreads();
-    const int n = (int)(tile.end - tile.begin);
-    for (int x = threadIdx.x; x < n; x += blockDim.x) {
-        const int32_t i = g.e_lo[tile.begin + x], j = g.e_hi[tile.begin + x];
+__device__ __forceinline__ void order_by_types(const GraphView &g, const Tile &tile, TileOrder<L * L> &o, bool by_caller,
+                                               const int32_t *__restrict__ old_of) {
+    tile_order(tile.begin, (int)(tile.end - tile.begin), o, [&](int64_t e) {
+        const int32_t i = g.e_lo[e], j = g.e_hi[e];
         const bool swap = by_caller && old_of[i] > old_of[j];
-        const int p = g.ty[swap ? j : i], q = g.ty[swap ? i : j];
-        o.key[x] = (uint8_t)(p * L + q);
-        atomicAdd(&o.count[p * L + q], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int run = 0;
-        for (int b = 0; b < LL; b += 32) {
-            const int k = b + threadIdx.x;
-            const int c = k < LL ? o.count[k] : 0;
-            int inc = c;
-            for (int d = 1; d < 32; d <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, inc, d);
-                if ((int)threadIdx.x >= d) inc += y;
-            }
-            if (k < LL) o.next[k] = run + inc - c;
-            run += __shfl_sync(0xffffffffu, inc, 31);
-        }
-    }
-    __syncthreads();
-    for (int x = threadIdx.x; x < n; x += blockDim.x) o.order[atomicAdd(&o.next[o.key[x]], 1)] = (uint16_t)x;
-    __syncthreads();
-}
-
-// the share of slice s of E of a tile's n grouped edges
-__device__ __forceinline__ void slice_of(int n, int s, int E, int &b, int &e) {
-    b = (int)((int64_t)n * s / E);
-    e = (int)((int64_t)n * (s + 1) / E);
+        return g.ty[swap ? j : i] * L + g.ty[swap ? i : j];
+    });
 }
 
 // ------------------------------------------------------------ slot rows
@@ -248,7 +209,7 @@ __global__ void __launch_bounds__(kEpiThreads, 3) k_epi4(GraphView g, CountView 
     constexpr int LL = L * L, P = L * (L + 1) / 2, S = 2 * L + 10 * P;
     constexpr int E = kEpiThreads / P;                      // edges in flight per CTA
     extern __shared__ unsigned long long hist[];
-    __shared__ TileOrder o;
+    __shared__ TileOrder<LL> o;
     const int G = (int)global_slots(L, 4);
     uint16_t *rank2 = reinterpret_cast<uint16_t *>(hist + G);
     uint16_t *rank3 = rank2 + LL;
@@ -277,7 +238,7 @@ __global__ void __launch_bounds__(kEpiThreads, 3) k_epi4(GraphView g, CountView 
     int cur_graph = -1;
     for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
         const Tile tile = tiles[ti];
-        tile_order<L>(g, tile, o, false, nullptr);
+        order_by_types<L>(g, tile, o, false, nullptr);
         if (tile.graph != cur_graph) {
             if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph);
             __syncthreads();
@@ -374,7 +335,7 @@ __global__ void __launch_bounds__(kEpiThreads) k_edge3(GraphView g, CountView cv
                                                        unsigned long long *gacc) {
     constexpr int LL = L * L, S = 2 * L, E = kEpiThreads / L;
     extern __shared__ unsigned long long hist[];
-    __shared__ TileOrder o;
+    __shared__ TileOrder<LL> o;
     const int G = (int)global_slots(L, 3);
     for (int s = threadIdx.x; s < G; s += blockDim.x) hist[s] = 0;
     const int off1 = gblock_off(L, 1), off2 = gblock_off(L, 2);
@@ -382,7 +343,7 @@ __global__ void __launch_bounds__(kEpiThreads) k_edge3(GraphView g, CountView cv
     int cur_graph = -1;
     for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
         const Tile tile = tiles[ti];
-        tile_order<L>(g, tile, o, false, nullptr);
+        order_by_types<L>(g, tile, o, false, nullptr);
         if (tile.graph != cur_graph) {
             if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph);
             __syncthreads();
@@ -457,7 +418,7 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
     constexpr int LL = L * L, P = L * (L + 1) / 2, E = kEpiThreads / P;
     constexpr int kOrdered = 9, kPairs = 6;
     extern __shared__ unsigned long long hist[];
-    __shared__ TileOrder o;
+    __shared__ TileOrder<LL> o;
     const int S = pv.S, G = pv.G;
     for (int s = threadIdx.x; s < G; s += blockDim.x) hist[s] = 0;
     const int slice = threadIdx.x / P, pi = threadIdx.x % P;
@@ -471,7 +432,7 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
     int cur_graph = -1;
     for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
         const Tile tile = tiles[ti];
-        tile_order<L>(g, tile, o, true, pv.old_of);
+        order_by_types<L>(g, tile, o, true, pv.old_of);
         if (tile.graph != cur_graph) {
             if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph);
             __syncthreads();

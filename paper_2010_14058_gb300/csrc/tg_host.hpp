@@ -153,13 +153,14 @@ struct Graph {
     };
     std::vector<std::unique_ptr<HubPlan>> hub_plans;
     DBuf hub_tables;
-    // directed counts (tg_directed.cu): slot signs, typed out-degrees, class tables
-    DBuf dsign, doutdeg, dcls, darcs, dgacc;
+    // directed counts (tg_directed.cu): edge labels, typed out-degrees, class tables, triangle cells
+    DBuf dlab, doutdeg, dcls, darcs, dgacc, dcell;
     int64_t d_global = 0;
     bool directed = false;
-    // edge-typed counts (tg_edge_typed.cu): edge type per slot, per-node
-    // neighbour counts by (node type, edge type), the totals' accumulator
-    DBuf etype, etdeg, etgacc;
+    // edge-typed counts (tg_edge_typed.cu): edge type per edge, per-node
+    // neighbour counts by (node type, edge type), the totals' accumulator,
+    // triangle cells when there are no rows to hold them
+    DBuf etype, etdeg, etgacc, etcell;
     int32_t et_X = 0;
     int64_t et_global = 0;
     bool edge_typed = false;
@@ -196,7 +197,6 @@ struct Graph {
     GraphView view() const {
         GraphView v;
         v.ngraphs = ngraphs; v.L = L; v.n = n; v.nnz = nnz; v.m = m;
-        v.isect_modes = opt.isect_modes;
         v.node_off = node_off.as<int64_t>();
         v.edge_off = edge_off.as<int64_t>();
         v.rp = rp.as<int64_t>();
@@ -245,7 +245,7 @@ struct Graph {
         return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
-                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dsign, &doutdeg, &dcls, &darcs, &dgacc, &etype, &etdeg, &etgacc, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
+                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dlab, &doutdeg, &dcls, &darcs, &dgacc, &dcell, &etype, &etdeg, &etgacc, &etcell, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
@@ -360,6 +360,9 @@ void prepare_edges(Graph &G, int k, cudaStream_t s);
 // stage recomputed (no cached state).  Returns the kernel launches.
 int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per_edge_out,
                   unsigned long long *gacc, bool full, cudaStream_t s);
+// edges per tile of the per-edge kernels (tg_count.cu)
+int64_t tile_edges(const Graph &G);
+
 // rows and raw sums of the edges of the tiles (tg_epi.cu)
 void prepare_epi(Graph &G);
 int64_t launch_edges3(Graph &G, const Tile *tiles, int64_t n_tiles, int64_t e_begin, uint32_t *per_edge_out,
