@@ -129,7 +129,7 @@ struct Graph {
     tg_options opt;
 
     // graph (built once)
-    DBuf node_off, edge_off, rp, adj, toff, pivot, nplus, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
+    DBuf node_off, edge_off, rp, adj, toff, tdeg, pivot, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
     DBuf plus_off, plus_adj, plus_eid;
     // nodes by |N+| (tg_local.cuh): mid, big, and larger than shared memory holds
     DBuf tri_list[3], local_scratch;
@@ -203,7 +203,7 @@ struct Graph {
         v.adj = adj.as<int32_t>();
         v.toff = toff.as<int32_t>();
         v.pivot = pivot.as<int32_t>();
-        v.nplus = nplus.as<int32_t>();
+        v.tdeg = tdeg.as<uint32_t>();
         v.ty = ty.as<uint8_t>();
         v.slot_eid = slot_eid.as<int32_t>();
         v.e_lo = e_lo.as<int32_t>();
@@ -242,7 +242,7 @@ struct Graph {
         return v;
     }
     std::vector<const DBuf *> cbuffers() const {
-        return {&node_off, &edge_off, &rp, &adj, &toff, &pivot, &nplus, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
+        return {&node_off, &edge_off, &rp, &adj, &toff, &tdeg, &pivot, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
                              &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dlab, &doutdeg, &dcls, &darcs, &dgacc, &dcell, &etype, &etdeg, &etgacc, &etcell, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
@@ -314,6 +314,8 @@ struct LocalClass {
 };
 LocalClass local_class(const Graph &G, int cls);
 
+// out[x][t][q] = sums of rows[index[s]][q] over x's slots s of type t
+int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, int64_t *out, cudaStream_t s);
 // shared-memory limits and scratch of launch_triangles (before any capture)
 void prepare_triangles(Graph &G);
 // typed triangles per edge and, with_tau, the per-node sums of the whole

@@ -56,7 +56,7 @@ __device__ __forceinline__ Stage stage_carve(uint32_t *mem, int L) {   // mem: 8
     return s;
 }
 
-// typed triangle counts of one edge
+// the first L words of row e (of typed triangle counts by edge, or typed degrees by node)
 __device__ __forceinline__ void load_c(const uint32_t *C, int64_t e, int L, uint32_t *out) {
     const uint4 *c = reinterpret_cast<const uint4 *>(C + e * kCRow);
     const uint4 lo = c[0], hi = L > 4 ? c[1] : make_uint4(0, 0, 0, 0);
@@ -74,13 +74,7 @@ __device__ __forceinline__ void load_c(const uint32_t *C, int64_t e, int L, uint
 __device__ __forceinline__ void load_vec(const GraphView &g, const uint32_t *C, uint32_t eid, int32_t id, int L,
                                          uint32_t *vec) {
     load_c(C, eid, L, vec);
-    const int32_t *o = g.toff + (int64_t)id * (L + 1);
-    int32_t prev = o[0];
-    for (int q = 0; q < L; ++q) {
-        const int32_t next = o[q + 1];
-        vec[L + q] = (uint32_t)(next - prev);
-        prev = next;
-    }
+    load_c(g.tdeg, id, L, vec + L);
 }
 
 // stages triangle number i of the warp (nq is filled in by the caller)

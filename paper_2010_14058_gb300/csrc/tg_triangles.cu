@@ -100,38 +100,106 @@ __global__ void __launch_bounds__(kThreadsT) k_tri_cta(GraphView g, uint32_t *C,
     }
 }
 
-// Warp per node x: tau_x[t][t'] = sum_{w in Gamma_x^t} c_{xw}^{t'}, the
-// ordered adjacent pairs inside Gamma_x by type.
-__global__ void __launch_bounds__(256) k_tau(GraphView g, CountView cv) {
-    const int lane = threadIdx.x & 31;
+// out[x][t][q] = sum over x's slots s of type t of rows[index[s]][q] (rows of
+// kCRow words): with the edges' typed triangle counts tau_x[t][t'] = sum_{w in
+// Gamma_x^t} c_{xw}^{t'}, the ordered adjacent pairs inside Gamma_x by type;
+// with the nodes' typed degrees delta_x[t][t'] = sum_{w in Gamma_x^t} d_w^t'.
+// Eight lanes read one row (a 32-byte sector), so a warp takes four slots at
+// a time and a type's sums need two shuffles (a lane per slot with L sums
+// each left most lanes idle in segments of a few slots and needed L 64-bit
+// warp sums per type: 3.7 ms for delta and 3.0 for tau on a 20 M-edge
+// Chung-Lu graph against 0.9 and 1.27).  Rows of more than kLongRow slots: a
+// CTA per node.
+constexpr int64_t kLongRow = 1024;
+
+__device__ __forceinline__ unsigned long long seg_row_sum(const int32_t *__restrict__ index,
+                                                          const uint32_t *__restrict__ rows, int64_t s, int64_t e,
+                                                          int64_t step, int q) {
+    unsigned long long acc = 0;
+    for (; s + 3 * step < e; s += 4 * step) {
+        uint32_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldg(rows + (int64_t)__ldg(index + s + k * step) * kCRow + q);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc += v[k];
+    }
+    for (; s < e; s += step) acc += __ldg(rows + (int64_t)__ldg(index + s) * kCRow + q);
+    return acc;
+}
+
+__global__ void __launch_bounds__(256) k_row_sums(GraphView g, const int32_t *__restrict__ index,
+                                                  const uint32_t *__restrict__ rows, int64_t *out) {
     const int L = g.L;
+    const int lane = threadIdx.x & 31, q = lane & 7, sub = lane >> 3;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t x = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; x < g.n; x += nw) {
+        const int64_t b = g.rp[x];
+        if (g.rp[x + 1] - b > kLongRow) continue;
+        int32_t to = lane <= L ? g.toff[x * (L + 1) + lane] : 0;
         for (int t = 0; t < L; ++t) {
-            unsigned long long acc[kMaxL];
-#pragma unroll
-            for (int q = 0; q < kMaxL; ++q) acc[q] = 0;
-            for (int64_t s = seg_begin(g, x, t) + lane; s < seg_end(g, x, t); s += 32) {
-                const uint4 *c = reinterpret_cast<const uint4 *>(cv.C + (int64_t)g.slot_eid[s] * kCRow);
-                const uint4 lo = c[0];
-                acc[0] += lo.x; acc[1] += lo.y; acc[2] += lo.z; acc[3] += lo.w;
-                if (L > 4) {
-                    const uint4 hi = c[1];
-                    acc[4] += hi.x; acc[5] += hi.y; acc[6] += hi.z; acc[7] += hi.w;
-                }
+            const int64_t s = b + __shfl_sync(0xffffffffu, to, t), e = b + __shfl_sync(0xffffffffu, to, t + 1);
+            unsigned long long acc = 0;
+            if (e > s) {
+                acc = seg_row_sum(index, rows, s + sub, e, 4, q);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 16);
             }
-#pragma unroll
-            for (int q = 0; q < kMaxL; ++q) {
-                if (q >= L) break;
-                unsigned long long v = acc[q];
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-                if (lane == 0) cv.tau[(x * L + t) * L + q] = (int64_t)v;
-            }
+            if (lane < L) out[(x * L + t) * L + lane] = (int64_t)acc;
         }
     }
 }
 
+__global__ void __launch_bounds__(256) k_row_sums_long(GraphView g, const int32_t *__restrict__ index,
+                                                       const uint32_t *__restrict__ rows, int64_t *out) {
+    __shared__ unsigned long long part[8][kMaxL];
+    __shared__ int64_t found[256];
+    __shared__ int n_found;
+    const int L = g.L;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, q = lane & 7, sub = lane >> 3;
+    // the CTA's nodes are gridDim apart (long rows are the last ids of a
+    // graph), looked over 256 at a time
+    for (int64_t x0 = blockIdx.x; x0 < g.n; x0 += (int64_t)gridDim.x * 256) {
+        if (threadIdx.x == 0) n_found = 0;
+        __syncthreads();
+        const int64_t y = x0 + (int64_t)threadIdx.x * gridDim.x;
+        if (y < g.n && g.rp[y + 1] - g.rp[y] > kLongRow) found[atomicAdd(&n_found, 1)] = y;
+        __syncthreads();
+        const int n = n_found;
+        for (int k = 0; k < n; ++k) {
+            const int64_t x = found[k];
+            for (int t = 0; t < L; ++t) {
+                const int64_t s = seg_begin(g, x, t), e = seg_end(g, x, t);
+                unsigned long long acc = seg_row_sum(index, rows, s + wid * 4 + sub, e, 32, q);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+                if (lane < kMaxL) part[wid][lane] = acc;
+                __syncthreads();
+                if (threadIdx.x < L) {
+                    unsigned long long sum = 0;
+                    for (int w = 0; w < 8; ++w) sum += part[w][threadIdx.x];
+                    out[(x * L + t) * L + threadIdx.x] = (int64_t)sum;
+                }
+                __syncthreads();
+            }
+        }
+        __syncthreads();                                    // the list is replaced next
+    }
+}
+
 }  // namespace
+
+int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, int64_t *out, cudaStream_t s) {
+    if (G.n == 0) return 0;
+    const int sms = sm_count();
+    k_row_sums<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sms * 64), 256, 0, s>>>(G.view(), index, rows, out);
+    int64_t launches = 1;
+    if (G.max_degree > kLongRow) {
+        k_row_sums_long<<<(unsigned)std::min<int64_t>(G.n, (int64_t)sms * 8), 256, 0, s>>>(G.view(), index, rows, out);
+        ++launches;
+    }
+    TG_CK(cudaGetLastError());
+    return launches;
+}
 
 LocalClass local_class(const Graph &G, int cls) {
     LocalClass c;
@@ -193,8 +261,7 @@ int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s) {
     }
     if (G.n > 0 && with_tau) {
         KernelTimer kt(G, s, "k_tau");
-        k_tau<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sms * 16), 256, 0, s>>>(gv, cv);
-        ++launches;
+        launches += launch_row_sums(G, G.slot_eid.as<int32_t>(), cv.C, cv.tau, s);
     }
     TG_CK(cudaGetLastError());
     return launches;
