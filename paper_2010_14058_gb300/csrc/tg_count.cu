@@ -41,6 +41,7 @@
 
 #include <cub/device/device_scan.cuh>
 
+#include <memory>
 #include <mutex>
 
 #include "tg_host.hpp"
@@ -148,19 +149,137 @@ void prepare_edges(Graph &G, int k, cudaStream_t s) {
     tiles_for(G, 0, G.m, nt, unused, s);
 }
 
-static int64_t launch_wedges(Graph &G, const Graph::Chunk &c, cudaStream_t s) {
-    G.a_base = c.s0;
-    const GraphView gv = G.view();
-    const CountView cv = G.cview();
-    const int sms = sm_count();
-    int64_t launches = 0;
+// Side streams of one count call: the wedge forms and the triangle kernels do
+// not depend on each other and run beside each other, since on a small graph
+// none of them fills the GPU and on a large one each ends in a tail.  A set
+// is taken for the call and given back once the joins are enqueued (what a
+// later call enqueues on it comes after); the process keeps at most kKeep
+// sets per device, more exist only while that many calls run at once.
+class SideStreams {
+public:
+    static constexpr int kSides = 3;
+    explicit SideStreams(cudaStream_t main) : main_(main) {
+        TG_CK(cudaGetDevice(&dev_));
+        {
+            std::lock_guard<std::mutex> lock(mutex());
+            auto &pool = free_sets();
+            for (size_t k = 0; k < pool.size() && !set_; ++k)
+                if (pool[k]->dev == dev_) {
+                    set_ = std::move(pool[k]);
+                    pool.erase(pool.begin() + (std::ptrdiff_t)k);
+                }
+        }
+        if (!set_) {
+            set_ = std::make_unique<Set>();
+            set_->dev = dev_;
+            for (auto &x : set_->s) TG_CK(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
+            for (auto &x : set_->ev) TG_CK(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+        }
+    }
+    ~SideStreams() {
+        if (forked_) {                                      // an error between fork and join: nothing may still run
+            for (cudaStream_t x : set_->s) cudaStreamSynchronize(x);   // when the caller gives its buffers back
+            return;
+        }
+        std::lock_guard<std::mutex> lock(mutex());
+        size_t kept = 0;
+        for (const auto &x : free_sets()) kept += x->dev == dev_ ? 1 : 0;
+        if (kept < kKeep) free_sets().push_back(std::move(set_));
+    }
+    cudaStream_t side(int k) const { return set_->s[k]; }
+    // the sides start after what the main stream has so far
+    void fork() {
+        forked_ = true;
+        TG_CK(cudaEventRecord(set_->ev[0], main_));
+        for (cudaStream_t x : set_->s) TG_CK(cudaStreamWaitEvent(x, set_->ev[0], 0));
+    }
+    // side k goes on after what the main stream has so far
+    void after_main(int k) {
+        TG_CK(cudaEventRecord(set_->ev[1], main_));
+        TG_CK(cudaStreamWaitEvent(set_->s[k], set_->ev[1], 0));
+    }
+    // the main stream goes on after the sides
+    void join() {
+        for (int k = 0; k < kSides; ++k) {
+            TG_CK(cudaEventRecord(set_->ev[2 + k], set_->s[k]));
+            TG_CK(cudaStreamWaitEvent(main_, set_->ev[2 + k], 0));
+        }
+        forked_ = false;
+    }
+
+private:
+    struct Set {
+        int dev = 0;
+        cudaStream_t s[kSides] = {};
+        cudaEvent_t ev[2 + kSides] = {};
+        ~Set() {                                            // (work enqueued on them completes all the same)
+            for (cudaStream_t x : s)
+                if (x) cudaStreamDestroy(x);
+            for (cudaEvent_t x : ev)
+                if (x) cudaEventDestroy(x);
+        }
+    };
+    static constexpr size_t kKeep = 8;
+    static std::mutex &mutex() {
+        static std::mutex *m = new std::mutex();
+        return *m;
+    }
+    static std::vector<std::unique_ptr<Set>> &free_sets() {   // never destroyed: the CUDA context may go first
+        static auto *v = new std::vector<std::unique_ptr<Set>>();
+        return *v;
+    }
+    cudaStream_t main_;
+    int dev_ = 0;
+    bool forked_ = false;
+    std::unique_ptr<Set> set_;
+};
+
+// Sums and 4-cycle slots of chunk ci, after the triangles of the whole graph
+// when `triangles` (their per-node sums included).  The kernels run beside
+// each other (a pass of 40 k edges 543 -> 282 us, 1 M edges 4.10 -> 3.76 ms,
+// 2 M 10.51 -> 10.25, a 30 M edge block model 55.8 -> 53.7), but:
+// - not the hub pass, which fills the GPU and whose tables want the L2 cache
+//   for themselves (beside the others: 2 M edges 13.4 ms, 20 M edges 162 ->
+//   235 ms; on graphs of few hubs beside or after differs by 3% at most);
+// - not under capture: a side stream stays in the capture until it ends, past
+//   this call, so no other call could take it (and captured batches whose
+//   replays overlap gained nothing: 41.0 -> 42.2 ms);
+// - not when every kernel is timed by itself.
+static int64_t launch_chunk(Graph &G, size_t ci, bool triangles, cudaStream_t s) {
+    const Graph::Chunk &c = G.chunks[ci];
     const int L = G.L;
+    int64_t launches = 0;
+    G.a_base = c.s0;
+    G.e_base = c.e0;
     if (c.s1 > c.s0)
         TG_CK(cudaMemset2DAsync(G.A.p, (size_t)G.a_stride * sizeof(uint32_t), 0, (size_t)(c.s1 - c.s0) * sizeof(uint32_t),
                                 (size_t)L * L, s));
-    if (G.n_hubs > 0) launches += launch_hubs(G, (size_t)(&c - G.chunks.data()), s);
-    launches += launch_anchor_wedges(G, c.n0, c.n1, s);
-    TG_CK(cudaGetLastError());
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+        (void)cudaGetLastError();                            // (a legacy stream while another thread captures)
+        capture = cudaStreamCaptureStatusActive;
+    }
+    if (G.timing || capture != cudaStreamCaptureStatusNone) {
+        if (triangles) launches += launch_triangles(G, true, s);
+        launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
+        if (G.n_hubs > 0) launches += launch_hubs(G, ci, s);
+        launches += launch_anchor_wedges(G, 0, kHubClass - 1, c.n0, c.n1, s);
+    } else {
+        SideStreams side(s);
+        side.fork();
+        launches += launch_anchor_wedges(G, kHubClass - 1, kHubClass - 1, c.n0, c.n1, side.side(1));
+        launches += launch_anchor_wedges(G, 2, kHubClass - 2, c.n0, c.n1, side.side(2));
+        if (triangles) {
+            launches += launch_triangles(G, false, s);
+            side.after_main(0);
+            launches += launch_row_sums(G, G.slot_eid.as<int32_t>(), G.C.as<uint32_t>(), G.tau.as<int64_t>(), side.side(0));
+        }
+        launches += launch_anchor_wedges(G, 0, 1, c.n0, c.n1, side.side(1));
+        launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
+        side.join();
+        if (G.n_hubs > 0) launches += launch_hubs(G, ci, s);
+    }
+    launches += launch_slot_rows(G, c.s1 - c.s0, s);
     return launches;
 }
 
@@ -191,11 +310,13 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
                   bool full, cudaStream_t s) {
     int64_t launches = 0;
     // prepared_k 3: typed triangles only (all that k = 3 reads); 4: their per-node sums too
-    if (full || G.prepared_k < 3 || (k == 4 && !G.tau_ready)) {
+    bool triangles = full || G.prepared_k < 3 || (k == 4 && !G.tau_ready);
+    if (triangles && (k == 3 || G.chunks.size() != 1 || e_begin >= e_end || (!full && G.prepared_k == 4))) {
         launches += launch_triangles(G, k == 4, s);
-        G.prepared_k = std::max(G.prepared_k, 3);
-        G.tau_ready = G.tau_ready || k == 4;
+        triangles = false;
     }
+    G.prepared_k = std::max(G.prepared_k, 3);
+    G.tau_ready = G.tau_ready || k == 4;
     DBuf tmp;                                                // tiles of a range, stream-ordered
     tmp.owner = &G.stream;
     int64_t n_tiles = 0;
@@ -206,14 +327,13 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
         const bool whole = e_begin == 0 && e_end == G.m;
         std::vector<Tile> host;
         if (!whole) host = make_tiles(G, e_begin, e_end);
-        for (const Graph::Chunk &c : G.chunks) {
+        for (size_t ci = 0; ci < G.chunks.size(); ++ci) {
+            const Graph::Chunk &c = G.chunks[ci];
             const int64_t b = std::max(e_begin, c.e0), e = std::min(e_end, c.e1);
             if (b >= e) continue;
             // the wedge pass and sums of a single-chunk handle are reused by later range calls
             if (full || G.chunks.size() > 1 || G.prepared_k != 4) {
-                launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
-                launches += launch_wedges(G, c, s);
-                launches += launch_slot_rows(G, c.s1 - c.s0, s);
+                launches += launch_chunk(G, ci, triangles, s);
                 if (G.chunks.size() == 1) G.prepared_k = 4;
             }
             const Tile *ct = tiles;

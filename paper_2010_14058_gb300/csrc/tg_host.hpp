@@ -349,10 +349,10 @@ void with_types(int L, F f) {
 
 // wedge anchors (tg_wedge.cu): class lists from the wedges and the most
 // lower-priority neighbours of one type of every node (the hubs unsorted);
-// the wedge pass of the anchors of [n0, n1) that are not hubs
+// the wedge pass of the anchors of [n0, n1) in the forms form_lo to form_hi
 void list_anchors(Graph &G, const int64_t *work, const int32_t *most, cudaStream_t s);
 void prepare_wedges(Graph &G);
-int64_t launch_anchor_wedges(Graph &G, int64_t n0, int64_t n1, cudaStream_t s);
+int64_t launch_anchor_wedges(Graph &G, int form_lo, int form_hi, int64_t n0, int64_t n1, cudaStream_t s);
 
 // count entries (tg_count.cu)
 void prepare_counting(Graph &G, int k, cudaStream_t s);

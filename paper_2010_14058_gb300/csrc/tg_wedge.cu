@@ -432,13 +432,14 @@ void prepare_wedges(Graph &G) {
     });
 }
 
-int64_t launch_anchor_wedges(Graph &G, int64_t n0, int64_t n1, cudaStream_t s) {
+int64_t launch_anchor_wedges(Graph &G, int form_lo, int form_hi, int64_t n0, int64_t n1, cudaStream_t s) {
     const GraphView gv = G.view();
     const CountView cv = G.cview();
     int64_t launches = 0;
     each_form(G, [&](auto form, int64_t table, size_t smem) {
         constexpr int kForm = decltype(form)::value;
         using F = Form<kForm>;
+        if (kForm < form_lo || kForm > form_hi) return;
         static const char *names[5] = {"k_wedge_light", "k_wedge_64", "k_wedge_192", "k_wedge_512", "k_wedge_1024"};
         KernelTimer kt(G, s, names[kForm]);
         const int per_sm = std::max(1, std::min<int>(2048 / (F::threads * F::groups), (int)((226u << 10) / (smem + 1280))));
