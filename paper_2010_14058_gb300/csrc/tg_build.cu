@@ -132,7 +132,7 @@ __global__ void k_gather_types(int64_t n, const int32_t *__restrict__ old_of, co
 // lower- and higher-priority neighbours
 __global__ void k_rows(int64_t n, int L, int nb, const int64_t *__restrict__ rp,
                        const unsigned long long *__restrict__ keys, int32_t *adj, int32_t *toff, uint32_t *tdeg,
-                       int32_t *pivot, int64_t *nplus, int32_t *most_lower, uint32_t *status) {
+                       int32_t *pivot, int64_t *nplus, int32_t *most_lower, int64_t *long_type, uint32_t *status) {
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp;
     int lane = threadIdx.x & (kWarp - 1);
     if (warp > n) return;
@@ -180,6 +180,7 @@ __global__ void k_rows(int64_t n, int L, int nb, const int64_t *__restrict__ rp,
         down = (int32_t)(lo - b) - sb;
     }
     if (lane < kCRow) tdeg[x * kCRow + lane] = (uint32_t)(se - sb);
+    if (se - sb >= kNarrowDegree) *long_type = 1;
     up = (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)up);
     down = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)down);
     if (lane == 0) {
@@ -438,6 +439,9 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
     G.pivot.alloc(sizeof(int32_t) * std::max<int64_t>(n * L, 1));
     G.plus_off.alloc(sizeof(int64_t) * (n + 1));
     G.ty.alloc(std::max<int64_t>(n, 1));
+    std::vector<int64_t> h_info(2 * (size_t)ngraphs + 4);    // see k_graph_info; last: a typed degree of kNarrowDegree or more
+    TBuf info(sizeof(int64_t) * h_info.size(), s);
+    TG_CK(cudaMemsetAsync(info.as<int64_t>() + 2 * ngraphs + 3, 0, sizeof(int64_t), s));
     TBuf nplus(sizeof(int64_t) * (n + 1), s), most(sizeof(int32_t) * std::max<int64_t>(n, 1), s);
     {
         TBuf keys(sizeof(unsigned long long) * std::max<int64_t>(nnz, 1), s), keys2(sizeof(unsigned long long) * std::max<int64_t>(nnz, 1), s);
@@ -456,7 +460,8 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
         ++G.last_launches;
         k_rows<<<blocks_for((n + 1) * kWarp, kThreads), kThreads, 0, s>>>(
             n, L, nb, G.rp.as<int64_t>(), keys2.as<unsigned long long>(), G.adj.as<int32_t>(), G.toff.as<int32_t>(),
-            G.tdeg.as<uint32_t>(), G.pivot.as<int32_t>(), nplus.as<int64_t>(), most.as<int32_t>(), status);
+            G.tdeg.as<uint32_t>(), G.pivot.as<int32_t>(), nplus.as<int64_t>(), most.as<int32_t>(),
+            info.as<int64_t>() + 2 * ngraphs + 3, status);
         TG_CK(cudaGetLastError());
     }
     // types by internal id
@@ -471,8 +476,6 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
     // slots, edges and largest degree per graph; graph g's edges are those whose smaller caller id lies in
     // graph g: with caller ids grouped by graph and lexicographic edge order they are contiguous, half of
     // its rows' entries
-    std::vector<int64_t> h_info(2 * (size_t)ngraphs + 3);
-    TBuf info(sizeof(int64_t) * h_info.size(), s);
     ++G.last_launches;
     k_graph_info<<<blocks_for(ngraphs + 1, kThreads), kThreads, 0, s>>>(
         G.view(), info.as<int64_t>(), info.as<int64_t>() + ngraphs + 1, info.as<int64_t>() + 2 * ngraphs + 1, status);
@@ -530,8 +533,9 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
     }
 
     // 5. per-node typed degree sums
-    G.delta.alloc(sizeof(int64_t) * std::max<int64_t>(n * L * L, 1));
-    G.last_launches += launch_row_sums(G, G.adj.as<int32_t>(), G.tdeg.as<uint32_t>(), G.delta.as<int64_t>(), s);
+    G.narrow = !h_info[2 * (size_t)ngraphs + 3] && nnz < kNarrowSlots && !G.wide_sums();
+    G.delta.alloc(G.node_sum_bytes() * std::max<int64_t>(n * L * L, 1));
+    G.last_launches += launch_row_sums(G, G.adj.as<int32_t>(), G.tdeg.as<uint32_t>(), G.delta.p, s);
 
     // 6. wedge anchors by class
     {

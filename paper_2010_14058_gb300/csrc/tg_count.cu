@@ -272,7 +272,7 @@ static int64_t launch_chunk(Graph &G, size_t ci, bool triangles, cudaStream_t s)
         if (triangles) {
             launches += launch_triangles(G, false, s);
             side.after_main(0);
-            launches += launch_row_sums(G, G.slot_eid.as<int32_t>(), G.C.as<uint32_t>(), G.tau.as<int64_t>(), side.side(0));
+            launches += launch_row_sums(G, G.slot_eid.as<int32_t>(), G.C.as<uint32_t>(), G.tau.p, side.side(0));
         }
         launches += launch_anchor_wedges(G, 0, 1, c.n0, c.n1, side.side(1));
         launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
@@ -289,7 +289,7 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
     const size_t m = (size_t)std::max<int64_t>(G.m, 1), n = (size_t)std::max<int64_t>(G.n, 1);
     if (G.C.bytes < m * kCRow * sizeof(uint32_t)) G.C.alloc(m * kCRow * sizeof(uint32_t));
     if (G.tri_any.bytes < n) G.tri_any.alloc(n);
-    if (G.tau.bytes < n * L * L * sizeof(int64_t)) G.tau.alloc(n * L * L * sizeof(int64_t));
+    if (G.tau.bytes < n * L * L * G.node_sum_bytes()) G.tau.alloc(n * L * L * G.node_sum_bytes());
     prepare_triangles(G);
     const size_t gbytes = (size_t)G.ngraphs * global_slots(L, 4) * sizeof(unsigned long long);
     if (G.gacc.bytes < gbytes) G.gacc.alloc(gbytes);

@@ -12,11 +12,15 @@
 // histogram in shared memory is touched once per group.
 // Measured on 20 M Chung-Lu edges (L = 5) and 30 M block-model edges (L = 4),
 // against a warp per edge with an atomic per value: 39.1 -> 26.8 and 50.3 ->
-// 29.7 ms, and with the slots' 4-cycle values read as rows (k_slot_rows, 1.5
-// and 1.2 ms) 11.7 and 9.8 ms; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
-// Bound now: latency of the gathers at 24 warps per SM (each edge reads two
+// 29.7 ms, with the slots' 4-cycle values read as rows (k_slot_rows, 1.5
+// and 1.2 ms) 11.7 and 9.8 ms, and with 32-bit values and node sums where
+// they fit (a narrow graph, kNarrowDegree; 64 registers instead of 80, so a
+// fourth CTA per SM, and half the bytes of the nodes' tables) 7.9
+// and 7.3 ms; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
+// Bound now: latency of the gathers at 32 warps per SM (each edge reads two
 // slot rows, its sums, and two nodes' tables) on top of the rows written
-// (12.8 GB, 1.9 ms at the measured copy rate).
+// (12.8 GB, 1.9 ms at the measured copy rate).  Narrow with 3 or 5 CTAs'
+// registers: 51.8 and 53.6 ms per pass of the block model against 51.3.
 #include <algorithm>
 
 #include "tg_host.hpp"
@@ -74,6 +78,7 @@ __device__ __forceinline__ void pair_types(int L, int pi, int &t, int &u) {
     u = t + (pi - pair_idx(L, t, t));
 }
 
+__device__ __forceinline__ uint32_t sat32(int32_t v, uint32_t *) { return (uint32_t)v; }   // (narrow: below 2^31)
 __device__ __forceinline__ uint32_t sat32(int64_t v, uint32_t *status) {
     if (v > 0xffffffffll) {
         set_status(status, ST_OVERFLOW);
@@ -132,37 +137,38 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_slot_rows(const uint32_t *__
 // ------------------------------------------------------------ one type pair
 // Every matrix entry of one edge at (t, u) [0] and (u, t) [1], i the first
 // endpoint (type p) and j the second (type q).
+template <class T>
 struct PairVals {
-    long long ct, cu, at, au, bt, bu;       // |T^t|, |S_i^t|, |S_j^t|
-    long long CTi[2], CTj[2], Q[2], Ri[2], Rj[2], G8[2], Wi, Wj, Ks;
+    T ct, cu, at, au, bt, bu;       // |T^t|, |S_i^t|, |S_j^t|
+    T CTi[2], CTj[2], Q[2], Ri[2], Rj[2], G8[2], Wi, Wj, Ks;
 };
 
-template <int L>
+template <int L, class T>
 __device__ __forceinline__ void pair_values(const GraphView &g, const CountView &cv, int64_t e, int32_t i, int32_t j,
-                                            int p, int q, bool swap, int t, int u, PairVals &v) {
+                                            int p, int q, bool swap, int t, int u, PairVals<T> &v) {
     // (e_lo, e_hi) = swap ? (j, i) : (i, j)
     constexpr int LL = L * L;
     const uint32_t *C = cv.C + e * kCRow;
-    v.ct = C[t];
-    v.cu = C[u];
+    v.ct = (T)C[t];
+    v.cu = (T)C[u];
     const int32_t *oi = g.toff + (int64_t)i * (L + 1), *oj = g.toff + (int64_t)j * (L + 1);
-    const long long dit = oi[t + 1] - oi[t], diu = oi[u + 1] - oi[u];
-    const long long djt = oj[t + 1] - oj[t], dju = oj[u + 1] - oj[u];
+    const T dit = oi[t + 1] - oi[t], diu = oi[u + 1] - oi[u];
+    const T djt = oj[t + 1] - oj[t], dju = oj[u + 1] - oj[u];
     v.at = dit - v.ct - (q == t ? 1 : 0);
     v.au = diu - v.cu - (q == u ? 1 : 0);
     v.bt = djt - v.ct - (p == t ? 1 : 0);
     v.bu = dju - v.cu - (p == u ? 1 : 0);
     // sums over T; rows of types without a triangle node are not kept
-    long long TC0[2] = {0, 0}, TC1[2] = {0, 0}, DT[2] = {0, 0}, K[2] = {0, 0};
+    T TC0[2] = {0, 0}, TC1[2] = {0, 0}, DT[2] = {0, 0}, K[2] = {0, 0};
     auto load = [&](auto x) {
         const auto *xs = x + (e - cv.e_base) * 4 * LL;
         if (v.ct) {
             const auto *r = xs + t * 4 * L + u;
-            TC0[0] = (long long)r[0]; TC1[0] = (long long)r[L]; DT[0] = (long long)r[2 * L]; K[0] = (long long)r[3 * L];
+            TC0[0] = (T)r[0]; TC1[0] = (T)r[L]; DT[0] = (T)r[2 * L]; K[0] = (T)r[3 * L];
         }
         if (v.cu) {
             const auto *r = xs + u * 4 * L + t;
-            TC0[1] = (long long)r[0]; TC1[1] = (long long)r[L]; DT[1] = (long long)r[2 * L]; K[1] = (long long)r[3 * L];
+            TC0[1] = (T)r[0]; TC1[1] = (T)r[L]; DT[1] = (T)r[2 * L]; K[1] = (T)r[3 * L];
         }
     };
     if (cv.wide) load(reinterpret_cast<const unsigned long long *>(cv.xsum));
@@ -171,11 +177,12 @@ __device__ __forceinline__ void pair_values(const GraphView &g, const CountView 
     const int k0 = t * L + u, k1 = u * L + t;
     // P[x][y]: slot i->j holds [type next to i][type next to j], slot j->i the reverse
     const uint32_t *Aij = cv.slot_rows + (swap ? s1 : s0) * LL, *Aji = cv.slot_rows + (swap ? s0 : s1) * LL;
-    const long long P0 = (long long)Aij[k1] + (long long)Aji[k0];
-    const long long P1 = (long long)Aij[k0] + (long long)Aji[k1];
-    const int64_t *tau_i = cv.tau + (int64_t)i * LL, *tau_j = cv.tau + (int64_t)j * LL;
-    const int64_t *del_i = g.delta + (int64_t)i * LL, *del_j = g.delta + (int64_t)j * LL;
-    const long long ti = tau_i[k0], tj = tau_j[k0];         // symmetric
+    const T P0 = (T)Aij[k1] + (T)Aji[k0];
+    const T P1 = (T)Aij[k0] + (T)Aji[k1];
+    const T *tau = static_cast<const T *>(cv.tau), *delta = static_cast<const T *>(g.delta);
+    const T *tau_i = tau + (int64_t)i * LL, *tau_j = tau + (int64_t)j * LL;
+    const T *del_i = delta + (int64_t)i * LL, *del_j = delta + (int64_t)j * LL;
+    const T ti = tau_i[k0], tj = tau_j[k0];         // symmetric
     v.Ks = (K[0] + K[1]) >> 1;                              // ordered adjacent pairs of T (K' counts each twice)
     v.CTi[0] = (swap ? TC1[0] : TC0[0]) - v.Ks - (u == q ? v.ct : 0);
     v.CTi[1] = (swap ? TC1[1] : TC0[1]) - v.Ks - (t == q ? v.cu : 0);
@@ -202,8 +209,8 @@ size_t epi4_smem_bytes(int L) {
            (size_t)(L * L + L * L * L + L * L * P + 1) * sizeof(uint16_t);
 }
 
-template <int L>
-__global__ void __launch_bounds__(kEpiThreads, 3) k_epi4(GraphView g, CountView cv, const Tile *__restrict__ tiles,
+template <int L, class T>
+__global__ void __launch_bounds__(kEpiThreads, sizeof(T) == 4 ? 4 : 3) k_epi4(GraphView g, CountView cv, const Tile *__restrict__ tiles,
                                                          int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
                                                          unsigned long long *gacc) {
     constexpr int LL = L * L, P = L * (L + 1) / 2, S = 2 * L + 10 * P;
@@ -272,9 +279,9 @@ __global__ void __launch_bounds__(kEpiThreads, 3) k_epi4(GraphView g, CountView 
                 if (key >= 0) flush();
                 key = k;
             }
-            PairVals v;
-            pair_values<L>(g, cv, e, g.e_lo[e], g.e_hi[e], k / L, k % L, false, t, u, v);
-            long long gv[10];
+            PairVals<T> v;
+            pair_values<L, T>(g, cv, e, g.e_lo[e], g.e_hi[e], k / L, k % L, false, t, u, v);
+            T gv[10];
             bool ok = v.at >= 0 && v.au >= 0 && v.bt >= 0 && v.bu >= 0;
             if (t != u) {
                 gv[0] = v.Ri[0] + v.Rj[0] + v.Ri[1] + v.Rj[1];         // g3
@@ -288,7 +295,7 @@ __global__ void __launch_bounds__(kEpiThreads, 3) k_epi4(GraphView g, CountView 
                 gv[6] = v.ct * (v.au + v.bu) + v.cu * (v.at + v.bt) - gv[7];   // Lemma 3
                 gv[8] = v.ct * v.cu - gv[9];                           // Lemma 4
             } else {
-                const long long w = v.Wi + v.Wj;
+                const T w = v.Wi + v.Wj;
                 ok = ok && !(w & 1) && !(v.Ks & 1);
                 gv[0] = v.Ri[0] + v.Rj[0];
                 gv[3] = v.Q[0];
@@ -315,11 +322,11 @@ __global__ void __launch_bounds__(kEpiThreads, 3) k_epi4(GraphView g, CountView 
 #pragma unroll
                 for (int b = 0; b < 10; ++b) row[2 * L + b * P + pi] = sat32(gv[b], cv.status);
             }
-            acc[0] += (unsigned long long)(gv[0] + gv[1]);             // 4-path: g3, g4
+            acc[0] += (unsigned long long)gv[0] + (unsigned long long)gv[1];             // 4-path: g3, g4
             acc[1] += (unsigned long long)gv[2];                       // 4-star: g5
             acc[2] += (unsigned long long)gv[3];                       // 4-cycle: g6
-            acc[3] += (unsigned long long)(gv[4] + gv[5] + gv[6]);     // tailed triangle: g7, g8, g9
-            acc[4] += (unsigned long long)(gv[7] + gv[8]);             // chordal cycle: g10, g11
+            acc[3] += (unsigned long long)gv[4] + (unsigned long long)gv[5] + (unsigned long long)gv[6];     // tailed triangle: g7, g8, g9
+            acc[4] += (unsigned long long)gv[7] + (unsigned long long)gv[8];             // chordal cycle: g10, g11
             acc[5] += (unsigned long long)gv[9];                       // 4-clique: g12
         }
         if (key >= 0) flush();
@@ -410,7 +417,7 @@ struct PaView {
     int32_t off[13];          // first slot of blocks O1..O12
 };
 
-template <int L>
+template <int L, class T>
 __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView cv, PaView pv,
                                                          const Tile *__restrict__ tiles, int64_t n_tiles,
                                                          int64_t row_base, uint32_t *per_edge_out,
@@ -479,11 +486,11 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
             int32_t i = g.e_lo[e], j = g.e_hi[e];
             const bool swap = pv.old_of[i] > pv.old_of[j];
             if (swap) { const int32_t y = i; i = j; j = y; }
-            PairVals v;
-            pair_values<L>(g, cv, e, i, j, k / L, k % L, swap, t, u, v);
+            PairVals<T> v;
+            pair_values<L, T>(g, cv, e, i, j, k / L, k % L, swap, t, u, v);
             uint32_t *row = per_edge_out ? per_edge_out + (e - row_base) * S : nullptr;
             bool ok = v.at >= 0 && v.au >= 0 && v.bt >= 0 && v.bu >= 0;
-            auto emit = [&](int slot, long long val, unsigned long long &a) {
+            auto emit = [&](int slot, T val, unsigned long long &a) {
                 ok = ok && val >= 0;
                 if (row) row[slot] = sat32(val, cv.status);
                 a += (unsigned long long)val;
@@ -497,10 +504,10 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
             for (int h = 0; h < 2; ++h) {                             // ordered blocks at (x, y) = (t, u), (u, t)
                 if (h == 1 && t == u) break;
                 const int xy = h == 0 ? ktu : u * L + t;
-                const long long cx = h == 0 ? v.ct : v.cu;
-                const long long ax = h == 0 ? v.at : v.au, ay = h == 0 ? v.au : v.at;
-                const long long by = h == 0 ? v.bu : v.bt;
-                const long long QT = v.Q[1 - h];
+                const T cx = h == 0 ? v.ct : v.cu;
+                const T ax = h == 0 ? v.at : v.au, ay = h == 0 ? v.au : v.at;
+                const T by = h == 0 ? v.bu : v.bt;
+                const T QT = v.Q[1 - h];
                 emit(so[0] + xy, v.Ri[h], acc_o[h][0]);               // inner endpoint lo: near x, far y
                 emit(so[1] + xy, v.Rj[h], acc_o[h][1]);
                 emit(so[2] + xy, ax * by - QT, acc_o[h][2]);          // lo's neighbour x, hi's y (Lemma 1)
@@ -511,7 +518,7 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
                 emit(so[7] + xy, v.CTi[h], acc_o[h][7]);              // chordal outer edge, degree-3 node lo
                 emit(so[8] + xy, v.CTj[h], acc_o[h][8]);
             }
-            long long star_i, star_j, tail_i, tail_j, chord, clique;
+            T star_i, star_j, tail_i, tail_j, chord, clique;
             if (t != u) {
                 star_i = v.at * v.au - v.Wi;                          // Lemma 2, centre lo
                 star_j = v.bt * v.bu - v.Wj;
@@ -568,19 +575,23 @@ PaView pa_view(const Graph &G) {
     return v;
 }
 
-unsigned epi_grid(const Graph &G, int64_t n_tiles) {
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_tiles, (int64_t)sm_count() * G.opt.ctas_per_sm));
+unsigned epi_grid(int64_t n_tiles, int per_sm) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_tiles, (int64_t)sm_count() * per_sm));
 }
 
 }  // namespace
 
 void prepare_epi(Graph &G) {
-    with_types(G.L, [&](auto l) { raise_smem_limit((const void *)k_epi4<decltype(l)::value>, epi4_smem_bytes(G.L)); });
+    with_types(G.L, [&](auto l) { 
+        raise_smem_limit((const void *)k_epi4<decltype(l)::value, int32_t>, epi4_smem_bytes(G.L));
+        raise_smem_limit((const void *)k_epi4<decltype(l)::value, int64_t>, epi4_smem_bytes(G.L));
+    });
 }
 
 void prepare_epi4_pa(Graph &G) {
     with_types(G.L, [&](auto l) {
-        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value>, (size_t)G.pa.G * sizeof(unsigned long long));
+        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value, int32_t>, (size_t)G.pa.G * sizeof(unsigned long long));
+        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value, int64_t>, (size_t)G.pa.G * sizeof(unsigned long long));
     });
 }
 
@@ -617,12 +628,17 @@ int64_t launch_edges4(Graph &G, const Tile *tiles, int64_t n_tiles, int64_t row_
     KernelTimer kt(G, s, G.pa_active ? "k_epi4_pa" : "k_epi4");
     with_types(G.L, [&](auto l) {
         constexpr int L = decltype(l)::value;
-        if (G.pa_active)
-            k_epi4_pa<L><<<epi_grid(G, n_tiles), kEpiThreads, (size_t)G.pa.G * sizeof(unsigned long long), s>>>(
-                G.view(), G.cview(), pa_view(G), tiles, n_tiles, row_base, per_edge_out, gacc);
-        else
-            k_epi4<L><<<epi_grid(G, n_tiles), kEpiThreads, epi4_smem_bytes(L), s>>>(G.view(), G.cview(), tiles, n_tiles,
-                                                                                    row_base, per_edge_out, gacc);
+        auto launch = [&](auto v) {
+            using T = decltype(v);
+            if (G.pa_active)
+                k_epi4_pa<L, T><<<epi_grid(n_tiles, G.opt.ctas_per_sm), kEpiThreads, (size_t)G.pa.G * sizeof(unsigned long long), s>>>(
+                    G.view(), G.cview(), pa_view(G), tiles, n_tiles, row_base, per_edge_out, gacc);
+            else
+                k_epi4<L, T><<<epi_grid(n_tiles, G.opt.ctas_per_sm + (G.narrow ? 1 : 0)), kEpiThreads, epi4_smem_bytes(L), s>>>(
+                    G.view(), G.cview(), tiles, n_tiles, row_base, per_edge_out, gacc);
+        };
+        if (G.narrow) launch(int32_t());
+        else launch(int64_t());
     });
     TG_CK(cudaGetLastError());
     return 1;

@@ -121,6 +121,7 @@ struct Graph {
     int64_t n = 0, nnz = 0, m = 0;
     int64_t max_graph_nodes = 0;
     int64_t max_degree = 0;
+    bool narrow = false;                                     // kNarrowDegree (tg_internal.cuh)
     std::vector<int64_t> h_node_off, h_edge_off, h_slot_off;
     // chunks of whole graphs counted one after another (bounds the 4-cycle array)
     struct Chunk { int32_t g0, g1; int64_t n0, n1, s0, s1, e0, e1, t0, t1; };
@@ -194,6 +195,7 @@ struct Graph {
 
     // sums over triangle nodes may reach 2^32 only when a degree reaches 2^16
     bool wide_sums() const { return max_degree >= (1 << 16); }
+    size_t node_sum_bytes() const { return narrow ? sizeof(uint32_t) : sizeof(int64_t); }   // of a delta or tau value
     GraphView view() const {
         GraphView v;
         v.ngraphs = ngraphs; v.L = L; v.n = n; v.nnz = nnz; v.m = m;
@@ -210,7 +212,8 @@ struct Graph {
         v.e_hi = e_hi.as<int32_t>();
         v.e_slot_lo = e_slot_lo.as<int64_t>();
         v.e_slot_hi = e_slot_hi.as<int64_t>();
-        v.delta = delta.as<int64_t>();
+        v.delta = delta.p;
+        v.narrow = narrow;
         v.plus_off = plus_off.as<int64_t>();
         v.plus_adj = plus_adj.as<int32_t>();
         v.plus_eid = plus_eid.as<int32_t>();
@@ -219,7 +222,7 @@ struct Graph {
     CountView cview() const {
         CountView c;
         c.C = C.as<uint32_t>();
-        c.tau = tau.as<int64_t>();
+        c.tau = tau.p;
         c.A = A.as<uint32_t>();
         c.slot_rows = slot_rows.as<uint32_t>();
         c.a_base = a_base;
@@ -315,7 +318,7 @@ struct LocalClass {
 LocalClass local_class(const Graph &G, int cls);
 
 // out[x][t][q] = sums of rows[index[s]][q] over x's slots s of type t
-int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, int64_t *out, cudaStream_t s);
+int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, void *out, cudaStream_t s);
 // shared-memory limits and scratch of launch_triangles (before any capture)
 void prepare_triangles(Graph &G);
 // typed triangles per edge and, with_tau, the per-node sums of the whole

@@ -59,6 +59,18 @@ struct HubSegment {
 };
 constexpr int64_t kHubTicketWords = 1 << 16;
 
+// A graph is narrow when no typed degree reaches kNarrowDegree, it has fewer
+// than kNarrowSlots adjacency entries and its sums over T are 32 bits wide:
+// every value of a 4-node row is then below 2^31.  Products: the largest,
+// c_t (a_u + b_u) + c_u (a_t + b_t) with c + a <= d_i and c + b <= d_j, and
+// a_t b_u + a_u b_t, are at most 2 (2^15 - 1)^2.  Sums: g3, the largest, is at
+// most delta_i[t][u] + delta_i[u][t] + the same of j; delta_x[t][u] and
+// delta_x[u][t] are sums of degrees over different neighbours, or of
+// different types' degrees, so their sum is at most the number of adjacency
+// entries, and twice that is below 2^30.
+constexpr int kNarrowDegree = 1 << 15;
+constexpr int64_t kNarrowSlots = (int64_t)1 << 29;
+
 // Edges of one graph that a CTA of the per-edge kernels takes at a time.
 struct Tile {
     int64_t begin, end;
@@ -84,7 +96,8 @@ struct GraphView {
     const int32_t *e_hi;       // [m] internal endpoint with the larger id
     const int64_t *e_slot_lo;  // [m] slot of e_hi inside row e_lo
     const int64_t *e_slot_hi;  // [m] slot of e_lo inside row e_hi
-    const int64_t *delta;      // [n*L*L] sum_{w in Gamma_x^t} d_w^t'
+    const void *delta;         // [n*L*L] sum_{w in Gamma_x^t} d_w^t': int64, or uint32 when narrow
+    bool narrow;               // delta and tau hold uint32 (kNarrowDegree)
     const int64_t *plus_off;   // [n+1] start of x's higher-priority neighbours in plus_adj
     const int32_t *plus_adj;   // [m] higher-priority neighbours of each node, (type << 29 | id),
                                // grouped by type in (type, id) order
@@ -94,7 +107,7 @@ struct GraphView {
 // Per-count working arrays.
 struct CountView {
     uint32_t *C;                // [m][kCRow] typed triangle counts c_e^t (t < L)
-    int64_t *tau;               // [n*L*L] ordered typed edges inside Gamma_x
+    void *tau;                  // [n*L*L] ordered typed edges inside Gamma_x: int64, or uint32 when narrow
     uint32_t *A;                // [L*L][a_stride] 4-cycle contributions per slot of the current chunk
     const uint32_t *slot_rows;  // [slots][L*L] the same by slot (k_slot_rows), read by the epilogue
     int64_t a_base;             // first adjacency slot of the current chunk

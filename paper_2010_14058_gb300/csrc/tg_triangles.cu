@@ -127,8 +127,9 @@ __device__ __forceinline__ unsigned long long seg_row_sum(const int32_t *__restr
     return acc;
 }
 
+template <class Out>
 __global__ void __launch_bounds__(256) k_row_sums(GraphView g, const int32_t *__restrict__ index,
-                                                  const uint32_t *__restrict__ rows, int64_t *out) {
+                                                  const uint32_t *__restrict__ rows, Out *out) {
     const int L = g.L;
     const int lane = threadIdx.x & 31, q = lane & 7, sub = lane >> 3;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -144,13 +145,14 @@ __global__ void __launch_bounds__(256) k_row_sums(GraphView g, const int32_t *__
                 acc += __shfl_xor_sync(0xffffffffu, acc, 8);
                 acc += __shfl_xor_sync(0xffffffffu, acc, 16);
             }
-            if (lane < L) out[(x * L + t) * L + lane] = (int64_t)acc;
+            if (lane < L) out[(x * L + t) * L + lane] = (Out)acc;
         }
     }
 }
 
+template <class Out>
 __global__ void __launch_bounds__(256) k_row_sums_long(GraphView g, const int32_t *__restrict__ index,
-                                                       const uint32_t *__restrict__ rows, int64_t *out) {
+                                                       const uint32_t *__restrict__ rows, Out *out) {
     __shared__ unsigned long long part[8][kMaxL];
     __shared__ int64_t found[256];
     __shared__ int n_found;
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(256) k_row_sums_long(GraphView g, const int32_
                 if (threadIdx.x < L) {
                     unsigned long long sum = 0;
                     for (int w = 0; w < 8; ++w) sum += part[w][threadIdx.x];
-                    out[(x * L + t) * L + threadIdx.x] = (int64_t)sum;
+                    out[(x * L + t) * L + threadIdx.x] = (Out)sum;
                 }
                 __syncthreads();
             }
@@ -188,15 +190,17 @@ __global__ void __launch_bounds__(256) k_row_sums_long(GraphView g, const int32_
 
 }  // namespace
 
-int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, int64_t *out, cudaStream_t s) {
+int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, void *out, cudaStream_t s) {
     if (G.n == 0) return 0;
     const int sms = sm_count();
-    k_row_sums<<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sms * 64), 256, 0, s>>>(G.view(), index, rows, out);
-    int64_t launches = 1;
-    if (G.max_degree > kLongRow) {
-        k_row_sums_long<<<(unsigned)std::min<int64_t>(G.n, (int64_t)sms * 8), 256, 0, s>>>(G.view(), index, rows, out);
-        ++launches;
-    }
+    auto launch = [&](auto *o) {
+        using Out = std::remove_pointer_t<decltype(o)>;
+        k_row_sums<Out><<<(unsigned)std::min<int64_t>((G.n + 7) / 8, (int64_t)sms * 64), 256, 0, s>>>(G.view(), index, rows, o);
+        if (G.max_degree <= kLongRow) return 1;
+        k_row_sums_long<Out><<<(unsigned)std::min<int64_t>(G.n, (int64_t)sms * 8), 256, 0, s>>>(G.view(), index, rows, o);
+        return 2;
+    };
+    const int64_t launches = G.narrow ? launch(static_cast<uint32_t *>(out)) : launch(static_cast<int64_t *>(out));
     TG_CK(cudaGetLastError());
     return launches;
 }
