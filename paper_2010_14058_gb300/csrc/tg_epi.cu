@@ -16,11 +16,12 @@
 // and 1.2 ms) 11.7 and 9.8 ms, and with 32-bit values and node sums where
 // they fit (a narrow graph, kNarrowDegree; 64 registers instead of 80, so a
 // fourth CTA per SM, and half the bytes of the nodes' tables) 7.9
-// and 7.3 ms; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
+// and 7.3 ms, with the tile's edges staged (stage_ends) 6.6 and 6.2; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
 // Bound now: latency of the gathers at 32 warps per SM (each edge reads two
 // slot rows, its sums, and two nodes' tables) on top of the rows written
 // (12.8 GB, 1.9 ms at the measured copy rate).  Narrow with 3 or 5 CTAs'
-// registers: 51.8 and 53.6 ms per pass of the block model against 51.3.
+// registers: 51.8 and 53.6 ms per pass of the block model against 51.3
+// (before the staging).
 #include <algorithm>
 
 #include "tg_host.hpp"
@@ -108,6 +109,25 @@ __device__ __forceinline__ void order_by_types(const GraphView &g, const Tile &t
     });
 }
 
+// By order: the endpoints of the tile's edges (by_caller's first if old_of, so
+// x > y says that they are swapped) and the edge's slots in rows e_lo and
+// e_hi, of the chunk; ends with a barrier.  Read once per edge here instead
+// of by each of its threads ahead of everything that they point to: k_epi4
+// 7.9 -> 7.1 (20 M Chung-Lu edges) and 7.3 -> 6.5 ms (30 M block model), and
+// with tiles of 1,024 edges instead of 2,048 6.6 and 6.2 (512: 6.6 and 6.3).
+template <int kKeys>
+__device__ __forceinline__ void stage_ends(const GraphView &g, const CountView &cv, const Tile &tile,
+                                           const TileOrder<kKeys> &o, uint4 *ends, const int32_t *__restrict__ old_of) {
+    for (int x = threadIdx.x; x < (int)(tile.end - tile.begin); x += blockDim.x) {
+        const int64_t e = tile.begin + o.order[x];
+        const int32_t i = g.e_lo[e], j = g.e_hi[e];
+        const bool swap = old_of && old_of[i] > old_of[j];
+        ends[x] = make_uint4((uint32_t)(swap ? j : i), (uint32_t)(swap ? i : j), (uint32_t)(g.e_slot_lo[e] - cv.a_base),
+                             (uint32_t)(g.e_slot_hi[e] - cv.a_base));
+    }
+    __syncthreads();
+}
+
 // ------------------------------------------------------------ slot rows
 // The wedge pass adds to one plane per type pair (consecutive slots of a plane
 // take its updates in whole sectors); an edge needs the L^2 values of two
@@ -145,8 +165,9 @@ struct PairVals {
 
 template <int L, class T>
 __device__ __forceinline__ void pair_values(const GraphView &g, const CountView &cv, int64_t e, int32_t i, int32_t j,
-                                            int p, int q, bool swap, int t, int u, PairVals<T> &v) {
-    // (e_lo, e_hi) = swap ? (j, i) : (i, j)
+                                            int p, int q, bool swap, int64_t s0, int64_t s1, int t, int u,
+                                            PairVals<T> &v) {
+    // (e_lo, e_hi) = swap ? (j, i) : (i, j); s0, s1: the edge's slots in rows e_lo and e_hi, of the chunk
     constexpr int LL = L * L;
     const uint32_t *C = cv.C + e * kCRow;
     v.ct = (T)C[t];
@@ -173,7 +194,6 @@ __device__ __forceinline__ void pair_values(const GraphView &g, const CountView 
     };
     if (cv.wide) load(reinterpret_cast<const unsigned long long *>(cv.xsum));
     else load(reinterpret_cast<const uint32_t *>(cv.xsum));
-    const int64_t s0 = g.e_slot_lo[e] - cv.a_base, s1 = g.e_slot_hi[e] - cv.a_base;
     const int k0 = t * L + u, k1 = u * L + t;
     // P[x][y]: slot i->j holds [type next to i][type next to j], slot j->i the reverse
     const uint32_t *Aij = cv.slot_rows + (swap ? s1 : s0) * LL, *Aji = cv.slot_rows + (swap ? s0 : s1) * LL;
@@ -201,21 +221,22 @@ __device__ __forceinline__ void pair_values(const GraphView &g, const CountView 
 }
 
 // ------------------------------------------------------------ typed rows
-// Shared memory of k_epi4: the histogram of G(L) u64, then the multiset rank
+// Shared memory of k_epi4: the tile's staged edges, the histogram of G(L) u64, then the multiset rank
 // tables rank2[p][q], rank3[p][q][t], rank4[p][q][pair] (uint16).
 size_t epi4_smem_bytes(int L) {
     const int P = L * (L + 1) / 2;
-    return (size_t)global_slots(L, 4) * sizeof(unsigned long long) +
+    return kTile * sizeof(uint4) + (size_t)global_slots(L, 4) * sizeof(unsigned long long) +
            (size_t)(L * L + L * L * L + L * L * P + 1) * sizeof(uint16_t);
 }
 
 template <int L, class T>
-__global__ void __launch_bounds__(kEpiThreads, sizeof(T) == 4 ? 4 : 3) k_epi4(GraphView g, CountView cv, const Tile *__restrict__ tiles,
-                                                         int64_t n_tiles, int64_t row_base, uint32_t *per_edge_out,
-                                                         unsigned long long *gacc) {
+__global__ void __launch_bounds__(kEpiThreads, sizeof(T) == 4 ? 4 : 3)
+    k_epi4(GraphView g, CountView cv, const Tile *__restrict__ tiles, int64_t n_tiles, int64_t row_base,
+           uint32_t *per_edge_out, unsigned long long *gacc) {
     constexpr int LL = L * L, P = L * (L + 1) / 2, S = 2 * L + 10 * P;
     constexpr int E = kEpiThreads / P;                      // edges in flight per CTA
-    extern __shared__ unsigned long long hist[];
+    extern __shared__ __align__(16) uint4 ends[];           // by order: nodes and slots of the tile's edges
+    unsigned long long *hist = reinterpret_cast<unsigned long long *>(ends + kTile);
     __shared__ TileOrder<LL> o;
     const int G = (int)global_slots(L, 4);
     uint16_t *rank2 = reinterpret_cast<uint16_t *>(hist + G);
@@ -246,6 +267,7 @@ __global__ void __launch_bounds__(kEpiThreads, sizeof(T) == 4 ? 4 : 3) k_epi4(Gr
     for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
         const Tile tile = tiles[ti];
         order_by_types<L>(g, tile, o, false, nullptr);
+        stage_ends(g, cv, tile, o, ends, nullptr);
         if (tile.graph != cur_graph) {
             if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph);
             __syncthreads();
@@ -280,7 +302,8 @@ __global__ void __launch_bounds__(kEpiThreads, sizeof(T) == 4 ? 4 : 3) k_epi4(Gr
                 key = k;
             }
             PairVals<T> v;
-            pair_values<L, T>(g, cv, e, g.e_lo[e], g.e_hi[e], k / L, k % L, false, t, u, v);
+            const uint4 at = ends[x];
+            pair_values<L, T>(g, cv, e, (int32_t)at.x, (int32_t)at.y, k / L, k % L, false, at.z, at.w, t, u, v);
             T gv[10];
             bool ok = v.at >= 0 && v.au >= 0 && v.bt >= 0 && v.bu >= 0;
             if (t != u) {
@@ -424,7 +447,8 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
                                                          unsigned long long *gacc) {
     constexpr int LL = L * L, P = L * (L + 1) / 2, E = kEpiThreads / P;
     constexpr int kOrdered = 9, kPairs = 6;
-    extern __shared__ unsigned long long hist[];
+    extern __shared__ __align__(16) uint4 ends[];
+    unsigned long long *hist = reinterpret_cast<unsigned long long *>(ends + kTile);
     __shared__ TileOrder<LL> o;
     const int S = pv.S, G = pv.G;
     for (int s = threadIdx.x; s < G; s += blockDim.x) hist[s] = 0;
@@ -440,6 +464,7 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
     for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
         const Tile tile = tiles[ti];
         order_by_types<L>(g, tile, o, true, pv.old_of);
+        stage_ends(g, cv, tile, o, ends, pv.old_of);
         if (tile.graph != cur_graph) {
             if (cur_graph >= 0) flush_hist(hist, G, gacc, cur_graph);
             __syncthreads();
@@ -483,11 +508,9 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi4_pa(GraphView g, CountView 
                 if (key >= 0) flush();
                 key = k;
             }
-            int32_t i = g.e_lo[e], j = g.e_hi[e];
-            const bool swap = pv.old_of[i] > pv.old_of[j];
-            if (swap) { const int32_t y = i; i = j; j = y; }
+            const uint4 at = ends[x];
             PairVals<T> v;
-            pair_values<L, T>(g, cv, e, i, j, k / L, k % L, swap, t, u, v);
+            pair_values<L, T>(g, cv, e, (int32_t)at.x, (int32_t)at.y, k / L, k % L, at.x > at.y, at.z, at.w, t, u, v);
             uint32_t *row = per_edge_out ? per_edge_out + (e - row_base) * S : nullptr;
             bool ok = v.at >= 0 && v.au >= 0 && v.bt >= 0 && v.bu >= 0;
             auto emit = [&](int slot, T val, unsigned long long &a) {
@@ -575,6 +598,8 @@ PaView pa_view(const Graph &G) {
     return v;
 }
 
+size_t pa_smem_bytes(const Graph &G) { return kTile * sizeof(uint4) + (size_t)G.pa.G * sizeof(unsigned long long); }
+
 unsigned epi_grid(int64_t n_tiles, int per_sm) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_tiles, (int64_t)sm_count() * per_sm));
 }
@@ -590,8 +615,8 @@ void prepare_epi(Graph &G) {
 
 void prepare_epi4_pa(Graph &G) {
     with_types(G.L, [&](auto l) {
-        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value, int32_t>, (size_t)G.pa.G * sizeof(unsigned long long));
-        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value, int64_t>, (size_t)G.pa.G * sizeof(unsigned long long));
+        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value, int32_t>, pa_smem_bytes(G));
+        raise_smem_limit((const void *)k_epi4_pa<decltype(l)::value, int64_t>, pa_smem_bytes(G));
     });
 }
 
@@ -631,7 +656,7 @@ int64_t launch_edges4(Graph &G, const Tile *tiles, int64_t n_tiles, int64_t row_
         auto launch = [&](auto v) {
             using T = decltype(v);
             if (G.pa_active)
-                k_epi4_pa<L, T><<<epi_grid(n_tiles, G.opt.ctas_per_sm), kEpiThreads, (size_t)G.pa.G * sizeof(unsigned long long), s>>>(
+                k_epi4_pa<L, T><<<epi_grid(n_tiles, G.opt.ctas_per_sm), kEpiThreads, pa_smem_bytes(G), s>>>(
                     G.view(), G.cview(), pa_view(G), tiles, n_tiles, row_base, per_edge_out, gacc);
             else
                 k_epi4<L, T><<<epi_grid(n_tiles, G.opt.ctas_per_sm + (G.narrow ? 1 : 0)), kEpiThreads, epi4_smem_bytes(L), s>>>(

@@ -76,7 +76,7 @@ struct Tile {
     int64_t begin, end;
     int32_t graph, pad;
 };
-constexpr int kTile = 2048;                 // most edges per tile
+constexpr int kTile = 1024;                 // most edges per tile
 
 // Read-only view of a built graph, passed to kernels by value.
 struct GraphView {
