@@ -289,11 +289,12 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
     const size_t m = (size_t)std::max<int64_t>(G.m, 1), n = (size_t)std::max<int64_t>(G.n, 1);
     if (G.C.bytes < m * kCRow * sizeof(uint32_t)) G.C.alloc(m * kCRow * sizeof(uint32_t));
     if (G.tri_any.bytes < n) G.tri_any.alloc(n);
-    if (G.tau.bytes < n * L * L * G.node_sum_bytes()) G.tau.alloc(n * L * L * G.node_sum_bytes());
     prepare_triangles(G);
     const size_t gbytes = (size_t)G.ngraphs * global_slots(L, 4) * sizeof(unsigned long long);
     if (G.gacc.bytes < gbytes) G.gacc.alloc(gbytes);
     if (k == 4) {
+        if (!G.anchors_ready) prepare_anchors(G, s);
+        if (G.tau.bytes < n * L * L * G.node_sum_bytes()) G.tau.alloc(n * L * L * G.node_sum_bytes());
         if (G.chunks.empty()) plan_chunks(G);
         const size_t ab = (size_t)G.a_stride * L * L * sizeof(uint32_t);
         if (G.A.bytes < ab) G.A.alloc(ab);

@@ -131,6 +131,7 @@ struct Graph {
 
     // graph (built once)
     DBuf node_off, edge_off, rp, adj, toff, tdeg, pivot, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
+    DBuf most_lower;                            // most lower-priority neighbours of one type, until prepare_anchors
     DBuf plus_off, plus_adj, plus_eid;
     // nodes by |N+| (tg_local.cuh): mid, big, and larger than shared memory holds
     DBuf tri_list[3], local_scratch;
@@ -141,6 +142,7 @@ struct Graph {
     // hub anchors in (graph, type, id) order and the pieces of their wedges (tg_hub.cu)
     DBuf hubs, hub_base, hub_nlow, hub_piece;
     int64_t n_hubs = 0;
+    bool anchors_ready = false;                 // delta, anchors and hubs (prepare_anchors)
     std::vector<int32_t> h_hub_id;      // hub node ids
     std::vector<int64_t> h_hub_wedges;  // wedges of each hub
     // persistent hub pass (tg_hub.cu): per chunk, its ticket queue; the
@@ -246,7 +248,7 @@ struct Graph {
     }
     std::vector<const DBuf *> cbuffers() const {
         return {&node_off, &edge_off, &rp, &adj, &toff, &tdeg, &pivot, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
-                             &e_slot_lo, &e_slot_hi, &delta, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
+                             &e_slot_lo, &e_slot_hi, &delta, &most_lower, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
                              &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dlab, &doutdeg, &dcls, &darcs, &dgacc, &dcell, &etype, &etdeg, &etgacc, &etcell, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
                 &pa_cls, &pa_gacc};
@@ -353,6 +355,7 @@ void with_types(int L, F f) {
 // wedge anchors (tg_wedge.cu): class lists from the wedges and the most
 // lower-priority neighbours of one type of every node (the hubs unsorted);
 // the wedge pass of the anchors of [n0, n1) in the forms form_lo to form_hi
+void prepare_anchors(Graph &G, cudaStream_t s);          // tg_build.cu, before any capture
 void list_anchors(Graph &G, const int64_t *work, const int32_t *most, cudaStream_t s);
 void prepare_wedges(Graph &G);
 int64_t launch_anchor_wedges(Graph &G, int form_lo, int form_hi, int64_t n0, int64_t n1, cudaStream_t s);

@@ -485,7 +485,6 @@ void list_anchors(Graph &G, const int64_t *work, const int32_t *most, cudaStream
     for (int c = 0; c < kHubClass; ++c) G.anchors[c].alloc(sizeof(int32_t) * std::max<int64_t>(n, 1));
     G.hubs.alloc(sizeof(int32_t) * std::max<int64_t>(n, 1));
     if (n > 0) {
-        ++G.last_launches;
         k_anchor_lists<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
             n, G.L, lim, work, most, G.anchors[0].as<int32_t>(), G.anchors[1].as<int32_t>(), G.anchors[2].as<int32_t>(),
             G.anchors[3].as<int32_t>(), G.anchors[4].as<int32_t>(), G.hubs.as<int32_t>(), counts.as<unsigned long long>(),
