@@ -152,11 +152,13 @@ struct EdgeTypedCells {
 
 constexpr int kRowThreads = 256;
 
-// zeroes the cells of every edge
-__global__ void k_et_zero(int64_t m, int64_t stride, int words, uint32_t *cell) {
-    const int64_t n = m * words;
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-        cell[x / words * stride + x % words] = 0u;
+// zeroes the cells of every edge, a warp per edge (a thread per cell spent its
+// time on the 64-bit division of its number)
+__global__ void __launch_bounds__(256) k_et_zero(int64_t m, int64_t stride, int words, uint32_t *cell) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; e < m; e += nw)
+        for (int x = lane; x < words; x += 32) cell[e * stride + x] = 0u;
 }
 
 // Thread per (edge, slot): the 3-path slot from the typed degrees and the
@@ -171,6 +173,7 @@ __global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, co
                                                                  unsigned long long *gacc, uint32_t *status) {
     extern __shared__ unsigned long long ehist[];
     __shared__ TileOrder<L * L * X> o;
+    __shared__ int2 ends[kTile];                            // by order: rows of etdeg of the edges' endpoints
     constexpr int P = X * (X + 1) / 2, S = L * X + L * P, E = kRowThreads / S;
     const int64_t off1 = mchoose(L, 2) * X, off2 = off1 + mchoose(L, 3) * mchoose(X, 2);
     const int64_t w2 = mchoose(X, 2), w3 = mchoose(X, 3);
@@ -208,6 +211,11 @@ __global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, co
     for (int64_t b = blockIdx.x * tile; b < g.m; b += gridDim.x * tile) {
         const int n = (int)min(tile, g.m - b);
         tile_order(b, n, o, [&](int64_t e) { return (g.ty[g.e_lo[e]] * L + g.ty[g.e_hi[e]]) * X + xi[e]; });
+        for (int x = threadIdx.x; x < n; x += blockDim.x) {
+            const int64_t e = b + o.order[x];
+            ends[x] = make_int2(g.e_lo[e], g.e_hi[e]);
+        }
+        __syncthreads();
         for (int k = threadIdx.x; k < L * L * X; k += blockDim.x)
             if (o.count[k]) {
                 int n2[2] = {k / X / L, k / X % L};
@@ -237,7 +245,7 @@ __global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, co
             int64_t v;
             if (path) {
                 const int pi = k / X / L, pj = k / X % L, xij = k % X;
-                v = (int64_t)etdeg[((int64_t)g.e_lo[e] * L + t) * X + x0] + etdeg[((int64_t)g.e_hi[e] * L + t) * X + x0] -
+                v = (int64_t)etdeg[((int64_t)ends[x].x * L + t) * X + x0] + etdeg[((int64_t)ends[x].y * L + t) * X + x0] -
                     ((pj == t && xij == x0) ? 1 : 0) - ((pi == t && xij == x0) ? 1 : 0);
 #pragma unroll
                 for (int z = 0; z < X; ++z) v -= (int64_t)c[x_at[z]] * (z == x0 ? 2 : 1);
@@ -330,7 +338,7 @@ int64_t run_edge_typed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, c
         }
         {
             KernelTimer kt(G, s, "k_edge_typed_cells");
-            k_et_zero<<<(unsigned)std::min<int64_t>((G.m * L * P + 255) / 256, (int64_t)sm_count() * 32), 256, 0, s>>>(
+            k_et_zero<<<(unsigned)std::min<int64_t>((G.m + 7) / 8, (int64_t)sm_count() * 64), 256, 0, s>>>(
                 G.m, stride, L * P, cell);
             launches += 1 + visit_triangles(G, EdgeTypedCells{cell, stride, G.etype.as<uint8_t>(), X, P}, s);
         }
