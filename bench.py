@@ -191,20 +191,7 @@ def load_peaks():
 # DRAM bytes (read + write) per launch of a kernel, from the ncu capture
 # summarised under profiles/ for that workload and the current kernel code
 # (an entry is removed when its kernel changes).
-TRAFFIC = {("cl_large", "k_wedge_hub"): 283.908528e9}
-
-# Issue-limited peak of the 4-clique lookups: 152 SMs x 4 schedulers x 32
-# lanes x the maximum SM clock give the lane-instruction rate; one lookup
-# (load the N+ entry, mask its id, distance to the largest member clamped
-# to the window, word index, one 32-bit shared-memory load, bit extract,
-# the typed hit count in three, the hash-range check in three) takes at
-# least LOOKUP_INSTR of them.
-LOOKUP_INSTR = 15
-
-
-def alu_peak_lookups(sm_mhz: float, sms: int = 152) -> float:
-    return sms * 4 * 32 * sm_mhz * 1e6 / LOOKUP_INSTR
-
+TRAFFIC = {}
 
 def w_alg_bytes(g: dict, tsize, S: int) -> dict:
     """The algorithmic traffic model W_alg = sum_e [4(d_i + d_j) +
@@ -282,7 +269,7 @@ def kernel_units(g: dict, light_anchor_max: int = 64, hub_min: int = 1 << 14) ->
 def clique_units(pe, L: int, big_t: int = 256, chunk: int = 1 << 22) -> dict:
     """|T_e| (sum of the triangle slots) and K_e (sum of the 4-clique orbit
     slots g12) of every edge, read from the per-edge rows, summed over the
-    edges counted by k_clique (|T| <= big_t) and by k_clique_big."""
+    edges of at most and of more than big_t triangles."""
     import torch
     P = L * (L + 1) // 2
     k0 = 2 * L + 9 * P
@@ -300,43 +287,38 @@ def clique_units(pe, L: int, big_t: int = 256, chunk: int = 1 << 22) -> dict:
     return out
 
 
-def algorithmic_bytes(u: dict, m: int, L: int, S: int, t_nodes: int, cu: dict | None = None) -> dict:
+def algorithmic_bytes(u: dict, m: int, L: int, S: int, t_nodes: int) -> dict:
     """Bytes each count kernel must move at least once in this formulation
     (reads of its inputs and writes of its outputs, intermediates included),
     per launch over the whole graph:
-      k_tri       per edge: endpoints 8, the shorter side of each typed
-                  intersection 4 B/entry, its typed triangle row 4L;
-      k_wedge_*   per wedge: the far node's id 4 + its 4-cycle slot 4 read +
+      k_tri       per edge: its entry of the N+ lists read 8 (id, edge id);
+                  its row of typed triangle counts zeroed and read or
+                  written 64; per triangle three counts read and written 24
+                  (the scan of the lists, which L2 serves, is not counted);
+      k_sum       per triangle three rows of triangle counts read 96, per
+                  triangle node of an edge its typed sums read and written
+                  24L; k_sum_zero clears 16L^2 per edge that has triangles;
+      k_wedge_light, k_wedge_64 to k_wedge_1024 (one line, k_wedge_shared):
+                  per wedge the far node's id 4 + its 4-cycle slot 4 read +
                   4 written; per (anchor, neighbour) pair: L slots 8 B each;
-                  k_wedge_hub, when the library's work counters give them:
-                  per hub wedge its far node's id 4, per nonzero 4-cycle
-                  slot update (a wedge and a type of the fourth node, or a
-                  (hub, neighbour, type) sum) the slot read and written 8;
-      k_tsum      per edge: endpoints 8, shorter sides as k_tri, C row 4L,
-                  the three L x L sums 24 L^2; per triangle node: its id
-                  written 4, two edge ids 8, two typed-triangle rows 8L,
-                  its type offsets 4(L+1);
-      k_clique, k_clique_big (edges with |T| up to / above max(light edge
-                  degree, 32)): per triangle node its id read 4, per adjacent
-                  pair inside T one adjacency entry read 4, per edge K written
-                  8L^2 (a lower bound: the misses of the N+ scans are not
-                  counted);
-      k_epi4      per edge: endpoints and slots 24, C row 4L, two type
-                  offset rows 8(L+1), tsum 24L^2, K 8L^2, the two 4-cycle
-                  slot columns 8L^2, tau and delta of both endpoints 32L^2,
-                  its output row 4S."""
+      k_wedge_hub when the library's work counters give them: per hub wedge
+                  its far node's id 4, per nonzero 4-cycle slot update (a
+                  wedge and a type of the fourth node, or a (hub, neighbour,
+                  type) sum) the slot read and written 8;
+      k_slot_rows per adjacency slot L^2 values read and written 8L^2;
+      k_epi4      per edge: endpoints and slots 24, C row 32, two type
+                  offset rows 8(L+1), two rows of 4-cycle values 8L^2, delta
+                  and tau of both endpoints 16L^2 (32-bit), its output row
+                  4S; per triangle node of an edge its sums 16L."""
     LL = L * L
     return {
-        "k_tri": 8.0 * m + 4.0 * u["typed_min_sum"] + 4.0 * L * m,
-        "k_wedge_light": 12.0 * u["wedges_light"] + 8.0 * L * u["pairs_light"],
-        "k_wedge_heavy": 12.0 * u["wedges_heavy"] + 8.0 * L * u["pairs_heavy"],
+        "k_tri": 72.0 * m + 8.0 * t_nodes,
+        "k_sum": (32.0 + 24.0 * L) * t_nodes,
+        "k_wedge_shared": 12.0 * (u["wedges_light"] + u["wedges_heavy"]) + 8.0 * L * (u["pairs_light"] + u["pairs_heavy"]),
         "k_wedge_hub": 4.0 * u["hub_wedges_counted"] + 8.0 * u["hub_slot_updates"] if "hub_slot_updates" in u else
         12.0 * u["wedges_hub"] + 8.0 * L * u["pairs_hub"],
-        "k_tsum": (8.0 + 4 * L + 24 * LL) * m + 4.0 * u["typed_min_sum"] + (12.0 + 12 * L + 4) * t_nodes,
-        "k_clique": 4.0 * t_nodes + 8.0 * LL * m if cu is None else
-        4.0 * (cu["t_small"] + cu["k_small"]) + 8.0 * LL * (m - cu["edges_big"]),
-        "k_clique_big": None if cu is None else 4.0 * (cu["t_big"] + cu["k_big"]) + 8.0 * LL * cu["edges_big"],
-        "k_epi4": (24.0 + 4 * L + 8 * (L + 1) + 72 * LL + 4 * S) * m,
+        "k_slot_rows": 16.0 * LL * m,
+        "k_epi4": (24.0 + 32 + 8 * (L + 1) + 24 * LL + 4 * S) * m + 16.0 * L * t_nodes,
     }
 
 
@@ -509,11 +491,11 @@ def run_ours(args):
 
 
     # roofline: algorithmic bytes of each count kernel per step over its
-    # CUDA-event time per step (k_clique and k_clique_big share one bound)
+    # CUDA-event time per step
     peak, peak_kind = load_peaks()
     roofline, per_kernel, compulsory, count_alone, walg, work = None, {}, None, None, None, None
     if rank == 0:
-        # the 4-clique lookups of one count, from the library's work counters
+        # the hub wedges and 4-clique words of one count, from the library's work counters
         # (one extra, untimed count)
         h = tg.tg_build(rp, col, ty, L, stream=stream)
         tg.tg_set_work_counting(h, True)
@@ -528,8 +510,13 @@ def run_ours(args):
         if work.get("hub_wedges"):
             units.update({"hub_wedges_counted": float(work["hub_wedges"]),
                           "hub_slot_updates": float(work["hub_slot_updates"])})
-        abytes = algorithmic_bytes(units, m, L, S, t_nodes, cu)
-        for name, (kms, nl) in kernel_ms.items():
+        abytes = algorithmic_bytes(units, m, L, S, t_nodes)
+        # the shared-memory wedge forms share one bound
+        forms = [v for k, v in kernel_ms.items() if k.startswith("k_wedge_") and k != "k_wedge_hub"]
+        timed = {k: v for k, v in kernel_ms.items() if v not in forms}
+        if forms:
+            timed["k_wedge_shared"] = (sum(v[0] for v in forms), sum(v[1] for v in forms))
+        for name, (kms, nl) in timed.items():
             if abytes.get(name) is None or kms <= 0:
                 continue
             step_ms = kms / args.steps
@@ -537,27 +524,8 @@ def run_ours(args):
             per_kernel[name] = {"ms_per_step": round(step_ms, 3), "launches_per_step": nl // args.steps,
                                 "algorithmic_gb": round(abytes[name] / 1e9, 3), "achieved_gbs": round(gbs, 2),
                                 "frac": round(gbs / peak, 5)}
-        top = max(kernel_ms.items(), key=lambda kv: kv[1][0])[0]
-        sm_mhz = float(clk.get("sm_mhz") or 2070.0)
-        lookups = {"k_clique": work["clique_probes"] + work["clique_searches"],
-                   "k_clique_big": work["clique_big_probes"]}
-        for name, ops in lookups.items():
-            if name in kernel_ms and kernel_ms[name][0] > 0:
-                ms_k = kernel_ms[name][0] / args.steps
-                per_kernel.setdefault(name, {})["lookups"] = ops
-                per_kernel[name]["glookups_per_s"] = round(ops / (ms_k / 1e3) / 1e9, 2)
-                per_kernel[name]["alu_frac"] = round(ops / (ms_k / 1e3) / alu_peak_lookups(sm_mhz), 5)
-        if top in lookups:
-            ms_k = kernel_ms[top][0] / args.steps
-            ach = lookups[top] / (ms_k / 1e3) / 1e9
-            pk_alu = alu_peak_lookups(sm_mhz) / 1e9
-            roofline = {"kernel": top, "bound": "alu", "achieved": round(ach, 2), "peak": round(pk_alu, 1),
-                        "peak_kind": f"derived: 152 SMs x 128 lanes x {sm_mhz:.0f} MHz (median SM clock under "
-                                     f"load) / {LOOKUP_INSTR} lane instructions per lookup",
-                        "unit": "Glookups/s", "frac": round(ach / pk_alu, 5), "algorithmic_ops": lookups[top],
-                        "ops": "set-of-T lookups of the 4-clique scan, sum over edges of sum_{w in T} |N+(w)|",
-                        "ms_per_step": round(ms_k, 3), "traffic": TRAFFIC.get((args.workload, top))}
-        elif top in per_kernel and "achieved_gbs" in per_kernel[top]:
+        top = max(timed.items(), key=lambda kv: kv[1][0])[0]
+        if top in per_kernel and "achieved_gbs" in per_kernel[top]:
             pk = per_kernel[top]
             roofline = {"kernel": top, "bound": "hbm", "achieved": pk["achieved_gbs"], "peak": peak,
                         "peak_kind": peak_kind, "unit": "GB/s", "frac": pk["frac"],
@@ -666,7 +634,7 @@ def run_ours(args):
         directed = {"value": round(m * args.steps / (dms / 1e3), 1), "unit": UNIT,
                     "ms_per_step": round(dms / args.steps, 3), "status": tg.STATUS[d_status],
                     "per_edge_slots": lay_d["per_edge_slots"], "global_slots": lay_d["global_slots"],
-                    "k_directed3_ms_per_step": round(d_ms.get("k_directed3", 0.0) / args.steps, 3),
+                    "kernels_ms_per_step": {k: round(v / args.steps, 3) for k, v in d_ms.items()},
                     "step": "tg_build_directed + tg_count_directed3 + tg_free, device-resident; each edge of the "
                             "workload oriented by a seeded coin"}
 
@@ -708,7 +676,7 @@ def run_ours(args):
         edge_typed = {"value": round(m * args.steps / (xms / 1e3), 1), "unit": UNIT,
                       "ms_per_step": round(xms / args.steps, 3), "status": tg.STATUS[x_status], "edge_types": X,
                       "per_edge_slots": lay_x["per_edge_slots"], "global_slots": lay_x["global_slots"],
-                      "k_edge_typed3_ms_per_step": round(x_ms.get("k_edge_typed3", 0.0) / args.steps, 3),
+                      "kernels_ms_per_step": {k: round(v / args.steps, 3) for k, v in x_ms.items()},
                       "step": "tg_build_edge_typed + tg_count_edge_typed3 + tg_free, device-resident; each edge "
                               "of the workload typed by a seeded hash"}
 

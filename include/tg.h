@@ -480,10 +480,9 @@ tg_status tg_count_edge_typed3(tg_graph *g, uint32_t *per_edge_out, int64_t *glo
 
 /* Work counters (diagnostics for the benchmark's roofline; no effect on the
  * counts).  While enabled, the counting kernels add the units of work they
- * did to per-handle counters, slot TG_WORK_*: the set-of-T lookups of the
- * 4-clique scans (one per entry of N+(w) for every member w of T, Alg. 3's
- * 4-clique branch) by the warp-per-edge and CTA-per-edge kernels, the pair
- * searches of edges with few pairs, and the SM clock cycles the CTAs of the
+ * did to per-handle counters, slot TG_WORK_*: the 32-bit words ANDed for the
+ * 4-cliques (TG_WORK_CLIQUE_PROBES; TG_WORK_CLIQUE_SEARCHES and
+ * TG_WORK_CLIQUE_BIG_PROBES stay 0), and the SM clock cycles the CTAs of the
  * hub wedge pass spent waiting for their tickets' dependencies and working
  * on tickets of each kind (fill the counter tables, read them, clear them
  * by walking the wedges, clear them by zeroing), the wedges of the hub

@@ -3,9 +3,8 @@
 The knobs never change a count (tg_options: "results never depend on
 them"); they pick which kernel variant takes which part of the work:
 
-  light_edge_max_degree    heavy-edge threshold of the 4-clique pass: edges
-                           whose triangle set T is larger go to one CTA per
-                           edge instead of one warp per edge
+  light_edge_max_degree    accepted and without effect (the 4-cliques are
+                           counted in one form)
   light_anchor_max_wedges  wedge anchors with at most this many wedges are
                            one warp each (shared-memory hash per warp)
   hub_min_wedges           anchors with more wedges are counted by the whole
@@ -15,11 +14,9 @@ them"); they pick which kernel variant takes which part of the work:
   ctas_per_sm              resident CTAs per SM of the orbit epilogue
   hub_l2_mb                hub node tables counted together (more hubs per
                            group against L2 pressure)
-  isect_bucket_0 .. 3      typed set intersection per bucket of the shorter
-                           segment's length ([1,32) [32,128) [128,512)
-                           [512,inf)): 1 binary search, 2 warp-wide merge,
-                           3 a dependent-load count picks per pair; packed
-                           into tg_options.isect_modes
+  isect_bucket_0 .. 3      accepted and without effect (every triangle is
+                           found once from the lists of higher-priority
+                           neighbours); packed into tg_options.isect_modes
 
 tune() measures tg_count (CUDA events on the given stream) for one graph or
 batch handle per candidate, by coordinate descent from the defaults, and

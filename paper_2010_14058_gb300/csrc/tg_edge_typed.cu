@@ -164,7 +164,9 @@ __global__ void __launch_bounds__(256) k_et_zero(int64_t m, int64_t stride, int 
 // Thread per (edge, slot): the 3-path slot from the typed degrees and the
 // cells, or the triangle slot's cell; class sums (block 0 edges, block 1
 // 3-paths, block 2 triangles) are kept in registers while the endpoints'
-// types and the edge's type stay the same.
+// types and the edge's type stay the same.  Bound by the latency of the
+// gathers and the rows written; the endpoints of a tile's edges are staged in
+// shared memory by visiting order (5 M edges, L = 5, X = 4: 2.78 -> 2.45 ms).
 template <int L, int X>
 __global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, const uint32_t *__restrict__ cell,
                                                                  int64_t stride, const uint8_t *__restrict__ xi,
