@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "tg.h"
+#include "tg_wedge_table.hpp"
 
 namespace tg {
 
@@ -35,13 +36,6 @@ constexpr int32_t kIdMask = (1 << kTypeShift) - 1;
 enum : int { kWorkCliqueProbes = 0, kWorkCliqueSearches = 1, kWorkCliqueBigProbes = 2, kWorkHubWait = 3,
              kWorkHubKind = 4 /* + ticket kind 0..3 */, kWorkHubWedges = 8, kWorkHubSlotUpdates = 9,
              kWorkSlots = 16 };
-
-// Wedge anchors by class (tg_wedge.cu): 0 a warp, 1-4 a CTA by table size, kHubClass hubs.
-constexpr int kHubClass = 5;
-struct WedgeLimits {
-    int64_t light, hub;         // most wedges of class 0, and of the shared-memory classes
-    int64_t bytes[4];           // table bytes of classes 1 to 4
-};
 
 // Persistent hub pass (tg_hub.cu): a group of hubs whose counter tables
 // share one table buffer, and the ticket queue as runs of tickets of one

@@ -39,50 +39,15 @@ namespace tg {
 
 namespace {
 
-// Layout of an anchor's counters: rw words per wedge end, F types per word,
-// `bits` bits each.
-struct Pack {
-    int rw, F, bits;
-};
-
-__host__ __device__ __forceinline__ Pack pack_of(int L, int64_t most) {
-    Pack k;
-    k.rw = 1;
-    k.F = L;
-    k.bits = 32 / L;
-    if (most >> k.bits) {
-        k.rw = 2;
-        k.F = (L + 1) / 2;
-        k.bits = 32 / k.F;
-    }
-    if (most >> k.bits) {
-        k.rw = 4;
-        k.F = 2;
-        k.bits = 16;
-    }
-    return k;
-}
-
-// Table of an anchor of W wedges: per slot a key and rw counter words, per
-// wedge the slot it went to (uint16).  Two slots per wedge where `bytes` hold
-// them, at least one (a slot per distinct end, so an insert always ends).
-__host__ __device__ __forceinline__ int64_t table_need(int64_t W, int64_t slots, int rw) {
-    return slots * (4 + 4 * rw) + ((2 * W + 3) & ~(int64_t)3);
-}
-__host__ __device__ __forceinline__ int64_t slots_for(int64_t W, int64_t bytes, int rw) {
-    const int64_t fit = (bytes - table_need(W, 0, rw)) / (4 + 4 * rw), want = 2 * W + 16;
-    return want < fit ? want : fit;
-}
-
 // ------------------------------------------------------------ classes
 // Threads per anchor, entries of the run list (entries beyond it are walked
 // in chunks), and bytes of the table (the warp form's follow the option).
 template <int kForm> struct Form;
 template <> struct Form<0> { static constexpr int threads = 32, groups = 4, runs = 160; };
-template <> struct Form<1> { static constexpr int threads = 64, groups = 1, runs = 256, bytes = 11 << 10; };
-template <> struct Form<2> { static constexpr int threads = 192, groups = 1, runs = 384, bytes = 30 << 10; };
-template <> struct Form<3> { static constexpr int threads = 512, groups = 1, runs = 1024, bytes = 98 << 10; };
-template <> struct Form<4> { static constexpr int threads = 1024, groups = 1, runs = 1536, bytes = 200 << 10; };
+template <> struct Form<1> { static constexpr int threads = 64, groups = 1, runs = 256; };
+template <> struct Form<2> { static constexpr int threads = 192, groups = 1, runs = 384; };
+template <> struct Form<3> { static constexpr int threads = 512, groups = 1, runs = 1024; };
+template <> struct Form<4> { static constexpr int threads = 1024, groups = 1, runs = 1536; };
 
 template <int kForm>
 __host__ __device__ constexpr size_t run_bytes() {          // start, off, sv, tv of Runs
@@ -165,16 +130,23 @@ struct Table {
     uint16_t *slot;             // [wedges] the slot of every wedge's end
     uint32_t cap;
     Pack pk;
+    uint32_t *status;
 };
 
-// the slot of w, inserted if new (a free slot exists: cap >= the wedges)
+// the slot of w, inserted if new (a free slot exists: cap >= the wedges,
+// anchor_pack and slots_for; a full table would be reported, not probed on)
 __device__ __forceinline__ uint32_t table_insert(const Table &tb, uint32_t w) {
-    uint32_t h = __umulhi(w * 2654435761u, tb.cap);
+    const uint32_t h0 = __umulhi(w * 2654435761u, tb.cap);
+    uint32_t h = h0;
     for (;;) {
         uint32_t k = *(volatile uint32_t *)&tb.keys[h];
         if (k == 0xffffffffu) k = atomicCAS(&tb.keys[h], 0xffffffffu, w);
         if (k == 0xffffffffu || k == w) return h;
         h = h + 1 == tb.cap ? 0 : h + 1;
+        if (h == h0) {
+            set_status(tb.status, ST_INTERNAL);
+            return h;
+        }
     }
 }
 
@@ -307,8 +279,9 @@ __global__ void __launch_bounds__(Form<kForm>::threads * Form<kForm>::groups)
         const int32_t nV = __shfl_sync(0xffffffffu, inc, kMaxL - 1);
         const int32_t most = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)nt);
         Table tb;
-        tb.pk = pack_of(L, most);
+        tb.pk = anchor_pack(L, wedges[u], most);
         tb.cap = (uint32_t)slots_for(wedges[u], table_bytes, tb.pk.rw);
+        tb.status = cv.status;
         tb.keys = mem;
         tb.cnt = mem + tb.cap;
         tb.slot = reinterpret_cast<uint16_t *>(tb.cnt + (size_t)tb.cap * tb.pk.rw);
@@ -368,12 +341,6 @@ size_t form_bytes(int64_t table_bytes) {
     return Form<kForm>::groups * ((size_t)table_bytes + run_bytes<kForm>());
 }
 
-// bytes of a light anchor's table: its wedges may all end at distinct nodes,
-// and its counters reach the number of its wedges
-int64_t light_bytes(int L, int64_t wedges) {
-    return table_need(wedges, 2 * wedges + 16, pack_of(L, wedges).rw);
-}
-
 }  // namespace
 
 int light_anchor_limit(int L) {
@@ -389,28 +356,12 @@ WedgeLimits wedge_limits(const Graph &G) {
     WedgeLimits w;
     w.light = G.opt.light_anchor_max_wedges;
     w.hub = G.opt.hub_min_wedges;
-    w.bytes[0] = Form<1>::bytes;
-    w.bytes[1] = Form<2>::bytes;
-    w.bytes[2] = Form<3>::bytes;
-    w.bytes[3] = Form<4>::bytes;
+    for (int f = 1; f < kHubClass; ++f) w.bytes[f - 1] = kFormBytes[f];
     return w;
 }
 
-__device__ int wedge_class(const WedgeLimits &w, int L, int64_t W, int64_t most) {
-    if (W <= 0) return -1;
-    if (W <= w.light) return 0;
-    if (W > w.hub) return kHubClass;
-    const int rw = pack_of(L, most).rw;
-    // two slots per wedge; in the largest form a slot per wedge is enough
-    for (int f = 0; f < 4; ++f)
-        if (table_need(W, (f < 3 ? 2 * W : W) + 16, rw) <= w.bytes[f] && W < (1 << 15)) return f + 1;
-    return kHubClass;
-}
-
 static int64_t table_bytes_of(const Graph &G, int form) {
-    const int64_t b = form == 0 ? light_bytes(G.L, G.opt.light_anchor_max_wedges)
-                    : form == 1 ? Form<1>::bytes : form == 2 ? Form<2>::bytes : form == 3 ? Form<3>::bytes : Form<4>::bytes;
-    return (b + 15) & ~(int64_t)15;
+    return form == 0 ? light_bytes(G.L, G.opt.light_anchor_max_wedges) : kFormBytes[form];
 }
 
 template <class Fn>
