@@ -287,21 +287,19 @@ static int64_t launch_chunk(Graph &G, size_t ci, bool triangles, cudaStream_t s)
 void prepare_counting(Graph &G, int k, cudaStream_t s) {
     const int L = G.L;
     const size_t m = (size_t)std::max<int64_t>(G.m, 1), n = (size_t)std::max<int64_t>(G.n, 1);
-    if (G.C.bytes < m * kCRow * sizeof(uint32_t)) G.C.alloc(m * kCRow * sizeof(uint32_t));
-    if (G.tri_any.bytes < n) G.tri_any.alloc(n);
+    G.C.alloc_once(m * kCRow * sizeof(uint32_t));
+    G.tri_any.alloc_once(n);
     prepare_triangles(G);
-    const size_t gbytes = (size_t)G.ngraphs * global_slots(L, 4) * sizeof(unsigned long long);
-    if (G.gacc.bytes < gbytes) G.gacc.alloc(gbytes);
+    G.gacc.alloc_once((size_t)G.ngraphs * global_slots(L, 4) * sizeof(unsigned long long));
     if (k == 4) {
         if (!G.anchors_ready) prepare_anchors(G, s);
-        if (G.tau.bytes < n * L * L * G.node_sum_bytes()) G.tau.alloc(n * L * L * G.node_sum_bytes());
+        G.tau.alloc_once(n * L * L * G.node_sum_bytes());
         if (G.chunks.empty()) plan_chunks(G);
         const size_t ab = (size_t)G.a_stride * L * L * sizeof(uint32_t);
-        if (G.A.bytes < ab) G.A.alloc(ab);
-        if (G.slot_rows.bytes < ab) G.slot_rows.alloc(ab);
+        G.A.alloc_once(ab);
+        G.slot_rows.alloc_once(ab);
         const size_t me = (size_t)std::max<int64_t>(G.max_chunk_edges, 1);
-        const size_t xb = me * 4 * L * L * (G.wide_sums() ? sizeof(unsigned long long) : sizeof(uint32_t));
-        if (G.xsum.bytes < xb) G.xsum.alloc(xb);
+        G.xsum.alloc_once(me * 4 * L * L * (G.wide_sums() ? sizeof(unsigned long long) : sizeof(uint32_t)));
         prepare_sums(G);
         if (G.n_hubs > 0 && G.hub_plans.empty()) prepare_hubs(G, s);
     }

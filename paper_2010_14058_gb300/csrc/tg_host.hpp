@@ -69,6 +69,12 @@ struct DBuf {
         else TG_CK(cudaMalloc(&p, b));
         bytes = b;
     }
+    // for buffers that a captured batch points to: allocated once, and never
+    // replaced while the handle lives
+    void alloc_once(size_t b) {
+        if (!p) alloc(b);
+        else if (bytes < b) throw Error{TG_ERR_INTERNAL, "working array of another size"};
+    }
     void release() {
         if (p) {
             if (owner) cudaFreeAsync(p, *owner);
@@ -133,8 +139,9 @@ struct Graph {
     DBuf node_off, edge_off, rp, adj, toff, tdeg, pivot, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
     DBuf most_lower;                            // most lower-priority neighbours of one type, until prepare_anchors
     DBuf plus_off, plus_adj, plus_eid;
-    // nodes by |N+| (tg_local.cuh): mid, big, and larger than shared memory holds
-    DBuf tri_list[3], local_scratch;
+    // nodes by |N+| (tg_local.cuh): mid, big, and larger than shared memory
+    // holds; the slices of the CTAs that list triangles and of those that sum
+    DBuf tri_list[3], tri_scratch, sum_scratch;
     int64_t tri_count[3] = {0, 0, 0}, max_nplus = 0;
     // work lists
     DBuf anchors[kHubClass], anchor_wedges;     // wedge anchors by class (tg_wedge.cu); wedges of every node
@@ -250,7 +257,7 @@ struct Graph {
         return {&node_off, &edge_off, &rp, &adj, &toff, &tdeg, &pivot, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &most_lower, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
-                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dlab, &doutdeg, &dcls, &darcs, &dgacc, &dcell, &etype, &etdeg, &etgacc, &etcell, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &local_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
+                             &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dlab, &doutdeg, &dcls, &darcs, &dgacc, &dcell, &etype, &etdeg, &etgacc, &etcell, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &tri_scratch, &sum_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,
                 &pa_cls, &pa_gacc};
     }
     int64_t device_bytes() const {
@@ -323,6 +330,8 @@ LocalClass local_class(const Graph &G, int cls);
 int64_t launch_row_sums(Graph &G, const int32_t *index, const uint32_t *rows, void *out, cudaStream_t s);
 // shared-memory limits and scratch of launch_triangles (before any capture)
 void prepare_triangles(Graph &G);
+// G.tri_scratch, of one size whichever kernels list the triangles
+void prepare_tri_scratch(Graph &G);
 // typed triangles per edge and, with_tau, the per-node sums of the whole
 // graph (tg_triangles.cu); returns the kernel launches
 int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s);

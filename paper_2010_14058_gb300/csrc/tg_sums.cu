@@ -383,14 +383,16 @@ SumShape shape_of(const Graph &G, const LocalClass &c, int cls) {
 template <class Acc, int kL>
 void prepare(Graph &G) {
     raise_smem_limit((const void *)k_sum_warp<Acc, kL>, warp_bytes(G.L));
+    size_t scratch = 0;
     for (int cls = 0; cls < 3; ++cls) {
         const LocalClass c = local_class(G, cls);
         if (c.n == 0) continue;
         const SumShape r = shape_of(G, c, cls);
         if (cls == 0) raise_smem_limit((const void *)k_sum_cta<Acc, kL, kTriMidThreads, true>, r.smem);
         else if (cls == 1) raise_smem_limit((const void *)k_sum_cta<Acc, kL, kTriBigThreads, true>, r.smem);
-        if (G.local_scratch.bytes < r.slice * (size_t)r.ctas) G.local_scratch.alloc(r.slice * (size_t)r.ctas);
+        scratch = std::max(scratch, r.slice * (size_t)r.ctas);
     }
+    if (scratch) G.sum_scratch.alloc_once(scratch);
 }
 
 template <class Acc, int kL>
@@ -422,7 +424,7 @@ int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStr
         ++launches;
         auto run = [&](auto kern) {
             kern<<<(unsigned)r.ctas, c.threads, r.smem, s>>>(gv, cv, c.list, c.n, n0, n1, c.cap, c.lgf,
-                                                             G.local_scratch.as<unsigned char>(), (int64_t)r.slice);
+                                                             G.sum_scratch.as<unsigned char>(), (int64_t)r.slice);
         };
         if (cls == 0) run(k_sum_cta<Acc, kL, kTriMidThreads, true>);
         else if (cls == 1) run(k_sum_cta<Acc, kL, kTriBigThreads, true>);

@@ -250,14 +250,19 @@ static size_t tri_bytes(const Graph &G, const LocalClass &c) {
     return ((size_t)c.cap * G.L * 4 + local_bytes(c.cap, c.lgf, c.threads / 32) + 15) & ~(size_t)15;
 }
 
+void prepare_tri_scratch(Graph &G) {
+    const LocalClass c = local_class(G, 2);
+    if (c.n > 0) G.tri_scratch.alloc_once(tri_bytes(G, c) * (size_t)std::min<int64_t>(c.n, sm_count()));
+}
+
 void prepare_triangles(Graph &G) {
-    for (int cls = 0; cls < 3; ++cls) {
+    prepare_tri_scratch(G);
+    for (int cls = 0; cls < 2; ++cls) {
         const LocalClass c = local_class(G, cls);
         if (c.n == 0) continue;
         const size_t bytes = tri_bytes(G, c);
         if (cls == 0) raise_smem_limit((const void *)k_tri_cta<kTriMidThreads, true>, bytes);
-        else if (cls == 1) raise_smem_limit((const void *)k_tri_cta<kTriBigThreads, true>, bytes);
-        else if (G.local_scratch.bytes < bytes * (size_t)sm_count()) G.local_scratch.alloc(bytes * (size_t)sm_count());
+        else raise_smem_limit((const void *)k_tri_cta<kTriBigThreads, true>, bytes);
     }
 }
 
@@ -283,7 +288,7 @@ int64_t launch_triangles(Graph &G, bool with_tau, cudaStream_t s) {
             if (cls == 2) {
                 const int64_t grid = std::min<int64_t>(c.n, sms);
                 k_tri_cta<kTriBigThreads, false><<<(unsigned)grid, kTriBigThreads, 0, s>>>(
-                    gv, cv.C, cv.tri_any, c.list, c.n, c.cap, c.lgf, G.local_scratch.as<unsigned char>(), (int64_t)bytes);
+                    gv, cv.C, cv.tri_any, c.list, c.n, c.cap, c.lgf, G.tri_scratch.as<unsigned char>(), (int64_t)bytes);
                 continue;
             }
             auto launch = [&](auto kern) {

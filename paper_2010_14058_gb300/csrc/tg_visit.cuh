@@ -86,9 +86,9 @@ int64_t visit_triangles(Graph &G, V v, cudaStream_t s) {
         ++launches;
         if (cls == 2) {
             const int64_t grid = std::min<int64_t>(c.n, sms);
-            if (G.local_scratch.bytes < bytes * (size_t)grid) G.local_scratch.alloc(bytes * (size_t)grid);
+            prepare_tri_scratch(G);
             k_visit_cta<kTriBigThreads, false, V><<<(unsigned)grid, kTriBigThreads, 0, s>>>(
-                gv, v, c.list, c.n, c.cap, c.lgf, G.local_scratch.as<unsigned char>(), (int64_t)bytes);
+                gv, v, c.list, c.n, c.cap, c.lgf, G.tri_scratch.as<unsigned char>(), (int64_t)bytes);
             continue;
         }
         auto run = [&](auto kern) {
