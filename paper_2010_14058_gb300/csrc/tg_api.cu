@@ -79,7 +79,7 @@ void build_common(int32_t ngraphs, const int64_t *node_off, int64_t n, int64_t n
     try {
         tg::build_graph(h->g, ngraphs, node_off, n, nnz, row_ptr, col, types, L, o, (cudaStream_t)stream);
     } catch (...) {
-        cudaStreamSynchronize((cudaStream_t)stream);
+        tg::forget(cudaStreamSynchronize((cudaStream_t)stream));
         h->g.stream = nullptr;
         delete h;
         throw;
@@ -356,7 +356,7 @@ tg_status tg_count_edge_typed3(tg_graph *gh, uint32_t *per_edge_out, int64_t *gl
 
 void tg_free(tg_graph *g) {
     if (!g) return;
-    cudaStreamSynchronize(g->g.stream);
+    tg::forget(cudaStreamSynchronize(g->g.stream));
     g->g.stream = nullptr;          // release on the legacy stream: the caller's may be gone later
     delete g;
 }
@@ -564,7 +564,7 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
                           G.batch_stream == s;
         if (!same) {
             if (G.batch_exec) {
-                cudaGraphExecDestroy(G.batch_exec);
+                tg::forget(cudaGraphExecDestroy(G.batch_exec));
                 G.batch_exec = nullptr;
             }
             tg::prepare_counting(G, k, s);
@@ -578,13 +578,13 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
                 launches += tg::run_count(G, k, 0, G.m, per_edge_out, G.gacc.as<unsigned long long>(), true, s);
                 if (global_out) launches += tg::launch_finalize(G, k, global_out, s);
             } catch (...) {
-                cudaStreamEndCapture(s, &graph);
-                if (graph) cudaGraphDestroy(graph);
+                tg::forget(cudaStreamEndCapture(s, &graph));
+                if (graph) tg::forget(cudaGraphDestroy(graph));
                 throw;
             }
             TG_CK(cudaStreamEndCapture(s, &graph));
             cudaError_t ie = cudaGraphInstantiate(&G.batch_exec, graph, 0);
-            cudaGraphDestroy(graph);
+            tg::forget(cudaGraphDestroy(graph));
             TG_CK(ie);
             G.batch_k = k;
             G.batch_pe = per_edge_out;

@@ -178,7 +178,7 @@ public:
     }
     ~SideStreams() {
         if (forked_) {                                      // an error between fork and join: nothing may still run
-            for (cudaStream_t x : set_->s) cudaStreamSynchronize(x);   // when the caller gives its buffers back
+            for (cudaStream_t x : set_->s) forget(cudaStreamSynchronize(x));   // when the caller gives its buffers back
             return;
         }
         std::lock_guard<std::mutex> lock(mutex());
@@ -214,9 +214,9 @@ private:
         cudaEvent_t ev[2 + kSides] = {};
         ~Set() {                                            // (work enqueued on them completes all the same)
             for (cudaStream_t x : s)
-                if (x) cudaStreamDestroy(x);
+                if (x) forget(cudaStreamDestroy(x));
             for (cudaEvent_t x : ev)
-                if (x) cudaEventDestroy(x);
+                if (x) forget(cudaEventDestroy(x));
         }
     };
     static constexpr size_t kKeep = 8;

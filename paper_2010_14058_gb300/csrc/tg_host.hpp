@@ -45,6 +45,12 @@ int light_anchor_limit(int L);
 
 #define TG_CK(call) ::tg::throw_cuda((call), #call)
 
+// For calls of destructors, which may run because an earlier call failed: an
+// error of theirs must not be what the next entry's cudaGetLastError finds.
+inline void forget(cudaError_t e) {
+    if (e != cudaSuccess) (void)cudaGetLastError();
+}
+
 // Stream-ordered memory pool of the current device, owned by the library
 // (release threshold kept at its maximum, so freed blocks are reused instead
 // of returned to the CUDA driver).  Defined in tg_build.cu.
@@ -77,8 +83,7 @@ struct DBuf {
     }
     void release() {
         if (p) {
-            if (owner) cudaFreeAsync(p, *owner);
-            else cudaFree(p);
+            forget(owner ? cudaFreeAsync(p, *owner) : cudaFree(p));
         }
         p = nullptr;
         bytes = 0;
@@ -98,7 +103,7 @@ struct TBuf {
     }
     TBuf(const TBuf &) = delete;
     TBuf &operator=(const TBuf &) = delete;
-    ~TBuf() { if (p) cudaFreeAsync(p, s); }
+    ~TBuf() { if (p) forget(cudaFreeAsync(p, s)); }
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
@@ -266,9 +271,9 @@ struct Graph {
         return s;
     }
     ~Graph() {
-        if (batch_exec) cudaGraphExecDestroy(batch_exec);
+        if (batch_exec) forget(cudaGraphExecDestroy(batch_exec));
         for (auto &r : timer_pending) { event_pool.push_back(r.a); event_pool.push_back(r.b); }
-        for (cudaEvent_t e : event_pool) cudaEventDestroy(e);
+        for (cudaEvent_t e : event_pool) forget(cudaEventDestroy(e));
     }
     cudaEvent_t take_event() {
         if (!event_pool.empty()) { cudaEvent_t e = event_pool.back(); event_pool.pop_back(); return e; }
@@ -288,14 +293,18 @@ struct KernelTimer {
     KernelTimer(Graph &g, cudaStream_t st, const char *nm) : G(g), s(st), name(nm) {
         if (!G.timing) return;
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return;
+        const cudaError_t e = cudaStreamIsCapturing(s, &cs);
+        forget(e);
+        if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone) return;
         a = G.take_event();
         b = G.take_event();
         TG_CK(cudaEventRecord(a, s));
     }
     ~KernelTimer() {
         if (!a) return;
-        if (cudaEventRecord(b, s) == cudaSuccess) G.timer_pending.push_back(Graph::TimerRec{name, a, b});
+        const cudaError_t e = cudaEventRecord(b, s);
+        if (e == cudaSuccess) G.timer_pending.push_back(Graph::TimerRec{name, a, b});
+        else forget(e);
     }
 };
 
