@@ -560,6 +560,7 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
         G.stream = s;
+        tg::CountGuard guard(G);
         const bool same = G.batch_exec && G.batch_k == k && G.batch_pe == per_edge_out && G.batch_gl == global_out &&
                           G.batch_stream == s;
         if (!same) {
@@ -583,9 +584,11 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
                 throw;
             }
             TG_CK(cudaStreamEndCapture(s, &graph));
-            cudaError_t ie = cudaGraphInstantiate(&G.batch_exec, graph, 0);
+            cudaGraphExec_t exec = nullptr;
+            cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
             tg::forget(cudaGraphDestroy(graph));
             TG_CK(ie);
+            G.batch_exec = exec;
             G.batch_k = k;
             G.batch_pe = per_edge_out;
             G.batch_gl = global_out;
@@ -593,6 +596,7 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
             G.last_launches = launches;
         }
         TG_CK(cudaGraphLaunch(G.batch_exec, s));
+        guard.done = true;
     });
 }
 

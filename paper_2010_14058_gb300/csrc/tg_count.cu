@@ -308,14 +308,15 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
 int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per_edge_out, unsigned long long *gacc,
                   bool full, cudaStream_t s) {
     int64_t launches = 0;
+    CountGuard guard(G);
     // prepared_k 3: typed triangles only (all that k = 3 reads); 4: their per-node sums too
     bool triangles = full || G.prepared_k < 3 || (k == 4 && !G.tau_ready);
     if (triangles && (k == 3 || G.chunks.size() != 1 || e_begin >= e_end || (!full && G.prepared_k == 4))) {
         launches += launch_triangles(G, k == 4, s);
         triangles = false;
+        G.prepared_k = std::max(G.prepared_k, 3);
+        G.tau_ready = G.tau_ready || k == 4;
     }
-    G.prepared_k = std::max(G.prepared_k, 3);
-    G.tau_ready = G.tau_ready || k == 4;
     DBuf tmp;                                                // tiles of a range, stream-ordered
     tmp.owner = &G.stream;
     int64_t n_tiles = 0;
@@ -334,6 +335,7 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
             if (full || G.chunks.size() > 1 || G.prepared_k != 4) {
                 launches += launch_chunk(G, ci, triangles, s);
                 if (G.chunks.size() == 1) G.prepared_k = 4;
+                G.tau_ready = G.tau_ready || triangles;
             }
             const Tile *ct = tiles;
             int64_t nct = n_tiles;
@@ -354,6 +356,7 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
         }
     }
     if (tmp.p) TG_CK(cudaStreamSynchronize(s));
+    guard.done = true;
     return launches;
 }
 

@@ -283,6 +283,20 @@ struct Graph {
     }
 };
 
+// What a count leaves in the handle's working arrays (prepared_k, tau_ready)
+// is recorded once the launches that make it are enqueued; a count that ends
+// with an error leaves nothing that a later one may rely on.
+struct CountGuard {
+    Graph &G;
+    bool done = false;
+    explicit CountGuard(Graph &g) : G(g) {}
+    ~CountGuard() {
+        if (done) return;
+        G.prepared_k = 0;
+        G.tau_ready = false;
+    }
+};
+
 // Brackets one kernel launch with events when timing is on and the stream
 // is not being captured.
 struct KernelTimer {

@@ -1,6 +1,8 @@
-"""A call that fails on the host leaves a handle and a runtime that count on.
-The failure is the runtime's own: synchronising a stream that is being
-captured, which it refuses; no kernel of the failed call runs."""
+"""A call that fails on the host leaves a handle and a runtime that count on:
+what the failed call had not launched is launched by the next one.  The
+failures are the runtime's own: capturing the legacy stream, and synchronising
+a stream that is being captured, both of which it refuses; no kernel of the
+failed calls runs."""
 import ctypes
 
 import numpy as np
@@ -17,6 +19,7 @@ if not torch.cuda.is_available():
 
 import paper_2010_14058_gb300 as tg  # noqa: E402
 
+LEGACY = 1                                                   # cudaStreamLegacy
 RELAXED = 2                                                  # cudaStreamCaptureModeRelaxed
 
 
@@ -63,6 +66,30 @@ def test_a_count_after_a_failed_range(graph):
         s.synchronize()
         failing_range(h, out, totals, s)
         tg.tg_count(h, 4, out, totals, stream=s)
+        s.synchronize()
+        np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32).astype(np.int64), rows)
+        assert tg.tg_query_status(h) == 0
+        h.free()
+
+
+@pytest.mark.parametrize("before", [None, 3])
+def test_a_range_after_a_failed_range(graph, before):
+    g, rows = graph
+    rp, col, ty = tg.to_device(g)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    lay = tg.tg_layout(g["L"], 4)
+    with torch.cuda.stream(s):
+        out = torch.full((g["m"], lay["per_edge_slots"]), -1, dtype=torch.int32, device="cuda")
+        totals = torch.zeros(lay["global_slots"], dtype=torch.int64, device="cuda")
+        h = tg.tg_build(rp, col, ty, g["L"], stream=s)
+        if before:                                           # triangle counts without their sums per node
+            tg.tg_count(h, before, None, totals, stream=s)
+        s.synchronize()
+        with pytest.raises(tg.TGError):                      # every working array is there, and nothing is counted
+            tg.tg_count_batch(h, 4, out, totals, stream=LEGACY)
+        failing_range(h, out, totals, s)
+        tg.tg_count_range(h, 4, 0, h.m, out, stream=s)
         s.synchronize()
         np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32).astype(np.int64), rows)
         assert tg.tg_query_status(h) == 0
