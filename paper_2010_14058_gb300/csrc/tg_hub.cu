@@ -477,7 +477,7 @@ void prepare_hubs(Graph &G, cudaStream_t s) {
 
     // ticket queues
     const int64_t ctas = (int64_t)sm_count() * kHubCtasPerSm;
-    G.hub_plans.clear();
+    std::vector<std::unique_ptr<Graph::HubPlan>> plans;     // the handle gets all of them or, on an error, none
     for (size_t c = 0; c < G.chunks.size(); ++c) {
         auto plan = std::make_unique<Graph::HubPlan>();
         for (DBuf *d : {&plan->segs, &plan->groups, &plan->ntick, &plan->ctr}) d->owner = &G.stream;
@@ -551,8 +551,9 @@ void prepare_hubs(Graph &G, cudaStream_t s) {
             TG_CK(cudaMemcpyAsync(plan->ntick.p, ntick.data(), sizeof(int64_t) * ntick.size(), cudaMemcpyHostToDevice,
                                   s));
         }
-        G.hub_plans.push_back(std::move(plan));
+        plans.push_back(std::move(plan));
     }
+    G.hub_plans = std::move(plans);
 }
 
 int64_t launch_hubs(Graph &G, size_t ci, cudaStream_t s) {
