@@ -264,7 +264,7 @@ tg_status tg_count_directed3(tg_graph *gh, uint32_t *per_edge_out, int64_t *glob
         if (!gh || !gh->g.directed) throw Error{TG_ERR_INVALID_ARG, "not a directed handle"};
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         const size_t pe_bytes = (size_t)G.m * 8 * G.L * sizeof(uint32_t);
         const size_t gl_bytes = (size_t)G.d_global * sizeof(int64_t);
         bool pe_staged = false, gl_staged = false;
@@ -340,7 +340,7 @@ tg_status tg_count_edge_typed3(tg_graph *gh, uint32_t *per_edge_out, int64_t *gl
         if (!gh || !gh->g.edge_typed) throw Error{TG_ERR_INVALID_ARG, "not an edge-typed handle"};
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         const int64_t X = G.et_X, P = X * (X + 1) / 2;
         const size_t pe_bytes = (size_t)G.m * (size_t)(G.L * X + G.L * P) * sizeof(uint32_t);
         const size_t gl_bytes = (size_t)G.et_global * sizeof(int64_t);
@@ -401,7 +401,7 @@ tg_status tg_count(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_t *glo
         if (!gh || (k != 3 && k != 4)) throw Error{TG_ERR_INVALID_ARG, "k"};
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         tg::prepare_counting(G, k, s);
         tg::prepare_edges(G, k, s);
         const size_t pe_bytes = (size_t)G.m * tg::per_edge_slots(G.L, k) * sizeof(uint32_t);
@@ -440,7 +440,7 @@ tg_status tg_count_position_aware(tg_graph *gh, uint32_t *per_edge_out, int64_t 
         if (!gh) throw Error{TG_ERR_INVALID_ARG, "NULL"};
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         tg::prepare_counting(G, 4, s);
         tg::prepare_edges(G, 4, s);
         tg::prepare_position_aware(G, s);
@@ -471,7 +471,7 @@ tg_status tg_count_range(tg_graph *gh, int32_t k, int64_t e_begin, int64_t e_end
         Graph &G = gh->g;
         if (e_begin < 0 || e_end < e_begin || e_end > G.m) throw Error{TG_ERR_INVALID_ARG, "range"};
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         tg::prepare_counting(G, k, s);
         tg::prepare_edges(G, k, s);
         int64_t launches = 0;
@@ -483,7 +483,7 @@ tg_status tg_count_range(tg_graph *gh, int32_t k, int64_t e_begin, int64_t e_end
         if (gl_staged) TG_CK(cudaMemcpyAsync(gl, global_accum, gl_bytes, cudaMemcpyHostToDevice, s));
         unsigned long long *acc = gl ? reinterpret_cast<unsigned long long *>(gl) : nullptr;
         tg::DBuf scratch;
-        scratch.owner = &G.stream;
+        scratch.owner = &G;
         if (!acc) {
             scratch.alloc(gl_bytes);
             TG_CK(cudaMemsetAsync(scratch.p, 0, gl_bytes, s));
@@ -506,7 +506,7 @@ tg_status tg_count_sparse(tg_graph *gh, int32_t k, int64_t *row_off, uint16_t *s
             if (p && !tg::is_device_pointer(p)) throw Error{TG_ERR_INVALID_ARG, "sparse arrays must be device memory"};
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         tg::prepare_counting(G, k, s);
         tg::prepare_edges(G, k, s);
         const size_t gl_bytes = (size_t)G.ngraphs * tg::global_slots(G.L, k) * sizeof(int64_t);
@@ -529,7 +529,7 @@ tg_status tg_graphlet_weights(tg_graph *gh, int32_t k, const uint32_t *per_edge_
         for (const void *p : {(const void *)per_edge_rows, (const void *)weights, (const void *)degree})
             if (p && !tg::is_device_pointer(p)) throw Error{TG_ERR_INVALID_ARG, "arrays must be device memory"};
         Graph &G = gh->g;
-        G.stream = (cudaStream_t)stream;
+        G.on((cudaStream_t)stream);
         tg::launch_weights(G, k, per_edge_rows, block, rank, weights, degree, G.stream);
     });
 }
@@ -559,7 +559,7 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
             throw Error{TG_ERR_INVALID_ARG, "batched outputs must be device memory"};
         Graph &G = gh->g;
         cudaStream_t s = (cudaStream_t)stream;
-        G.stream = s;
+        G.on(s);
         tg::CountGuard guard(G);
         const bool same = G.batch_exec && G.batch_k == k && G.batch_pe == per_edge_out && G.batch_gl == global_out &&
                           G.batch_stream == s;
@@ -612,6 +612,7 @@ tg_status tg_set_work_counting(tg_graph *gh, int32_t on) {
         if (!gh) throw Error{TG_ERR_INVALID_ARG, "NULL"};
         Graph &G = gh->g;
         if (on && !G.work.p) {
+            G.on(G.stream);
             G.work.alloc(sizeof(unsigned long long) * tg::kWorkSlots);
             TG_CK(cudaMemsetAsync(G.work.p, 0, sizeof(unsigned long long) * tg::kWorkSlots, G.stream));
         }

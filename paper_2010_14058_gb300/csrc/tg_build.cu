@@ -359,7 +359,7 @@ int sm_count() {
 void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_t n, int64_t nnz,
                  const int64_t *row_ptr, const int32_t *col, const uint8_t *types, int32_t L,
                  const tg_options &opt, cudaStream_t s) {
-    G.stream = s;
+    G.on(s);
     G.last_launches = 0;
     G.ngraphs = ngraphs;
     G.L = L;

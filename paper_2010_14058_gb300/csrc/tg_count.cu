@@ -114,11 +114,7 @@ static const Tile *tiles_for(Graph &G, int64_t e_begin, int64_t e_end, int64_t &
     std::vector<Tile> tiles = make_tiles(G, e_begin, e_end);
     n_tiles = (int64_t)tiles.size();
     DBuf &dst = full ? G.tiles_full : tmp;
-    dst.alloc(sizeof(Tile) * std::max<size_t>(tiles.size(), 1));
-    if (!tiles.empty()) {
-        TG_CK(cudaMemcpyAsync(dst.p, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice, s));
-        TG_CK(cudaStreamSynchronize(s));   // the host vector goes out of scope
-    }
+    dst.upload(tiles.data(), sizeof(Tile) * tiles.size(), s);
     if (full) G.n_tiles_full = n_tiles;
     return dst.as<Tile>();
 }
@@ -144,7 +140,7 @@ void prepare_edges(Graph &G, int k, cudaStream_t s) {
     if (k == 4) prepare_epi(G);
     if (k == 4) prepare_wedges(G);
     DBuf unused;
-    unused.owner = &G.stream;
+    unused.owner = &G;
     int64_t nt = 0;
     tiles_for(G, 0, G.m, nt, unused, s);
 }
@@ -318,7 +314,7 @@ int64_t run_count(Graph &G, int k, int64_t e_begin, int64_t e_end, uint32_t *per
         G.tau_ready = G.tau_ready || k == 4;
     }
     DBuf tmp;                                                // tiles of a range, stream-ordered
-    tmp.owner = &G.stream;
+    tmp.owner = &G;
     int64_t n_tiles = 0;
     const Tile *tiles = tiles_for(G, e_begin, e_end, n_tiles, tmp, s);
     if (k == 3) {

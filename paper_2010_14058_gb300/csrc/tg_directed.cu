@@ -373,7 +373,7 @@ int64_t run_directed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, cud
     int64_t launches = 0;
     if (G.m > 0) {
         const size_t bytes = sizeof(uint32_t) * 4 * (size_t)G.L * (size_t)G.m;
-        if (G.dcell.bytes < bytes) G.dcell.alloc(bytes);
+        G.dcell.alloc_once(bytes);
         {
             KernelTimer kt(G, s, "k_directed_cells");
             TG_CK(cudaMemsetAsync(G.dcell.p, 0, bytes, s));

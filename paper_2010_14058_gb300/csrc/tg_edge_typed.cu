@@ -334,8 +334,7 @@ int64_t run_edge_typed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, c
         uint32_t *cell = per_edge_out ? per_edge_out + L * X : nullptr;
         const int64_t stride = per_edge_out ? S : L * P;
         if (!cell) {
-            const size_t bytes = sizeof(uint32_t) * (size_t)(stride * G.m);
-            if (G.etcell.bytes < bytes) G.etcell.alloc(bytes);
+            G.etcell.alloc_once(sizeof(uint32_t) * (size_t)(stride * G.m));
             cell = G.etcell.as<uint32_t>();
         }
         {

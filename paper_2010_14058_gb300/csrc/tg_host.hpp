@@ -56,14 +56,47 @@ inline void forget(cudaError_t e) {
 // of returned to the CUDA driver).  Defined in tg_build.cu.
 cudaMemPool_t device_pool();
 
+// Whether `s` is being captured into a CUDA graph.
+inline bool stream_captured(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    forget(e);
+    return e == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
+// cudaMalloc and cudaFree are refused on a thread that captures a stream
+// unless it asks for them.
+template <class F>
+cudaError_t relaxed(F f) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    forget(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = f();
+    forget(cudaThreadExchangeStreamCaptureMode(&mode));
+    return e;
+}
+
+// Stream of a handle's last call, and whether it was captured then (asked once
+// per call, not per buffer: a small build has forty of them).
+struct OwnerStream {
+    cudaStream_t stream = nullptr;
+    bool captured = false;
+    void on(cudaStream_t s) {
+        stream = s;
+        captured = stream_captured(s);
+    }
+};
+
 // Device buffer owned by a handle; freed by release() or the destructor.
-// With an owner stream (the handle's stream) it is allocated and freed
-// stream-ordered from the library pool, so no call synchronises the device;
-// without one it falls back to cudaMalloc / cudaFree.
+// With an owner (the handle) it is allocated and freed stream-ordered on its
+// stream from the library pool, so no call synchronises the device; without
+// one, and while that stream is captured, it is cudaMalloc's and cudaFree's:
+// an allocation that a capture takes up has memory behind it only while the
+// captured graph runs, and the handle keeps the buffer.
 struct DBuf {
     void *p = nullptr;
     size_t bytes = 0;
-    const cudaStream_t *owner = nullptr;
+    const OwnerStream *owner = nullptr;
+    bool plain = false;         // of cudaMalloc
     DBuf() = default;
     DBuf(const DBuf &) = delete;
     DBuf &operator=(const DBuf &) = delete;
@@ -71,9 +104,20 @@ struct DBuf {
     void alloc(size_t b) {
         release();
         if (b == 0) b = 16;
-        if (owner) TG_CK(cudaMallocFromPoolAsync(&p, b, device_pool(), *owner));
-        else TG_CK(cudaMalloc(&p, b));
+        plain = !owner || owner->captured;
+        const cudaError_t e = plain ? relaxed([&] { return cudaMalloc(&p, b); })
+                                    : cudaMallocFromPoolAsync(&p, b, device_pool(), owner->stream);
+        if (e != cudaSuccess) p = nullptr;
+        throw_cuda(e, "device memory of the handle");
         bytes = b;
+    }
+    // a copy of host memory, complete on return; after an error there is no buffer
+    void upload(const void *src, size_t b, cudaStream_t s) {
+        alloc(b);
+        cudaError_t e = b ? cudaMemcpyAsync(p, src, b, cudaMemcpyHostToDevice, s) : cudaSuccess;
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) release();
+        throw_cuda(e, "upload");
     }
     // for buffers that a captured batch points to: allocated once, and never
     // replaced while the handle lives
@@ -83,7 +127,7 @@ struct DBuf {
     }
     void release() {
         if (p) {
-            forget(owner ? cudaFreeAsync(p, *owner) : cudaFree(p));
+            forget(plain ? relaxed([&] { return cudaFree(p); }) : cudaFreeAsync(p, owner->stream));
         }
         p = nullptr;
         bytes = 0;
@@ -125,9 +169,8 @@ struct PaLayout {
     int64_t boff[10] = {0};             // first class of each global block; boff[9] = G
 };
 
-struct Graph {
+struct Graph : OwnerStream {
     int device = 0;
-    cudaStream_t stream = nullptr;      // stream of the last call
     int32_t ngraphs = 1, L = 1;
     int64_t n = 0, nnz = 0, m = 0;
     int64_t max_graph_nodes = 0;
@@ -251,7 +294,7 @@ struct Graph {
         return c;
     }
     Graph() {
-        for (DBuf *b : buffers()) b->owner = &stream;
+        for (DBuf *b : buffers()) b->owner = this;
     }
     std::vector<DBuf *> buffers() {
         std::vector<DBuf *> v;

@@ -480,7 +480,7 @@ void prepare_hubs(Graph &G, cudaStream_t s) {
     std::vector<std::unique_ptr<Graph::HubPlan>> plans;     // the handle gets all of them or, on an error, none
     for (size_t c = 0; c < G.chunks.size(); ++c) {
         auto plan = std::make_unique<Graph::HubPlan>();
-        for (DBuf *d : {&plan->segs, &plan->groups, &plan->ntick, &plan->ctr}) d->owner = &G.stream;
+        for (DBuf *d : {&plan->segs, &plan->groups, &plan->ntick, &plan->ctr}) d->owner = &G;
         std::vector<HubGroup> &groups = plan->h_groups;
         std::vector<int64_t> &ntick = plan->h_ntick;
         auto below = [&](int64_t n) {                       // hubs of earlier graphs (hub order is by graph first)

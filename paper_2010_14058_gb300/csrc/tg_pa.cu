@@ -214,12 +214,10 @@ void prepare_position_aware(Graph &G, cudaStream_t s) {
         const PaLayout Y = pa_layout(G.L);
         const std::vector<int32_t> table = pa_class_table(Y);
         G.pa = Y;
-        G.pa_cls.alloc(table.size() * sizeof(int32_t));
-        TG_CK(cudaMemcpyAsync(G.pa_cls.p, table.data(), table.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-        TG_CK(cudaStreamSynchronize(s));                   // the table lives on this stack frame
+        G.pa_cls.upload(table.data(), table.size() * sizeof(int32_t), s);
     }
     const size_t gbytes = (size_t)G.ngraphs * G.pa.G * sizeof(unsigned long long);
-    if (G.pa_gacc.bytes < gbytes) G.pa_gacc.alloc(gbytes);
+    G.pa_gacc.alloc_once(gbytes);
     prepare_epi4_pa(G);
 }
 

@@ -77,14 +77,14 @@ int64_t count_sparse(Graph &G, int k, int64_t *row_off, uint16_t *slot, uint32_t
     const int64_t m = G.m;
     const int64_t window = std::max<int64_t>(1, std::min<int64_t>(m, (int64_t)(kWindowBytes / (S * sizeof(uint32_t)))));
     DBuf dense, cnt, local;
-    dense.owner = cnt.owner = local.owner = &G.stream;
+    dense.owner = cnt.owner = local.owner = &G;
     dense.alloc((size_t)window * S * sizeof(uint32_t));
     cnt.alloc((size_t)(window + 1) * sizeof(int64_t));
     local.alloc((size_t)(window + 1) * sizeof(int64_t));
     size_t tb = 0;
     TG_CK(cub::DeviceScan::ExclusiveSum(nullptr, tb, cnt.as<int64_t>(), local.as<int64_t>(), window + 1, s));
     DBuf tmp;
-    tmp.owner = &G.stream;
+    tmp.owner = &G;
     tmp.alloc(std::max<size_t>(tb, 16));
     G.prepared_k = 0;                                     // fresh triangle and wedge passes
     int64_t base = 0;

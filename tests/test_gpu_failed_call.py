@@ -3,13 +3,12 @@ what the failed call had not launched is launched by the next one.  The
 failures are the runtime's own: capturing the legacy stream, and synchronising
 a stream that is being captured, both of which it refuses; no kernel of the
 failed calls runs."""
-import ctypes
-
 import numpy as np
 import pytest
 
 import graphgen
 import oracle
+from capture import captured
 
 pytestmark = pytest.mark.gpu
 
@@ -20,30 +19,12 @@ if not torch.cuda.is_available():
 import paper_2010_14058_gb300 as tg  # noqa: E402
 
 LEGACY = 1                                                   # cudaStreamLegacy
-RELAXED = 2                                                  # cudaStreamCaptureModeRelaxed
-
-
-def cudart():
-    for name in ("libcudart.so.13", "/usr/local/cuda/lib64/libcudart.so"):
-        try:
-            return ctypes.CDLL(name)
-        except OSError:
-            pass
-    pytest.skip("needs the CUDA runtime as a shared library")
 
 
 def failing_range(h, out, totals, s):
     """A range whose tiles are copied and synchronised while `s` is captured."""
-    rt, handle, graph = cudart(), ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
-    assert rt.cudaStreamBeginCapture(handle, RELAXED) == 0
-    try:
-        with pytest.raises(tg.TGError):
-            tg.tg_count_range(h, 4, 1, h.m - 1, out, totals, stream=s)
-    finally:
-        rt.cudaStreamEndCapture(handle, ctypes.byref(graph))
-        if graph.value:
-            rt.cudaGraphDestroy(graph)
-        rt.cudaGetLastError()
+    with captured(s), pytest.raises(tg.TGError):
+        tg.tg_count_range(h, 4, 1, h.m - 1, out, totals, stream=s)
 
 
 @pytest.fixture(scope="module")
