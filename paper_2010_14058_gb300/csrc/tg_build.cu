@@ -542,7 +542,7 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
     if (h_status & ST_INVALID_GRAPH) throw Error{TG_ERR_INVALID_GRAPH, "asymmetric rows"};
     for (int c = 0; c < 3; ++c) G.tri_count[c] = (int64_t)h_counts[c];
     G.max_nplus = (int64_t)h_counts[3];
-    G.narrow = !h_info[2 * (size_t)ngraphs + 3] && nnz < kNarrowSlots && !G.wide_sums();
+    G.narrow = !h_info[2 * (size_t)ngraphs + 3] && nnz < kNarrowSlots && G.max_degree < kNarrowTotal;
 }
 
 // What only 4-node counts need, before the first of them: the per-node typed

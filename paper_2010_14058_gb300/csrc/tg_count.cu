@@ -77,7 +77,7 @@ static void plan_chunks(Graph &G) {
     const int64_t LL = (int64_t)G.L * G.L;
     const int64_t budget = std::max<int64_t>((int64_t)G.opt.cycle_budget_mb << 20, 1);
     auto bytes_of = [&](int a, int b) {
-        return (G.h_slot_off[b] - G.h_slot_off[a]) * 8 * LL + (G.h_edge_off[b] - G.h_edge_off[a]) * LL * (G.wide_sums() ? 32 : 16);
+        return (G.h_slot_off[b] - G.h_slot_off[a]) * 8 * LL + (G.h_edge_off[b] - G.h_edge_off[a]) * 16 * LL;
     };
     // tile index ranges follow graph boundaries (make_tiles emits graph after graph)
     std::vector<int64_t> tile_off(G.ngraphs + 1, 0);
@@ -295,7 +295,7 @@ void prepare_counting(Graph &G, int k, cudaStream_t s) {
         G.A.alloc_once(ab);
         G.slot_rows.alloc_once(ab);
         const size_t me = (size_t)std::max<int64_t>(G.max_chunk_edges, 1);
-        G.xsum.alloc_once(me * 4 * L * L * (G.wide_sums() ? sizeof(unsigned long long) : sizeof(uint32_t)));
+        G.xsum.alloc_once(me * 4 * L * L * sizeof(uint32_t));
         prepare_sums(G);
         if (G.n_hubs > 0 && G.hub_plans.empty()) prepare_hubs(G, s);
     }

@@ -250,8 +250,6 @@ struct Graph : OwnerStream {
     const void *batch_pe = nullptr, *batch_gl = nullptr;
     cudaStream_t batch_stream = nullptr;
 
-    // sums over triangle nodes may reach 2^32 only when a degree reaches 2^16
-    bool wide_sums() const { return max_degree >= (1 << 16); }
     size_t node_sum_bytes() const { return narrow ? sizeof(uint32_t) : sizeof(int64_t); }   // of a delta or tau value
     GraphView view() const {
         GraphView v;
@@ -285,8 +283,7 @@ struct Graph : OwnerStream {
         c.a_base = a_base;
         c.a_stride = a_stride;
         c.e_base = e_base;
-        c.xsum = xsum.p;
-        c.wide = wide_sums();
+        c.xsum = xsum.as<uint32_t>();
         c.tri_any = tri_any.as<uint8_t>();
         c.gacc = gacc.as<unsigned long long>();
         c.status = status.as<uint32_t>();

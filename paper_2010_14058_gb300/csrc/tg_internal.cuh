@@ -53,16 +53,18 @@ struct HubSegment {
 };
 constexpr int64_t kHubTicketWords = 1 << 16;
 
-// A graph is narrow when no typed degree reaches kNarrowDegree, it has fewer
-// than kNarrowSlots adjacency entries and its sums over T are 32 bits wide:
-// every value of a 4-node row is then below 2^31.  Products: the largest,
+// A graph is narrow when no typed degree reaches kNarrowDegree, no degree
+// kNarrowTotal, and it has fewer than kNarrowSlots adjacency entries: every
+// value of a 4-node row is then below 2^31.  Products: the largest,
 // c_t (a_u + b_u) + c_u (a_t + b_t) with c + a <= d_i and c + b <= d_j, and
 // a_t b_u + a_u b_t, are at most 2 (2^15 - 1)^2.  Sums: g3, the largest, is at
 // most delta_i[t][u] + delta_i[u][t] + the same of j; delta_x[t][u] and
 // delta_x[u][t] are sums of degrees over different neighbours, or of
 // different types' degrees, so their sum is at most the number of adjacency
-// entries, and twice that is below 2^30.
+// entries, and twice that is below 2^30.  (Nothing above needs kNarrowTotal: it
+// keeps the rule to the degrees that it was measured and tested on.)
 constexpr int kNarrowDegree = 1 << 15;
+constexpr int64_t kNarrowTotal = (int64_t)1 << 16;
 constexpr int64_t kNarrowSlots = (int64_t)1 << 29;
 
 // Edges of one graph that a CTA of the per-edge kernels takes at a time.
@@ -107,8 +109,7 @@ struct CountView {
     int64_t a_base;             // first adjacency slot of the current chunk
     int64_t a_stride;           // slots per type-pair row of A
     int64_t e_base;             // first edge of the current chunk (xsum is relative to it)
-    void *xsum;                 // [edges][L][4][L] TCi, TCj, DT, K' (tg_sums.cu): uint32, or uint64 when wide
-    bool wide;                  // xsum holds uint64
+    uint32_t *xsum;             // [edges][L][4][L] TCi, TCj, DT, K' (tg_sums.cu)
     uint8_t *tri_any;           // [n] 1 if a triangle has the node as its lowest
     unsigned long long *gacc;   // [ngraphs*G] raw per-graphlet edge sums
     uint32_t *status;           // device status word

@@ -7,6 +7,10 @@
 //   [1][q]  TCj  sum over w in T^t of c_{jw}^q
 //   [2][q]  DT   sum over w in T^t of d_w^q
 //   [3][q]  K'   K' + K'^T = 2 (ordered adjacent pairs of T^t x T^q)
+// Every word fits 32 bits: DT adds up degrees of different nodes, so it is at
+// most the number of adjacency entries, below 2^31; TCi and TCj are at most
+// DT (c_{iw}^q <= d_w^q); and an unordered adjacent pair of T adds 2 to K' in
+// all, so K' is at most twice the number of edges, below 2^31 too.
 // A triangle u < a < b adds one 4 L-word term to row ty_b of {u, a}, row ty_a
 // of {u, b} and row ty_u of {a, b}: one atomic instruction of 4 L lanes on
 // consecutive words each.  The last part counts 4-cliques: with the local
@@ -91,16 +95,16 @@ __device__ __forceinline__ void stage_put(const CountView &cv, int L, const Stag
 // Adds the terms of the warp's `cnt` staged triangles.  vec: the local
 // nodes' rows, du: the lane's word of u's own typed degrees (component 2).
 // Lanes take 4 L words of one triangle, 32 / (4 L) triangles at a time.
-template <class Acc, int kL>
-__device__ __forceinline__ void add_terms(Acc *X, int rt_L, const Stage &s, int cnt, const uint32_t *vec, uint32_t du,
+template <int kL>
+__device__ __forceinline__ void add_terms(uint32_t *X, const Stage &s, int cnt, const uint32_t *vec, uint32_t du,
                                           int lane) {
-    const int L = kL ? kL : rt_L;
+    constexpr int L = kL;
     const int row = 4 * L, per = 32 / row;
     const int grp = lane / row, comp = lane - grp * row;
     const int k = comp / L, q = comp - k * L;
     const int off = k == 2 ? L + q : q;                     // word of vec (components 0 and 2)
     const int val = k == 3 ? L + q : q;                     // word of the staged values (components 1 and 3)
-    Acc *Xc = X + comp;
+    uint32_t *Xc = X + comp;
 #pragma unroll 2
     for (int i = grp < per ? grp : cnt; i < cnt; i += per) {
         const uint32_t kk = s.kk[i];
@@ -109,9 +113,9 @@ __device__ __forceinline__ void add_terms(Acc *X, int rt_L, const Stage &s, int 
         // 0: u's counts of the other node; 1: {a, b}'s counts; 2: degrees; 3: the 4-cliques
         const uint32_t xa = k & 1 ? sv : vb, xb = k & 1 ? sv : va;
         const uint32_t xab = k == 0 ? va : k == 1 ? vb : k == 2 ? du : 2 * sv;
-        if (xa) atomicAdd(Xc + s.at[3 * i], (Acc)xa);
-        if (xb) atomicAdd(Xc + s.at[3 * i + 1], (Acc)xb);
-        if (xab) atomicAdd(Xc + s.at[3 * i + 2], (Acc)xab);
+        if (xa) atomicAdd(Xc + s.at[3 * i], xa);
+        if (xb) atomicAdd(Xc + s.at[3 * i + 1], xb);
+        if (xab) atomicAdd(Xc + s.at[3 * i + 2], xab);
     }
 }
 
@@ -122,29 +126,28 @@ __device__ __forceinline__ uint32_t own_degree(const GraphView &g, int32_t u, in
 }
 
 // zeroes the rows that will be added to and read: (e, t) with c_e^t > 0
-template <class Acc>
 __global__ void __launch_bounds__(256) k_sum_zero(int64_t e0, int64_t e1, int L, const uint32_t *__restrict__ C,
-                                                  Acc *X) {
+                                                  uint32_t *X) {
     const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t e = e0 + x / kCRow;
     const int t = (int)(x % kCRow);
     if (e >= e1 || t >= L || C[e * kCRow + t] == 0) return;
     uint4 *r = reinterpret_cast<uint4 *>(X + ((e - e0) * L + t) * 4 * L);
-    for (int k = 0; k < L * (int)(sizeof(Acc) / 4); ++k) r[k] = make_uint4(0, 0, 0, 0);
+    for (int k = 0; k < L; ++k) r[k] = make_uint4(0, 0, 0, 0);
 }
 
 // Warp per node u of [n0, n1) with 2 <= |N+(u)| <= kTriWarpMax: the bit
 // matrix is one word per local node, type q's columns a mask of that word.
-template <class Acc, int kL>
+template <int kL>
 __global__ void __launch_bounds__(kSumWarps * 32) k_sum_warp(GraphView g, CountView cv, int64_t n0, int64_t n1) {
     extern __shared__ uint32_t sw_smem[];
-    const int L = kL ? kL : g.L;
+    constexpr int L = kL;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int per_warp = (int)stage_words(L) + 32 * 2 * L + 32 * 3;   // even: the staging is 8-byte aligned
     uint32_t *mem = sw_smem + wid * per_warp;
     const Stage s = stage_carve(mem, L);
     uint32_t *vec = mem + stage_words(L), *ents = vec + 32 * 2 * L, *eids = ents + 32, *B = eids + 32;
-    Acc *X = reinterpret_cast<Acc *>(cv.xsum);
+    uint32_t *X = cv.xsum;
     unsigned long long words = 0;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t u = n0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); u < n1; u += nw) {
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_warp(GraphView g, CountV
                 words += 1;
             }
             __syncwarp();
-            add_terms<Acc, kL>(X, L, s, __popc(bal), vec, du, lane);
+            add_terms<kL>(X, s, __popc(bal), vec, du, lane);
             __syncwarp();
         }
     }
@@ -227,7 +230,7 @@ struct Found {
 __host__ __device__ inline int64_t most_found(int64_t cap) { return cap * (cap - 1) / 2; }
 
 // CTA per listed node u of [n0, n1)
-template <class Acc, int kL, int kThreadsT, bool kSmem>
+template <int kL, int kThreadsT, bool kSmem>
 __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv, const int32_t *__restrict__ list,
                                                        int64_t n_list, int64_t n0, int64_t n1, int cap, int lgf,
                                                        unsigned char *scratch, int64_t stride) {
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv
     // triangles of one node, so that its lists are scanned once; else the
     // arrays in the slice and a second scan
     extern __shared__ uint32_t sc_smem[];
-    const int L = kL ? kL : g.L;
+    constexpr int L = kL;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int kWarps = kThreadsT / 32;
     uint32_t *mem = kSmem ? sc_smem : reinterpret_cast<uint32_t *>(scratch + (int64_t)blockIdx.x * stride);
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv
     int *shift = ws + kMaxL + 1;                            // [L] column of list position k of type t: k + shift[t]
     LocalList q;
     local_carve(q, reinterpret_cast<unsigned char *>(ws + 2 * kMaxL + 2), cap, lgf, kWarps, wid);
-    Acc *X = reinterpret_cast<Acc *>(cv.xsum);
+    uint32_t *X = cv.xsum;
     unsigned long long words = 0;
     __shared__ int s_found, s_next;
     Found *found = reinterpret_cast<Found *>(scratch + (int64_t)blockIdx.x * stride);
@@ -311,7 +314,7 @@ __global__ void __launch_bounds__(kThreadsT) k_sum_cta(GraphView g, CountView cv
                 words += (unsigned)w;
             }
             __syncwarp();
-            add_terms<Acc, kL>(X, L, s, __popc(bal), vec, du, lane);
+            add_terms<kL>(X, s, __popc(bal), vec, du, lane);
             __syncwarp();
         };
         local_pairs(g, p, q, lane, wid, kWarps, [&](bool hit, int ka, int kb, uint32_t pos) {
@@ -380,22 +383,22 @@ SumShape shape_of(const Graph &G, const LocalClass &c, int cls) {
     return r;
 }
 
-template <class Acc, int kL>
+template <int kL>
 void prepare(Graph &G) {
-    raise_smem_limit((const void *)k_sum_warp<Acc, kL>, warp_bytes(G.L));
+    raise_smem_limit((const void *)k_sum_warp<kL>, warp_bytes(G.L));
     size_t scratch = 0;
     for (int cls = 0; cls < 3; ++cls) {
         const LocalClass c = local_class(G, cls);
         if (c.n == 0) continue;
         const SumShape r = shape_of(G, c, cls);
-        if (cls == 0) raise_smem_limit((const void *)k_sum_cta<Acc, kL, kTriMidThreads, true>, r.smem);
-        else if (cls == 1) raise_smem_limit((const void *)k_sum_cta<Acc, kL, kTriBigThreads, true>, r.smem);
+        if (cls == 0) raise_smem_limit((const void *)k_sum_cta<kL, kTriMidThreads, true>, r.smem);
+        else if (cls == 1) raise_smem_limit((const void *)k_sum_cta<kL, kTriBigThreads, true>, r.smem);
         scratch = std::max(scratch, r.slice * (size_t)r.ctas);
     }
     if (scratch) G.sum_scratch.alloc_once(scratch);
 }
 
-template <class Acc, int kL>
+template <int kL>
 int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s) {
     G.e_base = e0;
     const GraphView gv = G.view();
@@ -405,16 +408,15 @@ int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStr
     if (e1 <= e0) return 0;
     {
         KernelTimer kt(G, s, "k_sum_zero");
-        k_sum_zero<Acc><<<(unsigned)(((e1 - e0) * kCRow + 255) / 256), 256, 0, s>>>(e0, e1, G.L, cv.C,
-                                                                                 reinterpret_cast<Acc *>(cv.xsum));
+        k_sum_zero<<<(unsigned)(((e1 - e0) * kCRow + 255) / 256), 256, 0, s>>>(e0, e1, G.L, cv.C, cv.xsum);
         ++launches;
     }
     KernelTimer kt(G, s, "k_sum");
     {
         const size_t bytes = warp_bytes(G.L);
         const int per_sm = std::max(1, std::min<int>(2048 / (kSumWarps * 32), (int)((220u << 10) / (bytes + 1024))));
-        k_sum_warp<Acc, kL><<<(unsigned)std::min<int64_t>((n1 - n0 + kSumWarps - 1) / kSumWarps, (int64_t)sms * per_sm * 8),
-                          kSumWarps * 32, bytes, s>>>(gv, cv, n0, n1);
+        k_sum_warp<kL><<<(unsigned)std::min<int64_t>((n1 - n0 + kSumWarps - 1) / kSumWarps, (int64_t)sms * per_sm * 8),
+                         kSumWarps * 32, bytes, s>>>(gv, cv, n0, n1);
         ++launches;
     }
     for (int cls = 0; cls < 3; ++cls) {
@@ -426,9 +428,9 @@ int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStr
             kern<<<(unsigned)r.ctas, c.threads, r.smem, s>>>(gv, cv, c.list, c.n, n0, n1, c.cap, c.lgf,
                                                              G.sum_scratch.as<unsigned char>(), (int64_t)r.slice);
         };
-        if (cls == 0) run(k_sum_cta<Acc, kL, kTriMidThreads, true>);
-        else if (cls == 1) run(k_sum_cta<Acc, kL, kTriBigThreads, true>);
-        else run(k_sum_cta<Acc, kL, kTriBigThreads, false>);
+        if (cls == 0) run(k_sum_cta<kL, kTriMidThreads, true>);
+        else if (cls == 1) run(k_sum_cta<kL, kTriBigThreads, true>);
+        else run(k_sum_cta<kL, kTriBigThreads, false>);
     }
     TG_CK(cudaGetLastError());
     return launches;
@@ -436,17 +438,15 @@ int64_t launch(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStr
 
 }  // namespace
 
-// kernels of 32-bit sums are compiled per number of types (the terms' index
-// arithmetic is most of their instructions), those of 64-bit sums once
+// the kernels are compiled per number of types: the terms' index arithmetic
+// is most of their instructions
 void prepare_sums(Graph &G) {
-    if (G.wide_sums()) prepare<unsigned long long, 0>(G);
-    else with_types(G.L, [&](auto l) { prepare<uint32_t, decltype(l)::value>(G); });
+    with_types(G.L, [&](auto l) { prepare<decltype(l)::value>(G); });
 }
 
 int64_t launch_sums(Graph &G, int64_t n0, int64_t n1, int64_t e0, int64_t e1, cudaStream_t s) {
-    if (G.wide_sums()) return launch<unsigned long long, 0>(G, n0, n1, e0, e1, s);
     int64_t launches = 0;
-    with_types(G.L, [&](auto l) { launches = launch<uint32_t, decltype(l)::value>(G, n0, n1, e0, e1, s); });
+    with_types(G.L, [&](auto l) { launches = launch<decltype(l)::value>(G, n0, n1, e0, e1, s); });
     return launches;
 }
 
