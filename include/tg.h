@@ -32,6 +32,8 @@
  * Streams: every call that takes `stream` (a cudaStream_t, NULL = legacy
  *   default stream) is stream-ordered.  Device outputs are complete when the
  *   stream reaches the call's end.
+ *   Kernels of one 4-node count that do not depend on each other run on
+ *   streams of the library's beside it, of the same priority as `stream`.
  *
  * Edge ids: the edges {u,v}, u < v in the caller's node ids, numbered
  *   0..m-1 in lexicographic order of (u,v).  For a batch (tg_build_batch)

@@ -45,6 +45,7 @@
 #include <mutex>
 
 #include "tg_host.hpp"
+#include "tg_side.hpp"
 
 namespace tg {
 
@@ -144,91 +145,6 @@ void prepare_edges(Graph &G, int k, cudaStream_t s) {
     int64_t nt = 0;
     tiles_for(G, 0, G.m, nt, unused, s);
 }
-
-// Side streams of one count call: the wedge forms and the triangle kernels do
-// not depend on each other and run beside each other, since on a small graph
-// none of them fills the GPU and on a large one each ends in a tail.  A set
-// is taken for the call and given back once the joins are enqueued (what a
-// later call enqueues on it comes after); the process keeps at most kKeep
-// sets per device, more exist only while that many calls run at once.
-class SideStreams {
-public:
-    static constexpr int kSides = 3;
-    explicit SideStreams(cudaStream_t main) : main_(main) {
-        TG_CK(cudaGetDevice(&dev_));
-        {
-            std::lock_guard<std::mutex> lock(mutex());
-            auto &pool = free_sets();
-            for (size_t k = 0; k < pool.size() && !set_; ++k)
-                if (pool[k]->dev == dev_) {
-                    set_ = std::move(pool[k]);
-                    pool.erase(pool.begin() + (std::ptrdiff_t)k);
-                }
-        }
-        if (!set_) {
-            set_ = std::make_unique<Set>();
-            set_->dev = dev_;
-            for (auto &x : set_->s) TG_CK(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
-            for (auto &x : set_->ev) TG_CK(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
-        }
-    }
-    ~SideStreams() {
-        if (forked_) {                                      // an error between fork and join: nothing may still run
-            for (cudaStream_t x : set_->s) forget(cudaStreamSynchronize(x));   // when the caller gives its buffers back
-            return;
-        }
-        std::lock_guard<std::mutex> lock(mutex());
-        size_t kept = 0;
-        for (const auto &x : free_sets()) kept += x->dev == dev_ ? 1 : 0;
-        if (kept < kKeep) free_sets().push_back(std::move(set_));
-    }
-    cudaStream_t side(int k) const { return set_->s[k]; }
-    // the sides start after what the main stream has so far
-    void fork() {
-        forked_ = true;
-        TG_CK(cudaEventRecord(set_->ev[0], main_));
-        for (cudaStream_t x : set_->s) TG_CK(cudaStreamWaitEvent(x, set_->ev[0], 0));
-    }
-    // side k goes on after what the main stream has so far
-    void after_main(int k) {
-        TG_CK(cudaEventRecord(set_->ev[1], main_));
-        TG_CK(cudaStreamWaitEvent(set_->s[k], set_->ev[1], 0));
-    }
-    // the main stream goes on after the sides
-    void join() {
-        for (int k = 0; k < kSides; ++k) {
-            TG_CK(cudaEventRecord(set_->ev[2 + k], set_->s[k]));
-            TG_CK(cudaStreamWaitEvent(main_, set_->ev[2 + k], 0));
-        }
-        forked_ = false;
-    }
-
-private:
-    struct Set {
-        int dev = 0;
-        cudaStream_t s[kSides] = {};
-        cudaEvent_t ev[2 + kSides] = {};
-        ~Set() {                                            // (work enqueued on them completes all the same)
-            for (cudaStream_t x : s)
-                if (x) forget(cudaStreamDestroy(x));
-            for (cudaEvent_t x : ev)
-                if (x) forget(cudaEventDestroy(x));
-        }
-    };
-    static constexpr size_t kKeep = 8;
-    static std::mutex &mutex() {
-        static std::mutex *m = new std::mutex();
-        return *m;
-    }
-    static std::vector<std::unique_ptr<Set>> &free_sets() {   // never destroyed: the CUDA context may go first
-        static auto *v = new std::vector<std::unique_ptr<Set>>();
-        return *v;
-    }
-    cudaStream_t main_;
-    int dev_ = 0;
-    bool forked_ = false;
-    std::unique_ptr<Set> set_;
-};
 
 // Sums and 4-cycle slots of chunk ci, after the triangles of the whole graph
 // when `triangles` (their per-node sums included).  The kernels run beside

@@ -12,26 +12,10 @@
 #include <cuda_runtime.h>
 
 #include "tg.h"
+#include "tg_error.hpp"
 #include "tg_internal.cuh"
 
 namespace tg {
-
-// Internal error carrying a tg_status; caught at every extern "C" entry.
-struct Error {
-    tg_status status;
-    const char *what;
-    bool from_cuda = false;     // message already recorded by throw_cuda
-};
-
-// Text of the calling thread's last failed entry (tg_last_error).
-inline thread_local char tl_last_error[256] = "";
-
-inline void throw_cuda(cudaError_t e, const char *what) {
-    if (e == cudaSuccess) return;
-    (void)cudaGetLastError();   // clear the sticky-free error state
-    std::snprintf(tl_last_error, sizeof tl_last_error, "%s: %s", what, cudaGetErrorString(e));
-    throw Error{e == cudaErrorMemoryAllocation ? TG_ERR_OOM : TG_ERR_CUDA, what, true};
-}
 
 // Raises (never lowers) a kernel's dynamic shared-memory limit.  The limit
 // is a process-wide attribute of the function, so handles counted
@@ -42,14 +26,6 @@ void raise_smem_limit(const void *func, size_t bytes);
 // Largest light_anchor_max_wedges whose per-warp hashes of k_wedge_light fit
 // one CTA's shared memory for L types.  Defined in tg_wedge.cu.
 int light_anchor_limit(int L);
-
-#define TG_CK(call) ::tg::throw_cuda((call), #call)
-
-// For calls of destructors, which may run because an earlier call failed: an
-// error of theirs must not be what the next entry's cudaGetLastError finds.
-inline void forget(cudaError_t e) {
-    if (e != cudaSuccess) (void)cudaGetLastError();
-}
 
 // Stream-ordered memory pool of the current device, owned by the library
 // (release threshold kept at its maximum, so freed blocks are reused instead
