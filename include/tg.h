@@ -123,7 +123,9 @@ typedef struct {
                                          or a hub table) */
     int32_t ctas_per_sm;              /* resident CTAs per SM for the per-edge kernels */
     int32_t cycle_budget_mb;          /* device memory for the per-slot 4-cycle array; a batch whose
-                                         array would exceed it is counted in chunks of whole graphs */
+                                         array would exceed it is counted in chunks of whole graphs, and
+                                         directed and edge-typed counts whose triangle cells would exceed
+                                         four times as much in windows of edges */
     int32_t hub_min_wedges;           /* anchors with more wedges than this, or than a CTA's shared memory
                                          holds, are hubs: each is counted by the whole GPU against one
                                          node table shared by all CTAs */

@@ -185,11 +185,14 @@ __global__ void k_arc_labels(GraphView g, const int8_t *__restrict__ sign, const
 // ---------------------------------------------------------------- count
 // cells [edge][type of the third node][sign at lower endpoint - ? 2 : 0 |
 // sign at higher endpoint - ? 1 : 0]
+template <bool kWindow>
 struct DirectedCells {
-    uint32_t *cell;
+    uint32_t *cell;                                         // of edge 0 (the array starts at e0's)
     const uint8_t *lab;
     int L;
+    int64_t e0, e1;                                         // kWindow: edges with cells
     __device__ __forceinline__ void add(int64_t e, int t, bool minus_lo, bool minus_hi) const {
+        if (kWindow && (e < e0 || e >= e1)) return;
         atomicAdd(&cell[(e * L + t) * 4 + (minus_lo ? 2 : 0) + (minus_hi ? 1 : 0)], 1u);
     }
     __device__ __forceinline__ void operator()(int64_t ua, int64_t ub, int64_t ab, int tu, int ta, int tb) const {
@@ -211,15 +214,16 @@ __global__ void __launch_bounds__(kRowThreads) k_directed_rows(GraphView g, cons
                                                                const uint8_t *__restrict__ lab,
                                                                const int32_t *__restrict__ outdeg,
                                                                const int32_t *__restrict__ slot_class, int G,
-                                                               int64_t tile, uint32_t *per_edge_out,
+                                                               int64_t tile, int64_t e0, int64_t e1,
+                                                               uint32_t *per_edge_out,
                                                                unsigned long long *gacc, uint32_t *status) {
     constexpr int LL = L * L, E = kRowThreads / L;
     extern __shared__ unsigned long long dhist[];
     __shared__ TileOrder<2 * LL> o;
     for (int s = threadIdx.x; s < G; s += blockDim.x) dhist[s] = 0;
     const int slice = threadIdx.x / L, t = threadIdx.x % L;
-    for (int64_t b = blockIdx.x * tile; b < g.m; b += gridDim.x * tile) {
-        const int n = (int)min(tile, g.m - b);
+    for (int64_t b = e0 + blockIdx.x * tile; b < e1; b += gridDim.x * tile) {
+        const int n = (int)min(tile, e1 - b);
         // key ((phi_i * L + phi_j) * 2 + o), o = 0: i -> j
         tile_order(b, n, o, [&](int64_t e) {
             const int l = lab[e];
@@ -372,24 +376,29 @@ int64_t run_directed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, cud
     const size_t smem = sizeof(unsigned long long) * (size_t)Gs;
     int64_t launches = 0;
     if (G.m > 0) {
-        const size_t bytes = sizeof(uint32_t) * 4 * (size_t)G.L * (size_t)G.m;
-        G.dcell.alloc_once(bytes);
-        {
-            KernelTimer kt(G, s, "k_directed_cells");
-            TG_CK(cudaMemsetAsync(G.dcell.p, 0, bytes, s));
-            launches += visit_triangles(G, DirectedCells{G.dcell.as<uint32_t>(), G.dlab.as<uint8_t>(), G.L}, s);
-        }
-        KernelTimer kt(G, s, "k_directed_rows");
+        const size_t edge_bytes = sizeof(uint32_t) * 4 * (size_t)G.L;
+        const int64_t window = cell_window(G, G.dcell, edge_bytes);
         const int64_t tile = tile_edges(G);
-        const unsigned grid = (unsigned)std::min<int64_t>((G.m + tile - 1) / tile, (int64_t)sm_count() * 6);
-        with_types(G.L, [&](auto l) {
-            constexpr int L = decltype(l)::value;
-            raise_smem_limit((const void *)k_directed_rows<L>, smem);
-            k_directed_rows<L><<<grid, kRowThreads, smem, s>>>(
-                G.view(), G.dcell.as<uint32_t>(), G.dlab.as<uint8_t>(), G.doutdeg.as<int32_t>(), G.dcls.as<int32_t>(), Gs,
-                tile, per_edge_out, G.dgacc.as<unsigned long long>(), G.status.as<uint32_t>());
-        });
-        ++launches;
+        for (int64_t e0 = 0; e0 < G.m; e0 += window) {
+            const int64_t e1 = std::min(G.m, e0 + window);
+            uint32_t *cell = G.dcell.as<uint32_t>() - e0 * 4 * G.L;
+            {
+                KernelTimer kt(G, s, "k_directed_cells");
+                TG_CK(cudaMemsetAsync(G.dcell.p, 0, edge_bytes * (size_t)(e1 - e0), s));
+                if (window >= G.m) launches += visit_triangles(G, DirectedCells<false>{cell, G.dlab.as<uint8_t>(), G.L, e0, e1}, s);
+                else launches += visit_triangles(G, DirectedCells<true>{cell, G.dlab.as<uint8_t>(), G.L, e0, e1}, s);
+            }
+            KernelTimer kt(G, s, "k_directed_rows");
+            const unsigned grid = (unsigned)std::min<int64_t>((e1 - e0 + tile - 1) / tile, (int64_t)sm_count() * 6);
+            with_types(G.L, [&](auto l) {
+                constexpr int L = decltype(l)::value;
+                raise_smem_limit((const void *)k_directed_rows<L>, smem);
+                k_directed_rows<L><<<grid, kRowThreads, smem, s>>>(
+                    G.view(), cell, G.dlab.as<uint8_t>(), G.doutdeg.as<int32_t>(), G.dcls.as<int32_t>(), Gs, tile, e0, e1,
+                    per_edge_out, G.dgacc.as<unsigned long long>(), G.status.as<uint32_t>());
+            });
+            ++launches;
+        }
     }
     if (global_out) {
         k_directed_finalize<<<(unsigned)((Gs + 255) / 256), 256, 0, s>>>(Gs, G.L * G.L, G.dgacc.as<unsigned long long>(),

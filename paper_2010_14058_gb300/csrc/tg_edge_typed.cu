@@ -137,16 +137,22 @@ __device__ __forceinline__ int x_pair(int X, int x, int y) {
 }
 
 // cells [edge][type of the third node][pair of its edges' types]
+template <bool kWindow>
 struct EdgeTypedCells {
-    uint32_t *cell;
+    uint32_t *cell;             // of edge 0 (the array starts at e0's)
     int64_t stride;             // words from edge to edge
     const uint8_t *xi;
     int X, P;
+    int64_t e0, e1;             // kWindow: edges with cells
+    __device__ __forceinline__ void add(int64_t e, int slot) const {
+        if (kWindow && (e < e0 || e >= e1)) return;
+        atomicAdd(&cell[e * stride + slot], 1u);
+    }
     __device__ __forceinline__ void operator()(int64_t ua, int64_t ub, int64_t ab, int tu, int ta, int tb) const {
         const int xa = xi[ua], xb = xi[ub], xab = xi[ab];
-        atomicAdd(&cell[ua * stride + tb * P + x_pair(X, xb, xab)], 1u);
-        atomicAdd(&cell[ub * stride + ta * P + x_pair(X, xa, xab)], 1u);
-        atomicAdd(&cell[ab * stride + tu * P + x_pair(X, xa, xb)], 1u);
+        add(ua, tb * P + x_pair(X, xb, xab));
+        add(ub, ta * P + x_pair(X, xa, xab));
+        add(ab, tu * P + x_pair(X, xa, xb));
     }
 };
 
@@ -171,6 +177,7 @@ template <int L, int X>
 __global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, const uint32_t *__restrict__ cell,
                                                                  int64_t stride, const uint8_t *__restrict__ xi,
                                                                  const int32_t *__restrict__ etdeg, int G, int64_t tile,
+                                                                 int64_t e0, int64_t e1,
                                                                  uint32_t *per_edge_out,
                                                                  unsigned long long *gacc, uint32_t *status) {
     extern __shared__ unsigned long long ehist[];
@@ -210,8 +217,8 @@ __global__ void __launch_bounds__(kRowThreads) k_edge_typed_rows(GraphView g, co
     }
 #pragma unroll
     for (int z = 0; z < X; ++z) x_at[z] = x_pair(X, x0, z);
-    for (int64_t b = blockIdx.x * tile; b < g.m; b += gridDim.x * tile) {
-        const int n = (int)min(tile, g.m - b);
+    for (int64_t b = e0 + blockIdx.x * tile; b < e1; b += gridDim.x * tile) {
+        const int n = (int)min(tile, e1 - b);
         tile_order(b, n, o, [&](int64_t e) { return (g.ty[g.e_lo[e]] * L + g.ty[g.e_hi[e]]) * X + xi[e]; });
         for (int x = threadIdx.x; x < n; x += blockDim.x) {
             const int64_t e = b + o.order[x];
@@ -331,35 +338,37 @@ int64_t run_edge_typed3(Graph &G, uint32_t *per_edge_out, int64_t *global_out, c
     if (G.m > 0) {
         const int P = X * (X + 1) / 2, S = L * X + L * P;
         // the rows hold the cells; without rows, a buffer of the handle
-        uint32_t *cell = per_edge_out ? per_edge_out + L * X : nullptr;
         const int64_t stride = per_edge_out ? S : L * P;
-        if (!cell) {
-            G.etcell.alloc_once(sizeof(uint32_t) * (size_t)(stride * G.m));
-            cell = G.etcell.as<uint32_t>();
-        }
-        {
-            KernelTimer kt(G, s, "k_edge_typed_cells");
-            k_et_zero<<<(unsigned)std::min<int64_t>((G.m + 7) / 8, (int64_t)sm_count() * 64), 256, 0, s>>>(
-                G.m, stride, L * P, cell);
-            launches += 1 + visit_triangles(G, EdgeTypedCells{cell, stride, G.etype.as<uint8_t>(), X, P}, s);
-        }
-        KernelTimer kt(G, s, "k_edge_typed_rows");
+        const int64_t window = per_edge_out ? G.m : cell_window(G, G.etcell, sizeof(uint32_t) * (size_t)stride);
         const int64_t tile = tile_edges(G);
-        const unsigned grid = (unsigned)std::min<int64_t>((G.m + tile - 1) / tile, (int64_t)sm_count() * 6);
-        with_types(L, [&](auto l) {
-            constexpr int kL = decltype(l)::value;
-            auto run = [&](auto kern) {
-                raise_smem_limit((const void *)kern, smem);
-                kern<<<grid, kRowThreads, smem, s>>>(G.view(), cell, stride, G.etype.as<uint8_t>(), G.etdeg.as<int32_t>(),
-                                                     Gs, tile, per_edge_out, G.etgacc.as<unsigned long long>(),
-                                                     G.status.as<uint32_t>());
-            };
-            if (X == 1) run(k_edge_typed_rows<kL, 1>);
-            else if (X == 2) run(k_edge_typed_rows<kL, 2>);
-            else if (X == 3) run(k_edge_typed_rows<kL, 3>);
-            else run(k_edge_typed_rows<kL, 4>);
-        });
-        ++launches;
+        for (int64_t e0 = 0; e0 < G.m; e0 += window) {
+            const int64_t e1 = std::min(G.m, e0 + window);
+            uint32_t *first = per_edge_out ? per_edge_out + L * X : G.etcell.as<uint32_t>(), *cell = first - e0 * stride;
+            {
+                KernelTimer kt(G, s, "k_edge_typed_cells");
+                k_et_zero<<<(unsigned)std::min<int64_t>((e1 - e0 + 7) / 8, (int64_t)sm_count() * 64), 256, 0, s>>>(
+                    e1 - e0, stride, L * P, first);
+                const uint8_t *xi = G.etype.as<uint8_t>();
+                if (window >= G.m) launches += 1 + visit_triangles(G, EdgeTypedCells<false>{cell, stride, xi, X, P, e0, e1}, s);
+                else launches += 1 + visit_triangles(G, EdgeTypedCells<true>{cell, stride, xi, X, P, e0, e1}, s);
+            }
+            KernelTimer kt(G, s, "k_edge_typed_rows");
+            const unsigned grid = (unsigned)std::min<int64_t>((e1 - e0 + tile - 1) / tile, (int64_t)sm_count() * 6);
+            with_types(L, [&](auto l) {
+                constexpr int kL = decltype(l)::value;
+                auto run = [&](auto kern) {
+                    raise_smem_limit((const void *)kern, smem);
+                    kern<<<grid, kRowThreads, smem, s>>>(G.view(), cell, stride, G.etype.as<uint8_t>(), G.etdeg.as<int32_t>(),
+                                                         Gs, tile, e0, e1, per_edge_out, G.etgacc.as<unsigned long long>(),
+                                                         G.status.as<uint32_t>());
+                };
+                if (X == 1) run(k_edge_typed_rows<kL, 1>);
+                else if (X == 2) run(k_edge_typed_rows<kL, 2>);
+                else if (X == 3) run(k_edge_typed_rows<kL, 3>);
+                else run(k_edge_typed_rows<kL, 4>);
+            });
+            ++launches;
+        }
     }
     if (global_out) {
         const int64_t off1 = mchoose(L, 2) * X, off2 = off1 + mchoose(L, 3) * mchoose(X, 2);

@@ -12,6 +12,7 @@
 
 #include "tg_host.hpp"
 #include "tg_local.cuh"
+#include "tg_visit.cuh"
 
 namespace tg {
 
@@ -248,6 +249,25 @@ LocalClass local_class(const Graph &G, int cls) {
 
 static size_t tri_bytes(const Graph &G, const LocalClass &c) {
     return ((size_t)c.cap * G.L * 4 + local_bytes(c.cap, c.lgf, c.threads / 32) + 15) & ~(size_t)15;
+}
+
+int64_t cell_window(Graph &G, DBuf &cells, size_t edge_bytes) {
+    if (!cells.p) {
+        const int64_t budget = std::max<int64_t>((int64_t)G.opt.cycle_budget_mb << 22, 1);
+        int64_t n = std::min<int64_t>(G.m, std::max<int64_t>(budget / (int64_t)edge_bytes, kTile));
+        for (;;) {
+            try {
+                cells.alloc(edge_bytes * (size_t)n);
+                break;
+            } catch (const Error &e) {                      // no room: half as many edges at a time
+                if (e.status != TG_ERR_OOM || n <= kTile) throw;
+                n = std::max<int64_t>((n + 1) / 2, kTile);
+            }
+        }
+    }
+    const int64_t most = (int64_t)(cells.bytes / edge_bytes);
+    const int64_t windows = (G.m + most - 1) / most;
+    return (G.m + windows - 1) / windows;
 }
 
 void prepare_tri_scratch(Graph &G) {

@@ -72,6 +72,13 @@ __global__ void __launch_bounds__(kThreadsT) k_visit_cta(GraphView g, V v, const
     }
 }
 
+// Edges whose cells are counted together: all of them where their cells fit
+// four times the handle's working budget (cycle_budget_mb) and device memory
+// has room, else windows of equal numbers of edges, each with a visit of the
+// triangles of its own (a functor of a window passes other edges by).
+// Allocates `cells` at the handle's first such count.
+int64_t cell_window(Graph &G, DBuf &cells, size_t edge_bytes);
+
 // launches the functor over every triangle of the handle's graph; returns the launches
 template <class V>
 int64_t visit_triangles(Graph &G, V v, cudaStream_t s) {
