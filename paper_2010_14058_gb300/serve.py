@@ -33,9 +33,39 @@ import numpy as np
 from . import tg
 
 # device bytes a request needs while it is counted, per edge and per node
-# (handle arrays plus per-edge intermediates of the 4-node stage, L = 8 bound)
+# (handle arrays plus per-edge intermediates of the 4-node stage, L = 8 bound;
+# measured, graphs of average degree 10 take 0.24 to 0.92 of it)
 BYTES_PER_EDGE = 40 * 64 + 96
-BYTES_PER_NODE = 2 * 8 * 64 + 64
+BYTES_PER_NODE = 2 * 8 * 64 + 192
+DENSE = 16                                # edges per node from which handle_bytes is asked too: cliques of 100 to
+                                          # 1,500 nodes took 1.02 to 1.42 times the bytes above at L = 8
+CTAS = 320                                # at most two CTAs of the sums per SM
+
+
+def handle_bytes(deg: np.ndarray, m: int, L: int) -> int:
+    """Upper bound of a handle's device bytes after a 4-node count, from the degrees: the arrays per edge and node,
+    the tables of the hub anchors and the scratch of the lists of higher-priority neighbours.  All members of
+    such a list have at least its node's degree, so the longest has at most h entries, h the largest number such that
+    h nodes have degree h or more, and the d nodes of the highest degrees have lists of less than d."""
+    n, top = len(deg), int(deg.max(initial=0))
+    base = (32 * L * L + 160) * m + (16 * L * L + 192) * n
+    at_least = np.cumsum(np.bincount(deg, minlength=1)[::-1])[::-1]          # nodes of degree d or more
+    h = int((at_least >= np.arange(len(at_least))).sum()) - 1
+    over = lambda d: int(at_least[d + 1]) if d < top else 0                  # noqa: E731
+    # an anchor beyond shared memory has more than 9,000 wedges, which end at less than degree^2 places
+    hubs, row = over(94), 4 * ((L + 1) // 2 if top < 1 << 16 else L)
+    base += 3 * min(hubs * n * row, max(96 << 20, n * row)) + (16 + 16 * L) * min(2 * m, hubs * top)
+    scratch = 0
+    if h > 32:                            # 8 bytes per pair of a list's capacity and CTA
+        scratch = min(over(32) - 32, 8 * CTAS) * 4 * 128 * 127
+    if h > 128:
+        cap = min(h + 31, 704)
+        scratch = max(scratch, min(over(128) - 128, CTAS) * 4 * cap * cap)
+    if h > 704:                           # the lists' arrays in global memory: of the sums and of the triangles
+        arrays = h * (32 + 4 * L) + (1 << 20)
+        scratch = max(scratch, min((over(704) - 704) * (h * (h // 8 + 60 + 8 * L) + arrays), 4 << 30))
+        scratch += min(over(704) - 704, CTAS // 2) * arrays
+    return base + scratch
 
 
 @dataclass
@@ -47,6 +77,7 @@ class Request:
     types: np.ndarray
     arrival: float = 0.0                  # seconds after the start of the run
     key: object = None                    # identity of the graph (None: never kept resident)
+    _bytes: int = 0                       # bytes_needed, worked out once
 
     @property
     def n(self) -> int:
@@ -57,7 +88,11 @@ class Request:
         return int(self.col.shape[0]) // 2
 
     def bytes_needed(self) -> int:
-        return BYTES_PER_EDGE * self.m + BYTES_PER_NODE * self.n + (1 << 20)
+        if not self._bytes:
+            self._bytes = (1 << 20) + BYTES_PER_EDGE * self.m + BYTES_PER_NODE * self.n
+            if self.m >= DENSE * self.n:
+                self._bytes = max(self._bytes, (1 << 20) + handle_bytes(np.diff(self.row_ptr), self.m, self.L))
+        return self._bytes
 
 
 @dataclass
