@@ -369,9 +369,6 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
     G.opt = opt;
     TG_CK(cudaGetDevice(&G.device));
     G.h_node_off.assign(node_off_host, node_off_host + ngraphs + 1);
-    G.max_graph_nodes = 0;
-    for (int g = 0; g < ngraphs; ++g)
-        G.max_graph_nodes = std::max(G.max_graph_nodes, G.h_node_off[g + 1] - G.h_node_off[g]);
 
     G.status.alloc(sizeof(uint32_t));
     TG_CK(cudaMemsetAsync(G.status.p, 0, sizeof(uint32_t), s));
@@ -496,8 +493,6 @@ void build_graph(Graph &G, int32_t ngraphs, const int64_t *node_off_host, int64_
         G.max_degree = std::max(G.max_degree, h_info[(size_t)ngraphs + 1 + g]);
     }
     if (G.h_edge_off[ngraphs] != m) throw Error{TG_ERR_INVALID_GRAPH, "edge count per graph"};
-    G.edge_off.alloc(sizeof(int64_t) * (ngraphs + 1));
-    TG_CK(cudaMemcpyAsync(G.edge_off.p, G.h_edge_off.data(), sizeof(int64_t) * (ngraphs + 1), cudaMemcpyHostToDevice, s));
 
     // 4. higher-priority neighbour lists (one entry per edge), and the edges in caller order
     G.slot_eid.alloc(sizeof(int32_t) * std::max<int64_t>(nnz, 1));

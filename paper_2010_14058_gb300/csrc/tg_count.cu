@@ -37,12 +37,8 @@
 // with v, w, x all of lower priority; the wedge work is
 // sum_{(u,v) in E} min(d_u, d_v).
 #include <algorithm>
-#include <vector>
-
-#include <cub/device/device_scan.cuh>
-
-#include <memory>
 #include <mutex>
+#include <vector>
 
 #include "tg_host.hpp"
 #include "tg_side.hpp"

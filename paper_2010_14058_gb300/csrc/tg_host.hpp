@@ -5,7 +5,6 @@
 #include <cstdio>
 #include <cstring>
 #include <memory>
-#include <string>
 #include <type_traits>
 #include <utility>
 #include <vector>
@@ -149,7 +148,6 @@ struct Graph : OwnerStream {
     int device = 0;
     int32_t ngraphs = 1, L = 1;
     int64_t n = 0, nnz = 0, m = 0;
-    int64_t max_graph_nodes = 0;
     int64_t max_degree = 0;
     bool narrow = false;                                     // kNarrowDegree (tg_internal.cuh)
     std::vector<int64_t> h_node_off, h_edge_off, h_slot_off;
@@ -160,7 +158,7 @@ struct Graph : OwnerStream {
     tg_options opt;
 
     // graph (built once)
-    DBuf node_off, edge_off, rp, adj, toff, tdeg, pivot, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
+    DBuf node_off, rp, adj, toff, tdeg, pivot, ty, old_of, slot_eid, e_lo, e_hi, e_slot_lo, e_slot_hi, delta;
     DBuf most_lower;                            // most lower-priority neighbours of one type, until prepare_anchors
     DBuf plus_off, plus_adj, plus_eid;
     // nodes by |N+| (tg_local.cuh): mid, big, and larger than shared memory
@@ -231,7 +229,6 @@ struct Graph : OwnerStream {
         GraphView v;
         v.ngraphs = ngraphs; v.L = L; v.n = n; v.nnz = nnz; v.m = m;
         v.node_off = node_off.as<int64_t>();
-        v.edge_off = edge_off.as<int64_t>();
         v.rp = rp.as<int64_t>();
         v.adj = adj.as<int32_t>();
         v.toff = toff.as<int32_t>();
@@ -275,7 +272,7 @@ struct Graph : OwnerStream {
         return v;
     }
     std::vector<const DBuf *> cbuffers() const {
-        return {&node_off, &edge_off, &rp, &adj, &toff, &tdeg, &pivot, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
+        return {&node_off, &rp, &adj, &toff, &tdeg, &pivot, &ty, &old_of, &slot_eid, &e_lo, &e_hi,
                              &e_slot_lo, &e_slot_hi, &delta, &most_lower, &anchors[0], &anchors[1], &anchors[2], &anchors[3], &anchors[4],
                              &anchor_wedges, &C, &tau, &A, &gacc, &status, &tiles_full, &stage_pe,
                              &stage_gl, &xsum, &tri_any, &slot_rows, &work, &hub_tables, &dlab, &doutdeg, &dcls, &darcs, &dgacc, &dcell, &etype, &etdeg, &etgacc, &etcell, &plus_off, &plus_adj, &plus_eid, &tri_list[0], &tri_list[1], &tri_list[2], &tri_scratch, &sum_scratch, &hubs, &hub_base, &hub_nlow, &hub_piece,

@@ -80,7 +80,6 @@ struct GraphView {
     int32_t L;
     int64_t n, nnz, m;
     const int64_t *node_off;   // [ngraphs+1] internal node id ranges per graph
-    const int64_t *edge_off;   // [ngraphs+1] edge id ranges per graph
     const int64_t *rp;         // [n+1]
     const int32_t *adj;        // [nnz] internal ids, rows sorted by (type, id)
     const int32_t *toff;       // [n*(L+1)] type segment starts, relative to rp[x]
@@ -182,15 +181,6 @@ __device__ __forceinline__ int graph_of_node(const GraphView &g, int64_t x) {
     while (hi - lo > 1) {
         int mid = (lo + hi) >> 1;
         if (g.node_off[mid] <= x) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ int graph_of_edge(const GraphView &g, int64_t e) {
-    int lo = 0, hi = g.ngraphs;
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (g.edge_off[mid] <= e) lo = mid; else hi = mid;
     }
     return lo;
 }
