@@ -287,43 +287,48 @@ def clique_units(pe, L: int, big_t: int = 256, chunk: int = 1 << 22) -> dict:
     return out
 
 
-def algorithmic_bytes(u: dict, m: int, L: int, S: int, t_nodes: int) -> dict:
+def algorithmic_bytes(u: dict, n: int, m: int, L: int, S: int, tri_rows: int) -> dict:
     """Bytes each count kernel must move at least once in this formulation
-    (reads of its inputs and writes of its outputs, intermediates included),
-    per launch over the whole graph:
+    (every element of its inputs read once, however often L2 serves it again,
+    and every element of its outputs written once), per launch over the whole
+    graph; tri_rows: (edge, type) pairs with a triangle, whose rows of sums are
+    kept.
       k_tri       per edge: its entry of the N+ lists read 8 (id, edge id);
-                  its row of typed triangle counts zeroed and read or
-                  written 64; per triangle three counts read and written 24
-                  (the scan of the lists, which L2 serves, is not counted);
-      k_sum       per triangle three rows of triangle counts read 96, per
-                  triangle node of an edge its typed sums read and written
-                  24L; k_sum_zero clears 16L^2 per edge that has triangles;
+                  its row of typed triangle counts zeroed and written 64;
+      k_sum_zero  per edge its row of triangle counts read 32, per kept row
+                  16L written;
+      k_sum       per edge its entry of the N+ lists 8 and row of triangle
+                  counts 32, per node its typed degrees 32, per kept row its
+                  sums read and written 32L;
+      k_slot_rows per adjacency slot L^2 values read and written 8L^2;
+      k_epi4      per edge: endpoints and slots 24, its row of triangle counts
+                  32, two rows of 4-cycle values 8L^2, its output row 4S; per
+                  node its type offsets 4(L+1), delta and tau 8L^2 (32-bit);
+                  per kept row its sums 16L.
+    Of the wedge kernels, whose updates scatter over more than L2 holds, the
+    accesses instead:
       k_wedge_light, k_wedge_64 to k_wedge_1024 (one line, k_wedge_shared):
                   per wedge the far node's id 4 + its 4-cycle slot 4 read +
                   4 written; per (anchor, neighbour) pair: L slots 8 B each;
       k_wedge_hub when the library's work counters give them: per hub wedge
                   its far node's id 4, per nonzero 4-cycle slot update (a
                   wedge and a type of the fourth node, or a (hub, neighbour,
-                  type) sum) the slot read and written 8;
-      k_slot_rows per adjacency slot L^2 values read and written 8L^2;
-      k_epi4      per edge: endpoints and slots 24, C row 32, two type
-                  offset rows 8(L+1), two rows of 4-cycle values 8L^2, delta
-                  and tau of both endpoints 16L^2 (32-bit), its output row
-                  4S; per triangle node of an edge its sums 16L."""
+                  type) sum) the slot read and written 8."""
     LL = L * L
     return {
-        "k_tri": 72.0 * m + 8.0 * t_nodes,
-        "k_sum": (32.0 + 24.0 * L) * t_nodes,
+        "k_tri": 72.0 * m,
+        "k_sum_zero": 32.0 * m + 16.0 * L * tri_rows,
+        "k_sum": 40.0 * m + 32.0 * n + 32.0 * L * tri_rows,
         "k_wedge_shared": 12.0 * (u["wedges_light"] + u["wedges_heavy"]) + 8.0 * L * (u["pairs_light"] + u["pairs_heavy"]),
         "k_wedge_hub": 4.0 * u["hub_wedges_counted"] + 8.0 * u["hub_slot_updates"] if "hub_slot_updates" in u else
         12.0 * u["wedges_hub"] + 8.0 * L * u["pairs_hub"],
         "k_slot_rows": 16.0 * LL * m,
-        "k_epi4": (24.0 + 32 + 8 * (L + 1) + 24 * LL + 4 * S) * m + 16.0 * L * t_nodes,
+        "k_epi4": (24.0 + 32 + 8 * LL + 4 * S) * m + (4.0 * (L + 1) + 8 * LL) * n + 16.0 * L * tri_rows,
     }
 
 
 def count_only(m: int, count_ms: float, step_ms: float) -> dict | None:
-    """Edges per second of tg_count alone (its kernels' CUDA-event time per
+    """Edges per second of tg_count alone (CUDA events around the call, per
     step) and the rest of the step (tg_build, tg_free) in milliseconds."""
     if count_ms <= 0:
         return None
@@ -367,28 +372,59 @@ def run_ours(args):
         if dist is not None:
             dist.barrier()
 
-    kernel_ms = {}
+    kernel_ms, count_ms_sum = {}, [0.0]
+    ksteps = min(args.steps, 5)
     launches = [0]
 
-    def step(timing: bool):
-        h = tg.tg_build(rp, col, ty, L, stream=stream)
+    def one(build, count, kernels=None, events=None):
+        """build, count, status, free; `kernels`: with the library's per-kernel timing, which runs the kernels one
+        after another; `events`: recorded around the count."""
+        h = build()
         launches[0] += h.last_launch_count
-        if timing:
+        if kernels is not None:
             tg.tg_set_timing(h, True)
-        tg.tg_count(h, 4, pe, gl, stream=stream)
+        if events:
+            events[0].record(stream)
+        count(h)
+        if events:
+            events[1].record(stream)
         launches[0] += h.last_launch_count
-        if timing:
+        if kernels is not None:
             for name, (ms, n) in tg.tg_get_timing(h).items():
-                a = kernel_ms.setdefault(name, [0.0, 0])
+                a = kernels.setdefault(name, [0.0, 0])
                 a[0] += ms
                 a[1] += n
-        st = tg.tg_query_status(h) if timing else 0
+        st = tg.tg_query_status(h)
+        if events:
+            count_ms_sum[0] += events[0].elapsed_time(events[1])
         h.free()
         return st
 
+    def timed_steps(build, count, kernels):
+        """Milliseconds of args.steps steps after the warm-up, and their status; then, untimed, the kernels' times."""
+        for _ in range(args.warmup):
+            one(build, count)
+        torch.cuda.synchronize()
+        a = torch.cuda.Event(enable_timing=True)
+        b = torch.cuda.Event(enable_timing=True)
+        a.record(stream)
+        st = 0
+        for _ in range(args.steps):
+            st = one(build, count) or st
+        b.record(stream)
+        torch.cuda.synchronize()
+        for _ in range(ksteps):
+            st = one(build, count, kernels=kernels) or st
+        return a.elapsed_time(b), st
+
+    def step(kernels=None, events=None):
+        return one(lambda: tg.tg_build(rp, col, ty, L, stream=stream),
+                   lambda h: tg.tg_count(h, 4, pe, gl, stream=stream), kernels, events)
+
     for _ in range(args.warmup):
-        step(False)
+        step()
     status = 0
+    count_ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
     # timed region
     clocks = ClockSampler(torch.cuda.current_device())
     barrier()
@@ -399,11 +435,12 @@ def run_ours(args):
     launches[0] = 0
     t0.record(stream)
     for _ in range(args.steps):
-        st = step(True)
+        st = step(events=count_ev)
         status = status or st
     t1.record(stream)
     torch.cuda.synchronize()
     barrier()
+    n_launches = launches[0]
     clk = clocks.stop()
     ms = t0.elapsed_time(t1)
     ms_t = torch.tensor([ms], dtype=torch.float64, device=dev)
@@ -491,10 +528,13 @@ def run_ours(args):
 
 
     # roofline: algorithmic bytes of each count kernel per step over its
-    # CUDA-event time per step
+    # CUDA-event time per step (untimed steps of their own: per-kernel timing
+    # runs the kernels one after another)
     peak, peak_kind = load_peaks()
     roofline, per_kernel, compulsory, count_alone, walg, work = None, {}, None, None, None, None
     if rank == 0:
+        for _ in range(ksteps):
+            status = step(kernels=kernel_ms) or status
         # the hub wedges and 4-clique words of one count, from the library's work counters
         # (one extra, untimed count)
         h = tg.tg_build(rp, col, ty, L, stream=stream)
@@ -502,15 +542,13 @@ def run_ours(args):
         tg.tg_count(h, 4, pe, gl, stream=stream)
         work = tg.tg_get_work(h)
         h.free()
-        gl_host = gl.cpu().numpy()
-        b2 = lay["global_block_offset"][2]
-        t_nodes = 3 * int(gl_host[b2:b2 + lay["global_block_size"][2]].sum())   # sum_e |T_e|
         cu = clique_units(pe, L)
         units.update({"clique": cu})
         if work.get("hub_wedges"):
             units.update({"hub_wedges_counted": float(work["hub_wedges"]),
                           "hub_slot_updates": float(work["hub_slot_updates"])})
-        abytes = algorithmic_bytes(units, m, L, S, t_nodes)
+        tri_rows = sum(int((pe[a:a + (1 << 22), L:2 * L] != 0).sum()) for a in range(0, m, 1 << 22))
+        abytes = algorithmic_bytes(units, g["n"], m, L, S, tri_rows)
         # the shared-memory wedge forms share one bound
         forms = [v for k, v in kernel_ms.items() if k.startswith("k_wedge_") and k != "k_wedge_hub"]
         timed = {k: v for k, v in kernel_ms.items() if v not in forms}
@@ -519,9 +557,9 @@ def run_ours(args):
         for name, (kms, nl) in timed.items():
             if abytes.get(name) is None or kms <= 0:
                 continue
-            step_ms = kms / args.steps
+            step_ms = kms / ksteps
             gbs = abytes[name] / (step_ms / 1e3) / 1e9
-            per_kernel[name] = {"ms_per_step": round(step_ms, 3), "launches_per_step": nl // args.steps,
+            per_kernel[name] = {"ms_per_step": round(step_ms, 3), "launches_per_step": nl // ksteps,
                                 "algorithmic_gb": round(abytes[name] / 1e9, 3), "achieved_gbs": round(gbs, 2),
                                 "frac": round(gbs / peak, 5)}
         top = max(timed.items(), key=lambda kv: kv[1][0])[0]
@@ -537,7 +575,7 @@ def run_ours(args):
         # compulsory traffic of the whole count: CSR and types read once,
         # outputs written once -- the headline "% of HBM roofline"
         cb = 8.0 * m + 8.0 * g["n"] + g["n"] + 4.0 * S * m + 8.0 * G
-        count_ms = sum(v[0] for v in kernel_ms.values()) / args.steps
+        count_ms = count_ms_sum[0] / args.steps
         compulsory = {"bound": "hbm", "bytes": cb, "count_ms": round(count_ms, 3), "peak": peak,
                       "peak_kind": peak_kind, "unit": "GB/s",
                       "achieved": round(cb / (count_ms / 1e3) / 1e9, 2),
@@ -558,36 +596,13 @@ def run_ours(args):
         pe_pa = torch.empty((m, lay_pa["per_edge_slots"]), dtype=torch.int32, device=dev)
         gl_pa = torch.empty(lay_pa["global_slots"], dtype=torch.int64, device=dev)
         pa_ms = {}
-
-        def pa_step(timing: bool):
-            h = tg.tg_build(rp, col, ty, L, stream=stream)
-            if timing:
-                tg.tg_set_timing(h, True)
-            tg.tg_count_position_aware(h, pe_pa, gl_pa, stream=stream)
-            if timing:
-                for name, (kms, n) in tg.tg_get_timing(h).items():
-                    pa_ms[name] = pa_ms.get(name, 0.0) + kms
-            st = tg.tg_query_status(h) if timing else 0
-            h.free()
-            return st
-
-        for _ in range(args.warmup):
-            pa_step(False)
-        torch.cuda.synchronize()
-        a0 = torch.cuda.Event(enable_timing=True)
-        a1 = torch.cuda.Event(enable_timing=True)
-        a0.record(stream)
-        pa_status = 0
-        for _ in range(args.steps):
-            pa_status = pa_status or pa_step(True)
-        a1.record(stream)
-        torch.cuda.synchronize()
-        pms = a0.elapsed_time(a1)
+        pms, pa_status = timed_steps(lambda: tg.tg_build(rp, col, ty, L, stream=stream),
+                                     lambda h: tg.tg_count_position_aware(h, pe_pa, gl_pa, stream=stream), pa_ms)
         position_aware = {"value": round(m * args.steps / (pms / 1e3), 1), "unit": UNIT,
                           "ms_per_step": round(pms / args.steps, 3), "status": tg.STATUS[pa_status],
                           "per_edge_slots": lay_pa["per_edge_slots"], "global_slots": lay_pa["global_slots"],
-                          "k_epi4_pa_ms_per_step": round(pa_ms.get("k_epi4_pa", 0.0) / args.steps, 3),
-                          "k_epi4_ms_per_step": round(kernel_ms.get("k_epi4", [0.0])[0] / args.steps, 3),
+                          "k_epi4_pa_ms_per_step": round(pa_ms.get("k_epi4_pa", [0.0])[0] / ksteps, 3),
+                          "k_epi4_ms_per_step": round(kernel_ms.get("k_epi4", [0.0])[0] / ksteps, 3),
                           "step": "tg_build + tg_count_position_aware + tg_free, device-resident"}
 
     # directed typed 3-node counts (Sec. 4.8) of the same edges, each oriented
@@ -606,35 +621,12 @@ def run_ours(args):
         pe_d = torch.empty((m, lay_d["per_edge_slots"]), dtype=torch.int32, device=dev)
         gl_d = torch.empty(lay_d["global_slots"], dtype=torch.int64, device=dev)
         d_ms = {}
-
-        def d_step(timing: bool):
-            h = tg.tg_build_directed(d_rp, d_col, ty, L, stream=stream)
-            if timing:
-                tg.tg_set_timing(h, True)
-            tg.tg_count_directed3(h, pe_d, gl_d, stream=stream)
-            if timing:
-                for name, (kms, nl) in tg.tg_get_timing(h).items():
-                    d_ms[name] = d_ms.get(name, 0.0) + kms
-            st = tg.tg_query_status(h) if timing else 0
-            h.free()
-            return st
-
-        for _ in range(args.warmup):
-            d_step(False)
-        torch.cuda.synchronize()
-        b0 = torch.cuda.Event(enable_timing=True)
-        b1 = torch.cuda.Event(enable_timing=True)
-        b0.record(stream)
-        d_status = 0
-        for _ in range(args.steps):
-            d_status = d_status or d_step(True)
-        b1.record(stream)
-        torch.cuda.synchronize()
-        dms = b0.elapsed_time(b1)
+        dms, d_status = timed_steps(lambda: tg.tg_build_directed(d_rp, d_col, ty, L, stream=stream),
+                                    lambda h: tg.tg_count_directed3(h, pe_d, gl_d, stream=stream), d_ms)
         directed = {"value": round(m * args.steps / (dms / 1e3), 1), "unit": UNIT,
                     "ms_per_step": round(dms / args.steps, 3), "status": tg.STATUS[d_status],
                     "per_edge_slots": lay_d["per_edge_slots"], "global_slots": lay_d["global_slots"],
-                    "kernels_ms_per_step": {k: round(v / args.steps, 3) for k, v in d_ms.items()},
+                    "kernels_ms_per_step": {k: round(v[0] / ksteps, 3) for k, v in d_ms.items()},
                     "step": "tg_build_directed + tg_count_directed3 + tg_free, device-resident; each edge of the "
                             "workload oriented by a seeded coin"}
 
@@ -648,35 +640,12 @@ def run_ours(args):
         pe_x = torch.empty((m, lay_x["per_edge_slots"]), dtype=torch.int32, device=dev)
         gl_x = torch.empty(lay_x["global_slots"], dtype=torch.int64, device=dev)
         x_ms = {}
-
-        def x_step(timing: bool):
-            h = tg.tg_build_edge_typed(rp, col, ty, xi, L, X, stream=stream)
-            if timing:
-                tg.tg_set_timing(h, True)
-            tg.tg_count_edge_typed3(h, pe_x, gl_x, stream=stream)
-            if timing:
-                for name, (kms, nl) in tg.tg_get_timing(h).items():
-                    x_ms[name] = x_ms.get(name, 0.0) + kms
-            st = tg.tg_query_status(h) if timing else 0
-            h.free()
-            return st
-
-        for _ in range(args.warmup):
-            x_step(False)
-        torch.cuda.synchronize()
-        b0 = torch.cuda.Event(enable_timing=True)
-        b1 = torch.cuda.Event(enable_timing=True)
-        b0.record(stream)
-        x_status = 0
-        for _ in range(args.steps):
-            x_status = x_status or x_step(True)
-        b1.record(stream)
-        torch.cuda.synchronize()
-        xms = b0.elapsed_time(b1)
+        xms, x_status = timed_steps(lambda: tg.tg_build_edge_typed(rp, col, ty, xi, L, X, stream=stream),
+                                    lambda h: tg.tg_count_edge_typed3(h, pe_x, gl_x, stream=stream), x_ms)
         edge_typed = {"value": round(m * args.steps / (xms / 1e3), 1), "unit": UNIT,
                       "ms_per_step": round(xms / args.steps, 3), "status": tg.STATUS[x_status], "edge_types": X,
                       "per_edge_slots": lay_x["per_edge_slots"], "global_slots": lay_x["global_slots"],
-                      "kernels_ms_per_step": {k: round(v / args.steps, 3) for k, v in x_ms.items()},
+                      "kernels_ms_per_step": {k: round(v[0] / ksteps, 3) for k, v in x_ms.items()},
                       "step": "tg_build_edge_typed + tg_count_edge_typed3 + tg_free, device-resident; each edge "
                               "of the workload typed by a seeded hash"}
 
@@ -698,7 +667,7 @@ def run_ours(args):
             "count_only": count_alone, "kernel_share": kernel_share,
             "units": units,
             "cpu_baseline": cpu, "e2e": e2e, "e2e_sparse": e2e_sparse, "clocks": clk,
-            "gpu_launches": int(launches[0]),
+            "gpu_launches": int(n_launches),
         }
         if position_aware is not None:
             line["position_aware"] = position_aware
