@@ -672,6 +672,10 @@ tg_status tg_query_status(tg_graph *gh) {
         TG_CK(cudaStreamSynchronize(G.stream));
         TG_CK(cudaMemcpy(&v, G.status.p, sizeof(uint32_t), cudaMemcpyDeviceToHost));
         TG_CK(cudaMemset(G.status.p, 0, sizeof(uint32_t)));
+        if ((v & tg::ST_TIMEOUT) && G.hub_tables.p) {       // skipped tickets leave counters in the hub tables
+            TG_CK(cudaMemsetAsync(G.hub_tables.p, 0, G.hub_tables.bytes, G.stream));
+            TG_CK(cudaStreamSynchronize(G.stream));
+        }
     });
     if (st != TG_OK) return st;
     if (v & tg::ST_INVALID_GRAPH) return TG_ERR_INVALID_GRAPH;
