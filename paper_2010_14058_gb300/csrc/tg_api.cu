@@ -573,16 +573,19 @@ tg_status tg_count_batch(tg_graph *gh, int32_t k, uint32_t *per_edge_out, int64_
             TG_CK(cudaStreamSynchronize(s));
             cudaGraph_t graph = nullptr;
             TG_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+            G.captured = true;
             int64_t launches = 0;
             try {
                 TG_CK(cudaMemsetAsync(G.gacc.p, 0, (size_t)G.ngraphs * tg::global_slots(G.L, 4) * sizeof(unsigned long long), s));
                 launches += tg::run_count(G, k, 0, G.m, per_edge_out, G.gacc.as<unsigned long long>(), true, s);
                 if (global_out) launches += tg::launch_finalize(G, k, global_out, s);
             } catch (...) {
+                G.captured = false;
                 tg::forget(cudaStreamEndCapture(s, &graph));
                 if (graph) tg::forget(cudaGraphDestroy(graph));
                 throw;
             }
+            G.captured = false;
             TG_CK(cudaStreamEndCapture(s, &graph));
             cudaGraphExec_t exec = nullptr;
             cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);

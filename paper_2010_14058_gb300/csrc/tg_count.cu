@@ -162,12 +162,7 @@ static int64_t launch_chunk(Graph &G, size_t ci, bool triangles, cudaStream_t s)
     if (c.s1 > c.s0)
         TG_CK(cudaMemset2DAsync(G.A.p, (size_t)G.a_stride * sizeof(uint32_t), 0, (size_t)(c.s1 - c.s0) * sizeof(uint32_t),
                                 (size_t)L * L, s));
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
-        (void)cudaGetLastError();                            // (a legacy stream while another thread captures)
-        capture = cudaStreamCaptureStatusActive;
-    }
-    if (G.timing || capture != cudaStreamCaptureStatusNone) {
+    if (G.timing || G.captured) {
         if (triangles) launches += launch_triangles(G, true, s);
         launches += launch_sums(G, c.n0, c.n1, c.e0, c.e1, s);
         if (G.n_hubs > 0) launches += launch_hubs(G, ci, s);

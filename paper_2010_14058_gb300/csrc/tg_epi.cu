@@ -17,9 +17,10 @@
 // they fit (a narrow graph, kNarrowDegree; 64 registers instead of 80, so a
 // fourth CTA per SM, and half the bytes of the nodes' tables) 7.9
 // and 7.3 ms, with the tile's edges staged (stage_ends) 6.6 and 6.2; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
-// Bound now: latency of the gathers at 32 warps per SM (each edge reads two
-// slot rows, its sums, and two nodes' tables) on top of the rows written
-// (12.8 GB, 1.9 ms at the measured copy rate).  Narrow with 3 or 5 CTAs'
+// Bound now: DRAM at 0.82 of the measured copy rate (36.5 GB on the 20 M
+// edges of the benchmark graph: 12.9 of rows written, 23.6 read, of which the
+// two nodes' tables of every edge, which do not stay in L2, are the most) at
+// 32 warps per SM.  Narrow with 3 or 5 CTAs'
 // registers: 51.8 and 53.6 ms per pass of the block model against 51.3
 // (before the staging).
 #include <algorithm>
