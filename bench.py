@@ -191,7 +191,8 @@ def load_peaks():
 # DRAM bytes (read + write) per launch of a kernel, from the ncu capture
 # summarised under profiles/ for that workload and the current kernel code
 # (an entry is removed when its kernel changes).
-TRAFFIC = {}
+TRAFFIC = {("cl_large", "k_wedge_hub"): 230.590e9, ("cl_large", "k_sum"): 52.625e9, ("cl_large", "k_epi4"): 36.473e9}
+
 
 def w_alg_bytes(g: dict, tsize, S: int) -> dict:
     """The algorithmic traffic model W_alg = sum_e [4(d_i + d_j) +

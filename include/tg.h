@@ -151,9 +151,8 @@ void tg_default_options(tg_options *opt);
  * its inputs when the stream reaches the end of the call.  On the device it
  * validates the graph, orders nodes by (degree, id), sorts every adjacency
  * list by (type, id) with per-type offsets (typed neighbourhoods Gamma_i^t
- * and typed degrees d_i^t), numbers the edges and precomputes per-node
- * typed degree sums.  opt may be NULL.  Synchronises `stream` once (to size
- * work lists).  Errors: TG_ERR_INVALID_ARG, TG_ERR_TOO_MANY_TYPES,
+ * and typed degrees d_i^t) and numbers the edges.  opt may be NULL.
+ * Synchronises `stream` (to validate and to size arrays).  Errors: TG_ERR_INVALID_ARG, TG_ERR_TOO_MANY_TYPES,
  * TG_ERR_INVALID_GRAPH, TG_ERR_OOM, TG_ERR_TOO_LARGE, TG_ERR_CUDA; on error
  * *out is NULL. */
 tg_status tg_build(int64_t n, int64_t nnz, const int64_t *row_ptr, const int32_t *col,
@@ -195,7 +194,10 @@ tg_status tg_edge_offsets(const tg_graph *g, int64_t *out);
  *          Table 3) and the six typed 4-node graphlets (Sec. 4.4).
  * per_edge_out: uint32 [m][S(L)] or NULL (global totals only).
  * global_out:   int64 [ngraphs][G(L)] or NULL.
- * Working memory is allocated on the first call and kept by the handle.
+ * Working memory is allocated on the first call and kept by the handle; the
+ * first call with k = 4 also makes what only 4-node counts need (per-node
+ * typed degree sums, work lists) and synchronises `stream`.  Later calls
+ * with device outputs do not, and can be captured into a CUDA graph.
  * Errors: TG_ERR_INVALID_ARG, TG_ERR_OOM, TG_ERR_CUDA (device-detected
  * errors go to the status word). */
 tg_status tg_count(tg_graph *g, int32_t k, uint32_t *per_edge_out, int64_t *global_out,
@@ -363,6 +365,8 @@ int64_t tg_last_launch_count(const tg_graph *g);
 /* Per-kernel timing.  While enabled, every kernel that tg_count or
  * tg_count_range launches is bracketed by a CUDA event pair recorded on the
  * launching stream, and the elapsed times are accumulated per kernel name.
+ * The kernels of a count then run one after another on `stream`, so that
+ * each is timed by itself: a timed count takes longer than others.
  * (Not recorded inside tg_count_batch's captured graph.) */
 tg_status tg_set_timing(tg_graph *g, int32_t on);
 

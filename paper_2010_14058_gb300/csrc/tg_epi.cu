@@ -16,7 +16,8 @@
 // and 1.2 ms) 11.7 and 9.8 ms, and with 32-bit values and node sums where
 // they fit (a narrow graph, kNarrowDegree; 64 registers instead of 80, so a
 // fourth CTA per SM, and half the bytes of the nodes' tables) 7.9
-// and 7.3 ms, with the tile's edges staged (stage_ends) 6.6 and 6.2; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
+// and 7.3 ms, with the tile's edges staged (stage_ends) 6.6 and 6.2, with 32-bit
+// sums throughout 6.7 and 6.0; 3-node rows of 10 M edges 3.0 -> 0.56 ms.
 // Bound now: DRAM at 0.82 of the measured copy rate (36.5 GB on the 20 M
 // edges of the benchmark graph: 12.9 of rows written, 23.6 read, of which the
 // two nodes' tables of every edge, which do not stay in L2, are the most) at

@@ -29,7 +29,10 @@
 // What it took, on the block model: the new tables with a search and a lookup
 // per wedge and phase 54 ms; with the slot of every wedge kept (phase 1 reads
 // its counter at once, and a wedge that is alone at its end stops there) and
-// the runs followed instead of searched 26.5 ms.  Bound now: instructions of
+// the runs followed instead of searched 26.5 ms; compiled to 56 registers
+// since the insert is bounded 23.3 ms (six CTAs of 192 threads fit an SM, as
+// launched; five did at 64: 6.0 -> 3.4 ms; Chung-Lu edges 8.6, dense graphs
+// 7.3).  Bound now: instructions of
 // the inserts (probes diverge) and the barriers between an anchor's phases.
 #include <algorithm>
 
