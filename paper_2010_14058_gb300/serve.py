@@ -26,7 +26,7 @@ import queue
 import threading
 import time
 from collections import OrderedDict
-from dataclasses import dataclass
+from dataclasses import dataclass, field
 
 import numpy as np
 
@@ -77,7 +77,7 @@ class Request:
     types: np.ndarray
     arrival: float = 0.0                  # seconds after the start of the run
     key: object = None                    # identity of the graph (None: never kept resident)
-    _bytes: int = 0                       # bytes_needed, worked out once
+    _bytes: int = field(default=0, init=False, repr=False, compare=False)   # bytes_needed, worked out once
 
     @property
     def n(self) -> int:
